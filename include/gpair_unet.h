@@ -64,6 +64,11 @@ gpair_status gpair_pool2_bwd(const gpair_bf16* dout, int D, int H, int W, int C,
 gpair_status gpair_up2_fwd(const gpair_bf16* in, int D, int H, int W, int C, gpair_bf16* out, void* stream);
 gpair_status gpair_up2_bwd(const gpair_bf16* dout, int D, int H, int W, int C, gpair_bf16* din, void* stream);
 
+/* the two in one pass: out[v] = (a upsampled from (D, H, W) to (2D, 2H, 2W) (Ca channels), b[v] (Cb channels)),
+ * b and out on (2D, 2H, 2W) -- the decoder's upsampling and skip connection. */
+gpair_status gpair_up2_concat_fwd(const gpair_bf16* a, int D, int H, int W, int Ca, const gpair_bf16* b, int Cb,
+                                  gpair_bf16* out, void* stream);
+
 /* channel concatenation out[v] = (a[v] (Ca channels), b[v] (Cb channels)) over nv voxels, and split. */
 gpair_status gpair_concat_fwd(const gpair_bf16* a, int Ca, const gpair_bf16* b, int Cb, int64_t nv, gpair_bf16* out,
                               void* stream);

@@ -39,6 +39,7 @@ def _unet_lib():
         lib.gpair_pool2_bwd.argtypes = [P, i32, i32, i32, i32, P, P]
         lib.gpair_up2_fwd.argtypes = [P, i32, i32, i32, i32, P, P]
         lib.gpair_up2_bwd.argtypes = [P, i32, i32, i32, i32, P, P]
+        lib.gpair_up2_concat_fwd.argtypes = [P, i32, i32, i32, i32, P, i32, P, P]
         lib.gpair_concat_fwd.argtypes = [P, i32, P, i32, i64, P, P]
         lib.gpair_concat_bwd.argtypes = [P, i32, i32, i64, P, P, P]
         lib.gpair_add_bf16.argtypes = [P, P, P, i64, P]
@@ -117,6 +118,10 @@ def gpair_up2_fwd(x, dims, C, out):
 
 def gpair_up2_bwd(dout, dims, C, din):
     _ck("gpair_up2_bwd", _unet_lib().gpair_up2_bwd(_p(dout), *dims, C, _p(din), _s()))
+
+
+def gpair_up2_concat_fwd(a, dims, Ca, b, Cb, out):
+    _ck("gpair_up2_concat_fwd", _unet_lib().gpair_up2_concat_fwd(_p(a), *dims, Ca, _p(b), Cb, _p(out), _s()))
 
 
 def gpair_concat_fwd(a, Ca, b, Cb, nv, out):
@@ -228,19 +233,18 @@ class UNet3D:
         a["e3a"], a["e3b"] = bf16((nv[2], c3), self.dev), bf16((nv[2], c3), self.dev)
         a["p3"] = bf16((nv[3], c3), self.dev)
         a["b4a"], a["b4b"] = bf16((nv[3], c4), self.dev), bf16((nv[3], c4), self.dev)
-        a["u3"] = bf16((nv[2], c4), self.dev)
         a["k3"] = bf16((nv[2], c4 + c3), self.dev)
         a["d3a"], a["d3b"] = bf16((nv[2], c3), self.dev), bf16((nv[2], c3), self.dev)
-        a["u2"] = bf16((nv[1], c3), self.dev)
         a["k2"] = bf16((nv[1], c3 + c2), self.dev)
         a["d2a"], a["d2b"] = bf16((nv[1], c2), self.dev), bf16((nv[1], c2), self.dev)
-        a["u1"] = bf16((nv[0], c2), self.dev)
         a["k1"] = bf16((nv[0], c2 + c1), self.dev)
         a["d1a"], a["d1b"] = bf16((nv[0], c1), self.dev), bf16((nv[0], c1), self.dev)
         a["out"] = bf16((nv[0], COUT_PAD), self.dev)
         self.act = a
         # gradient buffers (same shapes); reused across steps
         self.grad = {k: torch.empty_like(v) for k, v in a.items() if k != "x"}
+        for q, c in ((0, c2), (1, c3), (2, c4)):      # the upsampled half of each concatenation
+            self.grad["u%d" % (q + 1)] = bf16((nv[q], c), self.dev)
         # pooled-path gradient of each encoder output before it is added to the skip gradient
         self.tmp = {0: bf16((nv[0], c1), self.dev), 1: bf16((nv[1], c2), self.dev), 2: bf16((nv[2], c3), self.dev)}
         self.loss = torch.zeros(1, dtype=torch.float64, device=self.dev)
@@ -268,16 +272,13 @@ class UNet3D:
         gpair_pool2_fwd(a["e3b"], L[2], c3, a["p3"])
         self._conv("b4a", a["p3"], L[3], a["b4a"])
         self._conv("b4b", a["b4a"], L[3], a["b4b"])
-        gpair_up2_fwd(a["b4b"], L[3], c4, a["u3"])
-        gpair_concat_fwd(a["u3"], c4, a["e3b"], c3, self.nv[2], a["k3"])
+        gpair_up2_concat_fwd(a["b4b"], L[3], c4, a["e3b"], c3, a["k3"])
         self._conv("d3a", a["k3"], L[2], a["d3a"])
         self._conv("d3b", a["d3a"], L[2], a["d3b"])
-        gpair_up2_fwd(a["d3b"], L[2], c3, a["u2"])
-        gpair_concat_fwd(a["u2"], c3, a["e2b"], c2, self.nv[1], a["k2"])
+        gpair_up2_concat_fwd(a["d3b"], L[2], c3, a["e2b"], c2, a["k2"])
         self._conv("d2a", a["k2"], L[1], a["d2a"])
         self._conv("d2b", a["d2a"], L[1], a["d2b"])
-        gpair_up2_fwd(a["d2b"], L[1], c2, a["u1"])
-        gpair_concat_fwd(a["u1"], c2, a["e1b"], c1, self.nv[0], a["k1"])
+        gpair_up2_concat_fwd(a["d2b"], L[1], c2, a["e1b"], c1, a["k1"])
         self._conv("d1a", a["k1"], L[0], a["d1a"])
         self._conv("d1b", a["d1a"], L[0], a["d1b"])
         self._conv("out", a["d1b"], L[0], a["out"])

@@ -142,6 +142,40 @@ def test_pool_up_concat_relu():
     unet.gpair_relu_bwd(xd, g)
     assert torch.equal(g.cpu(), (x.float() > 0).to(torch.bfloat16))
 
+def test_up2_concat_equals_its_two_passes():
+    """The fused upsampling and concatenation, and the 16-byte forms of pooling, packing and ReLU backward,
+    against torch, for channel counts that allow 16-byte accesses and for ones that do not."""
+    gen = torch.Generator().manual_seed(11)
+    for (D, H, W), ca, cb in (((1, 2, 3), 8, 16), ((2, 3, 5), 32, 8), ((3, 1, 2), 5, 3), ((2, 2, 70), 16, 16)):
+        a, nv = _bf((D * H * W, ca), gen), 8 * D * H * W
+        b = _bf((nv, cb), gen)
+        out = torch.empty((nv, ca + cb), dtype=torch.bfloat16, device="cuda")
+        unet.gpair_up2_concat_fwd(a.cuda(), (D, H, W), ca, b.cuda(), cb, out)
+        up = a.reshape(D, H, W, ca).repeat_interleave(2, 0).repeat_interleave(2, 1).repeat_interleave(2, 2)
+        ref = torch.cat([up.reshape(nv, ca), b], 1)
+        assert torch.equal(out.cpu(), ref)
+        cat = torch.empty_like(out)
+        unet.gpair_concat_fwd(up.reshape(nv, ca).contiguous().cuda(), ca, b.cuda(), cb, nv, cat)
+        assert torch.equal(cat.cpu(), ref)
+        p = torch.empty((D * H * W, ca + cb), dtype=torch.bfloat16, device="cuda")
+        unet.gpair_pool2_fwd(out, (2 * D, 2 * H, 2 * W), ca + cb, p)
+        c8 = ref.float().reshape(D, 2, H, 2, W, 2, ca + cb).permute(0, 2, 4, 1, 3, 5, 6).reshape(-1, 8, ca + cb)
+        acc = torch.zeros(c8.shape[0], ca + cb)
+        for q in range(8):
+            acc = acc + c8[:, q]
+        assert torch.equal(p.cpu(), (0.125 * acc).to(torch.bfloat16))
+        x = torch.randn(nv, generator=gen)
+        packed = torch.full((nv, ca + cb), 7.0, dtype=torch.bfloat16, device="cuda")
+        unet.gpair_pack_input(x.cuda(), 0.3, nv, ca + cb, packed)
+        want = torch.zeros(nv, ca + cb)
+        want[:, 0] = torch.tensor(0.3, dtype=torch.float32) * x
+        assert torch.equal(packed.cpu(), want.to(torch.bfloat16))
+        for off in (0, 1):                       # an unaligned view takes the element-wise form
+            act, g = out.reshape(-1)[off:], _bf((nv * (ca + cb) - off,), gen)
+            gd = torch.cat([torch.zeros(off, dtype=torch.bfloat16), g]).cuda()[off:]
+            unet.gpair_relu_bwd(act, gd)
+            assert torch.equal(gd.cpu(), torch.where(ref.reshape(-1)[off:].float() > 0, g, torch.zeros_like(g)))
+
 
 def test_unet_forward_backward_matches_fp64_reference():
     """The whole network against the FP64 reference that stores activations and gradients in BF16
