@@ -249,255 +249,203 @@ int device_sms() {
 // Frobenius sum, D_pq = D_qp); Neumann boundaries (neighbour indices clamped per axis); unit voxel
 // spacing; eps inside each square root.  Image x fastest.
 
-__device__ __forceinline__ int64_t vox(int ix, int iy, int iz, int nx, int ny) {
-    return ((int64_t)iz * ny + iy) * nx + ix;
-}
-
-// One fused pass marching along z.  A CTA owns a column of VM_TX x VM_TY voxels and a chunk of
-// VM_ZC planes.  Per step it stages one plane of x with two voxels of halo in x and y (neighbour
-// indices clamped per axis: the Neumann reading) into a ring of three planes, forms the weighted
-// fields of the previous plane on the column plus one voxel per side,
+// One fused pass marching along z.  A CTA covers 32 x VM_PY field positions, one thread each (a warp is
+// a row), of which the inner 30 x (VM_PY - 2) are the voxels it owns, and a chunk of planes.  Per step it
+// has one plane of x in shared memory (with one more voxel of halo, neighbour indices clamped per
+// axis: the Neumann reading); each thread reads its eight neighbours there once and keeps what the
+// stencils need of them for three planes in registers.  From planes z - 1, z, z + 1 it forms its
+// weighted fields at plane z,
 //   F_k = m_k (D_k x) / sqrt(sH + eps)  (k = xx, yy, zz, xy, xz, yz; m = 1, 1, 1, 2, 2, 2),
 //   F_{6+d} = beta (D_d x) / sqrt(sT + eps),
-// sH = sum_{p,q} (D_pq x)^2, sT = sum_d (D_d x)^2, into a ring of three field planes, and adds
-// lam (sum_k D_k^T F_k) to g on the plane before that.  (D^T F)[j] sums c F[i] over the stencil
-// entries (o, c) and every i whose clamped neighbour i + o is j: inside the volume i = j - o, and
-// on a face the clamp adds i = j.  Fields are zero outside the volume, so the gather over j - o
-// needs no masks and a face voxel adds only the terms that take j itself.  Only x and g cross
-// HBM; the fields stay in shared memory.  The value sum sqrt(sH + eps) + beta sqrt(sT + eps) over
-// the CTA's own voxels is compensated FP32 per thread and FP64 per CTA (partial[blockIdx.x]).
-constexpr int VM_TX = 32, VM_TY = 8, VM_ZC = 16;
-constexpr int VM_XW = VM_TX + 4, VM_XH = VM_TY + 4, VM_XN = VM_XW * VM_XH;   // staged x plane
-constexpr int VM_FW = VM_TX + 2, VM_FH = VM_TY + 2, VM_FN = VM_FW * VM_FH;   // field plane
-static_assert(VM_TX * VM_TY == RED_THREADS, "one thread per column position");
-struct VcrMarchSmem {
-    float x[3][VM_XN];
-    float F[3][9][VM_FN];
-};
+// sH = sum_{p,q} (D_pq x)^2, sT = sum_d (D_d x)^2, zero outside the volume, and hands the ones that
+// neighbours along y need on through shared memory, along x through warp shuffles.
+// The gradient sum_k D_k^T F_k is separable per axis: with S_o the clamped shift, (S_o^T F)[j] =
+// F[j - o], plus F[j] itself where j + o leaves the volume.  So along an axis, with lo / hi telling
+// whether j is its first / last node,
+//   (S_+ - S_-)^T F      = F[j-1] - F[j+1] + (hi - lo) F[j],
+//   (S_+ - 2 + S_-)^T F  = F[j-1] + F[j+1] + (hi + lo - 2) F[j],
+// exact on faces, edges and corners alike; the mixed fields take the first form along both axes.  The
+// z part of plane z goes to planes z - 1, z and z + 1: each thread carries the sums of two pending
+// planes.  Only x and g cross HBM.  Two sets of buffers: one barrier per plane.
+// What bounds it: shared-memory and shuffle issue, 25 accesses per position and plane, and the plane's
+// chain of loads, square roots and one barrier.  256 x 256 x 128: 109 us, where the form with nine field
+// planes in shared memory (72 accesses per voxel, two barriers a plane) took 214.  Rows per CTA x CTAs per
+// SM: 16 x 2 109 us, 16 x 3 (40 registers, spills) 125, 32 x 1 110, 8 x 4 118.
+// The value sum sqrt(sH + eps) + beta sqrt(sT + eps) over the CTA's own voxels is compensated FP32 per
+// thread and FP64 per CTA (partial[blockIdx.x]).
+constexpr int VM_PY = 16, VM_CTAS = 2;                 // field rows of a CTA, CTAs per SM
+constexpr int VM_THREADS = 32 * VM_PY;
+constexpr int VM_OX = 30, VM_OY = VM_PY - 2;           // voxels owned
+constexpr int VM_XW = 34, VM_XH = VM_PY + 2, VM_XN = VM_XW * VM_XH;   // staged x plane
+constexpr int VM_STAGE = (VM_XN + VM_THREADS - 1) / VM_THREADS;
 
-// Stencil entries of the nine operators: field k, neighbour offset, coefficient.
-struct VcrEntry {
-    signed char k, ox, oy, oz;
-    float c;
-};
-__constant__ VcrEntry c_vcr[27] = {
-    {0, 1, 0, 0, 1.f}, {0, 0, 0, 0, -2.f}, {0, -1, 0, 0, 1.f},
-    {1, 0, 1, 0, 1.f}, {1, 0, 0, 0, -2.f}, {1, 0, -1, 0, 1.f},
-    {2, 0, 0, 1, 1.f}, {2, 0, 0, 0, -2.f}, {2, 0, 0, -1, 1.f},
-    {3, 1, 1, 0, .25f}, {3, 1, -1, 0, -.25f}, {3, -1, 1, 0, -.25f}, {3, -1, -1, 0, .25f},
-    {4, 1, 0, 1, .25f}, {4, 1, 0, -1, -.25f}, {4, -1, 0, 1, -.25f}, {4, -1, 0, -1, .25f},
-    {5, 0, 1, 1, .25f}, {5, 0, 1, -1, -.25f}, {5, 0, -1, 1, -.25f}, {5, 0, -1, -1, .25f},
-    {6, 1, 0, 0, .5f}, {6, -1, 0, 0, -.5f},
-    {7, 0, 1, 0, .5f}, {7, 0, -1, 0, -.5f},
-    {8, 0, 0, 1, .5f}, {8, 0, 0, -1, -.5f},
-};
-
-// Extra terms of (sum_k D_k^T F_k)[j] for a voxel on an edge or corner of the volume.  Along one
-// axis the preimages of j under the clamped offset o are j - o (when inside) and j itself when
-// j + o falls outside; the gather over j - o with zero fields outside the volume already holds
-// the products of the first kind, so this adds every product that takes j itself along at least
-// one axis.  Fplane[d + 1] is the field plane at z = jz + d ([9][VM_FN] each).
-__device__ __noinline__ float vcr_fold_terms(const float* Fm, const float* F0, const float* Fp, int jx, int jy, int jz,
-                                             int nx, int ny, int nz, int X0, int Y0) {
-    const float* Fplane[3] = {Fm, F0, Fp};
-    float s = 0.f;
-    for (int e = 0; e < 27; ++e) {
-        const VcrEntry E = c_vcr[e];
-        const bool fx = jx + E.ox < 0 || jx + E.ox >= nx, fy = jy + E.oy < 0 || jy + E.oy >= ny,
-                   fz = jz + E.oz < 0 || jz + E.oz >= nz;
-        if (!(fx || fy || fz)) continue;
-        float sum = 0.f;
-        for (int m = 1; m < 8; ++m) {          // bit set: that axis takes j itself
-            if (((m & 1) && !fx) || ((m & 2) && !fy) || ((m & 4) && !fz)) continue;
-            const int px = (m & 1) ? jx : jx - E.ox, py = (m & 2) ? jy : jy - E.oy, pz = (m & 4) ? jz : jz - E.oz;
-            // an axis that shifts outside the volume reads a zero field: skip it
-            if (px < 0 || px >= nx || py < 0 || py >= ny || pz < 0 || pz >= nz) continue;
-            sum += Fplane[pz - jz + 1][E.k * VM_FN + (py - Y0 + 1) * VM_FW + (px - X0 + 1)];
-        }
-        s = fmaf(E.c, sum, s);
-    }
+__device__ __forceinline__ double block_sum_n(double v, double* red, int warps) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double s = 0.0;
+    if (threadIdx.x == 0)
+        for (int k = 0; k < warps; ++k) s += red[k];
     return s;
 }
 
 template <bool GRAD>
-__global__ void __launch_bounds__(RED_THREADS, 4)
+__global__ void __launch_bounds__(VM_THREADS, VM_CTAS)
 vcr_march_kernel(const float* __restrict__ x, int nx, int ny, int nz, float beta, float eps, float lam,
-                 float* __restrict__ g, double* __restrict__ partial, unsigned item_mul) {
-    extern __shared__ __align__(16) unsigned char vcr_smem[];
-    VcrMarchSmem& S = *reinterpret_cast<VcrMarchSmem*>(vcr_smem);
-    __shared__ double red[RED_THREADS / 32];
-    const int tx = threadIdx.x % VM_TX, ty = threadIdx.x / VM_TX;
-    const unsigned ncx = (nx + VM_TX - 1) / VM_TX, ncy = (ny + VM_TY - 1) / VM_TY, ncz = (nz + VM_ZC - 1) / VM_ZC;
-    const unsigned nitems = ncx * ncy * ncz;                  // < 2^31 (checked on the host)
-    // Item k of this CTA is (blockIdx.x + k gridDim.x) item_mul mod nitems, stepped by one add:
-    // item_mul is coprime to nitems, so every item is visited once, and the face columns, which
-    // carry extra terms, spread over the CTAs.
-    const unsigned step = (unsigned)(((unsigned long long)gridDim.x * item_mul) % nitems);
-    unsigned it = (unsigned)(((unsigned long long)blockIdx.x * item_mul) % nitems);
+                 float* __restrict__ g, double* __restrict__ partial, int zc, unsigned nitems) {
+    __shared__ float xs[2][VM_XN];
+    __shared__ float fs[GRAD ? 2 : 1][GRAD ? 4 : 1][GRAD ? VM_THREADS : 1];   // A, B, yz, xy rows (see below)
+    __shared__ double red[VM_PY];
+    const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
+    const unsigned ncx = (nx + VM_OX - 1) / VM_OX, ncy = (ny + VM_OY - 1) / VM_OY;
+    const int64_t plane = (int64_t)nx * ny;
     KahanF acc;    // this thread's own voxels; FP64 from the CTA sum on
-    constexpr int SY = VM_FW;
-    for (unsigned k = blockIdx.x; k < nitems; k += gridDim.x) {
+    for (unsigned it = blockIdx.x; it < nitems; it += gridDim.x) {
         const unsigned cx = it % ncx, rest = it / ncx;
-        const int X0 = (int)cx * VM_TX, Y0 = (int)(rest % ncy) * VM_TY, Z0 = (int)(rest / ncy) * VM_ZC;
-        const int Z1 = min(Z0 + VM_ZC, nz);
-        it += step;
-        if (it >= nitems) it -= nitems;
-        const int jx = X0 + tx, jy = Y0 + ty;
-        // this thread's staging entries q = threadIdx.x + u RED_THREADS of a plane, loaded one step
-        // ahead into registers so that the loads overlap the previous step's work
-        constexpr int VM_STAGE = (VM_XN + RED_THREADS - 1) / RED_THREADS;
+        const int X0 = (int)cx * VM_OX, Y0 = (int)(rest % ncy) * VM_OY, Z0 = (int)(rest / ncy) * zc;
+        const int Z1 = min(Z0 + zc, nz);
+        const int px = X0 - 1 + lane, py = Y0 - 1 + row;               // this thread's field position
+        const bool inside = px >= 0 && px < nx && py >= 0 && py < ny;
+        const bool own = inside && lane >= 1 && lane <= VM_OX && row >= 1 && row <= VM_OY;
+        const float hix = px == nx - 1 ? 1.f : 0.f, lox = px == 0 ? 1.f : 0.f;
+        const float hiy = py == ny - 1 ? 1.f : 0.f, loy = py == 0 ? 1.f : 0.f;
+        const float ex = hix - lox, ax = hix + lox - 2.f, ey = hiy - loy, ay = hiy + loy - 2.f;
+        // this thread's staging entries: offsets in a plane, the same for every plane of the item
+        int64_t off[VM_STAGE];
+#pragma unroll
+        for (int u = 0; u < VM_STAGE; ++u) {
+            const int q = threadIdx.x + u * VM_THREADS, a = q % VM_XW, b = q / VM_XW;
+            const int ix = min(max(X0 - 2 + a, 0), nx - 1), iy = min(max(Y0 - 2 + b, 0), ny - 1);
+            off[u] = q < VM_XN ? (int64_t)iy * nx + ix : -1;
+        }
         float pre[VM_STAGE];
         auto load_plane = [&](int zi) {
-            const int zc = min(max(zi, 0), nz - 1);
-            const float* xp = x + (int64_t)zc * ny * nx;
+            const float* xp = x + (int64_t)min(max(zi, 0), nz - 1) * plane;
 #pragma unroll
-            for (int u = 0; u < VM_STAGE; ++u) {
-                const int q = threadIdx.x + u * RED_THREADS;
-                const int a = q % VM_XW, b = q / VM_XW;
-                const int ix = min(max(X0 - 2 + a, 0), nx - 1), iy = min(max(Y0 - 2 + b, 0), ny - 1);
-                pre[u] = q < VM_XN ? __ldg(xp + (int64_t)iy * nx + ix) : 0.f;
-            }
+            for (int u = 0; u < VM_STAGE; ++u) pre[u] = off[u] >= 0 ? __ldg(xp + off[u]) : 0.f;
         };
+        auto store_plane = [&](int s) {
+#pragma unroll
+            for (int u = 0; u < VM_STAGE; ++u)
+                if (off[u] >= 0) xs[s & 1][threadIdx.x + u * VM_THREADS] = pre[u];
+        };
+        // Step s reads x plane Z0 - 2 + s, forms the fields of plane zf = Z0 - 3 + s (s >= 2) and finishes
+        // the gradient of plane zf - 1 (s >= 4); x plane s + 1 is stored and plane s + 2 loaded meanwhile.
         load_plane(Z0 - 2);
-        // step s stages x plane Z0 - 2 + s, forms the fields of plane Z0 - 3 + s (s >= 2) and the
-        // gradient of plane Z0 - 4 + s (s >= 4)
+        __syncthreads();                 // the previous item's readers are done
+        store_plane(0);
+        load_plane(Z0 - 1);
+        __syncthreads();
+        // of x: the centre and the x and y differences of the last three planes, and the in-plane second
+        // differences of the last two
+        float c0 = 0.f, cm = 0.f, dx0 = 0.f, dxm = 0.f, dy0 = 0.f, dym = 0.f, hxx0 = 0.f, hyy0 = 0.f, hxy0 = 0.f;
+        float hold = 0.f, zplus = 0.f;   // gradient of plane zf - 1 without its part from zf; part of zf - 1 for zf
         for (int s = 0; Z0 - 4 + s < Z1; ++s) {
-            const int zi = Z0 - 2 + s;
-            __syncthreads();   // the readers of the slots overwritten below are done
-            {
-                float* xs = S.x[s % 3];
-#pragma unroll
-                for (int u = 0; u < VM_STAGE; ++u) {
-                    const int q = threadIdx.x + u * RED_THREADS;
-                    if (q < VM_XN) xs[q] = pre[u];
+            const float* xp = &xs[s & 1][(row + 1) * VM_XW + lane + 1];
+            const float cp = xp[0];
+            const float xr = xp[1], xl = xp[-1], yr = xp[VM_XW], yl = xp[-VM_XW];
+            const float dxp = xr - xl, dyp = yr - yl;
+            const float hxxp = (xr - cp) + (xl - cp), hyyp = (yr - cp) + (yl - cp);
+            const float hxyp = 0.25f * ((xp[VM_XW + 1] - xp[1 - VM_XW]) - (xp[VM_XW - 1] - xp[-VM_XW - 1]));
+            if (s + 1 < Z1 - Z0 + 4) store_plane(s + 1);
+            if (s + 2 < Z1 - Z0 + 4) load_plane(Z0 + s);
+            const int zf = Z0 - 3 + s;
+            float fzz = 0.f, fz = 0.f, fxz = 0.f, fyz = 0.f, fxy = 0.f, fxx = 0.f, fx = 0.f, fyy = 0.f, fy = 0.f;
+            if (s >= 2 && inside && zf >= 0 && zf < nz) {
+                const float hzz = (cp - c0) + (cm - c0), d1z = 0.5f * (cp - cm);
+                const float hxz = 0.25f * (dxp - dxm), hyz = 0.25f * (dyp - dym);
+                const float d1x = 0.5f * dx0, d1y = 0.5f * dy0;
+                const float sH = hxx0 * hxx0 + hyy0 * hyy0 + hzz * hzz + 2.f * (hxy0 * hxy0 + hxz * hxz + hyz * hyz) + eps;
+                const float sT = d1x * d1x + d1y * d1y + d1z * d1z + eps;
+                if (GRAD) {
+                    const float wH = rsqrtf(sH), wT = 0.5f * beta * rsqrtf(sT);
+                    fxx = wH * hxx0; fyy = wH * hyy0; fzz = wH * hzz;
+                    const float wM = 0.5f * wH;              // the factor 2 of the mixed fields and the 1/4 of their stencil
+                    fxy = wM * hxy0; fxz = wM * hxz; fyz = wM * hyz;
+                    fx = wT * d1x; fy = wT * d1y; fz = wT * d1z;     // with the 1/2 of their stencil
                 }
+                if (own && zf >= Z0 && zf < Z1) acc.add(sqrtf(sH) + beta * sqrtf(sT));
             }
-            if (Z0 - 4 + s + 1 < Z1) load_plane(zi + 1);
+            if constexpr (GRAD) {
+                float (*F)[VM_THREADS] = fs[s & 1];
+                F[0][threadIdx.x] = fyy + fy;                // A: what the row above adds
+                F[1][threadIdx.x] = fyy - fy;                // B: what the row below adds
+                F[2][threadIdx.x] = fyz;
+                F[3][threadIdx.x] = fxy;
+            }
             __syncthreads();
-            const int zf = zi - 1;
-            if (s >= 2) {
-                const float* xm = S.x[(s + 1) % 3];     // plane zf - 1
-                const float* x0 = S.x[(s + 2) % 3];     // plane zf
-                const float* xq = S.x[s % 3];           // plane zf + 1
-                float* Fz = &S.F[s % 3][0][0];
-                const bool zin = zf >= 0 && zf < nz;
-                const bool zown = zf >= Z0 && zf < Z1;
-                for (int q = threadIdx.x; q < VM_FN; q += RED_THREADS) {
-                    const int a = q % VM_FW, b = q / VM_FW;
-                    const int px = X0 - 1 + a, py = Y0 - 1 + b;
-                    const bool inside = zin && px >= 0 && px < nx && py >= 0 && py < ny;
-                    const bool own = inside && zown && a >= 1 && a <= VM_TX && b >= 1 && b <= VM_TY;
-                    if (!inside) {
-                        if (GRAD)
-#pragma unroll
-                            for (int f = 0; f < 9; ++f) Fz[f * VM_FN + q] = 0.f;
-                        continue;
-                    }
-                    if (!GRAD && !own) continue;
-                    const int o = (b + 1) * VM_XW + (a + 1);   // the position in the staged planes
-                    const float c0 = x0[o];
-                    const float vxp = x0[o + 1], vxm = x0[o - 1];
-                    const float vyp = x0[o + VM_XW], vym = x0[o - VM_XW];
-                    const float vzp = xq[o], vzm = xm[o];
-                    const float d1x = 0.5f * (vxp - vxm), d1y = 0.5f * (vyp - vym), d1z = 0.5f * (vzp - vzm);
-                    const float hxx = (vxp - c0) + (vxm - c0), hyy = (vyp - c0) + (vym - c0), hzz = (vzp - c0) + (vzm - c0);
-                    const float hxy = 0.25f * ((x0[o + 1 + VM_XW] - x0[o + 1 - VM_XW]) - (x0[o - 1 + VM_XW] - x0[o - 1 - VM_XW]));
-                    const float hxz = 0.25f * ((xq[o + 1] - xm[o + 1]) - (xq[o - 1] - xm[o - 1]));
-                    const float hyz = 0.25f * ((xq[o + VM_XW] - xm[o + VM_XW]) - (xq[o - VM_XW] - xm[o - VM_XW]));
-                    const float sH = hxx * hxx + hyy * hyy + hzz * hzz + 2.f * (hxy * hxy + hxz * hxz + hyz * hyz);
-                    const float sT = d1x * d1x + d1y * d1y + d1z * d1z;
-                    if (GRAD) {
-                        const float wH = rsqrtf(sH + eps), wT = beta * rsqrtf(sT + eps);
-                        Fz[0 * VM_FN + q] = wH * hxx;
-                        Fz[1 * VM_FN + q] = wH * hyy;
-                        Fz[2 * VM_FN + q] = wH * hzz;
-                        Fz[3 * VM_FN + q] = 2.f * wH * hxy;
-                        Fz[4 * VM_FN + q] = 2.f * wH * hxz;
-                        Fz[5 * VM_FN + q] = 2.f * wH * hyz;
-                        Fz[6 * VM_FN + q] = wT * d1x;
-                        Fz[7 * VM_FN + q] = wT * d1y;
-                        Fz[8 * VM_FN + q] = wT * d1z;
-                    }
-                    if (own) acc.add(sqrtf(sH + eps) + beta * sqrtf(sT + eps));
+            if constexpr (GRAD) if (s >= 2) {
+                float (*F)[VM_THREADS] = fs[s & 1];
+                const int up = max((int)threadIdx.x - 32, 0), dn = min((int)threadIdx.x + 32, VM_THREADS - 1);  // rows 0 and VM_PY - 1 own nothing
+                // along y, then x, the mixed xy field; the terms that take j itself only on the faces
+                float q = F[3][up] - F[3][dn];
+                float in = F[0][up] + F[1][dn] + ay * fyy;
+                float by = F[2][up] - F[2][dn];
+                if (ey != 0.f) {
+                    q += ey * fxy;
+                    in += ey * fy;
+                    by += ey * fyz;
                 }
-            }
-            if (!GRAD) continue;
-            __syncthreads();
-            const int jz = zi - 2;
-            if (s >= 4 && jz >= Z0 && jx < nx && jy < ny) {
-                const float* Fm = &S.F[(s + 1) % 3][0][0];    // fields of plane jz - 1
-                const float* F0 = &S.F[(s + 2) % 3][0][0];    // plane jz
-                const float* Fp = &S.F[s % 3][0][0];          // plane jz + 1
-                const int f0 = (ty + 1) * VM_FW + (tx + 1);
-                auto A = [&](const float* P, int f, int d) { return P[f * VM_FN + f0 + d]; };
-                // the entries of c_vcr with i = j - o, written out
-                float sg = (A(F0, 0, -1) + A(F0, 0, 1)) - 2.f * A(F0, 0, 0);
-                sg += (A(F0, 1, -SY) + A(F0, 1, SY)) - 2.f * A(F0, 1, 0);
-                sg += (A(Fm, 2, 0) + A(Fp, 2, 0)) - 2.f * A(F0, 2, 0);
-                sg += 0.25f * ((A(F0, 3, -1 - SY) - A(F0, 3, -1 + SY)) - (A(F0, 3, 1 - SY) - A(F0, 3, 1 + SY)));
-                sg += 0.25f * ((A(Fm, 4, -1) - A(Fp, 4, -1)) - (A(Fm, 4, 1) - A(Fp, 4, 1)));
-                sg += 0.25f * ((A(Fm, 5, -SY) - A(Fp, 5, -SY)) - (A(Fm, 5, SY) - A(Fp, 5, SY)));
-                sg += 0.5f * (A(F0, 6, -1) - A(F0, 6, 1));
-                sg += 0.5f * (A(F0, 7, -SY) - A(F0, 7, SY));
-                sg += 0.5f * (A(Fm, 8, 0) - A(Fp, 8, 0));
-                const int fxs = jx == 0 ? -1 : (jx == nx - 1 ? 1 : 0);   // outward offset on a face, else 0
-                const int fys = jy == 0 ? -1 : (jy == ny - 1 ? 1 : 0);
-                const int fzs = jz == 0 ? -1 : (jz == nz - 1 ? 1 : 0);
-                const int nf = (fxs != 0) + (fys != 0) + (fzs != 0);
-                if (nf == 1 && (fxs ? nx : fys ? ny : nz) > 1) {
-                    // one face, axis a with outward offset: the entries whose offset along a is that
-                    // offset also take j itself along a (the other axes shift as inside)
-                    const float h = 0.25f * (float)(fxs + fys + fzs);
-                    if (fxs) sg += A(F0, 0, 0) + h * ((A(F0, 3, -SY) - A(F0, 3, SY)) + (A(Fm, 4, 0) - A(Fp, 4, 0)) + 2.f * A(F0, 6, 0));
-                    else if (fys) sg += A(F0, 1, 0) + h * ((A(F0, 3, -1) - A(F0, 3, 1)) + (A(Fm, 5, 0) - A(Fp, 5, 0)) + 2.f * A(F0, 7, 0));
-                    else sg += A(F0, 2, 0) + h * ((A(F0, 4, -1) - A(F0, 4, 1)) + (A(F0, 5, -SY) - A(F0, 5, SY)) + 2.f * A(F0, 8, 0));
-                } else if (nf != 0) {
-                    sg += vcr_fold_terms(Fm, F0, Fp, jx, jy, jz, nx, ny, nz, X0, Y0);
+                in += __shfl_up_sync(0xffffffffu, fxx + fx, 1) + __shfl_down_sync(0xffffffffu, fxx - fx, 1) + ax * fxx;
+                in += __shfl_up_sync(0xffffffffu, q, 1) - __shfl_down_sync(0xffffffffu, q, 1);
+                float b = __shfl_up_sync(0xffffffffu, fxz, 1) - __shfl_down_sync(0xffffffffu, fxz, 1);
+                if (ex != 0.f) {
+                    in += ex * (fx + q);
+                    b += ex * fxz;
                 }
-                const int64_t j = vox(jx, jy, jz, nx, ny);
-                g[j] = fmaf(lam, sg, g[j]);
+                b += by + fz;                        // what plane zf gives its neighbours along z
+                const float hiz = zf == nz - 1 ? 1.f : 0.f, loz = zf == 0 ? 1.f : 0.f;
+                in += (hiz + loz - 2.f) * fzz;
+                if (hiz != loz) in += (hiz - loz) * b;
+                const int jz = zf - 1;
+                if (own && jz >= Z0 && jz < Z1) {
+                    const int64_t j = (int64_t)jz * plane + (int64_t)py * nx + px;
+                    g[j] = fmaf(lam, hold + (fzz - b), g[j]);
+                }
+                hold = zplus + in;
+                zplus = fzz + b;
             }
+            cm = c0; c0 = cp;
+            dxm = dx0; dx0 = dxp;
+            dym = dy0; dy0 = dyp;
+            hxx0 = hxxp; hyy0 = hyyp; hxy0 = hxyp;
         }
     }
-    const double tot = block_sum((double)acc.s - (double)acc.c, red);
+    const double tot = block_sum_n((double)acc.s - (double)acc.c, red, VM_PY);
     if (threadIdx.x == 0) partial[blockIdx.x] = tot;
 }
 
-int64_t vcr_items(int nx, int ny, int nz) {
-    return (int64_t)((nx + VM_TX - 1) / VM_TX) * ((ny + VM_TY - 1) / VM_TY) * ((nz + VM_ZC - 1) / VM_ZC);
+// Planes per item and the item count: the chunk length whose waves of CTAs take the fewest plane
+// steps (a chunk of zc planes takes zc + 4).
+static int vcr_chunk(int nx, int ny, int nz, int slots, int64_t& items) {
+    const int64_t cols = (int64_t)((nx + VM_OX - 1) / VM_OX) * ((ny + VM_OY - 1) / VM_OY);
+    int best = nz;
+    int64_t cost = INT64_MAX;
+    for (int n = 1; n <= 64 && n <= nz; ++n) {
+        const int zc = (nz + n - 1) / n;
+        const int64_t its = cols * ((nz + zc - 1) / zc), c = (its + slots - 1) / slots * (zc + 4);
+        if (c < cost) { cost = c; best = zc; }
+    }
+    items = cols * ((nz + best - 1) / best);
+    return best;
 }
-
-// Multiplier of the item permutation: an odd prime that does not divide the item count.
-unsigned vcr_item_mul(int nx, int ny, int nz) {
-    const int64_t n = vcr_items(nx, ny, nz);
-    const int64_t primes[] = {7919, 7927, 7933, 7937, 7949};
-    for (int64_t p : primes)
-        if (n % p != 0) return p % n == 0 ? 1u : (unsigned)p;
-    return 1u;
-}
-
-size_t vcr_smem_bytes(bool grad) { return grad ? sizeof(VcrMarchSmem) : sizeof(float) * 3 * VM_XN; }
 
 // value_out (device, may be NULL): R_VCR(x) in FP64.  g (may be NULL): g += lam grad R_VCR(x).
 // partial: RED_BLOCKS doubles.
 cudaError_t launch_vcr(const float* x, int nx, int ny, int nz, float beta, float eps, float lam, double* partial,
                        double* value_out, float* g, cudaStream_t st) {
-    if (vcr_items(nx, ny, nz) >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
-    cudaError_t e;
-    const unsigned mul = vcr_item_mul(nx, ny, nz);
-    if (g) {
-        const size_t sm = vcr_smem_bytes(true);
-        if ((e = cudaFuncSetAttribute(vcr_march_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) !=
-            cudaSuccess)
-            return e;
-        vcr_march_kernel<true><<<RED_BLOCKS, RED_THREADS, sm, st>>>(x, nx, ny, nz, beta, eps, lam, g, partial, mul);
-    } else {
-        vcr_march_kernel<false><<<RED_BLOCKS, RED_THREADS, vcr_smem_bytes(false), st>>>(x, nx, ny, nz, beta, eps, lam,
-                                                                                       nullptr, partial, mul);
-    }
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const int slots = VM_CTAS * device_sms();
+    int64_t items = 0;
+    const int zc = vcr_chunk(nx, ny, nz, slots, items);
+    if (items >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
+    const int nb = (int)(items < slots ? items : slots);
+    if (g) vcr_march_kernel<true><<<nb, VM_THREADS, 0, st>>>(x, nx, ny, nz, beta, eps, lam, g, partial, zc, (unsigned)items);
+    else vcr_march_kernel<false><<<nb, VM_THREADS, 0, st>>>(x, nx, ny, nz, beta, eps, lam, nullptr, partial, zc, (unsigned)items);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
     if (value_out) {
-        finish_kernel<<<1, RED_THREADS, 0, st>>>(partial, RED_BLOCKS, 1, 1, value_out);
+        finish_kernel<<<1, RED_THREADS, 0, st>>>(partial, nb, 1, 1, value_out);
         e = cudaGetLastError();
     }
     return e;

@@ -37,6 +37,20 @@ def test_value_and_gradient(dims, beta):
     assert rel_l2(gt.cpu().numpy() - g0, expect - g0) < 1e-5
 
 
+@pytest.mark.parametrize("dims", [(3, 14, 30), (4, 15, 31), (37, 13, 29), (70, 29, 61), (1, 1, 1), (1, 40, 64), (130, 3, 2)])
+def test_tile_edges(dims):
+    """Columns that end on, before and after a CTA's 30 x 14 voxels, one-voxel axes, and chunks along z."""
+    rng = np.random.default_rng(sum(dims))
+    x = rng.uniform(0.1, 1.0, dims).astype(np.float32)
+    val_o, g_o = vcr.value_and_grad(x.astype(np.float64), 0.5)
+    gt = torch.zeros(dims, device="cuda")
+    val = _lib.gpair_vcr(torch.as_tensor(x, device="cuda"), dims, 0.5, 1e-8, 1.0, gt)
+    assert abs(val - val_o) <= 1e-6 * val_o
+    got, scale = gt.cpu().numpy(), max(np.abs(g_o).max(), 1e-3)
+    assert np.abs(got - g_o).max() <= 1e-4 * scale              # every voxel: faces, edges and corners
+    assert np.linalg.norm(got - g_o) <= 1e-5 * np.linalg.norm(g_o) + 1e-6
+
+
 def test_value_only_leaves_no_gradient_and_zero_lambda():
     dims = (4, 5, 6)
     x = np.random.default_rng(1).uniform(0, 1, dims).astype(np.float32)
