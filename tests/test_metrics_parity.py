@@ -63,3 +63,11 @@ def test_paper_scale_volume():
     exp_mse = metrics.mse(xd, rd)
     assert abs(got["mse"] - exp_mse) <= 1e-6 * exp_mse
     assert abs(got["ssim"] - metrics.ssim(xd, rd, win=7)) <= 1e-5
+
+
+@pytest.mark.parametrize("win", [3, 5, 7, 9, 11])
+@pytest.mark.parametrize("dims", [(11, 12, 56), (14, 13, 57), (23, 33, 130), (1, 14, 63), (1, 40, 125)])
+def test_metrics_at_tile_edges(dims, win):
+    """Columns that end on, before and after a CTA's block of outputs for every window it takes, and 11, which
+    takes the other kernel."""
+    test_metrics_against_oracle(dims, win)
