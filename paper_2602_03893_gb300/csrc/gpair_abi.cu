@@ -73,7 +73,9 @@ cudaError_t launch_schedule(const SchedParams& p, StepSched* sd, cudaStream_t st
 cudaError_t launch_set_step(StepSched* sd, int t, const SchedParams& p, cudaStream_t st);
 int red_blocks();
 bool vox_is_lattice(const GaussDev& g, const gpair_grid& og);
-cudaError_t launch_voxelize(const GaussDev& g, const gpair_grid& og, float k, float* vol, float* tmp, cudaStream_t st);
+size_t vox_tile_bytes(const GaussDev& g, const gpair_grid& og);
+cudaError_t launch_voxelize(const GaussDev& g, const gpair_grid& og, float k, float* vol, float* tmp, void* prep,
+                            cudaStream_t st);
 }  // namespace gp
 
 using namespace gp;
@@ -92,8 +94,25 @@ struct Scratch {
 
 std::mutex g_pool_mu;
 std::unordered_map<uint64_t, Scratch> g_pool;
+std::mutex g_vox_mu;              // the voxelisation's own scratch, see gpair_voxelize
+std::unordered_map<uint64_t, Scratch> g_vox_pool;
 
 uint64_t pool_key(int dev, cudaStream_t st) { return ((uint64_t)(uint32_t)dev << 48) ^ (uint64_t)(uintptr_t)st; }
+
+// At least `bytes` in s.buf; the stream's earlier work is done with a buffer that is replaced.
+gpair_status grow_scratch(Scratch& s, cudaStream_t st, size_t bytes) {
+    if (s.cap >= bytes) return GPAIR_OK;
+    if (s.buf) {
+        cudaStreamSynchronize(st);
+        cudaFree(s.buf);
+        s.buf = nullptr;
+        s.cap = 0;
+    }
+    const size_t want = bytes + bytes / 8 + 4096;
+    if (cudaMalloc(&s.buf, want) != cudaSuccess) { s.buf = nullptr; cudaGetLastError(); return GPAIR_ERR_NOMEM; }
+    s.cap = want;
+    return GPAIR_OK;
+}
 
 gpair_status get_scratch(cudaStream_t st, size_t bytes, void** out_buf, int** out_status) {
     int dev = 0;
@@ -104,17 +123,8 @@ gpair_status get_scratch(cudaStream_t st, size_t bytes, void** out_buf, int** ou
         if (cudaMalloc(&s.status, sizeof(int)) != cudaSuccess) { s.status = nullptr; return GPAIR_ERR_NOMEM; }
         if (cudaMemsetAsync(s.status, 0, sizeof(int), st) != cudaSuccess) return GPAIR_ERR_CUDA;
     }
-    if (s.cap < bytes) {
-        if (s.buf) {
-            cudaStreamSynchronize(st);
-            cudaFree(s.buf);
-            s.buf = nullptr;
-            s.cap = 0;
-        }
-        size_t want = bytes + bytes / 8 + 4096;
-        if (cudaMalloc(&s.buf, want) != cudaSuccess) { s.buf = nullptr; cudaGetLastError(); return GPAIR_ERR_NOMEM; }
-        s.cap = want;
-    }
+    const gpair_status g = grow_scratch(s, st, bytes);
+    if (g != GPAIR_OK) return g;
     if (out_buf) *out_buf = s.buf;
     if (out_status) *out_status = s.status;
     return GPAIR_OK;
@@ -782,12 +792,28 @@ gpair_status gpair_voxelize(const gpair_gaussians* gi, const gpair_grid* og, flo
     if (!og || !vol || og->nx <= 0 || og->ny <= 0 || og->nz <= 0 || !finite_pos(og->dx) || !finite_pos(window_k))
         return GPAIR_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    void* tmp = nullptr;
     if (vox_is_lattice(g, *og)) {
+        void* tmp = nullptr;
         size_t bytes = (size_t)og->nx * og->ny * og->nz * 4;
         if ((s = get_scratch(st, bytes, &tmp, nullptr)) != GPAIR_OK) return s;
+        return cuda_status(launch_voxelize(g, *og, window_k, vol, static_cast<float*>(tmp), nullptr, st));
     }
-    return cuda_status(launch_voxelize(g, *og, window_k, vol, static_cast<float*>(tmp), st));
+    // Any other set.  The tile path keeps its scratch per stream, under a lock that also covers its
+    // launches: calls of several threads on one stream follow one another in it.  The scatter needs no
+    // scratch; it takes captured calls (a graph must not hold a buffer that a later call may replace),
+    // and those that find no memory.
+    const size_t bytes = vox_tile_bytes(g, *og);
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (bytes && cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess) return GPAIR_ERR_CUDA;
+        std::lock_guard<std::mutex> lk(g_vox_mu);
+        Scratch& b = g_vox_pool[pool_key(dev, st)];
+        if (grow_scratch(b, st, bytes) == GPAIR_OK)
+            return cuda_status(launch_voxelize(g, *og, window_k, vol, nullptr, b.buf, st));
+    }
+    cudaGetLastError();
+    return cuda_status(launch_voxelize(g, *og, window_k, vol, nullptr, nullptr, st));
 }
 
 gpair_status gpair_reduce_f64(const float* a, const float* b, const float* c, int64_t n, double* out, void* stream) {
@@ -990,17 +1016,21 @@ gpair_status gpair_wait_selftest(int polls, void* stream) {
 void gpair_release_scratch(void) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return;
-    std::lock_guard<std::mutex> lk(g_pool_mu);
-    for (auto it = g_pool.begin(); it != g_pool.end();) {
-        if ((it->first >> 48) == (uint64_t)(uint32_t)dev) {
-            cudaDeviceSynchronize();
-            if (it->second.buf) cudaFree(it->second.buf);
-            if (it->second.status) cudaFree(it->second.status);
-            it = g_pool.erase(it);
-        } else {
-            ++it;
+    auto release = [dev](std::mutex& mu, std::unordered_map<uint64_t, Scratch>& pool) {
+        std::lock_guard<std::mutex> lk(mu);
+        for (auto it = pool.begin(); it != pool.end();) {
+            if ((it->first >> 48) == (uint64_t)(uint32_t)dev) {
+                cudaDeviceSynchronize();
+                if (it->second.buf) cudaFree(it->second.buf);
+                if (it->second.status) cudaFree(it->second.status);
+                it = pool.erase(it);
+            } else {
+                ++it;
+            }
         }
-    }
+    };
+    release(g_pool_mu, g_pool);
+    release(g_vox_mu, g_vox_pool);
 }
 
 }  // extern "C"

@@ -227,8 +227,8 @@ __global__ void so_gather_kernel(GaussDev g, const int* __restrict__ perm, float
     out[4 * M + i] = g.A[j];
 }
 
-// gp: g with its arrays replaced by the permuted copies in scratch (spatial_order_bytes(g.M)).
-cudaError_t launch_spatial_order(const GaussDev& g, void* scratch, GaussDev& gp, cudaStream_t st) {
+// perm: the order as indices of g, in scratch (spatial_order_bytes(g.M)).
+cudaError_t launch_spatial_perm(const GaussDev& g, void* scratch, const int** perm, cudaStream_t st) {
     const int64_t M = g.M;
     if (M > 0x7FFFFFFF) return cudaErrorNotSupported;
     const size_t a = align256_sz((size_t)M * 4);
@@ -239,8 +239,6 @@ cudaError_t launch_spatial_order(const GaussDev& g, void* scratch, GaussDev& gp,
     int* hist = reinterpret_cast<int*>(p + 4 * a);
     float* boxp = reinterpret_cast<float*>(p + 4 * a + align256_sz((size_t)SO_RADIX * nb * 4));
     float* box = boxp + SO_BB_BLOCKS * 6;
-    float* out = reinterpret_cast<float*>(p + 4 * a + align256_sz((size_t)SO_RADIX * nb * 4) +
-                                          align256_sz((size_t)(SO_BB_BLOCKS + 1) * 6 * 4));
     so_box_partial_kernel<<<SO_BB_BLOCKS, SO_THREADS, 0, st>>>(g, boxp);
     so_box_final_kernel<<<1, SO_BB_BLOCKS, 0, st>>>(boxp, box);
     const unsigned eb = (unsigned)((M + 255) / 256);
@@ -253,7 +251,19 @@ cudaError_t launch_spatial_order(const GaussDev& g, void* scratch, GaussDev& gp,
                                                      vals[in ^ 1]);
     }
     static_assert(SO_PASSES % 2 == 0, "the order ends in buffer 0");
-    so_gather_kernel<<<eb, 256, 0, st>>>(g, vals[0], out);
+    *perm = vals[0];
+    return cudaGetLastError();
+}
+
+// gp: g with its arrays replaced by the permuted copies in scratch (spatial_order_bytes(g.M)).
+cudaError_t launch_spatial_order(const GaussDev& g, void* scratch, GaussDev& gp, cudaStream_t st) {
+    const int64_t M = g.M;
+    const int* perm = nullptr;
+    const cudaError_t e = launch_spatial_perm(g, scratch, &perm, st);
+    if (e != cudaSuccess) return e;
+    float* out = reinterpret_cast<float*>(static_cast<char*>(scratch) + spatial_order_bytes(M) -
+                                          5 * align256_sz((size_t)M * 4));
+    so_gather_kernel<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(g, perm, out);
     gp = g;
     gp.cx = out;
     gp.cy = out + M;

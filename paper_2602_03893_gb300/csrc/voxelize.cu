@@ -4,10 +4,14 @@
 // Lattice case (Gaussians on the output lattice, shared sigma): the field is A convolved with
 // the 1-D taps exp(-(m h)^2 / 2 sigma^2), |m h| <= k sigma, along x, y and z in turn -- three
 // separable gather passes, each one coalesced read and write of the volume (HBM-bound).
-// Any other Gaussian set: each Gaussian scatters its separable box of factors into the volume.
+// Any other Gaussian set: tiles of the volume gather the separable boxes of factors of the Gaussians that
+// reach them; very large sets, and calls under stream capture, scatter them instead.
 #include "gpair_internal.cuh"
 
 namespace gp {
+
+size_t spatial_order_bytes(int64_t M);
+cudaError_t launch_spatial_perm(const GaussDev& g, void* scratch, const int** perm, cudaStream_t st);
 
 constexpr int VOX_MAXTAP = 64;
 
@@ -201,23 +205,29 @@ __global__ void zero_kernel(float* p, int64_t n) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) p[i] = 0.f;
 }
 
-// One thread per Gaussian: scatter A prod_a f_a into the box of voxels within k sigma per axis.
-__global__ void vox_scatter_kernel(GaussDev g, gpair_grid og, float k, float* __restrict__ vol) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= g.M) return;
-    const float A = g.A[i];
-    if (A == 0.f) return;
-    float cx, cy, cz, s;
+// Gaussian i of the set: centre, width and amplitude.
+struct VoxG { float A, cx, cy, cz, s; };
+__device__ __forceinline__ VoxG vox_gaussian(const GaussDev& g, int64_t i) {
+    VoxG q;
+    q.A = g.A[i];
     if (g.grid) {
         const int ix = (int)(i % g.nx), iy = (int)((i / g.nx) % g.ny), iz = (int)(i / ((int64_t)g.nx * g.ny));
-        cx = (float)(g.ox + (ix + 0.5) * (double)g.h);
-        cy = (float)(g.oy + (iy + 0.5) * (double)g.h);
-        cz = (float)(g.oz + (iz + 0.5) * (double)g.h);
-        s = g.sigma;
+        q.cx = (float)(g.ox + (ix + 0.5) * (double)g.h);
+        q.cy = (float)(g.oy + (iy + 0.5) * (double)g.h);
+        q.cz = (float)(g.oz + (iz + 0.5) * (double)g.h);
+        q.s = g.sigma;
     } else {
-        cx = g.cx[i]; cy = g.cy[i]; cz = g.cz[i]; s = g.sg[i];
+        q.cx = g.cx[i]; q.cy = g.cy[i]; q.cz = g.cz[i]; q.s = g.sg[i];
     }
-    const float half = k * s * (1.f + 1e-6f), c2 = -0.72134752044448170368f / (s * s);
+    return q;
+}
+__device__ __forceinline__ float vox_half(float k, float s) { return k * s * (1.f + 1e-6f); }
+__device__ __forceinline__ float vox_c2(float s) { return -0.72134752044448170368f / (s * s); }
+
+// Add A prod_a f_a to the box of voxels within k sigma per axis, voxel by voxel.
+__device__ __forceinline__ void vox_scatter_one(const VoxG& q, const gpair_grid& og, float k, float* __restrict__ vol) {
+    const float cx = q.cx, cy = q.cy, cz = q.cz;
+    const float half = vox_half(k, q.s), c2 = vox_c2(q.s);
     const float inv = 1.f / og.dx;
     const int xa = max(0, (int)floorf((cx - half - og.ox) * inv - 0.5f)), xb = min(og.nx - 1, (int)ceilf((cx + half - og.ox) * inv - 0.5f));
     const int ya = max(0, (int)floorf((cy - half - og.oy) * inv - 0.5f)), yb = min(og.ny - 1, (int)ceilf((cy + half - og.oy) * inv - 0.5f));
@@ -225,7 +235,7 @@ __global__ void vox_scatter_kernel(GaussDev g, gpair_grid og, float k, float* __
     for (int iz = za; iz <= zb; ++iz) {
         const float rz = og.oz + (iz + 0.5f) * og.dx - cz;
         if (fabsf(rz) > half) continue;
-        const float fz = A * ex2_approx(rz * rz * c2);
+        const float fz = q.A * ex2_approx(rz * rz * c2);
         for (int iy = ya; iy <= yb; ++iy) {
             const float ry = og.oy + (iy + 0.5f) * og.dx - cy;
             if (fabsf(ry) > half) continue;
@@ -239,6 +249,260 @@ __global__ void vox_scatter_kernel(GaussDev g, gpair_grid og, float k, float* __
     }
 }
 
+// One thread per Gaussian: scatter its box into the volume.
+__global__ void vox_scatter_kernel(GaussDev g, gpair_grid og, float k, float* __restrict__ vol) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= g.M) return;
+    const VoxG q = vox_gaussian(g, i);
+    if (q.A == 0.f) return;
+    vox_scatter_one(q, og, k, vol);
+}
+
+// ------------------------------------------------------------------------------------------
+// The same sum by gathering.  The volume is cut into tiles of 8^3 voxels, one CTA each, whose warps
+// keep the whole tile in registers (16 voxels a lane: x = lane % 8, two rows of y, eight planes of z)
+// and share the Gaussians that reach it; the warps' tiles are added in shared memory and every voxel
+// is written once.  A Gaussian costs a tile 24 exponentials (8 per axis, zero outside its box)
+// and 512 FMAs of their outer product, against one exponential and one L2 atomic per voxel of its box.
+//
+// Finding them: the entries come in a spatially compact order (free centres: the Morton order; a
+// lattice: its 8 x 8 x 4 bricks), every 32 of them under one bounding box and every 1024 under another,
+// in voxel units.  A warp tests 32 boxes at a time, one to a lane, and goes down through the ones
+// that meet the tile; the entries found wait in the warp's queue until 32 are there, one to
+// a lane for the factors.
+//
+// Bound by FMA issue and shared-memory reads, no longer by the L2's atomics: 262,144 Gaussians of 3 to
+// 24 voxels a side into 128^3 took 3955 us as a scatter (857 M atomics) and take 488 us, 140 of them
+// the order.
+//
+// The scatter stays for sets whose prepared entries would need more than about a gigabyte
+// (VOX_TILE_MAX) and where Gaussians crowd the voxels (more than VOX_TILE_PER_VOXEL each): there are
+// too few tiles then to fill the chip, and boxes are a few voxels.
+constexpr int64_t VOX_TILE_MAX = (int64_t)1 << 24;
+constexpr int64_t VOX_TILE_PER_VOXEL = 8;
+constexpr int VT = 8;                         // tile side, voxels
+constexpr int VT_N = VT * VT * VT;
+constexpr int VT_WARPS = 8;
+constexpr int VT_ROW = 28;                    // factor row of one Gaussian: x 0-7, y 8-15 as (y, y + 4) pairs,
+                                              // z 16-23, 4 words of padding (conflict-free 16-byte stores)
+constexpr int VT_GROUP = 32, VT_SUPER = 1024;
+constexpr float VT_MARGIN = 0.25f;            // voxels by which the boxes exceed the exact test of a factor
+
+struct VoxBox { float lo[3], hi[3], pad[2]; };          // 32 bytes, two 16-byte loads
+struct VoxSet {                               // the prepared entries (scratch)
+    float4* u;                                // centre and half width in voxel units (half width < 0: skipped)
+    float4* c;                                // centre, k sigma
+    float2* w;                                // amplitude, -1 / (2 sigma^2 ln 2)
+    VoxBox *gbox, *sbox;                      // per 32 and per 1024 entries
+    int* odd;                                 // per 1024 entries: 1 when one of them is not finite
+    int64_t n;                                // entries, a multiple of VT_SUPER
+};
+
+// Entry e -> Gaussian, -1: none.
+__device__ __forceinline__ int64_t vox_entry(const GaussDev& g, const int* perm, int64_t e) {
+    if (!g.grid) return e < g.M ? (perm ? perm[e] : e) : -1;
+    const int64_t t = e / TILE;
+    if (t >= g.ntiles) return -1;
+    const int l = (int)(e % TILE);
+    const int ix = (int)(t % g.ntx) * BX + (l & (BX - 1)), iy = (int)((t / g.ntx) % g.nty) * BY + ((l / BX) & (BY - 1)),
+              iz = (int)(t / ((int64_t)g.ntx * g.nty)) * BZ + l / (BX * BY);
+    return ix < g.nx && iy < g.ny && iz < g.nz ? ((int64_t)iz * g.ny + iy) * g.nx + ix : -1;
+}
+
+// A Gaussian with a value that is not finite reaches voxels outside its box through the zeros of the
+// outer product; these few go voxel by voxel afterwards (vox_odd_kernel).
+// So do those whose place in voxel units is not.
+__device__ __forceinline__ bool vox_finite(const VoxG& q, const gpair_grid& og, float half, float c2) {
+    const float inv = 1.f / og.dx;
+    return isfinite(q.A) && isfinite(half * inv) && isfinite(c2) && isfinite((q.cx - og.ox) * inv) &&
+           isfinite((q.cy - og.oy) * inv) && isfinite((q.cz - og.oz) * inv);
+}
+
+__global__ void __launch_bounds__(VT_SUPER)
+vox_prepare_kernel(GaussDev g, gpair_grid og, float k, const int* __restrict__ perm, VoxSet V) {
+    __shared__ float sb[6][32];
+    const int64_t e = blockIdx.x * (int64_t)VT_SUPER + threadIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t i = vox_entry(g, perm, e);
+    float4 u = make_float4(0.f, 0.f, 0.f, -INFINITY), c = make_float4(0.f, 0.f, 0.f, -1.f);
+    float2 w = make_float2(0.f, 0.f);
+    float b[6] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY};
+    bool odd = false;
+    if (i >= 0) {
+        const VoxG q = vox_gaussian(g, i);
+        const float half = vox_half(k, q.s), c2 = vox_c2(q.s);
+        odd = q.A != 0.f && !vox_finite(q, og, half, c2);
+        if (q.A != 0.f && !odd && half >= 0.f) {
+            const float inv = 1.f / og.dx;
+            u = make_float4((q.cx - og.ox) * inv - 0.5f, (q.cy - og.oy) * inv - 0.5f, (q.cz - og.oz) * inv - 0.5f,
+                            half * inv + VT_MARGIN);
+            c = make_float4(q.cx, q.cy, q.cz, half);
+            w = make_float2(q.A, c2);
+            b[0] = u.x - u.w; b[1] = u.y - u.w; b[2] = u.z - u.w;
+            b[3] = u.x + u.w; b[4] = u.y + u.w; b[5] = u.z + u.w;
+        }
+    }
+    V.u[e] = u;
+    V.c[e] = c;
+    V.w[e] = w;
+    auto join = [&] {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+                const float v = __shfl_xor_sync(0xffffffffu, b[q], o);
+                b[q] = q < 3 ? fminf(b[q], v) : fmaxf(b[q], v);
+            }
+    };
+    auto store = [&](VoxBox* p) {
+        reinterpret_cast<float4*>(p)[0] = make_float4(b[0], b[1], b[2], b[3]);
+        reinterpret_cast<float2*>(p)[2] = make_float2(b[4], b[5]);
+    };
+    join();
+    if (lane == 0) {
+        store(V.gbox + e / VT_GROUP);
+#pragma unroll
+        for (int q = 0; q < 6; ++q) sb[q][warp] = b[q];
+    }
+    const int any_odd = __syncthreads_or(odd);
+    if (warp == 0) {
+#pragma unroll
+        for (int q = 0; q < 6; ++q) b[q] = sb[q][lane];
+        join();
+        if (lane == 0) {
+            store(V.sbox + blockIdx.x);
+            V.odd[blockIdx.x] = any_odd;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(VT_WARPS * 32)
+vox_tile_kernel(gpair_grid og, VoxSet V, int ntx, int nty, float* __restrict__ vol) {
+    __shared__ __align__(16) float F[VT_WARPS][VT_GROUP * VT_ROW];
+    __shared__ int queue[VT_WARPS][2 * VT_GROUP];
+    static_assert(VT_GROUP * VT_ROW >= VT_N, "the warps' tiles take the factors' place at the end");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int tx = blockIdx.x % ntx, ty = (blockIdx.x / ntx) % nty, tz = blockIdx.x / (ntx * nty);
+    const int x0 = tx * VT, y0 = ty * VT, z0 = tz * VT;
+    const float tlo[3] = {(float)x0, (float)y0, (float)z0};
+    const float thi[3] = {(float)(x0 + VT - 1), (float)(y0 + VT - 1), (float)(z0 + VT - 1)};
+    auto meets = [&](const VoxBox* p) {
+        const float4 a = __ldg(reinterpret_cast<const float4*>(p));
+        const float2 h = __ldg(reinterpret_cast<const float2*>(p) + 2);
+        return a.x <= thi[0] && a.y <= thi[1] && a.z <= thi[2] && a.w >= tlo[0] && h.x >= tlo[1] && h.y >= tlo[2];
+    };
+    float* Fw = F[warp];
+    int* qw = queue[warp];
+    const uint32_t lt = (1u << lane) - 1u;
+    // acc[p][r]: planes 2p and 2p + 1 of row y = lane / 8 + 4 r
+    float2 acc[VT / 2][2];
+#pragma unroll
+    for (int p = 0; p < VT / 2; ++p) acc[p][0] = acc[p][1] = make_float2(0.f, 0.f);
+
+    // the first n (<= 32) entries of the queue: factors by the lanes, then their outer products
+    auto batch = [&](int n) {
+        if (lane < n) {
+            const int e = qw[lane];
+            const float4 c = __ldg(V.c + e);
+            const float2 w = __ldg(V.w + e);
+            float f[3 * VT];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const float o = q == 0 ? og.ox : (q == 1 ? og.oy : og.oz), cc = q == 0 ? c.x : (q == 1 ? c.y : c.z);
+                const int i0 = q == 0 ? x0 : (q == 1 ? y0 : z0);
+#pragma unroll
+                for (int m = 0; m < VT; ++m) {
+                    const float r = o + ((float)(i0 + m) + 0.5f) * og.dx - cc;
+                    const float v = fabsf(r) <= c.w ? ex2_approx(r * r * w.y) : 0.f;
+                    f[q * VT + (q == 1 ? (m & 3) * 2 + (m >> 2) : m)] = q == 2 ? w.x * v : v;
+                }
+            }
+            float4* row = reinterpret_cast<float4*>(Fw + lane * VT_ROW);
+#pragma unroll
+            for (int m = 0; m < 3 * VT / 4; ++m) row[m] = make_float4(f[4 * m], f[4 * m + 1], f[4 * m + 2], f[4 * m + 3]);
+        }
+        __syncwarp();
+#pragma unroll 4
+        for (int j = 0; j < n; ++j) {
+            const float* row = Fw + j * VT_ROW;
+            const float fx = row[lane & 7];
+            const float2 fy = *reinterpret_cast<const float2*>(row + VT + 2 * (lane >> 3));
+            const float4 za = *reinterpret_cast<const float4*>(row + 2 * VT), zb = *reinterpret_cast<const float4*>(row + 2 * VT + 4);
+            const float w0 = fx * fy.x, w1 = fx * fy.y;
+            const float2 W0 = make_float2(w0, w0), W1 = make_float2(w1, w1);
+            const float2 z[4] = {make_float2(za.x, za.y), make_float2(za.z, za.w), make_float2(zb.x, zb.y), make_float2(zb.z, zb.w)};
+#pragma unroll
+            for (int p = 0; p < VT / 2; ++p) {
+                acc[p][0] = __ffma2_rn(z[p], W0, acc[p][0]);
+                acc[p][1] = __ffma2_rn(z[p], W1, acc[p][1]);
+            }
+        }
+        __syncwarp();
+    };
+
+    const int ns = (int)(V.n / VT_SUPER);
+    int qn = 0, turn = 0;
+    for (int s0 = 0; s0 < ns; s0 += 32) {
+        uint32_t sm = __ballot_sync(0xffffffffu, s0 + lane < ns && meets(V.sbox + min(s0 + lane, ns - 1)));
+        while (sm) {
+            const int sup = s0 + __ffs(sm) - 1;
+            sm &= sm - 1;
+            uint32_t gm = __ballot_sync(0xffffffffu, meets(V.gbox + (int64_t)sup * (VT_SUPER / VT_GROUP) + lane));
+            while (gm) {                       // the groups in turn to the warps
+                const int grp = __ffs(gm) - 1;
+                gm &= gm - 1;
+                if ((turn++ & (VT_WARPS - 1)) != warp) continue;
+                const int e = sup * VT_SUPER + grp * VT_GROUP + lane;
+                const float4 u = __ldg(V.u + e);
+                const bool hit = u.x - u.w <= thi[0] && u.y - u.w <= thi[1] && u.z - u.w <= thi[2] &&
+                                 u.x + u.w >= tlo[0] && u.y + u.w >= tlo[1] && u.z + u.w >= tlo[2];
+                const uint32_t hm = __ballot_sync(0xffffffffu, hit);
+                if (hit) qw[qn + __popc(hm & lt)] = e;
+                qn += __popc(hm);
+                __syncwarp();
+                if (qn >= VT_GROUP) {
+                    batch(VT_GROUP);
+                    qn -= VT_GROUP;
+                    const int rest = lane < qn ? qw[VT_GROUP + lane] : 0;
+                    __syncwarp();
+                    if (lane < qn) qw[lane] = rest;
+                    __syncwarp();
+                }
+            }
+        }
+    }
+    if (qn) batch(qn);
+
+    // this warp's tile in place of its factors: voxel (z, y, x) at z * 64 + y * 8 + x
+#pragma unroll
+    for (int p = 0; p < VT / 2; ++p)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            Fw[(2 * p) * 64 + r * 32 + lane] = acc[p][r].x;
+            Fw[(2 * p + 1) * 64 + r * 32 + lane] = acc[p][r].y;
+        }
+    __syncthreads();
+#pragma unroll
+    for (int v = threadIdx.x; v < VT_N; v += VT_WARPS * 32) {
+        float s = 0.f;
+#pragma unroll
+        for (int q = 0; q < VT_WARPS; ++q) s += F[q][v];
+        const int x = x0 + (v & 7), y = y0 + ((v >> 3) & 7), z = z0 + (v >> 6);
+        if (x < og.nx && y < og.ny && z < og.nz) vol[((int64_t)z * og.ny + y) * og.nx + x] = s;
+    }
+}
+
+// The Gaussians that the tiles left out for a value that is not finite.
+__global__ void __launch_bounds__(VT_SUPER)
+vox_odd_kernel(GaussDev g, gpair_grid og, float k, const int* __restrict__ perm, const int* __restrict__ odd,
+               float* __restrict__ vol) {
+    if (!odd[blockIdx.x]) return;
+    const int64_t i = vox_entry(g, perm, blockIdx.x * (int64_t)VT_SUPER + threadIdx.x);
+    if (i < 0) return;
+    const VoxG q = vox_gaussian(g, i);
+    if (q.A != 0.f && !vox_finite(q, og, vox_half(k, q.s), vox_c2(q.s))) vox_scatter_one(q, og, k, vol);
+}
+
 static int vox_blocks(int64_t n) {
     int64_t b = (n + 255) / 256;
     if (b > (int64_t)device_sms() * 32) b = (int64_t)device_sms() * 32;
@@ -250,8 +514,53 @@ bool vox_is_lattice(const GaussDev& g, const gpair_grid& og) {
            (double)og.ox == g.ox && (double)og.oy == g.oy && (double)og.oz == g.oz;
 }
 
-// tmp: scratch volume of the same size (lattice case).
-cudaError_t launch_voxelize(const GaussDev& g, const gpair_grid& og, float k, float* vol, float* tmp, cudaStream_t st) {
+// Entries of the tile path: the Gaussians (a lattice's in whole bricks), in whole supers.
+static int64_t vox_entries(const GaussDev& g) {
+    const int64_t n = g.grid ? g.ntiles * TILE : g.M;
+    return (n + VT_SUPER - 1) / VT_SUPER * VT_SUPER;
+}
+
+// Free sets of up to this many Gaussians are not sorted: a tile's 256 threads test every one of them.
+constexpr int64_t VOX_SORT_MIN = 4096;
+
+static size_t vox_set_bytes(int64_t n) { return (size_t)n * 40 + (size_t)(n / VT_GROUP + n / VT_SUPER) * sizeof(VoxBox) + (size_t)(n / VT_SUPER) * 4; }
+
+// Scratch of the tile path, 0: the scatter takes the call.
+size_t vox_tile_bytes(const GaussDev& g, const gpair_grid& og) {
+    const int64_t n = vox_entries(g);
+    const int64_t nt = (int64_t)((og.nx + VT - 1) / VT) * ((og.ny + VT - 1) / VT) * ((og.nz + VT - 1) / VT);
+    if (n > VOX_TILE_MAX || nt > INT32_MAX || n > VOX_TILE_PER_VOXEL * (nt * VT_N)) return 0;
+    return vox_set_bytes(n) + 256 + (!g.grid && g.M > VOX_SORT_MIN ? spatial_order_bytes(g.M) : 0);
+}
+
+static cudaError_t launch_vox_tiles(const GaussDev& g, const gpair_grid& og, float k, float* vol, void* prep,
+                                    cudaStream_t st) {
+    VoxSet V;
+    V.n = vox_entries(g);
+    const int64_t ng = V.n / VT_GROUP, ns = V.n / VT_SUPER;
+    V.u = static_cast<float4*>(prep);
+    V.c = V.u + V.n;
+    V.gbox = reinterpret_cast<VoxBox*>(V.c + V.n);
+    V.sbox = V.gbox + ng;
+    V.w = reinterpret_cast<float2*>(V.sbox + ns);
+    V.odd = reinterpret_cast<int*>(V.w + V.n);
+    const int* perm = nullptr;
+    if (!g.grid && g.M > VOX_SORT_MIN) {
+        char* so = static_cast<char*>(prep) + ((vox_set_bytes(V.n) + 255) & ~(size_t)255);
+        const cudaError_t e = launch_spatial_perm(g, so, &perm, st);
+        if (e != cudaSuccess) return e;
+    }
+    vox_prepare_kernel<<<(unsigned)ns, VT_SUPER, 0, st>>>(g, og, k, perm, V);
+    const int ntx = (og.nx + VT - 1) / VT, nty = (og.ny + VT - 1) / VT, ntz = (og.nz + VT - 1) / VT;
+    vox_tile_kernel<<<(unsigned)((int64_t)ntx * nty * ntz), VT_WARPS * 32, 0, st>>>(og, V, ntx, nty, vol);
+    vox_odd_kernel<<<(unsigned)ns, VT_SUPER, 0, st>>>(g, og, k, perm, V.odd, vol);
+    return cudaGetLastError();
+}
+
+// tmp: scratch volume of the same size (lattice case); prep: vox_tile_bytes() of scratch (others;
+// null: the scatter).
+cudaError_t launch_voxelize(const GaussDev& g, const gpair_grid& og, float k, float* vol, float* tmp, void* prep,
+                            cudaStream_t st) {
     const int64_t nv = (int64_t)og.nx * og.ny * og.nz;
     if (vox_is_lattice(g, og)) {
         Taps taps;
@@ -279,6 +588,7 @@ cudaError_t launch_voxelize(const GaussDev& g, const gpair_grid& og, float k, fl
         }
         return cudaGetLastError();
     }
+    if (prep) return launch_vox_tiles(g, og, k, vol, prep, st);
     zero_kernel<<<vox_blocks(nv), 256, 0, st>>>(vol, nv);
     vox_scatter_kernel<<<(unsigned)((g.M + 255) / 256), 256, 0, st>>>(g, og, k, vol);
     return cudaGetLastError();

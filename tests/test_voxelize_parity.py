@@ -95,3 +95,69 @@ def test_lattice_paper_scale_sampled_crops():
         ref = full[z0 - za:z0 - za + C, y0 - ya:y0 - ya + C, x0 - xa:x0 - xa + C]
         got = v[z0:z0 + C, y0:y0 + C, x0:x0 + C]
         assert rel_l2(got, ref) < 1e-4, (x0, y0, z0, rel_l2(got, ref))
+
+
+# One entry, a partial group of 32, the last set that is not sorted, the first that is, and two radix blocks;
+# tiles of 8^3: a single voxel, whole tiles and remainders.
+@pytest.mark.parametrize("M", [1, 33, 4096, 4097, 9001])
+@pytest.mark.parametrize("dims", [(1, 1, 1), (16, 8, 24), (23, 9, 17), (40, 37, 33)])
+def test_free_gaussians_tiles(M, dims):
+    rng = np.random.default_rng(M + sum(dims))
+    dx = 0.07e-3
+    ext = np.array(dims) * dx
+    c = ((rng.uniform(-0.7, 0.7, (M, 3))) * ext).astype(np.float32)      # some lie outside the volume
+    sig = np.exp(rng.uniform(np.log(0.03e-3), np.log(0.2e-3), M)).astype(np.float32)
+    A = rng.uniform(0, 1, M).astype(np.float32)
+    A[::7] = 0.0
+    gs = _lib.Gaussians(A=_cuda(A), cx=_cuda(c[:, 0]), cy=_cuda(c[:, 1]), cz=_cuda(c[:, 2]), sigma=_cuda(sig))
+    o = [float(np.float32(-e / 2)) for e in ext]
+    og = _lib.Grid(*dims, *o, dx, dx)
+    vol = torch.full(dims[::-1], float("nan"), device="cuda")
+    _lib.gpair_voxelize(gs, og, 3.0, vol)
+    G = oracle.gaussians_from_soa(c[:, 0], c[:, 1], c[:, 2], sig, A)
+    ref = oracle.voxelize(G, 3.0, *dims, *o, float(np.float32(dx)))
+    got = vol.cpu().numpy()
+    # a voxel at a box's edge may count on one side only: a term below e^-4.5 of its amplitude
+    bad = np.abs(got - ref) > 1e-4 * max(1e-30, np.abs(ref).max())
+    assert bad.mean() < 1e-3 and np.linalg.norm((got - ref)[~bad]) <= 1e-4 * np.linalg.norm(ref) + 1e-30
+
+
+def _cuda(a):
+    return torch.as_tensor(np.ascontiguousarray(a), device="cuda")
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), -float("inf")])
+def test_free_gaussians_not_finite_stay_in_their_box(value):
+    """An amplitude that is not finite marks the voxels of its own box and no others of the tiles it meets."""
+    dx, n = 1e-4, 24
+    c = np.array([[0.5, 3.5, -2.5], [-6.5, 1.5, 2.5], [0.5, 0.5, 0.5]], np.float32) * np.float32(dx)
+    A = np.array([1.0, value, 2.0], np.float32)
+    sig = np.full(3, dx, np.float32)
+    gs = _lib.Gaussians(A=_cuda(A), cx=_cuda(c[:, 0]), cy=_cuda(c[:, 1]), cz=_cuda(c[:, 2]), sigma=_cuda(sig))
+    o = -n * dx / 2
+    vol = torch.zeros((n, n, n), device="cuda")
+    _lib.gpair_voxelize(gs, _lib.Grid(n, n, n, o, o, o, dx, dx), 2.5, vol)
+    at = np.arange(n) - n / 2 + 0.5
+    on = [np.abs(at - q) <= 2.5 for q in (-6.5, 1.5, 2.5)]
+    box = on[2][:, None, None] & on[1][None, :, None] & on[0][None, None, :]
+    assert np.array_equal(~np.isfinite(vol.cpu().numpy()), box)
+
+
+def test_free_gaussians_captured():
+    """A captured call (the scatter) gives the tiles' result."""
+    rng = np.random.default_rng(5)
+    M, n, dx = 300, 19, 1e-4
+    c = (rng.uniform(-0.5, 0.5, (M, 3)) * n * dx).astype(np.float32)
+    sig = rng.uniform(0.5e-4, 2e-4, M).astype(np.float32)
+    gs = _lib.Gaussians(A=_cuda(rng.uniform(0, 1, M).astype(np.float32)), cx=_cuda(c[:, 0]), cy=_cuda(c[:, 1]),
+                        cz=_cuda(c[:, 2]), sigma=_cuda(sig))
+    og = _lib.Grid(n, n, n, -n * dx / 2, -n * dx / 2, -n * dx / 2, dx, dx)
+    one, two = torch.empty((n, n, n), device="cuda"), torch.empty((n, n, n), device="cuda")
+    _lib.gpair_voxelize(gs, og, 3.0, one)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        _lib.gpair_voxelize(gs, og, 3.0, two)
+    graph.replay()
+    # the same terms in another order: 300 of them, in single precision
+    assert torch.allclose(one, two, rtol=300 * 2.0 ** -23, atol=300 * 2.0 ** -23 * float(one.max()))
