@@ -10,7 +10,11 @@
 // global atomics.  Free-centre Gaussians are taken in the order of their window length (a
 // counting sort of the tile in shared memory), so the 32 threads of a warp walk windows of about
 // the same length.
+#include <cooperative_groups.h>
+
 #include "gpair_internal.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace gp {
 
@@ -257,8 +261,10 @@ adj_kernel(GaussDev g, ArrDev a, const TileInfo* __restrict__ ti, const float* _
 // The table is split by term so that a warp's gathers of nearby window starts touch as few
 // cache lines as possible: Qa[j][b + L] holds Q_0 .. Q_3 (16 bytes), Qb[j][b + L] the rest (Q_4,
 // Q_5 as 8 bytes for P = 6; Q_4 .. Q_7 as 16 bytes for P = 7, 8), for window starts b in
-// [-L, N_t); the residual is zero outside the record.  Qb starts N_d (N_t + L) float4 after Qa.
-__host__ __device__ __forceinline__ size_t adj_qb_offset(int Nd, int Nt, int L) { return (size_t)Nd * (Nt + L); }
+// [-L, N_t]; the residual is zero outside the record, so the entries of b = N_t are zero and stand
+// for every start outside.  Qb starts N_d rows of float4 after Qa.
+__host__ __device__ __forceinline__ int adj_q_row(int Nt, int L) { return Nt + L + 1; }
+__host__ __device__ __forceinline__ size_t adj_qb_offset(int Nd, int Nt, int L) { return (size_t)Nd * adj_q_row(Nt, L); }
 
 template <int P>
 __global__ void __launch_bounds__(256)
@@ -274,7 +280,7 @@ adj_q_kernel(const float* __restrict__ delta, int Nt, const __grid_constant__ Mo
     }
     __syncthreads();
     const int b = b0 + (int)threadIdx.x;
-    if (b >= Nt) return;
+    if (b > Nt) return;
     float acc[MOM_P];
 #pragma unroll
     for (int p = 0; p < MOM_P; ++p) acc[p] = 0.f;     // acc[p >= P] stays 0
@@ -283,115 +289,228 @@ adj_q_kernel(const float* __restrict__ delta, int Nt, const __grid_constant__ Mo
 #pragma unroll
         for (int p = 0; p < P; ++p) acc[p] = fmaf(dl, T.c[m][p], acc[p]);
     }
-    const size_t e = (size_t)j * (Nt + L) + (b + L);
+    const size_t e = (size_t)j * adj_q_row(Nt, L) + (b + L);
     float4* Qa = reinterpret_cast<float4*>(Q);
     Qa[e] = make_float4(acc[0], acc[1], acc[2], acc[3]);
     if constexpr (P == 6) reinterpret_cast<float2*>(Qa + adj_qb_offset(gridDim.y, Nt, L))[e] = make_float2(acc[4], acc[5]);
     else (Qa + adj_qb_offset(gridDim.y, Nt, L))[e] = make_float4(acc[4], acc[5], acc[6], acc[7]);
 }
 
-// One CTA per brick of 256 grid Gaussians, one thread per Gaussian, all sensors in chunks of 32.
+// One CTA of 64 threads per brick of 256 grid Gaussians, four Gaussians to a thread: x and x + 4, two
+// planes each.  The two planes go through packed FP32 arithmetic (add/mul/fma .f32x2), which rounds
+// each half as the scalar operation does; the ceiling of the window start comes from one addition that
+// rounds up; a start outside the record reads the row's zero entry.
+//
+// Bound by instruction issue and by the gathers' L1 wavefronts.  With one Gaussian to a thread and scalar
+// arithmetic it took 57 instructions a pair: 14.96 ms for 256 x 256 x 128 Gaussians and 1024 sensors,
+// 10.5 ms now.
+//
+// A brick's sensors are divided over the CTAs of a cluster where there are too few bricks to fill the
+// chip; their sums meet in the first CTA's shared memory, in the order of the ranks.
+constexpr int ADJM_THREADS = 64, ADJM_PER = TILE / ADJM_THREADS;
+constexpr int ADJM_SC = 64;              // sensors per chunk; sums are compensated every 32
+constexpr int ADJM_CTAS = 12;            // resident per SM
+struct __align__(16) AdjmRef {
+    float v2x, v2y, v2z, R0;             // 2 (c0 - s), |c0 - s|
+    float phi0;
+    unsigned n0;                         // sample n0 + L, less ADJ_MAGIC_BITS (wrapping)
+    int j, pad;
+    const float4* qa;                    // the sensor's rows
+    const char* qb;
+};
+
+// Starts 2^22 samples and more from the centre's are beyond the rounding addition; FP32 no longer resolves
+// half a sample there.
 template <int P>
-__global__ void __launch_bounds__(ADJ_THREADS, 5)
+__global__ void __launch_bounds__(ADJM_THREADS, ADJM_CTAS)
 adj_moment_kernel(GaussDev g, ArrDev a, const float* __restrict__ delta, const float* __restrict__ Q,
-                  const __grid_constant__ MomentTable T, float* __restrict__ gA) {
-    __shared__ PairRef refs2[2][ADJ_SC];
+                  const __grid_constant__ MomentTable T, float* __restrict__ gA, int per) {
+    __shared__ AdjmRef refs2[2][ADJM_SC];
+    __shared__ float part[TILE];
     const int64_t t = blockIdx.x;
-    const int l = threadIdx.x, warp = l >> 5, lane = l & 31;
+    const int l = threadIdx.x;
     const int tx = (int)(t % g.ntx), ty = (int)((t / g.ntx) % g.nty), tz = (int)(t / ((int64_t)g.ntx * g.nty));
-    // warp w takes a 4 x 4 x 2 block of the 8 x 8 x 4 brick (w's bits: x half, y half, z pair), so
-    // that the window starts of its 32 Gaussians for one sensor -- the table rows it gathers -- stay
-    // close together for every direction of the cap
-    static_assert(BX == 8 && BY == 8 && BZ == 4 && ADJ_THREADS == 256, "brick of 8 x 8 x 4, 8 warps");
-    const int lx = (l & 3) | (((l >> 5) & 1) << 2), ly = ((l >> 2) & 3) | (((l >> 6) & 1) << 2),
-              lz = ((l >> 4) & 1) | (((l >> 7) & 1) << 1);
-    const int gx = tx * BX + lx, gy = ty * BY + ly, gz = tz * BZ + lz;
-    const bool valid = gx < g.nx && gy < g.ny && gz < g.nz;
-    const int64_t i = ((int64_t)gz * g.ny + gy) * g.nx + gx;
-    const float dx = ((float)lx - 0.5f * (BX - 1)) * g.h, dy = ((float)ly - 0.5f * (BY - 1)) * g.h,
-                dz = ((float)lz - 0.5f * (BZ - 1)) * g.h;
+    // a warp takes a 4 x 4 x 2 block of nodes per gather (planes 0 and 2, or 1 and 3), so that the window
+    // starts of its 32 Gaussians for one sensor -- the table rows it gathers -- stay close together for
+    // every direction of the cap
+    static_assert(BX == 8 && BY == 8 && BZ == 4 && ADJM_THREADS == 64, "brick of 8 x 8 x 4, 2 warps");
+    const int lx = l & 3, ly = ((l >> 2) & 3) | (((l >> 5) & 1) << 2), lz = ((l >> 4) & 1) << 1;
+    const float dx0 = ((float)lx - 0.5f * (BX - 1)) * g.h, dx1 = ((float)(lx + 4) - 0.5f * (BX - 1)) * g.h;
+    const float dy = ((float)ly - 0.5f * (BY - 1)) * g.h;
+    const float2 dz = make_float2(((float)lz - 0.5f * (BZ - 1)) * g.h, ((float)(lz + 1) - 0.5f * (BZ - 1)) * g.h);
+    const float2 dx[2] = {make_float2(dx0, dx0), make_float2(dx1, dx1)}, dy2 = make_float2(dy, dy);
+    float2 d2[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) d2[u] = __ffma2_rn(dx[u], dx[u], __ffma2_rn(dy2, dy2, __fmul2_rn(dz, dz)));
     const double c0x = g.ox + (tx * BX + BX / 2) * (double)g.h;
     const double c0y = g.oy + (ty * BY + BY / 2) * (double)g.h;
     const double c0z = g.oz + (tz * BZ + BZ / 2) * (double)g.h;
     const float ks = a.k * g.sigma, Delta = a.Delta, invDelta = a.invDelta;
+    const float ksi = ks * invDelta;
     const float c2 = -0.72134752044448170368f / (g.sigma * g.sigma);
     const int L = T.L, Nt = a.Nt;
+    const unsigned zero_row = (unsigned)(Nt + L);
     const float ED = (float)T.E * Delta;
-    const float ksi = ks * invDelta;
-    const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));   // references below carry 2 (c0 - s)
     const float4* Qa = reinterpret_cast<const float4*>(Q);
-    const size_t qb_off = adj_qb_offset(a.Nd, Nt, L);
-    KahanF kA;
-    // References are double-buffered: after each barrier the last warp forms the next chunk's
-    // FP64 references while the others already work on the current chunk.
-    if (warp == ADJ_THREADS / 32 - 1 && lane < min(ADJ_SC, a.Nd))
-        refs2[0][lane] = ref_doubled(make_ref(c0x, c0y, c0z, a.xyz[3 * lane], a.xyz[3 * lane + 1], a.xyz[3 * lane + 2], a));
+    const char* Qb = reinterpret_cast<const char*>(Qa + adj_qb_offset(a.Nd, Nt, L));
+    const int jb = blockIdx.y * per, je = min(a.Nd, jb + per);
+
+    auto ref = [&](int j) {
+        const PairRef p = ref_doubled(make_ref(c0x, c0y, c0z, a.xyz[3 * j], a.xyz[3 * j + 1], a.xyz[3 * j + 2], a));
+        AdjmRef r;
+        r.v2x = p.v0x; r.v2y = p.v0y; r.v2z = p.v0z;
+        r.R0 = p.R0;
+        r.phi0 = p.phi0;
+        r.n0 = (unsigned)(p.n0 + L) - (unsigned)ADJ_MAGIC_BITS;
+        r.j = j;
+        r.pad = 0;
+        r.qa = Qa + (size_t)j * adj_q_row(Nt, L);
+        r.qb = Qb + (size_t)j * adj_q_row(Nt, L) * (P == 6 ? 8 : 16);
+        return r;
+    };
+    auto both = [](float v) { return make_float2(v, v); };
+    const float2 magic = both(ADJ_MAGIC), mmagic = both(-ADJ_MAGIC), iD = both(invDelta), mksi = both(-ksi),
+                 mD = both(-Delta), mdstar = both(-T.dstar), ihalf = both(T.inv_half);
+    KahanF kA[ADJM_PER];
+    // References are double-buffered: after each barrier the threads form the next chunk's.
+    if (jb + l < je) refs2[0][l] = ref(jb + l);
     int cur = 0;
-    for (int j0 = 0; j0 < a.Nd; j0 += ADJ_SC, cur ^= 1) {
-        const int nsc = min(ADJ_SC, a.Nd - j0);
+    for (int j0 = jb; j0 < je; j0 += ADJM_SC, cur ^= 1) {
+        const int nsc = min(ADJM_SC, je - j0);
         __syncthreads();
-        if (warp == ADJ_THREADS / 32 - 1 && j0 + ADJ_SC + lane < a.Nd) {
-            const int j = j0 + ADJ_SC + lane;
-            refs2[cur ^ 1][lane] = ref_doubled(make_ref(c0x, c0y, c0z, a.xyz[3 * j], a.xyz[3 * j + 1], a.xyz[3 * j + 2], a));
-        }
-        const PairRef* refs = refs2[cur];
-        if (valid) {
-            float acc = 0.f;         // FP32 over the chunk's 32 sensors, Kahan across chunks
-            constexpr int UNROLL = P <= 7 ? 4 : 2;   // 8 terms need the registers of the deeper unroll
-#pragma unroll UNROLL
-            for (int q = 0; q < nsc; ++q) {
-                const PairRef r = refs[q];
-                float invR, phi;
-                pair_phase_pre(r, dx, dy, dz, d2, invR, phi);
-                const float mf = ceilf(fmaf(phi, invDelta, -ksi));   // as the forward
-                const int b = r.n0 + (int)mf;
-                if (b < -L || b >= Nt) continue;
-                const float d0 = fmaf(-mf, Delta, phi);
-                const float e = (d0 - T.dstar) * T.inv_half;
-                const size_t qe = (size_t)(j0 + q) * (Nt + L) + (b + L);
-                const float4 q0 = __ldg(Qa + qe);
-                float s;
-                if constexpr (P == 6) {
-                    const float2 q1 = __ldg(reinterpret_cast<const float2*>(Qa + qb_off) + qe);
-                    s = fmaf(q1.y, e, q1.x);
-                } else {
-                    const float4 q1 = __ldg(Qa + qb_off + qe);
-                    if constexpr (P == 8) s = fmaf(fmaf(fmaf(q1.w, e, q1.z), e, q1.y), e, q1.x);
-                    else s = fmaf(fmaf(q1.z, e, q1.y), e, q1.x);
+        if (j0 + ADJM_SC + l < je) refs2[cur ^ 1][l] = ref(j0 + ADJM_SC + l);
+        for (int q0 = 0; q0 < nsc; q0 += 32) {
+            float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};   // FP32 over 32 sensors
+            const AdjmRef* rp = refs2[cur] + q0;
+            const int nq = min(32, nsc - q0);
+#pragma unroll 1
+            for (int q = 0; q < nq; ++q) {
+                const AdjmRef r = rp[q];
+                const float2 R0 = both(r.R0);
+                float2 e[2], iR[2];
+                unsigned rel[ADJM_PER];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const float2 num = __ffma2_rn(dx[u], both(r.v2x), __ffma2_rn(dy2, both(r.v2y), __ffma2_rn(dz, both(r.v2z), d2[u])));
+                    const float2 R2 = __ffma2_rn(R0, R0, num);
+                    iR[u] = make_float2(rsqrtf(R2.x), rsqrtf(R2.y));
+                    const float2 den = __ffma2_rn(R2, iR[u], R0);
+                    float2 rc;
+                    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc.x) : "f"(den.x));
+                    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc.y) : "f"(den.y));
+                    const float2 phi = __ffma2_rn(num, rc, both(r.phi0));
+                    const float2 up = __fadd2_ru(__ffma2_rn(phi, iD, mksi), magic);      // as the forward
+                    const float2 mf = __fadd2_rn(up, mmagic);
+                    rel[2 * u] = (unsigned)__float_as_int(up.x) + r.n0;
+                    rel[2 * u + 1] = (unsigned)__float_as_int(up.y) + r.n0;
+                    const float2 d0 = __ffma2_rn(mf, mD, phi);
+                    e[u] = __fmul2_rn(__fadd2_rn(d0, mdstar), ihalf);
                 }
-                s = fmaf(s, e, q0.w);
-                s = fmaf(s, e, q0.z);
-                s = fmaf(s, e, q0.y);
-                s = fmaf(s, e, q0.x);
-                if (edge_corrected(T, e)) {            // edge position E: rare direct correction
-                    const float dE = d0 - ED;
-                    const int n = b + T.E;
-                    if (n >= 0 && n < Nt)
-                        s = fmaf(edge_factor(T) * delta[(size_t)(j0 + q) * Nt + n] * dE, ex2_approx(dE * dE * c2), s);
+                float s[ADJM_PER];
+#pragma unroll
+                for (int u = 0; u < ADJM_PER; ++u) {
+                    const float x = (u & 1) ? e[u >> 1].y : e[u >> 1].x;
+                    const unsigned at = min(rel[u], zero_row);
+                    const float4 q0v = __ldg(r.qa + at);
+                    float v;
+                    if constexpr (P == 6) {
+                        const float2 q1 = __ldg(reinterpret_cast<const float2*>(r.qb) + at);
+                        v = fmaf(q1.y, x, q1.x);
+                    } else {
+                        const float4 q1 = __ldg(reinterpret_cast<const float4*>(r.qb) + at);
+                        if constexpr (P == 8) v = fmaf(fmaf(fmaf(q1.w, x, q1.z), x, q1.y), x, q1.x);
+                        else v = fmaf(fmaf(q1.z, x, q1.y), x, q1.x);
+                    }
+                    s[u] = fmaf(fmaf(fmaf(fmaf(v, x, q0v.w), x, q0v.z), x, q0v.y), x, q0v.x);
                 }
-                acc = fmaf(s, invR, acc);
+                bool edge = false;
+#pragma unroll
+                for (int u = 0; u < ADJM_PER; ++u) edge |= edge_corrected(T, (u & 1) ? e[u >> 1].y : e[u >> 1].x);
+                if (edge) {            // edge position E: rare direct correction
+#pragma unroll
+                    for (int u = 0; u < ADJM_PER; ++u) {
+                        const float x = (u & 1) ? e[u >> 1].y : e[u >> 1].x;
+                        const int n = (int)(rel[u] - (unsigned)L) + T.E;
+                        if (edge_corrected(T, x) && n >= 0 && n < Nt) {
+                            const float dE = fmaf(x, 0.5f * Delta, T.dstar) - ED;
+                            s[u] = fmaf(edge_factor(T) * delta[(size_t)r.j * Nt + n] * dE, ex2_approx(dE * dE * c2), s[u]);
+                        }
+                    }
+                }
+                acc[0] = __ffma2_rn(make_float2(s[0], s[1]), iR[0], acc[0]);
+                acc[1] = __ffma2_rn(make_float2(s[2], s[3]), iR[1], acc[1]);
             }
-            kA.add(acc);
+            kA[0].add(acc[0].x); kA[1].add(acc[0].y);
+            kA[2].add(acc[1].x); kA[3].add(acc[1].y);
         }
     }
-    if (valid) gA[i] = kA.s;                 // the table carries the 1/2 of A / 2R
+    float sum[ADJM_PER];
+#pragma unroll
+    for (int u = 0; u < ADJM_PER; ++u) sum[u] = kA[u].s;
+    if (gridDim.y > 1) {
+        cg::cluster_group cl = cg::this_cluster();
+#pragma unroll
+        for (int u = 0; u < ADJM_PER; ++u) part[u * ADJM_THREADS + l] = sum[u];
+        cl.sync();
+        if (blockIdx.y == 0)
+            for (unsigned c = 1; c < gridDim.y; ++c) {
+                const float* other = cl.map_shared_rank(part, c);
+#pragma unroll
+                for (int u = 0; u < ADJM_PER; ++u) sum[u] += other[u * ADJM_THREADS + l];
+            }
+        cl.sync();                       // the others' shared memory stays until it has been read
+        if (blockIdx.y) return;
+    }
+#pragma unroll
+    for (int u = 0; u < ADJM_PER; ++u) {
+        const int gx = tx * BX + lx + (u >> 1) * 4, gy = ty * BY + ly, gz = tz * BZ + lz + (u & 1);
+        if (gx < g.nx && gy < g.ny && gz < g.nz)
+            gA[((int64_t)gz * g.ny + gy) * g.nx + gx] = sum[u];     // the table carries the 1/2 of A / 2R
+    }
 }
 
-size_t adj_moment_q_bytes(const ArrDev& a, int L) { return (size_t)a.Nd * (a.Nt + L) * MOM_P * sizeof(float); }
+size_t adj_moment_q_bytes(const ArrDev& a, int L) { return (size_t)a.Nd * adj_q_row(a.Nt, L) * MOM_P * sizeof(float); }
+
+// CTAs that share a tile's sensors: as many (1, 2, 4, 8) as keep the grid within one wave of `ctas` per
+// SM, with at least 8 sensors each.  16 bricks and 128 sensors: 74 us for the 16 CTAs, 40 us for 8 times as many,
+// each with an eighth of the sensors (20 steps of a 16^3 reconstruction 2476 -> 1778 us).
+int adj_split(int64_t ntiles, int Nd, int ctas) {
+    int split = 1;
+    while (split < 8 && ntiles * split * 2 <= (int64_t)device_sms() * ctas && Nd >= 16 * split) split *= 2;
+    return split;
+}
+
+template <typename... Args>
+static cudaError_t launch_split(void (*kern)(Args...), unsigned tiles, int split, int threads, size_t smem,
+                                cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(tiles, split);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 1;
+    at[0].val.clusterDim.y = split;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = split > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
 
 cudaError_t launch_adjoint_moment(const GaussDev& g, const ArrDev& a, const float* delta, float* gA,
                                   const MomentTable& T, float* Q, const cudaEvent_t* ev, cudaStream_t st) {
-    dim3 qgrid((a.Nt + T.L + 255) / 256, a.Nd);
+    dim3 qgrid((adj_q_row(a.Nt, T.L) + 255) / 256, a.Nd);
     if (T.P == 6) adj_q_kernel<6><<<qgrid, 256, (256 + T.L) * sizeof(float), st>>>(delta, a.Nt, T, Q);
     else if (T.P == 7) adj_q_kernel<7><<<qgrid, 256, (256 + T.L) * sizeof(float), st>>>(delta, a.Nt, T, Q);
     else adj_q_kernel<8><<<qgrid, 256, (256 + T.L) * sizeof(float), st>>>(delta, a.Nt, T, Q);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (ev && (e = cudaEventRecord(ev[0], st)) != cudaSuccess) return e;
-    if (T.P == 6) adj_moment_kernel<6><<<(unsigned)g.ntiles, ADJ_THREADS, 0, st>>>(g, a, delta, Q, T, gA);
-    else if (T.P == 7) adj_moment_kernel<7><<<(unsigned)g.ntiles, ADJ_THREADS, 0, st>>>(g, a, delta, Q, T, gA);
-    else adj_moment_kernel<8><<<(unsigned)g.ntiles, ADJ_THREADS, 0, st>>>(g, a, delta, Q, T, gA);
-    e = cudaGetLastError();
+    auto kern = T.P == 6 ? adj_moment_kernel<6> : T.P == 7 ? adj_moment_kernel<7> : adj_moment_kernel<8>;
+    const int split = adj_split(g.ntiles, a.Nd, ADJM_CTAS);
+    e = launch_split(kern, (unsigned)g.ntiles, split, ADJM_THREADS, 0, st, g, a, delta, (const float*)Q, T, gA,
+                     (a.Nd + split - 1) / split);
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], st);
     return e;
 }

@@ -102,3 +102,15 @@ def test_paper_scale_full_launch_sampled_gaussians():
     idx = np.sort(rng.choice(w.M, 3000, replace=False))
     rels = _check(w, delta, full=False, gauss_idx=idx)
     assert rels["A"] < 1e-4
+
+
+@pytest.mark.parametrize("nd", [1, 15, 16, 33, 97, 130])
+@pytest.mark.parametrize("sides", [(3, 2, 1), (11, 9, 6)])
+def test_moment_adjoint_few_tiles(nd, sides):
+    """One to eight CTAs share a brick's sensors: a lone sensor, the last count without a split, counts that
+    leave the last CTA short, and chunks of 64 with a remainder; records that end before the last windows."""
+    g = synth.centred_grid(*sides, 0.1e-3)
+    w = synth.Workload("few", g, synth.cap_sensors(nd, 15e-3, 150.0), 405, A=np.ones(g.M, np.float32))
+    delta = np.random.default_rng(nd).normal(size=(w.Nd, w.Nt)).astype(np.float32)
+    _check(w, delta, full=False, A=w.A)
+
