@@ -31,7 +31,6 @@ namespace gp {
 constexpr int ASSA_SPC = 8;
 constexpr int ASSA_THREADS = 32 * ASSA_SPC;
 constexpr int ASSA_RING = 4;
-constexpr int ASSA_ADJ_SC = 32;
 constexpr float ASSA_QMAX = 0.99f * 524288.f;      // 0.99 * 2^19: bound of a scaled mass
 constexpr int ASSA_FLUSH = 16;                     // bricks per integer band (16 * 256 = 2^12 pairs)
 
@@ -267,6 +266,9 @@ assa_fwd_kernel(GaussDev g, ArrDev a, const SlabInfo* __restrict__ slabs, float*
     }
 }
 
+// A sensor's row of dconv: its alpha N_t fine samples and a zero.
+__host__ __device__ __forceinline__ int assa_dconv_row(int alpha, int Nt) { return alpha * Nt + 1; }
+
 // dconv_j[k] = sum_n h[alpha n - k] delta_j[n], k = 0 .. alpha Nt - 1 (zero filling and the
 // correlation with the flipped pulse in one pass).  Block: 256 fine samples of one sensor.
 __device__ __forceinline__ int floor_div(int a, int b) { return (a >= 0) ? a / b : -((-a + b - 1) / b); }
@@ -287,69 +289,110 @@ __global__ void assa_dconv_kernel(const float* __restrict__ delta, int Nt, const
     }
     __syncthreads();
     const int k = k0 + (int)threadIdx.x;
-    if (k >= Nup) return;
+    if (k > Nup) return;
+    if (k == Nup) {              // the entry of every sample outside the record
+        dconv[(size_t)j * assa_dconv_row(alpha, Nt) + k] = 0.f;
+        return;
+    }
     const int n1 = -floor_div(-(k - K), alpha), n2 = floor_div(k + K, alpha);
     float acc = 0.f;
     for (int n = n1; n <= n2; ++n) acc = fmaf(T.hr[K - (alpha * n - k)], sd[n - na], acc);
-    dconv[(size_t)j * Nup + k] = acc;
+    dconv[(size_t)j * assa_dconv_row(alpha, Nt) + k] = acc;
 }
 
 size_t assa_dconv_smem(const AssaTable& T) { return (size_t)((255 + 2 * T.K) / T.alpha + 3) * sizeof(float); }
 
-// g_i = sum_j dconv_j[k_ij] / r_ij.  One CTA per brick, one thread per Gaussian, all sensors in
-// chunks of 32 with FP64 references prepared one chunk ahead by the last warp.
-__global__ void __launch_bounds__(TILE)
+// g_i = sum_j dconv_j[k_ij] / r_ij.  One CTA of 64 threads per brick, four Gaussians to a thread (x and
+// x + 4, two planes each; the planes through packed FP32 arithmetic, which rounds each half as the scalar
+// operation does).  The FP64 references of a chunk of 64 sensors, one to a thread, are
+// double-buffered.  A snapped sample outside the record reads the sensor's zero entry, one past its end.
+//
+// Bound by instruction issue.
+constexpr int ASSA_ADJ_THREADS = 64, ASSA_ADJ_PER = TILE / ASSA_ADJ_THREADS, ASSA_ADJ_CTAS = 16;
+constexpr int ASSA_ADJ_SC = 64;
+struct __align__(16) AssaRef {
+    float v2x, v2y, v2z, R0;     // 2 (c0 - s), |c0 - s|
+    float phi0;
+    unsigned base;               // alpha n0 - SNAP_BITS (wrapping)
+    const float* row;            // the sensor's row of dconv
+};
+static_assert(sizeof(AssaRef) == 32, "two 16-byte loads");
+
+__global__ void __launch_bounds__(ASSA_ADJ_THREADS, ASSA_ADJ_CTAS)
 assa_adj_kernel(GaussDev g, ArrDev a, const float* __restrict__ dconv, const __grid_constant__ AssaTable T,
                 float* __restrict__ gA) {
-    __shared__ AdjRef refs2[2][ASSA_ADJ_SC];
+    __shared__ AssaRef refs2[2][ASSA_ADJ_SC];
     const int64_t t = blockIdx.x;
-    const int l = threadIdx.x, warp = l >> 5, lane = l & 31;
+    const int l = threadIdx.x;
     const int tx = (int)(t % g.ntx), ty = (int)((t / g.ntx) % g.nty), tz = (int)(t / ((int64_t)g.ntx * g.nty));
-    // warp w takes a 4 x 4 x 2 block of the 8 x 8 x 4 brick, so that the snapped positions of its
-    // 32 Gaussians for one sensor -- the residual entries it gathers -- stay close together
-    static_assert(BX == 8 && BY == 8 && BZ == 4 && TILE == 256, "brick of 8 x 8 x 4, 8 warps");
-    const int lx = (l & 3) | (((l >> 5) & 1) << 2), ly = ((l >> 2) & 3) | (((l >> 6) & 1) << 2),
-              lz = ((l >> 4) & 1) | (((l >> 7) & 1) << 1);
-    const int gx = tx * BX + lx, gy = ty * BY + ly, gz = tz * BZ + lz;
-    const bool valid = gx < g.nx && gy < g.ny && gz < g.nz;
-    const int64_t i = ((int64_t)gz * g.ny + gy) * g.nx + gx;
-    const float dx = ((float)lx - 0.5f * (BX - 1)) * g.h, dy = ((float)ly - 0.5f * (BY - 1)) * g.h,
-                dz = ((float)lz - 0.5f * (BZ - 1)) * g.h;
+    // a warp takes a 4 x 4 x 2 block of nodes per gather (planes 0 and 2, or 1 and 3), so that the snapped
+    // positions of its 32 Gaussians for one sensor -- the residual entries it gathers -- stay close together
+    static_assert(BX == 8 && BY == 8 && BZ == 4 && ASSA_ADJ_THREADS == 64, "brick of 8 x 8 x 4, 2 warps");
+    const int lx = l & 3, ly = ((l >> 2) & 3) | (((l >> 5) & 1) << 2), lz = ((l >> 4) & 1) << 1;
+    const int alpha = T.alpha, Nt = a.Nt;
+    const float aInvD = (float)alpha * a.invDelta;
+    const float dx0 = ((float)lx - 0.5f * (BX - 1)) * g.h, dx1 = ((float)(lx + 4) - 0.5f * (BX - 1)) * g.h;
+    const float dy = ((float)ly - 0.5f * (BY - 1)) * g.h;
+    const float2 dz = make_float2(((float)lz - 0.5f * (BZ - 1)) * g.h, ((float)(lz + 1) - 0.5f * (BZ - 1)) * g.h);
+    const float2 dx[2] = {make_float2(dx0, dx0), make_float2(dx1, dx1)}, dy2 = make_float2(dy, dy);
+    float2 d2[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) d2[u] = __ffma2_rn(dx[u], dx[u], __ffma2_rn(dy2, dy2, __fmul2_rn(dz, dz)));
     const double c0x = g.ox + (tx * BX + BX / 2) * (double)g.h;
     const double c0y = g.oy + (ty * BY + BY / 2) * (double)g.h;
     const double c0z = g.oz + (tz * BZ + BZ / 2) * (double)g.h;
-    const int alpha = T.alpha;
-    const int Nup = alpha * a.Nt;
-    const float aInvD = (float)alpha * a.invDelta;
-    constexpr int LASTW = TILE / 32 - 1;
-    const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    // the shared references carry alpha n0 (clamped) and the sensor's row j alpha Nt of dconv
-    auto ref_fine = [&](int j) {
-        const PairRef r = make_ref(c0x, c0y, c0z, a.xyz[3 * j], a.xyz[3 * j + 1], a.xyz[3 * j + 2], a);
-        return adj_ref(r, (int)((unsigned)assa_an0(alpha, r.n0) - SNAP_BITS), j * Nup);   // see assa_snap
+    const unsigned zero_entry = (unsigned)(alpha * Nt);
+    auto ref = [&](int j) {
+        const PairRef p = ref_doubled(make_ref(c0x, c0y, c0z, a.xyz[3 * j], a.xyz[3 * j + 1], a.xyz[3 * j + 2], a));
+        AssaRef r;
+        r.v2x = p.v0x; r.v2y = p.v0y; r.v2z = p.v0z;
+        r.R0 = p.R0;
+        r.phi0 = p.phi0;
+        r.base = (unsigned)assa_an0(alpha, p.n0) - SNAP_BITS;         // see assa_snap
+        r.row = dconv + (size_t)j * assa_dconv_row(alpha, Nt);
+        return r;
     };
-    KahanF kA;                       // across chunks; FP32 within a chunk of 32 sensors
-    if (warp == LASTW && lane < min(ASSA_ADJ_SC, a.Nd)) refs2[0][lane] = ref_fine(lane);
+    auto both = [](float v) { return make_float2(v, v); };
+    const float2 magic = both(SNAP_MAGIC), aD = both(aInvD);
+    KahanF kA[ASSA_ADJ_PER];         // FP32 over 32 sensors, compensated from there on
+    if (l < a.Nd) refs2[0][l] = ref(l);
     int cur = 0;
     for (int j0 = 0; j0 < a.Nd; j0 += ASSA_ADJ_SC, cur ^= 1) {
         const int nsc = min(ASSA_ADJ_SC, a.Nd - j0);
         __syncthreads();
-        if (warp == LASTW && j0 + ASSA_ADJ_SC + lane < a.Nd) refs2[cur ^ 1][lane] = ref_fine(j0 + ASSA_ADJ_SC + lane);
-        const AdjRef* refs = refs2[cur];
-        if (valid) {
-            float acc = 0.f;
-#pragma unroll 4
-            for (int q = 0; q < nsc; ++q) {
-                const AdjRef r = refs[q];
-                float invR, phi;
-                pair_phase_r(r, dx, dy, dz, d2, invR, phi);
-                const int k = assa_snap(phi, aInvD, (unsigned)r.n0);
-                if ((unsigned)k < (unsigned)Nup) acc = fmaf(__ldg(dconv + (size_t)(unsigned)(r.row + k)), invR, acc);
+        if (j0 + ASSA_ADJ_SC + l < a.Nd) refs2[cur ^ 1][l] = ref(j0 + ASSA_ADJ_SC + l);
+        for (int q0 = 0; q0 < nsc; q0 += 32) {
+            float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+            const AssaRef* rp = refs2[cur] + q0;
+            const int nq = min(32, nsc - q0);
+#pragma unroll 2
+            for (int q = 0; q < nq; ++q) {
+                const AssaRef r = rp[q];
+                const float2 R0 = both(r.R0);
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const float2 num = __ffma2_rn(dx[u], both(r.v2x), __ffma2_rn(dy2, both(r.v2y), __ffma2_rn(dz, both(r.v2z), d2[u])));
+                    const float2 R2 = __ffma2_rn(R0, R0, num);
+                    const float2 iR = make_float2(rsqrtf(R2.x), rsqrtf(R2.y));
+                    const float2 den = __ffma2_rn(R2, iR, R0);
+                    float2 rc;
+                    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc.x) : "f"(den.x));
+                    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc.y) : "f"(den.y));
+                    const float2 s = __ffma2_rn(__ffma2_rn(num, rc, both(r.phi0)), aD, magic);
+                    const unsigned ka = min((unsigned)__float_as_int(s.x) + r.base, zero_entry);
+                    const unsigned kb = min((unsigned)__float_as_int(s.y) + r.base, zero_entry);
+                    acc[u] = __ffma2_rn(make_float2(__ldg(r.row + ka), __ldg(r.row + kb)), iR, acc[u]);
+                }
             }
-            kA.add(acc);
+            kA[0].add(acc[0].x); kA[1].add(acc[0].y);
+            kA[2].add(acc[1].x); kA[3].add(acc[1].y);
         }
     }
-    if (valid) gA[i] = kA.s;
+#pragma unroll
+    for (int u = 0; u < ASSA_ADJ_PER; ++u) {
+        const int gx = tx * BX + lx + (u >> 1) * 4, gy = ty * BY + ly, gz = tz * BZ + lz + (u & 1);
+        if (gx < g.nx && gy < g.ny && gz < g.nz) gA[((int64_t)gz * g.ny + gy) * g.nx + gx] = kA[u].s;
+    }
 }
 
 // ---- host side -----------------------------------------------------------------------------
@@ -379,16 +422,16 @@ cudaError_t launch_assa_forward(const GaussDev& g, const ArrDev& a, const SlabIn
     return e;
 }
 
-size_t assa_dconv_bytes(const ArrDev& a, const AssaTable& T) { return (size_t)a.Nd * T.alpha * a.Nt * sizeof(float); }
+size_t assa_dconv_bytes(const ArrDev& a, const AssaTable& T) { return (size_t)a.Nd * assa_dconv_row(T.alpha, a.Nt) * sizeof(float); }
 
 cudaError_t launch_assa_adjoint(const GaussDev& g, const ArrDev& a, const float* delta, float* gA, const AssaTable& T,
                                 float* dconv, const cudaEvent_t* ev, cudaStream_t st) {
-    dim3 dgrid((T.alpha * a.Nt + 255) / 256, a.Nd);
+    dim3 dgrid((T.alpha * a.Nt + 256) / 256, a.Nd);
     assa_dconv_kernel<<<dgrid, 256, assa_dconv_smem(T), st>>>(delta, a.Nt, T, dconv);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (ev && (e = cudaEventRecord(ev[0], st)) != cudaSuccess) return e;
-    assa_adj_kernel<<<(unsigned)g.ntiles, TILE, 0, st>>>(g, a, dconv, T, gA);
+    assa_adj_kernel<<<(unsigned)g.ntiles, ASSA_ADJ_THREADS, 0, st>>>(g, a, dconv, T, gA);
     e = cudaGetLastError();
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], st);
     return e;
