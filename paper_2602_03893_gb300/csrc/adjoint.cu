@@ -10,11 +10,8 @@
 // global atomics.  Free-centre Gaussians are taken in the order of their window length (a
 // counting sort of the tile in shared memory), so the 32 threads of a warp walk windows of about
 // the same length.
-#include <cooperative_groups.h>
-
+#include "adjoint_split.cuh"
 #include "gpair_internal.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace gp {
 
@@ -303,13 +300,13 @@ adj_q_kernel(const float* __restrict__ delta, int Nt, const __grid_constant__ Mo
 //
 // Bound by instruction issue and by the gathers' L1 wavefronts.  With one Gaussian to a thread and scalar
 // arithmetic it took 57 instructions a pair: 14.96 ms for 256 x 256 x 128 Gaussians and 1024 sensors,
-// 10.5 ms now.
+// 9.7 ms now.
 //
 // A brick's sensors are divided over the CTAs of a cluster where there are too few bricks to fill the
 // chip; their sums meet in the first CTA's shared memory, in the order of the ranks.
 constexpr int ADJM_THREADS = 64, ADJM_PER = TILE / ADJM_THREADS;
 constexpr int ADJM_SC = 64;              // sensors per chunk; sums are compensated every 32
-constexpr int ADJM_CTAS = 12;            // resident per SM
+constexpr int ADJM_CTAS = 16;            // resident per SM (12: 1 to 3 % slower)
 struct __align__(16) AdjmRef {
     float v2x, v2y, v2z, R0;             // 2 (c0 - s), |c0 - s|
     float phi0;
@@ -447,20 +444,7 @@ adj_moment_kernel(GaussDev g, ArrDev a, const float* __restrict__ delta, const f
     float sum[ADJM_PER];
 #pragma unroll
     for (int u = 0; u < ADJM_PER; ++u) sum[u] = kA[u].s;
-    if (gridDim.y > 1) {
-        cg::cluster_group cl = cg::this_cluster();
-#pragma unroll
-        for (int u = 0; u < ADJM_PER; ++u) part[u * ADJM_THREADS + l] = sum[u];
-        cl.sync();
-        if (blockIdx.y == 0)
-            for (unsigned c = 1; c < gridDim.y; ++c) {
-                const float* other = cl.map_shared_rank(part, c);
-#pragma unroll
-                for (int u = 0; u < ADJM_PER; ++u) sum[u] += other[u * ADJM_THREADS + l];
-            }
-        cl.sync();                       // the others' shared memory stays until it has been read
-        if (blockIdx.y) return;
-    }
+    if (gridDim.y > 1 && !split_sum<ADJM_PER>(sum, part)) return;
 #pragma unroll
     for (int u = 0; u < ADJM_PER; ++u) {
         const int gx = tx * BX + lx + (u >> 1) * 4, gy = ty * BY + ly, gz = tz * BZ + lz + (u & 1);
@@ -470,33 +454,6 @@ adj_moment_kernel(GaussDev g, ArrDev a, const float* __restrict__ delta, const f
 }
 
 size_t adj_moment_q_bytes(const ArrDev& a, int L) { return (size_t)a.Nd * adj_q_row(a.Nt, L) * MOM_P * sizeof(float); }
-
-// CTAs that share a tile's sensors: as many (1, 2, 4, 8) as keep the grid within one wave of `ctas` per
-// SM, with at least 8 sensors each.  16 bricks and 128 sensors: 74 us for the 16 CTAs, 40 us for 8 times as many,
-// each with an eighth of the sensors (20 steps of a 16^3 reconstruction 2476 -> 1778 us).
-int adj_split(int64_t ntiles, int Nd, int ctas) {
-    int split = 1;
-    while (split < 8 && ntiles * split * 2 <= (int64_t)device_sms() * ctas && Nd >= 16 * split) split *= 2;
-    return split;
-}
-
-template <typename... Args>
-static cudaError_t launch_split(void (*kern)(Args...), unsigned tiles, int split, int threads, size_t smem,
-                                cudaStream_t st, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(tiles, split);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 1;
-    at[0].val.clusterDim.y = split;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = split > 1 ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, args...);
-}
 
 cudaError_t launch_adjoint_moment(const GaussDev& g, const ArrDev& a, const float* delta, float* gA,
                                   const MomentTable& T, float* Q, const cudaEvent_t* ev, cudaStream_t st) {

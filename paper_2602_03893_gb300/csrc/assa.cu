@@ -24,6 +24,7 @@
 #include <cmath>
 #include <cstring>
 
+#include "adjoint_split.cuh"
 #include "gpair_internal.cuh"
 
 namespace gp {
@@ -306,9 +307,10 @@ size_t assa_dconv_smem(const AssaTable& T) { return (size_t)((255 + 2 * T.K) / T
 // x + 4, two planes each; the planes through packed FP32 arithmetic, which rounds each half as the scalar
 // operation does).  The FP64 references of a chunk of 64 sensors, one to a thread, are
 // double-buffered.  A snapped sample outside the record reads the sensor's zero entry, one past its end.
+// A brick's sensors may be divided over the CTAs of a cluster.
 //
 // Bound by instruction issue.
-constexpr int ASSA_ADJ_THREADS = 64, ASSA_ADJ_PER = TILE / ASSA_ADJ_THREADS, ASSA_ADJ_CTAS = 16;
+constexpr int ASSA_ADJ_THREADS = 64, ASSA_ADJ_PER = TILE / ASSA_ADJ_THREADS, ASSA_ADJ_CTAS = 14;
 constexpr int ASSA_ADJ_SC = 64;
 struct __align__(16) AssaRef {
     float v2x, v2y, v2z, R0;     // 2 (c0 - s), |c0 - s|
@@ -318,10 +320,12 @@ struct __align__(16) AssaRef {
 };
 static_assert(sizeof(AssaRef) == 32, "two 16-byte loads");
 
+template <bool SPLIT>
 __global__ void __launch_bounds__(ASSA_ADJ_THREADS, ASSA_ADJ_CTAS)
 assa_adj_kernel(GaussDev g, ArrDev a, const float* __restrict__ dconv, const __grid_constant__ AssaTable T,
-                float* __restrict__ gA) {
+                float* __restrict__ gA, int per) {
     __shared__ AssaRef refs2[2][ASSA_ADJ_SC];
+    __shared__ float part[SPLIT ? TILE : 1];
     const int64_t t = blockIdx.x;
     const int l = threadIdx.x;
     const int tx = (int)(t % g.ntx), ty = (int)((t / g.ntx) % g.nty), tz = (int)(t / ((int64_t)g.ntx * g.nty));
@@ -355,17 +359,18 @@ assa_adj_kernel(GaussDev g, ArrDev a, const float* __restrict__ dconv, const __g
     auto both = [](float v) { return make_float2(v, v); };
     const float2 magic = both(SNAP_MAGIC), aD = both(aInvD);
     KahanF kA[ASSA_ADJ_PER];         // FP32 over 32 sensors, compensated from there on
-    if (l < a.Nd) refs2[0][l] = ref(l);
+    const int jb = SPLIT ? blockIdx.y * per : 0, je = SPLIT ? min(a.Nd, jb + per) : a.Nd;
+    if (jb + l < je) refs2[0][l] = ref(jb + l);
     int cur = 0;
-    for (int j0 = 0; j0 < a.Nd; j0 += ASSA_ADJ_SC, cur ^= 1) {
-        const int nsc = min(ASSA_ADJ_SC, a.Nd - j0);
+    for (int j0 = jb; j0 < je; j0 += ASSA_ADJ_SC, cur ^= 1) {
+        const int nsc = min(ASSA_ADJ_SC, je - j0);
         __syncthreads();
-        if (j0 + ASSA_ADJ_SC + l < a.Nd) refs2[cur ^ 1][l] = ref(j0 + ASSA_ADJ_SC + l);
+        if (j0 + ASSA_ADJ_SC + l < je) refs2[cur ^ 1][l] = ref(j0 + ASSA_ADJ_SC + l);
         for (int q0 = 0; q0 < nsc; q0 += 32) {
             float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
             const AssaRef* rp = refs2[cur] + q0;
             const int nq = min(32, nsc - q0);
-#pragma unroll 2
+#pragma unroll 4
             for (int q = 0; q < nq; ++q) {
                 const AssaRef r = rp[q];
                 const float2 R0 = both(r.R0);
@@ -388,10 +393,15 @@ assa_adj_kernel(GaussDev g, ArrDev a, const float* __restrict__ dconv, const __g
             kA[2].add(acc[1].x); kA[3].add(acc[1].y);
         }
     }
+    float sum[ASSA_ADJ_PER];
+#pragma unroll
+    for (int u = 0; u < ASSA_ADJ_PER; ++u) sum[u] = kA[u].s;
+    if constexpr (SPLIT)
+        if (!split_sum<ASSA_ADJ_PER>(sum, part)) return;
 #pragma unroll
     for (int u = 0; u < ASSA_ADJ_PER; ++u) {
         const int gx = tx * BX + lx + (u >> 1) * 4, gy = ty * BY + ly, gz = tz * BZ + lz + (u & 1);
-        if (gx < g.nx && gy < g.ny && gz < g.nz) gA[((int64_t)gz * g.ny + gy) * g.nx + gx] = kA[u].s;
+        if (gx < g.nx && gy < g.ny && gz < g.nz) gA[((int64_t)gz * g.ny + gy) * g.nx + gx] = sum[u];
     }
 }
 
@@ -431,8 +441,9 @@ cudaError_t launch_assa_adjoint(const GaussDev& g, const ArrDev& a, const float*
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (ev && (e = cudaEventRecord(ev[0], st)) != cudaSuccess) return e;
-    assa_adj_kernel<<<(unsigned)g.ntiles, ASSA_ADJ_THREADS, 0, st>>>(g, a, dconv, T, gA);
-    e = cudaGetLastError();
+    const int split = adj_split(g.ntiles, a.Nd, ASSA_ADJ_CTAS);
+    e = launch_split(split > 1 ? assa_adj_kernel<true> : assa_adj_kernel<false>, (unsigned)g.ntiles, split, ASSA_ADJ_THREADS, 0, st, g, a, (const float*)dconv, T,
+                     gA, (a.Nd + split - 1) / split);
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], st);
     return e;
 }

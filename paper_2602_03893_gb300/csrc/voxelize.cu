@@ -376,7 +376,7 @@ vox_prepare_kernel(GaussDev g, gpair_grid og, float k, const int* __restrict__ p
     }
 }
 
-__global__ void __launch_bounds__(VT_WARPS * 32)
+__global__ void __launch_bounds__(VT_WARPS * 32, 4)
 vox_tile_kernel(gpair_grid og, VoxSet V, int ntx, int nty, float* __restrict__ vol) {
     __shared__ __align__(16) float F[VT_WARPS][VT_GROUP * VT_ROW];
     __shared__ int queue[VT_WARPS][2 * VT_GROUP];
