@@ -3,73 +3,91 @@
 // of a tile lie close together and the sensor-lane kernel's sample bands stay short.  The
 // forward is a sum over Gaussians, so the order changes its result only by FP32 summation order.
 //
-// The order is a stable LSD radix sort of 18-bit Morton keys (64 cells per axis, finer than a
-// tile of 256 Gaussians needs) in two passes of 9 bits: per-block histograms, one exclusive scan
-// in (digit, block) order, and a scatter whose ranks inside a block follow the index order
-// through warp-level match masks.  Deterministic: equal keys keep their index order.  Then one
-// gather writes the permuted centres, widths and amplitudes.
+// The order is a stable sort of 18-bit Morton keys (64 cells per axis, finer than a tile of 256
+// Gaussians needs): equal keys keep their index order, so the result is deterministic.
+// Up to SO_ONE_MAX Gaussians one CTA does all of it, a bitonic sort of (key, index) words in shared
+// memory: ten launches less.  Larger sets go through an LSD radix sort in two passes of 9 bits:
+// per-block digit counts, a scan of each digit's counts over the blocks, and a scatter whose
+// ranks inside a block follow the index order through warp-level match masks.  Then one gather
+// writes the permuted centres, widths and amplitudes.
+//
+// Latency and launches bound it at every size in use.  262,144 Gaussians: 131 us with blocks of 4096
+// keys (64 CTAs) and one CTA scanning all counts, 46 us now; 1500: 57 us, 20 us now.
 #include <cfloat>
 
 #include "gpair_internal.cuh"
 
 namespace gp {
 
-constexpr int SO_THREADS = 256;
-constexpr int SO_CHUNK = SO_THREADS * 16;   // keys per block of a radix pass
+constexpr int SO_THREADS = 256, SO_WARPS = SO_THREADS / 32;
 constexpr int SO_BB_BLOCKS = 256;           // blocks of the bounding-box reduction
 constexpr int SO_AXIS_BITS = 6;             // Morton key: 6 bits per axis
 constexpr int SO_DIGIT = 9, SO_RADIX = 1 << SO_DIGIT, SO_PASSES = 3 * SO_AXIS_BITS / SO_DIGIT;
+constexpr int SO_ONE_THREADS = 1024, SO_ONE_BITS = 13, SO_ONE_MAX = 1 << SO_ONE_BITS;
+static_assert(SO_ONE_BITS + 3 * SO_AXIS_BITS < 32, "key and index in one word, the last word free");
+static_assert(SO_BB_BLOCKS == SO_THREADS, "a block joins the boxes, one to a thread");
 
-__host__ __device__ __forceinline__ int so_blocks(int64_t M) { return (int)((M + SO_CHUNK - 1) / SO_CHUNK); }
+// Keys per block of a radix pass: 1024, more where that would be over 1024 blocks.
+inline int64_t so_chunk(int64_t M) {
+    int64_t c = 1024;
+    while ((M + c - 1) / c > 1024) c *= 2;
+    return c;
+}
+inline int so_blocks(int64_t M) { return (int)((M + so_chunk(M) - 1) / so_chunk(M)); }
 inline size_t align256_sz(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// scratch: keys[2][M], vals[2][M], histogram [radix][blocks], box partials, permuted arrays [5][M]
+// scratch: keys[2][M], vals[2][M], counts [radix][blocks] and [radix] totals, box partials, permuted arrays [5][M]
 size_t spatial_order_bytes(int64_t M) {
     const size_t a = align256_sz((size_t)M * 4);
-    return 4 * a + align256_sz((size_t)SO_RADIX * so_blocks(M) * 4) + align256_sz((size_t)(SO_BB_BLOCKS + 1) * 6 * 4) +
+    return 4 * a + align256_sz((size_t)SO_RADIX * (so_blocks(M) + 1) * 4) + align256_sz((size_t)SO_BB_BLOCKS * 6 * 4) +
            5 * a;
 }
 
-// Per-block minima and maxima of the centres (grid-stride), then their reduction by one block.
-__global__ void so_box_partial_kernel(GaussDev g, float* __restrict__ part) {
-    __shared__ float red[6][SO_THREADS];
-    float mn[3] = {FLT_MAX, FLT_MAX, FLT_MAX}, mx[3] = {-FLT_MAX, -FLT_MAX, -FLT_MAX};
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.M; i += (int64_t)gridDim.x * blockDim.x) {
-        const float c[3] = {g.cx[i], g.cy[i], g.cz[i]};
+struct SoBox { float mn[3], mx[3]; };
+
+__device__ __forceinline__ void so_join(SoBox& b, const SoBox& o) {
 #pragma unroll
-        for (int q = 0; q < 3; ++q) { mn[q] = fminf(mn[q], c[q]); mx[q] = fmaxf(mx[q], c[q]); }
-    }
-#pragma unroll
-    for (int q = 0; q < 3; ++q) { red[q][threadIdx.x] = mn[q]; red[3 + q][threadIdx.x] = mx[q]; }
-    __syncthreads();
-    for (int s = SO_THREADS / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s)
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                red[q][threadIdx.x] = fminf(red[q][threadIdx.x], red[q][threadIdx.x + s]);
-                red[3 + q][threadIdx.x] = fmaxf(red[3 + q][threadIdx.x], red[3 + q][threadIdx.x + s]);
-            }
-        __syncthreads();
-    }
-    if (threadIdx.x < 6) part[blockIdx.x * 6 + threadIdx.x] = red[threadIdx.x][0];
+    for (int q = 0; q < 3; ++q) { b.mn[q] = fminf(b.mn[q], o.mn[q]); b.mx[q] = fmaxf(b.mx[q], o.mx[q]); }
 }
 
-// One block of SO_BB_BLOCKS threads: thread b takes block b's partials, then a tree.
-__global__ void so_box_final_kernel(const float* __restrict__ part, float* __restrict__ box) {
-    __shared__ float red[6][SO_BB_BLOCKS];
+// Join over the block (every thread gets it); sh: one box per warp.
+__device__ __forceinline__ SoBox so_block_join(SoBox b, SoBox* sh) {
 #pragma unroll
-    for (int q = 0; q < 6; ++q) red[q][threadIdx.x] = part[threadIdx.x * 6 + q];
-    __syncthreads();
-    for (int s = SO_BB_BLOCKS / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s)
+    for (int o = 16; o > 0; o >>= 1) {
+        SoBox v;
 #pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                red[q][threadIdx.x] = fminf(red[q][threadIdx.x], red[q][threadIdx.x + s]);
-                red[3 + q][threadIdx.x] = fmaxf(red[3 + q][threadIdx.x], red[3 + q][threadIdx.x + s]);
-            }
-        __syncthreads();
+        for (int q = 0; q < 3; ++q) {
+            v.mn[q] = __shfl_xor_sync(0xffffffffu, b.mn[q], o);
+            v.mx[q] = __shfl_xor_sync(0xffffffffu, b.mx[q], o);
+        }
+        so_join(b, v);
     }
-    if (threadIdx.x < 6) box[threadIdx.x] = red[threadIdx.x][0];
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = b;
+    __syncthreads();
+    b = sh[0];
+    for (int w = 1; w < (int)blockDim.x / 32; ++w) so_join(b, sh[w]);
+    return b;
+}
+
+__device__ __forceinline__ SoBox so_empty() {
+    return {{FLT_MAX, FLT_MAX, FLT_MAX}, {-FLT_MAX, -FLT_MAX, -FLT_MAX}};
+}
+
+__device__ __forceinline__ SoBox so_range_box(const GaussDev& g, int64_t first, int64_t stride) {
+    SoBox b = so_empty();
+    for (int64_t i = first; i < g.M; i += stride) {
+        const float c[3] = {g.cx[i], g.cy[i], g.cz[i]};
+#pragma unroll
+        for (int q = 0; q < 3; ++q) { b.mn[q] = fminf(b.mn[q], c[q]); b.mx[q] = fmaxf(b.mx[q], c[q]); }
+    }
+    return b;
+}
+
+__global__ void __launch_bounds__(SO_THREADS) so_box_kernel(GaussDev g, SoBox* __restrict__ part) {
+    __shared__ SoBox sh[SO_WARPS];
+    const SoBox b = so_block_join(so_range_box(g, blockIdx.x * (int64_t)SO_THREADS + threadIdx.x,
+                                               (int64_t)gridDim.x * SO_THREADS), sh);
+    if (threadIdx.x == 0) part[blockIdx.x] = b;
 }
 
 // the axis bits spread three apart (bit b to bit 3b), for interleaving x, y, z from the lowest bit
@@ -80,145 +98,21 @@ __device__ __forceinline__ uint32_t spread_bits(uint32_t v) {
     return r;
 }
 
-__global__ void so_keys_kernel(GaussDev g, const float* __restrict__ box, uint32_t* __restrict__ keys,
-                               int* __restrict__ vals) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= g.M) return;
+__device__ __forceinline__ uint32_t so_key(const GaussDev& g, const SoBox& box, int64_t i) {
     const float c[3] = {g.cx[i], g.cy[i], g.cz[i]};
     uint32_t k = 0;
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
-        const float lo = box[q], ext = box[3 + q] - lo;
+        const float lo = box.mn[q], ext = box.mx[q] - lo;
         const float t = ext > 0.f ? (c[q] - lo) / ext : 0.f;
         const float top = (float)((1 << SO_AXIS_BITS) - 1);
         const uint32_t u = (uint32_t)fminf(fmaxf(t * top, 0.f), top);
         k |= spread_bits(u) << q;
     }
-    keys[i] = k;
-    vals[i] = (int)i;
+    return k;
 }
 
-// Radix pass, step 1: the block's digit counts, stored digit-major: hist[d * nblocks + block].
-__global__ void so_hist_kernel(const uint32_t* __restrict__ keys, int64_t n, int shift, int* __restrict__ hist) {
-    __shared__ int h[SO_RADIX];
-    for (int d = threadIdx.x; d < SO_RADIX; d += SO_THREADS) h[d] = 0;
-    __syncthreads();
-    const int64_t b0 = (int64_t)blockIdx.x * SO_CHUNK;
-    for (int q = threadIdx.x; q < SO_CHUNK; q += SO_THREADS) {
-        const int64_t i = b0 + q;
-        if (i < n) atomicAdd(&h[(keys[i] >> shift) & (SO_RADIX - 1)], 1);
-    }
-    __syncthreads();
-    for (int d = threadIdx.x; d < SO_RADIX; d += SO_THREADS) hist[(int64_t)d * gridDim.x + blockIdx.x] = h[d];
-}
-
-// Step 2: exclusive scan of the counts in (digit, block) order, i.e. of hist as one flat array.
-// One block walks the array in tiles of SO_SCAN_THREADS x SO_SCAN_ITEMS entries: each thread loads
-// its SO_SCAN_ITEMS consecutive entries (all loads of a tile in flight together), the block scans
-// the thread sums with warp shuffles, and each thread writes its entries' running offsets; a
-// carry takes the tile's total to the next tile.
-constexpr int SO_SCAN_THREADS = 1024;
-constexpr int SO_SCAN_ITEMS = 8;
-__global__ void __launch_bounds__(SO_SCAN_THREADS) so_scan_kernel(int* __restrict__ hist, int nb) {
-    __shared__ int wsum[SO_SCAN_THREADS / 32];
-    __shared__ int carry_s;
-    const int64_t N = (int64_t)SO_RADIX * nb;
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    constexpr int64_t TILE_N = (int64_t)SO_SCAN_THREADS * SO_SCAN_ITEMS;
-    int carry = 0;
-    for (int64_t base = 0; base < N; base += TILE_N) {
-        const int64_t a = base + (int64_t)t * SO_SCAN_ITEMS;
-        int v[SO_SCAN_ITEMS];
-        int s = 0;
-#pragma unroll
-        for (int k = 0; k < SO_SCAN_ITEMS; ++k) {
-            v[k] = a + k < N ? hist[a + k] : 0;
-            s += v[k];
-        }
-        int x = s;                                   // inclusive scan over the warp
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int u = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += u;
-        }
-        if (lane == 31) wsum[w] = x;
-        __syncthreads();
-        if (w == 0) {                                // inclusive scan of the warp totals
-            int y = wsum[lane];
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int u = __shfl_up_sync(0xffffffffu, y, o);
-                if (lane >= o) y += u;
-            }
-            wsum[lane] = y;
-            if (lane == 31) carry_s = y;             // the tile's total
-        }
-        __syncthreads();
-        int run = carry + x - s + (w ? wsum[w - 1] : 0);
-#pragma unroll
-        for (int k = 0; k < SO_SCAN_ITEMS; ++k) {
-            if (a + k < N) hist[a + k] = run;
-            run += v[k];
-        }
-        carry += carry_s;
-        __syncthreads();                             // wsum and carry_s are reused by the next tile
-    }
-}
-
-// Step 3: stable scatter.  The block takes its keys 256 at a time in index order; inside a warp
-// the lanes of equal digit find each other with a match mask (rank = lower lanes of the same
-// digit), the warps' counts per digit give each warp its start, and a running count per digit
-// carries the offsets from one round to the next.
-__global__ void so_scatter_kernel(const uint32_t* __restrict__ kin, const int* __restrict__ vin, int64_t n, int shift,
-                                  const int* __restrict__ hist, uint32_t* __restrict__ kout, int* __restrict__ vout) {
-    __shared__ int base[SO_RADIX], run[SO_RADIX];
-    __shared__ int wcnt[SO_THREADS / 32][SO_RADIX];
-    const int t = threadIdx.x, warp = t >> 5;
-    for (int d = t; d < SO_RADIX; d += SO_THREADS) {
-        base[d] = hist[(int64_t)d * gridDim.x + blockIdx.x];
-        run[d] = 0;
-        for (int w = 0; w < SO_THREADS / 32; ++w) wcnt[w][d] = 0;
-    }
-    __syncthreads();
-    uint32_t lt;
-    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(lt));
-    const int64_t b0 = (int64_t)blockIdx.x * SO_CHUNK;
-    for (int r = 0; r < SO_CHUNK / SO_THREADS; ++r) {
-        const int64_t i = b0 + r * SO_THREADS + t;
-        const bool ok = i < n;
-        const uint32_t key = ok ? kin[i] : 0u;
-        const int val = ok ? vin[i] : 0;
-        const int d = ok ? (int)((key >> shift) & (SO_RADIX - 1)) : SO_RADIX;     // SO_RADIX: no key
-        const uint32_t peers = __match_any_sync(0xffffffffu, d);
-        const int rank = __popc(peers & lt);
-        if (ok && rank == 0) wcnt[warp][d] = __popc(peers);
-        __syncthreads();
-        for (int dd = t; dd < SO_RADIX; dd += SO_THREADS) {   // each warp's start inside the block, then the running count
-            int acc = run[dd];
-            for (int w = 0; w < SO_THREADS / 32; ++w) {
-                const int c = wcnt[w][dd];
-                wcnt[w][dd] = acc;
-                acc += c;
-            }
-            run[dd] = acc;
-        }
-        __syncthreads();
-        if (ok) {
-            const int pos = base[d] + wcnt[warp][d] + rank;
-            kout[pos] = key;
-            vout[pos] = val;
-        }
-        __syncthreads();
-        for (int dd = t; dd < SO_RADIX; dd += SO_THREADS)
-            for (int w = 0; w < SO_THREADS / 32; ++w) wcnt[w][dd] = 0;
-        __syncthreads();
-    }
-}
-
-__global__ void so_gather_kernel(GaussDev g, const int* __restrict__ perm, float* __restrict__ out) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= g.M) return;
-    const int64_t j = perm[i];
+__device__ __forceinline__ void so_gather_one(const GaussDev& g, int64_t i, int64_t j, float* __restrict__ out) {
     const int64_t M = g.M;
     out[i] = g.cx[j];
     out[M + i] = g.cy[j];
@@ -227,43 +121,196 @@ __global__ void so_gather_kernel(GaussDev g, const int* __restrict__ perm, float
     out[4 * M + i] = g.A[j];
 }
 
-// perm: the order as indices of g, in scratch (spatial_order_bytes(g.M)).
-cudaError_t launch_spatial_perm(const GaussDev& g, void* scratch, const int** perm, cudaStream_t st) {
+// The whole order of up to SO_ONE_MAX Gaussians: Mp words (a power of two of at least 64) of dynamic
+// shared memory.  out (may be null): the permuted arrays.
+__global__ void __launch_bounds__(SO_ONE_THREADS)
+so_one_kernel(GaussDev g, int Mp, int* __restrict__ perm, float* __restrict__ out) {
+    extern __shared__ uint32_t so_word[];
+    __shared__ SoBox sh[SO_ONE_THREADS / 32];
+    const int M = (int)g.M, t = threadIdx.x;
+    const SoBox box = so_block_join(so_range_box(g, t, SO_ONE_THREADS), sh);
+    for (int i = t; i < Mp; i += SO_ONE_THREADS)
+        so_word[i] = i < M ? so_key(g, box, i) << SO_ONE_BITS | (uint32_t)i : 0xffffffffu;
+    __syncthreads();
+    for (int k = 2; k <= Mp; k <<= 1)
+        for (int h = k >> 1; h > 0; h >>= 1) {
+            for (int u = t; u < Mp / 2; u += SO_ONE_THREADS) {
+                const int i = ((u & ~(h - 1)) << 1) | (u & (h - 1));
+                const uint32_t a = so_word[i], b = so_word[i + h];
+                if ((a > b) == ((i & k) == 0)) { so_word[i] = b; so_word[i + h] = a; }
+            }
+            // pairs of up to 32 words apart stay inside a warp's 64 words
+            if (h > 32 || h == 1) __syncthreads(); else __syncwarp();
+        }
+    for (int i = t; i < M; i += SO_ONE_THREADS) {
+        const int j = (int)(so_word[i] & (SO_ONE_MAX - 1));
+        perm[i] = j;
+        if (out) so_gather_one(g, i, j, out);
+    }
+}
+
+// Radix pass, step 1: the block's digit counts, stored digit-major: hist[d * nblocks + block].  The
+// first pass (g.M > 0 keys to form) joins the boxes and writes the keys and indices too.
+template <bool FIRST>
+__global__ void __launch_bounds__(SO_THREADS)
+so_hist_kernel(GaussDev g, const SoBox* __restrict__ part, uint32_t* __restrict__ keys, int* __restrict__ vals,
+               int64_t chunk, int shift, int* __restrict__ hist) {
+    __shared__ int h[SO_RADIX];
+    __shared__ SoBox sh[SO_WARPS];
+    for (int d = threadIdx.x; d < SO_RADIX; d += SO_THREADS) h[d] = 0;
+    SoBox box;
+    if (FIRST) box = so_block_join(part[threadIdx.x], sh);
+    __syncthreads();
+    const int64_t b0 = blockIdx.x * chunk;
+    for (int64_t q = threadIdx.x; q < chunk; q += SO_THREADS) {
+        const int64_t i = b0 + q;
+        if (i >= g.M) break;
+        uint32_t k;
+        if (FIRST) {
+            k = so_key(g, box, i);
+            keys[i] = k;
+            vals[i] = (int)i;
+        } else {
+            k = keys[i];
+        }
+        atomicAdd(&h[(k >> shift) & (SO_RADIX - 1)], 1);
+    }
+    __syncthreads();
+    for (int d = threadIdx.x; d < SO_RADIX; d += SO_THREADS) hist[(int64_t)d * gridDim.x + blockIdx.x] = h[d];
+}
+
+// Step 2: one warp per digit: the exclusive scan of its counts over the blocks, and its total.
+__global__ void __launch_bounds__(SO_THREADS) so_scan_kernel(int* __restrict__ hist, int nb, int* __restrict__ total) {
+    const int d = blockIdx.x * SO_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    int* row = hist + (int64_t)d * nb;
+    int carry = 0;
+    for (int b0 = 0; b0 < nb; b0 += 32) {
+        const int v = b0 + lane < nb ? row[b0 + lane] : 0;
+        int x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += u;
+        }
+        if (b0 + lane < nb) row[b0 + lane] = carry + x - v;
+        carry += __shfl_sync(0xffffffffu, x, 31);
+    }
+    if (lane == 0) total[d] = carry;
+}
+
+// Step 3: stable scatter.  Each warp owns a contiguous eighth of the block's keys: it counts its
+// digits, the warps' counts give each its start per digit, and it then takes its keys 32 at a time
+// in index order, the lanes of equal digit ranked by a match mask.
+__global__ void __launch_bounds__(SO_THREADS)
+so_scatter_kernel(const uint32_t* __restrict__ kin, const int* __restrict__ vin, int64_t n, int64_t chunk, int shift,
+                  const int* __restrict__ hist, const int* __restrict__ total, uint32_t* __restrict__ kout,
+                  int* __restrict__ vout) {
+    __shared__ int cnt[SO_WARPS][SO_RADIX];
+    __shared__ int wsum[SO_WARPS];
+    static_assert(SO_RADIX == 2 * SO_THREADS, "two digits a thread");
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    for (int q = t; q < SO_WARPS * SO_RADIX; q += SO_THREADS) (&cnt[0][0])[q] = 0;
+    // where each digit begins: thread t scans the totals of digits 2t and 2t + 1
+    const int t0 = total[2 * t], t1 = total[2 * t + 1];
+    int x = t0 + t1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += u;
+    }
+    if (lane == 31) wsum[warp] = x;
+    __syncthreads();
+    const int64_t seg = chunk / SO_WARPS, s0 = blockIdx.x * chunk + warp * seg;
+    const int64_t s1 = s0 + seg < n ? s0 + seg : n;
+    for (int64_t i = s0 + lane; i < s1; i += 32) atomicAdd(&cnt[warp][(kin[i] >> shift) & (SO_RADIX - 1)], 1);
+    int start = x - t0 - t1;
+    for (int w = 0; w < warp; ++w) start += wsum[w];
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int d = 2 * t + k;
+        int acc = start + (k ? t0 : 0) + hist[(int64_t)d * gridDim.x + blockIdx.x];
+#pragma unroll
+        for (int w = 0; w < SO_WARPS; ++w) {
+            const int c = cnt[w][d];
+            cnt[w][d] = acc;
+            acc += c;
+        }
+    }
+    __syncthreads();
+    uint32_t lt;
+    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(lt));
+    for (int64_t i0 = s0; i0 < s1; i0 += 32) {
+        const int64_t i = i0 + lane;
+        const bool ok = i < s1;
+        const uint32_t key = ok ? kin[i] : 0u;
+        const int val = ok ? vin[i] : 0;
+        const int d = ok ? (int)((key >> shift) & (SO_RADIX - 1)) : SO_RADIX;     // SO_RADIX: no key
+        const uint32_t peers = __match_any_sync(0xffffffffu, d);
+        const int rank = __popc(peers & lt);
+        const int at = ok ? cnt[warp][d] : 0;
+        __syncwarp();
+        if (ok && rank == 0) cnt[warp][d] = at + __popc(peers);
+        if (ok) {
+            kout[at + rank] = key;
+            vout[at + rank] = val;
+        }
+        __syncwarp();
+    }
+}
+
+__global__ void so_gather_kernel(GaussDev g, const int* __restrict__ perm, float* __restrict__ out) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i < g.M) so_gather_one(g, i, perm[i], out);
+}
+
+// The order as indices of g, in scratch; out (may be null): the permuted arrays.
+static cudaError_t spatial_sort(const GaussDev& g, void* scratch, const int** perm, float* out, cudaStream_t st) {
     const int64_t M = g.M;
     if (M > 0x7FFFFFFF) return cudaErrorNotSupported;
     const size_t a = align256_sz((size_t)M * 4);
     char* p = static_cast<char*>(scratch);
     uint32_t* keys[2] = {reinterpret_cast<uint32_t*>(p), reinterpret_cast<uint32_t*>(p + a)};
     int* vals[2] = {reinterpret_cast<int*>(p + 2 * a), reinterpret_cast<int*>(p + 3 * a)};
+    *perm = vals[0];
+    if (M <= SO_ONE_MAX) {
+        int Mp = 64;
+        while (Mp < M) Mp <<= 1;
+        so_one_kernel<<<1, SO_ONE_THREADS, (size_t)Mp * 4, st>>>(g, Mp, vals[0], out);
+        return cudaGetLastError();
+    }
     const int nb = so_blocks(M);
+    const int64_t chunk = so_chunk(M);
     int* hist = reinterpret_cast<int*>(p + 4 * a);
-    float* boxp = reinterpret_cast<float*>(p + 4 * a + align256_sz((size_t)SO_RADIX * nb * 4));
-    float* box = boxp + SO_BB_BLOCKS * 6;
-    so_box_partial_kernel<<<SO_BB_BLOCKS, SO_THREADS, 0, st>>>(g, boxp);
-    so_box_final_kernel<<<1, SO_BB_BLOCKS, 0, st>>>(boxp, box);
-    const unsigned eb = (unsigned)((M + 255) / 256);
-    so_keys_kernel<<<eb, 256, 0, st>>>(g, box, keys[0], vals[0]);
+    int* total = hist + (size_t)SO_RADIX * nb;
+    SoBox* part = reinterpret_cast<SoBox*>(p + 4 * a + align256_sz((size_t)SO_RADIX * (nb + 1) * 4));
+    so_box_kernel<<<SO_BB_BLOCKS, SO_THREADS, 0, st>>>(g, part);
     for (int pass = 0; pass < SO_PASSES; ++pass) {
-        const int in = pass & 1;
-        so_hist_kernel<<<nb, SO_THREADS, 0, st>>>(keys[in], M, SO_DIGIT * pass, hist);
-        so_scan_kernel<<<1, SO_SCAN_THREADS, 0, st>>>(hist, nb);
-        so_scatter_kernel<<<nb, SO_THREADS, 0, st>>>(keys[in], vals[in], M, SO_DIGIT * pass, hist, keys[in ^ 1],
+        const int in = pass & 1, shift = SO_DIGIT * pass;
+        if (pass == 0) so_hist_kernel<true><<<nb, SO_THREADS, 0, st>>>(g, part, keys[in], vals[in], chunk, shift, hist);
+        else so_hist_kernel<false><<<nb, SO_THREADS, 0, st>>>(g, part, keys[in], vals[in], chunk, shift, hist);
+        so_scan_kernel<<<SO_RADIX / SO_WARPS, SO_THREADS, 0, st>>>(hist, nb, total);
+        so_scatter_kernel<<<nb, SO_THREADS, 0, st>>>(keys[in], vals[in], M, chunk, shift, hist, total, keys[in ^ 1],
                                                      vals[in ^ 1]);
     }
     static_assert(SO_PASSES % 2 == 0, "the order ends in buffer 0");
-    *perm = vals[0];
+    if (out) so_gather_kernel<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(g, vals[0], out);
     return cudaGetLastError();
+}
+
+// perm: the order as indices of g, in scratch (spatial_order_bytes(g.M)).
+cudaError_t launch_spatial_perm(const GaussDev& g, void* scratch, const int** perm, cudaStream_t st) {
+    return spatial_sort(g, scratch, perm, nullptr, st);
 }
 
 // gp: g with its arrays replaced by the permuted copies in scratch (spatial_order_bytes(g.M)).
 cudaError_t launch_spatial_order(const GaussDev& g, void* scratch, GaussDev& gp, cudaStream_t st) {
     const int64_t M = g.M;
     const int* perm = nullptr;
-    const cudaError_t e = launch_spatial_perm(g, scratch, &perm, st);
-    if (e != cudaSuccess) return e;
     float* out = reinterpret_cast<float*>(static_cast<char*>(scratch) + spatial_order_bytes(M) -
                                           5 * align256_sz((size_t)M * 4));
-    so_gather_kernel<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(g, perm, out);
+    const cudaError_t e = spatial_sort(g, scratch, &perm, out, st);
+    if (e != cudaSuccess) return e;
     gp = g;
     gp.cx = out;
     gp.cy = out + M;
