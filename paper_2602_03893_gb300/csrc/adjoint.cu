@@ -17,75 +17,73 @@ namespace gp {
 
 constexpr int ADJ_THREADS = TILE;
 constexpr int ADJ_SC = 32;   // sensors staged per chunk
+constexpr int ADJ_CTAS = 4;  // resident per SM
 constexpr int ADJ_KEYS = 64; // window-length keys of the free-centre ordering
 constexpr float ADJ_MAGIC = 12582912.0f;    // 1.5 * 2^23: x + MAGIC, rounded up (down), holds ceil(x) (floor(x))
 constexpr int ADJ_MAGIC_BITS = 0x4B400000;
 
 
 
-// Window sums of one pair: s1 = sum dl d e (amplitude gradient); with FULL also s0 = sum dl e,
-// s2 = sum dl d^2 e, s3 = sum dl d^3 e (centre and width gradients).  src[m] is the residual at
+// Window sums of one pair: s1 = sum dl d e (amplitude gradient); with FULL also sR = sum dl (1 - d^2 /
+// sigma^2) e and s3 = sum dl d^3 e (distance and width gradients).  src[m] is the residual at
 // sample n0 + m; d = phi - m Delta is the pair's phase there.  Samples go two at a time through
 // packed FP32 pairs (mul/add/fma .f32x2), the even and odd samples in the two halves of each
 // accumulator; an odd window's last pair has its second residual set to zero.
+constexpr float ADJ_2LN2 = 1.38629436111989061883f;     // d^2 / sigma^2 = -2 ln 2 (d^2 c2)
 template <bool FULL>
 __device__ __forceinline__ void window_sums(const float* __restrict__ src, int m_lo, int m_hi, float phi,
-                                            float Delta, float c2, float& s0, float& s1, float& s2, float& s3) {
+                                            float Delta, float c2, float& sR, float& s1, float& s3) {
     float2 fm = make_float2((float)m_lo, (float)(m_lo + 1));     // m as floats, stepped exactly
     const float2 two = make_float2(2.f, 2.f), nD = make_float2(-Delta, -Delta), cc = make_float2(c2, c2);
-    const float2 ph = make_float2(phi, phi);
-    float2 S0 = make_float2(0.f, 0.f), S1 = S0, S2 = S0, S3 = S0;
+    const float2 ph = make_float2(phi, phi), one = make_float2(1.f, 1.f), l2 = make_float2(ADJ_2LN2, ADJ_2LN2);
+    float2 SR = make_float2(0.f, 0.f), S1 = SR, S3 = SR;
     for (int m = m_lo; m <= m_hi; m += 2, fm = __fadd2_rn(fm, two)) {
         const float2 d = __ffma2_rn(fm, nD, ph);
-        const float2 E = __fmul2_rn(__fmul2_rn(d, d), cc);
+        const float2 dd = __fmul2_rn(d, d), E = __fmul2_rn(dd, cc);
         const float x0 = src[m], x1 = m + 1 <= m_hi ? src[m + 1] : 0.f;
         const float2 u = __fmul2_rn(make_float2(x0, x1), make_float2(ex2_approx(E.x), ex2_approx(E.y)));
         if (FULL) {
             const float2 ud = __fmul2_rn(u, d);
-            const float2 udd = __fmul2_rn(ud, d);
-            S0 = __fadd2_rn(S0, u);
+            SR = __ffma2_rn(u, __ffma2_rn(E, l2, one), SR);
             S1 = __fadd2_rn(S1, ud);
-            S2 = __fadd2_rn(S2, udd);
-            S3 = __ffma2_rn(udd, d, S3);
+            S3 = __ffma2_rn(ud, dd, S3);
         } else {
             S1 = __ffma2_rn(u, d, S1);
         }
     }
     s1 += S1.x + S1.y;
     if (FULL) {
-        s0 += S0.x + S0.y;
-        s2 += S2.x + S2.y;
+        sR += SR.x + SR.y;
         s3 += S3.x + S3.y;
     }
 }
 
 // The same sums over a window held in a staged band, in the scaled phase s = sc d
-// (sc = sqrt(log2(e) / 2) / sigma, so that exp(-d^2 / 2 sigma^2) = 2^(-s^2)): S0 = sum dl e,
-// S1 = sum dl s e, S2 = sum dl s^2 e, S3 = sum dl s^3 e.  band[c] is the residual at band index
+// (sc = sqrt(log2(e) / 2) / sigma, so that exp(-d^2 / 2 sigma^2) = 2^(-s^2)): SR = sum dl (1 - 2 ln 2
+// s^2) e, S1 = sum dl s e, S3 = sum dl s^3 e.  band[c] is the residual at band index
 // c; the window is [c_lo, c_hi] with s_lo the scaled phase at c_lo and step = sc Delta.  The walk
 // reads the band two samples at a time as one aligned float2, from the even index at or below
 // c_lo up to the pair holding c_hi (band[c_hi + 1] must exist): only the first and the last pair
 // can hold a sample outside the window, and only those two are masked.
 template <bool FULL>
 __device__ __forceinline__ void band_sums(const float* __restrict__ band, int c_lo, int c_hi, float s_lo, float step,
-                                          float& s0, float& s1, float& s2, float& s3) {
+                                          float& sR, float& s1, float& s3) {
     const int ca = c_lo & ~1;
     const int NI = ((c_hi - ca) >> 1) + 1;                      // pairs walked (c_hi >= c_lo)
     const float2* bp = reinterpret_cast<const float2*>(band + ca);
     const float sa = (c_lo & 1) ? s_lo + step : s_lo;           // scaled phase at index ca
     float2 s = make_float2(sa, sa - step);
-    const float2 ds = make_float2(-2.f * step, -2.f * step);
-    float2 S0 = make_float2(0.f, 0.f), S1 = S0, S2 = S0, S3 = S0;
+    const float2 ds = make_float2(-2.f * step, -2.f * step), one = make_float2(1.f, 1.f),
+                 l2 = make_float2(-ADJ_2LN2, -ADJ_2LN2);
+    float2 SR = make_float2(0.f, 0.f), S1 = SR, S3 = SR;
     auto pair = [&](float2 x) {
         const float2 ss = __fmul2_rn(s, s);
         const float2 u = __fmul2_rn(x, make_float2(ex2_approx(-ss.x), ex2_approx(-ss.y)));
         if (FULL) {
             const float2 us = __fmul2_rn(u, s);
-            const float2 uss = __fmul2_rn(us, s);
-            S0 = __fadd2_rn(S0, u);
+            SR = __ffma2_rn(u, __ffma2_rn(ss, l2, one), SR);
             S1 = __fadd2_rn(S1, us);
-            S2 = __fadd2_rn(S2, uss);
-            S3 = __ffma2_rn(uss, s, S3);
+            S3 = __ffma2_rn(us, ss, S3);
         } else {
             S1 = __ffma2_rn(u, s, S1);
         }
@@ -96,6 +94,7 @@ __device__ __forceinline__ void band_sums(const float* __restrict__ band, int c_
     if (c_lo & 1) x.x = 0.f;
     if (NI == 1 && last_hi > c_hi) x.y = 0.f;
     pair(x);
+#pragma unroll 2
     for (int q = 1; q < NI - 1; ++q) pair(bp[q]);
     if (NI > 1) {
         x = bp[NI - 1];
@@ -104,16 +103,15 @@ __device__ __forceinline__ void band_sums(const float* __restrict__ band, int c_
     }
     s1 += S1.x + S1.y;
     if (FULL) {
-        s0 += S0.x + S0.y;
-        s2 += S2.x + S2.y;
+        sR += SR.x + SR.y;
         s3 += S3.x + S3.y;
     }
 }
 
 template <bool GRID, bool FULL>
-__global__ void __launch_bounds__(ADJ_THREADS, 4)
+__global__ void __launch_bounds__(ADJ_THREADS, ADJ_CTAS)
 adj_kernel(GaussDev g, ArrDev a, const TileInfo* __restrict__ ti, const float* __restrict__ delta,
-           float* __restrict__ gA, float* __restrict__ gc, float* __restrict__ gs, int LBA) {
+           float* __restrict__ gA, float* __restrict__ gc, float* __restrict__ gs, int LBA, int per) {
     extern __shared__ __align__(16) float bands[];   // [ADJ_SC][LBA]
     __shared__ PairRef refs[ADJ_SC];
     __shared__ int nbs[ADJ_SC];
@@ -167,7 +165,7 @@ adj_kernel(GaussDev g, ArrDev a, const TileInfo* __restrict__ ti, const float* _
         c0x = rt.c0x; c0y = rt.c0y; c0z = rt.c0z;
     }
     const float c2 = -0.72134752044448170368f / (sig * sig);   // -log2(e) / (2 sigma^2)
-    const float inv_s2 = 1.f / (sig * sig), inv_s3 = inv_s2 / sig;
+    const float inv_s3 = 1.f / (sig * sig) / sig;
     const float ks = a.k * sig;
     const float Delta = a.Delta, invDelta = a.invDelta;
     const float sc = 0.84932180028801904272f / sig;             // sqrt(log2(e) / 2) / sigma
@@ -176,8 +174,9 @@ adj_kernel(GaussDev g, ArrDev a, const TileInfo* __restrict__ ti, const float* _
     const float reach = rt.rad + a.k * rt.smax;                // farthest |d| offset in the tile
 
     KahanF kA, kX, kY, kZ, kS;
-    for (int j0 = 0; j0 < a.Nd; j0 += ADJ_SC) {
-        const int nsc = min(ADJ_SC, a.Nd - j0);
+    const int jb = blockIdx.y * per, je = min(a.Nd, jb + per);      // this CTA's sensors
+    for (int j0 = jb; j0 < je; j0 += ADJ_SC) {
+        const int nsc = min(ADJ_SC, je - j0);
         if (warp == 0 && lane < nsc) {
             const int j = j0 + lane;
             const PairRef r = make_ref(c0x, c0y, c0z, a.xyz[3 * j], a.xyz[3 * j + 1], a.xyz[3 * j + 2], a);
@@ -204,25 +203,25 @@ adj_kernel(GaussDev g, ArrDev a, const TileInfo* __restrict__ ti, const float* _
                 const float ulo = __fadd_ru(tt - ksi, ADJ_MAGIC), uhi = __fadd_rd(tt + ksi, ADJ_MAGIC);
                 const int w_lo = __float_as_int(ulo) - ADJ_MAGIC_BITS, w_hi = __float_as_int(uhi) - ADJ_MAGIC_BITS;
                 const int off = r.n0 - nbs[q];
-                float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+                float sR = 0.f, s1 = 0.f, s3 = 0.f;
                 if (w_lo <= w_hi) {
                     if ((off + w_lo >= 0) && (off + w_hi + 1 < LBA)) {
                         // the band is zero outside the record: no clamp; sums in the scaled phase
                         band_sums<FULL>(bands + q * LBA, off + w_lo, off + w_hi,
-                                        sc * fmaf(-(ulo - ADJ_MAGIC), Delta, phi), step, s0, s1, s2, s3);
+                                        sc * fmaf(-(ulo - ADJ_MAGIC), Delta, phi), step, sR, s1, s3);
                         s1 *= isc;
-                        if (FULL) { s2 *= isc * isc; s3 *= isc * isc * isc; }
+                        if (FULL) s3 *= isc * isc * isc;
                     } else {
                         const int m_lo = max(w_lo, -r.n0), m_hi = min(w_hi, a.Nt - 1 - r.n0);
-                        window_sums<FULL>(delta + (size_t)(j0 + q) * a.Nt + r.n0, m_lo, m_hi, phi, Delta, c2, s0, s1,
-                                          s2, s3);
+                        window_sums<FULL>(delta + (size_t)(j0 + q) * a.Nt + r.n0, m_lo, m_hi, phi, Delta, c2, sR, s1,
+                                          s3);
                     }
                 }
                 const float inv2R = 0.5f * invR;
                 aA = fmaf(s1, inv2R, aA);
                 if (FULL) {
                     const float wA = Ai * inv2R;
-                    const float gR = wA * (s0 - s2 * inv_s2) - wA * s1 * invR;
+                    const float gR = wA * sR - wA * s1 * invR;
                     const float gRi = gR * invR;
                     aX = fmaf(gRi, r.v0x + dx, aX);
                     aY = fmaf(gRi, r.v0y + dy, aY);
@@ -235,15 +234,19 @@ adj_kernel(GaussDev g, ArrDev a, const TileInfo* __restrict__ ti, const float* _
         }
         __syncthreads();
     }
+    float sum[FULL ? 5 : 1];
+    sum[0] = kA.s;
+    if constexpr (FULL) { sum[1] = kX.s; sum[2] = kY.s; sum[3] = kZ.s; sum[4] = kS.s; }
+    if (gridDim.y > 1 && !split_sum(sum, bands, l)) return;         // the bands' memory is free
     if (valid) {
-        gA[i] = kA.s;
-        if (FULL) {
+        gA[i] = sum[0];
+        if constexpr (FULL) {
             if (gc) {
-                gc[i] = kX.s;
-                gc[g.M + i] = kY.s;
-                gc[2 * g.M + i] = kZ.s;
+                gc[i] = sum[1];
+                gc[g.M + i] = sum[2];
+                gc[2 * g.M + i] = sum[3];
             }
-            if (gs) gs[i] = kS.s;
+            if (gs) gs[i] = sum[4];
         }
     }
 }
@@ -444,7 +447,7 @@ adj_moment_kernel(GaussDev g, ArrDev a, const float* __restrict__ delta, const f
     float sum[ADJM_PER];
 #pragma unroll
     for (int u = 0; u < ADJM_PER; ++u) sum[u] = kA[u].s;
-    if (gridDim.y > 1 && !split_sum<ADJM_PER>(sum, part)) return;
+    if (gridDim.y > 1 && !split_sum<ADJM_PER>(sum, part, l)) return;
 #pragma unroll
     for (int u = 0; u < ADJM_PER; ++u) {
         const int gx = tx * BX + lx + (u >> 1) * 4, gy = ty * BY + ly, gz = tz * BZ + lz + (u & 1);
@@ -482,13 +485,17 @@ cudaError_t launch_adjoint(const GaussDev& g, const ArrDev& a, const TileInfo* t
                            float* gc, float* gs, int LBA, cudaStream_t st) {
     const bool full = gc != nullptr || gs != nullptr;
     size_t smem = (size_t)ADJ_SC * LBA * sizeof(float);
+    smem = smem < 5 * TILE * sizeof(float) ? 5 * TILE * sizeof(float) : smem;     // the split's sums
     unsigned blocks = (unsigned)g.ntiles;
+    const int split = adj_split(g.ntiles, a.Nd, ADJ_CTAS);
     cudaError_t e = cudaSuccess;
 #define GP_LAUNCH_ADJ(G, F)                                                                                   \
     do {                                                                                                      \
         e = cudaFuncSetAttribute(adj_kernel<G, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);   \
         if (e != cudaSuccess) return e;                                                                       \
-        adj_kernel<G, F><<<blocks, ADJ_THREADS, smem, st>>>(g, a, ti, delta, gA, gc, gs, LBA);               \
+        e = launch_split(adj_kernel<G, F>, blocks, split, ADJ_THREADS, smem, st, g, a, ti, delta, gA, gc, gs, LBA, \
+                         (a.Nd + split - 1) / split);                                                         \
+        if (e != cudaSuccess) return e;                                                                       \
     } while (0)
     if (g.grid) {
         if (full) GP_LAUNCH_ADJ(true, true); else GP_LAUNCH_ADJ(true, false);

@@ -8,32 +8,33 @@
 namespace gp {
 
 // Each thread's N sums over the cluster's CTAs, in the order of the ranks, by the first CTA's threads
-// (true there, false in the others).  part: N floats of shared memory per thread.
+// (true there, false in the others).  at: which of the tile's sums they are -- every CTA has a thread
+// for each, not always the same one.  part: N floats of shared memory per thread.
 template <int N>
-__device__ __forceinline__ bool split_sum(float (&sum)[N], float* part) {
+__device__ __forceinline__ bool split_sum(float (&sum)[N], float* part, int at) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
 #pragma unroll
-    for (int u = 0; u < N; ++u) part[u * blockDim.x + threadIdx.x] = sum[u];
+    for (int u = 0; u < N; ++u) part[u * blockDim.x + at] = sum[u];
     cl.sync();
     if (blockIdx.y == 0)
         for (unsigned c = 1; c < gridDim.y; ++c) {
             const float* other = cl.map_shared_rank(part, c);
 #pragma unroll
-            for (int u = 0; u < N; ++u) sum[u] += other[u * blockDim.x + threadIdx.x];
+            for (int u = 0; u < N; ++u) sum[u] += other[u * blockDim.x + at];
         }
     cl.sync();                       // the others' shared memory stays until it has been read
     return blockIdx.y == 0;
 }
 
 // CTAs that share a tile's sensors: a power of two up to 8, doubled while the grid stays within one wave
-// of `ctas` per SM and each CTA keeps at least 8 sensors.  16 bricks and 128 sensors: 74 us for the 16
+// of `ctas` per SM and each CTA keeps at least 4 sensors.  16 bricks and 128 sensors: 74 us for the 16
 // CTAs, 40 us for 8 times as many (20 steps of a 16^3 reconstruction 2476 -> 1778 us).  More than a wave
 // is not split: CTAs that walk the sensors in the same order share their rows in L1, and 4096 bricks split
 // eightfold for an even last wave took the mid workload's two discretised adjoints from 1.4 to 2.1 ms.
 inline int adj_split(int64_t ntiles, int Nd, int ctas) {
     int split = 1;
-    while (split < 8 && ntiles * split * 2 <= (int64_t)device_sms() * ctas && Nd >= 16 * split) split *= 2;
+    while (split < 8 && ntiles * split * 2 <= (int64_t)device_sms() * ctas && Nd >= 8 * split) split *= 2;
     return split;
 }
 

@@ -397,7 +397,7 @@ assa_adj_kernel(GaussDev g, ArrDev a, const float* __restrict__ dconv, const __g
 #pragma unroll
     for (int u = 0; u < ASSA_ADJ_PER; ++u) sum[u] = kA[u].s;
     if constexpr (SPLIT)
-        if (!split_sum<ASSA_ADJ_PER>(sum, part)) return;
+        if (!split_sum<ASSA_ADJ_PER>(sum, part, l)) return;
 #pragma unroll
     for (int u = 0; u < ASSA_ADJ_PER; ++u) {
         const int gx = tx * BX + lx + (u >> 1) * 4, gy = ty * BY + ly, gz = tz * BZ + lz + (u & 1);

@@ -28,7 +28,8 @@ cudaError_t launch_slab_order(SlabInfo* si, int S, cudaStream_t st);
 size_t spatial_order_bytes(int64_t M);
 cudaError_t launch_spatial_order(const GaussDev& g, void* scratch, GaussDev& gp, cudaStream_t st);
 cudaError_t launch_forward_free(const GaussDev& g, const ArrDev& a, const TileInfo* ti, const SlabInfo* si, int S,
-                                float* partial, int2* rows, int PL, int LB, int NW, cudaStream_t st);
+                                float* partial, int2* rows, int PL, int LB, int NW, int parts,
+                                cudaStream_t st);
 cudaError_t launch_slab_reduce_rows(const ArrDev& a, const float* partial, const int2* rows, int S, int PL, float* y,
                                     cudaStream_t st);
 size_t fwd_lanes_smem(int NW, int NZ, int LB, int P, int L);
@@ -226,7 +227,8 @@ gpair_status cuda_status(cudaError_t e) {
 // ---- forward plan ---------------------------------------------------------------------------
 
 struct FwdPlan {
-    int S;                 // slabs
+    int S;                 // slabs; partial rows a sensor has (slabs x parts)
+    int parts;             // lanes kernels: CTAs that share a slab's Gaussians
     int64_t tiles_per_slab;        // SoA mode
     int sbx, sby, sbz;     // grid mode: slab block size in bricks
     int LB;                // slab band entries per sensor (FP64 in shared memory)
@@ -287,6 +289,7 @@ void soa_plan_from_slabs(FwdPlan& p, const GaussDev& g, const ArrDev& a, int64_t
 FwdPlan plan_forward(const GaussDev& g, const ArrDev& a) {
     FwdPlan p;
     memset(&p, 0, sizeof(p));
+    p.parts = 1;
     const int ngroups = (a.Nd + SPC - 1) / SPC;
     const int64_t target_S = ((int64_t)device_sms() * 4 * 4 + ngroups - 1) / ngroups;
     if (g.grid) {
@@ -391,6 +394,7 @@ bool plan_forward_lanes(const GaussDev& g, const ArrDev& a, const MomentTable& T
     int sc[3] = {std::min(4, nc[0]), std::min(4, nc[1]), std::min(2, nc[2])};
     FwdPlan p;
     memset(&p, 0, sizeof(p));
+    p.parts = 1;
     if (!lanes_plan_from_blocks(p, g, a, T, sc)) return false;
     const int64_t target = (int64_t)device_sms() * 8;
     for (;;) {
@@ -403,6 +407,7 @@ bool plan_forward_lanes(const GaussDev& g, const ArrDev& a, const MomentTable& T
         sc[best] = (sc[best] + 1) / 2;
         FwdPlan t;
         memset(&t, 0, sizeof(t));
+        t.parts = 1;
         if (!lanes_plan_from_blocks(t, g, a, T, sc)) break;
         p = t;
     }
@@ -418,6 +423,7 @@ constexpr int FREE_LANES_WARPS = 8;    // warps (sensor groups of 32) per CTA of
 // allow (a sensor whose slab band is longer takes several passes).
 bool plan_forward_free(const GaussDev& g, const ArrDev& a, FwdPlan& p) {
     memset(&p, 0, sizeof(p));
+    p.parts = 1;
     p.NW = std::min(FREE_LANES_WARPS, (a.Nd + 31) / 32);
     const int groups = (a.Nd + 32 * p.NW - 1) / (32 * p.NW);
     int64_t S = ((int64_t)device_sms() * 4 + groups - 1) / groups;
@@ -431,6 +437,12 @@ bool plan_forward_free(const GaussDev& g, const ArrDev& a, FwdPlan& p) {
     const size_t per_warp = (SMEM_PER_CTA - fwd_free_smem(0, 0)) / p.NW;
     p.LB = std::min<int64_t>(p.PL, (int64_t)(per_warp / (32 * 4)) & ~(int64_t)3);
     if (p.LB < 64) return false;
+    // Few tiles leave the chip idle: up to 8 CTAs share a slab's Gaussians, while there is an SM for each
+    // (a CTA fills one) and the rows fit.
+    while (p.parts < 8 && (int64_t)p.S * groups * 2 <= device_sms() && 2 * p.S * row <= ((int64_t)2 << 30)) {
+        p.parts *= 2;
+        p.S *= 2;
+    }
     p.free_lanes = true;
     plan_offsets(p, g, a);
     p.off_sort = p.bytes;
@@ -491,10 +503,10 @@ gpair_status run_forward(const GaussDev& g, const ArrDev& a, float* y, cudaStrea
         GaussDev gp;
         e = launch_spatial_order(g, base + p.off_sort, gp, st);
         if (e == cudaSuccess) e = launch_tile_info(gp, ti, st);
-        if (e == cudaSuccess) e = launch_slab_info_soa(gp, gp.ntiles, p.tiles_per_slab, p.S, si, st);
-        if (e == cudaSuccess) e = launch_slab_order(si, p.S, st);
+        if (e == cudaSuccess) e = launch_slab_info_soa(gp, gp.ntiles, p.tiles_per_slab, p.S / p.parts, si, st);
+        if (e == cudaSuccess) e = launch_slab_order(si, p.S / p.parts, st);
         if (e == cudaSuccess && ev) e = cudaEventRecord(ev[0], st);
-        if (e == cudaSuccess) e = launch_forward_free(gp, a, ti, si, p.S, part, rows, p.PL, p.LB, p.NW, st);
+        if (e == cudaSuccess) e = launch_forward_free(gp, a, ti, si, p.S, part, rows, p.PL, p.LB, p.NW, p.parts, st);
         if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], st);
         if (e == cudaSuccess) e = launch_slab_reduce_rows(a, part, rows, p.S, p.PL, y, st);
         return cuda_status(e);

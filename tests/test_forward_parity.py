@@ -143,3 +143,13 @@ def test_free_gaussians_band_longer_than_shared_memory():
     w = synth.Workload("free-spread", g, synth.cap_sensors(8, 200e-3, 120.0), 8192, free=free)
     rel, y, yo = _check(w)
     assert np.abs(yo).max() > 0
+
+
+@pytest.mark.parametrize("sides", [(1, 1, 1), (16, 8, 2), (13, 10, 5), (20, 20, 21)])
+def test_free_gaussians_few_tiles(sides):
+    """One to eight CTAs share a tile of 256: a lone Gaussian, a whole tile, a part of a third one; and an order
+    of more than one CTA's words (8192)."""
+    g = synth.centred_grid(*sides, 0.1e-3)
+    free = synth.free_gaussians(g, 7, A=np.random.default_rng(8).uniform(0.2, 1.0, g.M))
+    w = synth.Workload("free-few", g, synth.cap_sensors(35, 20e-3, 160.0), 900, free=free)
+    _check(w)
