@@ -240,6 +240,8 @@ struct FwdPlan {
     int NW, NZ;            // warps per CTA of the lanes kernels; moment-band bins (grid)
     size_t off_ti, off_si, off_rows, off_part, bytes;
     size_t off_sort;       // free-centre lanes plan: the spatial order's scratch (after the rest)
+    bool has_mom;          // the expansion applies (grid mode); mom is its table
+    MomentTable mom;
 };
 
 void plan_offsets(FwdPlan& p, const GaussDev& g, const ArrDev& a) {
@@ -455,9 +457,11 @@ bool plan_forward_free(const GaussDev& g, const ArrDev& a, FwdPlan& p) {
 FwdPlan plan_forward_op(const GaussDev& g, const ArrDev& a) {
     MomentTable T;
     FwdPlan p;
-    if (g.grid && make_moment_table(g, a, T) && plan_forward_lanes(g, a, T, p)) return p;
-    if (!g.grid && plan_forward_free(g, a, p)) return p;
-    return plan_forward(g, a);
+    const bool has_mom = g.grid && make_moment_table(g, a, T);
+    if (!(has_mom && plan_forward_lanes(g, a, T, p)) && !(!g.grid && plan_forward_free(g, a, p))) p = plan_forward(g, a);
+    p.has_mom = has_mom;
+    if (has_mom) p.mom = T;
+    return p;
 }
 
 // The same within `cap` bytes of scratch (the allocation-free entry point): the lanes plan
@@ -466,7 +470,13 @@ FwdPlan plan_forward_op(const GaussDev& g, const ArrDev& a) {
 bool plan_forward_op_capped(const GaussDev& g, const ArrDev& a, size_t cap, FwdPlan& out) {
     MomentTable T;
     FwdPlan p;
-    if (g.grid && make_moment_table(g, a, T) && plan_forward_lanes(g, a, T, p)) {
+    const bool has_mom = g.grid && make_moment_table(g, a, T);
+    auto with_table = [&] {
+        out.has_mom = has_mom;
+        if (has_mom) out.mom = T;
+        return true;
+    };
+    if (has_mom && plan_forward_lanes(g, a, T, p)) {
         const int nc[3] = {(g.nx + CUBE_SIDE - 1) / CUBE_SIDE, (g.ny + CUBE_SIDE - 1) / CUBE_SIDE,
                            (g.nz + CUBE_SIDE - 1) / CUBE_SIDE};
         int sc[3] = {p.sbx, p.sby, p.sbz};
@@ -481,10 +491,10 @@ bool plan_forward_op_capped(const GaussDev& g, const ArrDev& a, size_t cap, FwdP
         }
         if (ok) {
             out = p;
-            return true;
+            return with_table();
         }
     }
-    return plan_forward_capped(g, a, cap, out);
+    return plan_forward_capped(g, a, cap, out) && with_table();
 }
 
 // ev (optional): two events recorded immediately before and after the slab kernel.
@@ -532,11 +542,9 @@ gpair_status run_forward(const GaussDev& g, const ArrDev& a, float* y, cudaStrea
         if (e == cudaSuccess) e = launch_slab_info_soa(g, g.ntiles, p.tiles_per_slab, p.S, si, st);
     }
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[0], st);
-    MomentTable mom;
-    const bool use_mom = g.grid && make_moment_table(g, a, mom);
     if (e == cudaSuccess)
         e = launch_forward(g, a, ti, si, p.S, part, rows, p.PL, p.LB, p.TB, p.binned, status, tma ? &map : nullptr,
-                           use_mom ? &mom : nullptr, st);
+                           p.has_mom ? &p.mom : nullptr, st);
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], st);
     if (e == cudaSuccess) e = launch_slab_reduce(g, a, part, rows, p.S, p.PL, y, st);
     return cuda_status(e);
@@ -552,8 +560,7 @@ gpair_status run_forward(const GaussDev& g, const ArrDev& a, float* y, cudaStrea
 // largest error, evaluated against the pulse at 257 offsets per position, is below 3e-7 of the
 // pulse's peak.  Returns false when the expansion does not apply (window longer than MOM_LMAX
 // samples, or Delta > sigma / 2).
-bool make_moment_table(const GaussDev& g, const ArrDev& a, MomentTable& T) {
-    if (!g.grid) return false;
+bool form_moment_table(const GaussDev& g, const ArrDev& a, MomentTable& T) {
     const double s = g.sigma, Delta = (double)a.Delta, k = a.k;
     const double X = 2.0 * k * s / Delta;
     const int E = (int)std::floor(X);
@@ -576,39 +583,61 @@ bool make_moment_table(const GaussDev& g, const ArrDev& a, MomentTable& T) {
         return 0.5 * d * std::exp(-0.5 * d * d / (s * s));
     };
     constexpr int NC = 64;                       // Chebyshev points
-    // monomial coefficients of the Chebyshev polynomials T_0 .. T_{MOM_P-1}
-    double Tm[MOM_P][MOM_P] = {};
-    Tm[0][0] = 1.0;
-    Tm[1][1] = 1.0;
-    for (int n = 2; n < MOM_P; ++n)
-        for (int q = 0; q < MOM_P; ++q) Tm[n][q] = (q > 0 ? 2.0 * Tm[n - 1][q - 1] : 0.0) - Tm[n - 2][q];
+    // cos(n th_i), the points' offsets among them, and the monomial coefficients of T_0 .. T_{MOM_P-1}
+    struct Basis { double cosn[MOM_P][NC], Tm[MOM_P][MOM_P]; };
+    static const Basis B = [] {
+        Basis b = {};
+        for (int n = 0; n < MOM_P; ++n)
+            for (int i = 0; i < NC; ++i) b.cosn[n][i] = std::cos(n * (M_PI * (i + 0.5) / NC));
+        b.Tm[0][0] = 1.0;
+        b.Tm[1][1] = 1.0;
+        for (int n = 2; n < MOM_P; ++n)
+            for (int q = 0; q < MOM_P; ++q) b.Tm[n][q] = (q > 0 ? 2.0 * b.Tm[n - 1][q - 1] : 0.0) - b.Tm[n - 2][q];
+        return b;
+    }();
+    // The pulse at the NQ offsets of the error, from one position to the next by two factors: with D = dstar -
+    // m Delta and t = e Delta / 2, exp(-(D + t)^2 / 2 s^2) = exp(-D^2 / 2 s^2) exp(-t^2 / 2 s^2 - dstar t / s^2)
+    // exp(Delta t / s^2)^m.
+    constexpr int NQ = 257;
+    static thread_local double cd[MOM_LMAX][MOM_P], ch[MOM_LMAX][MOM_P], ref[MOM_LMAX][NQ];
+    double at[NQ], fac[NQ], grow[NQ];
+    for (int q = 0; q < NQ; ++q) {
+        at[q] = -1.0 + q / 128.0;
+        const double t = 0.5 * Delta * at[q];
+        fac[q] = std::exp(-(0.5 * t + dstar) * t / (s * s));
+        grow[q] = std::exp(Delta * t / (s * s));
+    }
+    for (int m = 0; m < L; ++m) {
+        const double D = dstar - m * Delta, w = 0.5 * std::exp(-0.5 * D * D / (s * s));
+        for (int q = 0; q < NQ; ++q) {
+            ref[m][q] = w * (D + 0.5 * Delta * at[q]) * fac[q];
+            fac[q] *= grow[q];
+        }
+        for (int n = 0; n < MOM_P; ++n) ch[m][n] = 0.0;      // Chebyshev coefficients from the discrete orthogonality
+        for (int i = 0; i < NC; ++i) {
+            const double f = pulse(m, B.cosn[1][i]);
+            for (int n = 0; n < MOM_P; ++n) ch[m][n] += f * B.cosn[n][i];
+        }
+        for (int n = 0; n < MOM_P; ++n) ch[m][n] *= (n == 0 ? 1.0 : 2.0) / NC;
+    }
     const double peak = 0.5 * s * std::exp(-0.5);
-    static thread_local double cd[MOM_LMAX][MOM_P];
     int P = MOM_P;
     for (int PP = 6; PP <= MOM_P; ++PP) {
         double err = 0.0;
         for (int m = 0; m < L; ++m) {
-            double ch[MOM_P] = {};             // Chebyshev coefficients from the discrete orthogonality
-            for (int i = 0; i < NC; ++i) {
-                const double th = M_PI * (i + 0.5) / NC;
-                const double f = pulse(m, std::cos(th));
-                for (int n = 0; n < PP; ++n) ch[n] += f * std::cos(n * th);
-            }
-            for (int n = 0; n < PP; ++n) ch[n] *= (n == 0 ? 1.0 : 2.0) / NC;
             for (int q = 0; q < MOM_P; ++q) {
                 double c = 0.0;
-                for (int n = 0; n < PP; ++n) c += ch[n] * Tm[n][q];
+                for (int n = 0; n < PP; ++n) c += ch[m][n] * B.Tm[n][q];
                 cd[m][q] = q < PP ? c : 0.0;
             }
-            for (int q = 0; q <= 256; ++q) {
-                const double e = -1.0 + q / 128.0;
-                double ser = 0.0, ep = 1.0;
-                for (int p = 0; p < PP; ++p, ep *= e) ser += cd[m][p] * ep;
-                err = std::max(err, std::fabs(pulse(m, e) - ser) / peak);
-            }
+            double ser[NQ];
+            for (int q = 0; q < NQ; ++q) ser[q] = cd[m][PP - 1];
+            for (int p = PP - 2; p >= 0; --p)
+                for (int q = 0; q < NQ; ++q) ser[q] = ser[q] * at[q] + cd[m][p];
+            for (int q = 0; q < NQ; ++q) err = std::max(err, std::fabs(ref[m][q] - ser[q]));
         }
         P = PP;
-        if (err <= 3e-7) break;
+        if (err <= 3e-7 * peak) break;
     }
     T.P = P;
     for (int m = 0; m < L; ++m)
@@ -616,26 +645,34 @@ bool make_moment_table(const GaussDev& g, const ArrDev& a, MomentTable& T) {
     return true;
 }
 
+// The same, with each thread's last table kept by the three values it is made of: forming it takes about 50 us of a
+// host core, as long as a small operator's kernels.
+bool make_moment_table(const GaussDev& g, const ArrDev& a, MomentTable& T) {
+    if (!g.grid) return false;
+    struct Last { float sigma, Delta, k; bool ok; MomentTable T; };
+    static thread_local Last last = {};
+    if (!(last.sigma == g.sigma && last.Delta == a.Delta && last.k == a.k)) {
+        last.ok = form_moment_table(g, a, last.T);
+        last.sigma = g.sigma; last.Delta = a.Delta; last.k = a.k;
+    }
+    if (last.ok) T = last.T;
+    return last.ok;
+}
+
 int adjoint_band(const GaussDev& g, const ArrDev& a) {
     if (g.grid) return adj_band_len(brick_radius(g.h), g.sigma, a.k, a.invDelta);
     return 256;
 }
 
-// Bytes of the expansion table Q an amplitude-only grid adjoint needs (0 when it does not apply).
-size_t adjoint_q_bytes(const GaussDev& g, const ArrDev& a) {
-    MomentTable T;
-    if (!make_moment_table(g, a, T)) return 0;
-    return align256(adj_moment_q_bytes(a, T.L));
-}
+// Bytes of the table Q that an amplitude-only grid adjoint through the expansion T needs.
+size_t adjoint_q_bytes(const ArrDev& a, const MomentTable& T) { return align256(adj_moment_q_bytes(a, T.L)); }
 
-// qbuf (optional): adjoint_q_bytes() of device memory for the expansion path.
+// qbuf (optional): adjoint_q_bytes() of device memory for the expansion path, with its table T.
 gpair_status run_adjoint(const GaussDev& g, const ArrDev& a, const float* delta, float* gA, float* gc, float* gs,
-                         cudaStream_t st, void* scratch, const cudaEvent_t* ev = nullptr, void* qbuf = nullptr) {
-    if (qbuf && !gc && !gs) {
-        MomentTable T;
-        if (make_moment_table(g, a, T))
-            return cuda_status(launch_adjoint_moment(g, a, delta, gA, T, static_cast<float*>(qbuf), ev, st));
-    }
+                         cudaStream_t st, void* scratch, const cudaEvent_t* ev = nullptr, void* qbuf = nullptr,
+                         const MomentTable* T = nullptr) {
+    if (qbuf && !gc && !gs)
+        return cuda_status(launch_adjoint_moment(g, a, delta, gA, *T, static_cast<float*>(qbuf), ev, st));
     TileInfo* ti = static_cast<TileInfo*>(scratch);
     cudaError_t e = launch_tile_info(g, ti, st);
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[0], st);
@@ -714,10 +751,11 @@ gpair_status gpair_adjoint(const gpair_gaussians* gi, const gpair_array* ai, con
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     void* scratch = nullptr;
     const size_t ti_bytes = align256(sizeof(TileInfo) * (size_t)g.ntiles);
-    const size_t q_bytes = (gc || gsigma) ? 0 : adjoint_q_bytes(g, a);
+    MomentTable T;
+    const size_t q_bytes = !gc && !gsigma && make_moment_table(g, a, T) ? adjoint_q_bytes(a, T) : 0;
     if ((s = get_scratch(st, ti_bytes + q_bytes, &scratch, nullptr)) != GPAIR_OK) return s;
     return run_adjoint(g, a, delta, gA, gc, gsigma, st, scratch, nullptr,
-                       q_bytes ? static_cast<char*>(scratch) + ti_bytes : nullptr);
+                       q_bytes ? static_cast<char*>(scratch) + ti_bytes : nullptr, &T);
 }
 
 gpair_status gpair_shard_range(const gpair_grid* grid, int shard, int n_shards, int* z_begin, int* z_end) {
@@ -790,10 +828,11 @@ gpair_status gpair_adjoint_shard(const gpair_gaussians* gi, const gpair_array* a
     const GaussDev gs = zslab(g, z0, z1, gi->A);
     void* scratch = nullptr;
     const size_t ti_bytes = align256(sizeof(TileInfo) * (size_t)gs.ntiles);
-    const size_t q_bytes = adjoint_q_bytes(gs, a);
+    MomentTable T;
+    const size_t q_bytes = make_moment_table(gs, a, T) ? adjoint_q_bytes(a, T) : 0;
     if ((s = get_scratch(st, ti_bytes + q_bytes, &scratch, nullptr)) != GPAIR_OK) return s;
     return run_adjoint(gs, a, delta, gA + (int64_t)z0 * g.nx * g.ny, nullptr, nullptr, st, scratch, nullptr,
-                       q_bytes ? static_cast<char*>(scratch) + ti_bytes : nullptr);
+                       q_bytes ? static_cast<char*>(scratch) + ti_bytes : nullptr, &T);
 }
 
 gpair_status gpair_voxelize(const gpair_gaussians* gi, const gpair_grid* og, float window_k, float* vol,
@@ -1094,7 +1133,7 @@ gpair_status solver_forward(gpair_solver* S, float* y, const cudaEvent_t* ev, cu
 gpair_status solver_adjoint(gpair_solver* S, const float* delta, float* gA, const cudaEvent_t* ev, cudaStream_t st) {
     if (S->assa) return cuda_status(launch_assa_adjoint(S->g, S->a, delta, gA, S->T, S->dconv, ev, st));
     // the amplitude adjoint needs only the tile summaries of the forward scratch (same layout)
-    return run_adjoint(S->g, S->a, delta, gA, nullptr, nullptr, st, S->fwd_scratch, ev, S->qbuf);
+    return run_adjoint(S->g, S->a, delta, gA, nullptr, nullptr, st, S->fwd_scratch, ev, S->qbuf, &S->plan.mom);
 }
 }  // namespace
 
@@ -1139,7 +1178,7 @@ gpair_status gpair_solver_create(const gpair_gaussians* gi, const gpair_array* a
     const size_t M = (size_t)g.M, N = (size_t)a.Nd * a.Nt;
     if (assa) S->aa = assa_band_array(g, a, S->T);
     S->plan = assa ? plan_forward(g, S->aa) : plan_forward_op(g, a);
-    const size_t qbytes = assa ? 0 : adjoint_q_bytes(g, a);
+    const size_t qbytes = !assa && S->plan.has_mom ? adjoint_q_bytes(a, S->plan.mom) : 0;
     bool ok = cudaMalloc(&S->z, M * 4) == cudaSuccess && cudaMalloc(&S->m, M * 4) == cudaSuccess &&
               cudaMalloc(&S->v, M * 4) == cudaSuccess && cudaMalloc(&S->x, M * 4) == cudaSuccess &&
               cudaMalloc(&S->gx, M * 4) == cudaSuccess && cudaMalloc(&S->y, N * 4) == cudaSuccess &&
