@@ -27,14 +27,18 @@ __device__ __forceinline__ bool split_sum(float (&sum)[N], float* part, int at) 
     return blockIdx.y == 0;
 }
 
-// CTAs that share a tile's sensors: a power of two up to 8, doubled while the grid stays within one wave
-// of `ctas` per SM and each CTA keeps at least 4 sensors.  16 bricks and 128 sensors: 74 us for the 16
-// CTAs, 40 us for 8 times as many (20 steps of a 16^3 reconstruction 2476 -> 1778 us).  More than a wave
-// is not split: CTAs that walk the sensors in the same order share their rows in L1, and 4096 bricks split
-// eightfold for an even last wave took the mid workload's two discretised adjoints from 1.4 to 2.1 ms.
-inline int adj_split(int64_t ntiles, int Nd, int ctas) {
+// CTAs that share a tile's sensors, a power of two up to 8, for grids of less than one wave of `ctas` per SM: doubled
+// while the CTAs stay within a wave and keep `least` sensors each (idle SMs), and while they stay within four
+// waves and keep 64 (few warps on each SM).  The amplitude adjoint's time with 1, 2, 4, 8 CTAs a tile: 16 bricks, 128
+// sensors: 74 us for 1, 17 us for 8; 184 bricks, 33 sensors: 24, ..., 12, 19 us; 675 bricks, 952 sensors: 609, 600,
+// 441, 370 us; 1024 bricks, 512 sensors: 337, 316, 305, 279 us.  From a wave on it costs: CTAs that walk the
+// sensors in the same order share their rows in L1 (3900 bricks, 47 sensors: 76, ..., 154, 241 us).
+inline int adj_split(int64_t ntiles, int Nd, int ctas, int least) {
+    const int64_t wave = (int64_t)device_sms() * ctas;
     int split = 1;
-    while (split < 8 && ntiles * split * 2 <= (int64_t)device_sms() * ctas && Nd >= 8 * split) split *= 2;
+    while (split < 8 && ntiles < wave &&
+           ((ntiles * split * 2 <= wave && Nd >= 2 * least * split) || (ntiles * split * 2 <= 4 * wave && Nd >= 128 * split)))
+        split *= 2;
     return split;
 }
 

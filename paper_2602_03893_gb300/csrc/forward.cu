@@ -89,24 +89,8 @@ __global__ void slab_info_grid_kernel(GaussDev g, int sbx, int sby, int sbz, int
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= S) return;
     const int sx = s % nsx, sy = (s / nsx) % nsy, sz = s / (nsx * nsy);
-    SlabInfo o;
-    o.bx0 = sx * sbx; o.by0 = sy * sby; o.bz0 = sz * sbz;
-    o.bdx = min(sbx, g.ntx - o.bx0); o.bdy = min(sby, g.nty - o.by0); o.bdz = min(sbz, g.ntz - o.bz0);
-    const int ax = o.bx0 * BX, bxn = min(g.nx, (o.bx0 + o.bdx) * BX);
-    const int ay = o.by0 * BY, byn = min(g.ny, (o.by0 + o.bdy) * BY);
-    const int az = o.bz0 * BZ, bzn = min(g.nz, (o.bz0 + o.bdz) * BZ);
-    o.lo[0] = (float)(g.ox + (ax + 0.5) * g.h); o.hi[0] = (float)(g.ox + (bxn - 0.5) * g.h);
-    o.lo[1] = (float)(g.oy + (ay + 0.5) * g.h); o.hi[1] = (float)(g.oy + (byn - 0.5) * g.h);
-    o.lo[2] = (float)(g.oz + (az + 0.5) * g.h); o.hi[2] = (float)(g.oz + (bzn - 0.5) * g.h);
-    // widen by a few ulp so that float rounding of the box never cuts a centre off
-    for (int q = 0; q < 3; ++q) {
-        float pad = 1e-6f * (fabsf(o.lo[q]) + fabsf(o.hi[q])) + 1e-9f;
-        o.lo[q] -= pad; o.hi[q] += pad;
-    }
-    o.smax = g.sigma;
-    o.t_begin = 0; o.t_end = o.bdx * o.bdy * o.bdz;
-    o.pad = 0;
-    si[s] = o;
+    const int bx0 = sx * sbx, by0 = sy * sby, bz0 = sz * sbz;
+    si[s] = brick_block(g, bx0, by0, bz0, min(sbx, g.ntx - bx0), min(sby, g.nty - by0), min(sbz, g.ntz - bz0));
 }
 
 // SoA mode: the axis-aligned box of the Gaussian centres and the widest sigma of each contiguous
@@ -1052,48 +1036,55 @@ slab_reduce_banded_kernel(const float* __restrict__ partial, const int2* __restr
     if (n < Nt) y[(size_t)j * Nt + n] = acc;
 }
 
-// Banded rows, one block per (sensor, group of four 256-sample chunks): the sensor's row
-// descriptors are sorted by band start (bitonic sort of (start, slab) keys in shared memory), and
-// each chunk walks only the slabs whose bands can reach it -- those starting after the chunk's
-// first sample minus the longest band and before its end, a contiguous run of the sorted keys --
+// Banded rows, one block per (sensor, group of four 256-sample chunks): the descriptors of the sensor's rows that
+// reach the group are sorted by band start (bitonic sort of (start, slab) keys in shared memory), and
+// each warp walks only the slabs whose bands can reach its 32 samples -- those starting after the
+// first of them minus the longest band and before the last's end, a contiguous run of the sorted keys --
 // instead of testing every slab, eight slabs' loads at a time.  Each sample sums its slabs in the
 // order of their band starts, ties by slab index: a fixed order, so the result is deterministic.
+// Where that is too few blocks to fill the chip (seg > 1), a block takes 256 / seg samples and seg warps share
+// each 32 of them, a run of the slabs each, added in their order.
+//
+// Bound by the latency of the rows' loads.  512 slabs, 1024 sensors: 256 us with all rows sorted and runs for 256
+// samples, 195 us; 1300 slabs, 47 sensors: 256 us with a warp to 32 samples, ... us with four.
 constexpr int SRS_THREADS = 256;
 constexpr int SRS_MAX_S = 2048;             // sorted keys and descriptors: 32 KB
 constexpr int SRS_CHUNKS = 4;               // 256-sample chunks per block (blockIdx.y: chunk group)
 constexpr int SRS_UNROLL = 8;
 __global__ void __launch_bounds__(SRS_THREADS)
 slab_reduce_sorted_kernel(const float* __restrict__ partial, const int2* __restrict__ rows, int S, int Nd, int Nt,
-                          int PL, float* __restrict__ y) {
-    extern __shared__ unsigned long long srs_key[];     // [Sp] keys, then S descriptors
-    __shared__ int red[2][SRS_THREADS / 32];
+                          int PL, int chunks, int seg, float* __restrict__ y) {
+    extern __shared__ unsigned long long srs_key[];     // [S rounded up to a power of two] keys, then S descriptors
+    __shared__ int red[SRS_THREADS / 32], count;
     const int j = blockIdx.x, t = threadIdx.x;
     int Sp = 1;
     while (Sp < S) Sp <<= 1;
     int2* srow = reinterpret_cast<int2*>(srs_key + Sp);
-    int lbmax = 0, nvalid = 0;
-    for (int q = t; q < Sp; q += SRS_THREADS) {
-        unsigned long long k = ~0ull;                     // empty rows sort last
-        if (q < S) {
-            const int2 ri = rows[(size_t)q * Nd + j];
-            srow[q] = ri;
-            if (ri.y > 0) {
-                k = ((unsigned long long)(unsigned)ri.x << 32) | (unsigned)q;
-                lbmax = max(lbmax, ri.y);
-                ++nvalid;
-            }
-        }
-        srs_key[q] = k;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        lbmax = max(lbmax, __shfl_xor_sync(0xffffffffu, lbmax, o));
-        nvalid += __shfl_xor_sync(0xffffffffu, nvalid, o);
-    }
-    if ((t & 31) == 0) { red[0][t >> 5] = lbmax; red[1][t >> 5] = nvalid; }
+    __shared__ float seg_sum[SRS_THREADS];
+    const int span = SRS_THREADS / seg, c_begin = blockIdx.y * chunks * span, c_end = min(Nt, c_begin + chunks * span);
+    if (t == 0) count = 0;
     __syncthreads();
-    lbmax = 0; nvalid = 0;
+    // the rows that reach the block's samples, in any order (their keys differ)
+    int lbmax = 0;
+    for (int q = t; q < S; q += SRS_THREADS) {
+        const int2 ri = rows[(size_t)q * Nd + j];
+        srow[q] = ri;
+        if (ri.y > 0 && ri.x < c_end && ri.x + ri.y > c_begin) {
+            srs_key[atomicAdd(&count, 1)] = ((unsigned long long)(unsigned)ri.x << 32) | (unsigned)q;
+            lbmax = max(lbmax, ri.y);
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) lbmax = max(lbmax, __shfl_xor_sync(0xffffffffu, lbmax, o));
+    if ((t & 31) == 0) red[t >> 5] = lbmax;
+    __syncthreads();
+    const int nvalid = count;
+    Sp = 1;
+    while (Sp < nvalid) Sp <<= 1;
+    for (int q = nvalid + t; q < Sp; q += SRS_THREADS) srs_key[q] = ~0ull;
+    lbmax = 0;
 #pragma unroll
-    for (int w = 0; w < SRS_THREADS / 32; ++w) { lbmax = max(lbmax, red[0][w]); nvalid += red[1][w]; }
+    for (int w = 0; w < SRS_THREADS / 32; ++w) lbmax = max(lbmax, red[w]);
+    __syncthreads();
     for (int k = 2; k <= Sp; k <<= 1)                     // bitonic sort, ascending
         for (int h = k >> 1; h > 0; h >>= 1) {
             for (int i = t; i < Sp; i += SRS_THREADS) {
@@ -1105,9 +1096,9 @@ slab_reduce_sorted_kernel(const float* __restrict__ partial, const int2* __restr
             }
             __syncthreads();
         }
-    const int c_end = min(Nt, (blockIdx.y + 1) * SRS_CHUNKS * SRS_THREADS);
-    for (int n0 = blockIdx.y * SRS_CHUNKS * SRS_THREADS; n0 < c_end; n0 += SRS_THREADS) {
-        // the run of keys whose bands can reach the chunk: start in [n0 - lbmax + 1, n0 + 256)
+    const int warp_seg = (t >> 5) / (span / 32);
+    for (int n0 = c_begin + (t & ~31) % span; n0 < c_end; n0 += span) {
+        // the run of keys whose bands can reach the warp's samples: start in [n0 - lbmax + 1, n0 + 32)
         auto lower = [&](long long wv) {
             int lo = 0, hi = nvalid;
             while (lo < hi) {
@@ -1116,8 +1107,13 @@ slab_reduce_sorted_kernel(const float* __restrict__ partial, const int2* __restr
             }
             return lo;
         };
-        const int i0 = lower((long long)n0 - lbmax + 1), i1 = lower((long long)n0 + SRS_THREADS);
-        const int n = n0 + t;
+        int i0 = lower((long long)n0 - lbmax + 1), i1 = lower((long long)n0 + 32);
+        if (seg > 1) {
+            const int r0 = i0, len = i1 - i0;
+            i0 = r0 + warp_seg * len / seg;
+            i1 = r0 + (warp_seg + 1) * len / seg;
+        }
+        const int n = n0 + (t & 31);
         float acc = 0.f;
         // SRS_UNROLL slabs at a time, so that their loads are in flight together; a slab past the
         // run or missing the sample contributes an exact zero, so the sum is the slab-by-slab one
@@ -1135,7 +1131,16 @@ slab_reduce_sorted_kernel(const float* __restrict__ partial, const int2* __restr
 #pragma unroll
             for (int u = 0; u < SRS_UNROLL; ++u) acc += v[u];
         }
-        if (n < Nt) y[(size_t)j * Nt + n] = acc;
+        if (seg > 1) seg_sum[t] = acc;
+        else if (n < Nt) y[(size_t)j * Nt + n] = acc;
+    }
+    if (seg > 1) {           // one chunk: thread t < span has sample c_begin + t
+        __syncthreads();
+        if (t < span && c_begin + t < c_end) {
+            float acc = seg_sum[t];
+            for (int q = 1; q < seg; ++q) acc += seg_sum[q * span + t];
+            y[(size_t)j * Nt + c_begin + t] = acc;
+        }
     }
 }
 
@@ -1225,8 +1230,13 @@ cudaError_t launch_forward(const GaussDev& g, const ArrDev& a, const TileInfo* t
     return cudaGetLastError();
 }
 
+constexpr int SRS_SEG = 4;
+static bool slab_reduce_few(const ArrDev& a) {      // the grid of four chunks a block is under two blocks an SM
+    return (int64_t)a.Nd * ((a.Nt + SRS_CHUNKS * SRS_THREADS - 1) / (SRS_CHUNKS * SRS_THREADS)) <= (int64_t)device_sms() * 2;
+}
 static dim3 slab_reduce_sorted_grid(const ArrDev& a) {
-    return dim3(a.Nd, (a.Nt + SRS_CHUNKS * SRS_THREADS - 1) / (SRS_CHUNKS * SRS_THREADS));
+    const int per = slab_reduce_few(a) ? SRS_THREADS / SRS_SEG : SRS_CHUNKS * SRS_THREADS;
+    return dim3(a.Nd, (a.Nt + per - 1) / per);
 }
 
 static size_t slab_reduce_sorted_smem(int S) {
@@ -1241,7 +1251,7 @@ cudaError_t launch_slab_reduce_rows(const ArrDev& a, const float* partial, const
     dim3 rgrid((a.Nt + 255) / 256, a.Nd);
     if (S <= SRS_MAX_S && slab_reduce_sorted_grid(a).y <= 65535)
         slab_reduce_sorted_kernel<<<slab_reduce_sorted_grid(a), SRS_THREADS, slab_reduce_sorted_smem(S), st>>>(
-            partial, rows, S, a.Nd, a.Nt, PL, y);
+            partial, rows, S, a.Nd, a.Nt, PL, slab_reduce_few(a) ? 1 : SRS_CHUNKS, slab_reduce_few(a) ? SRS_SEG : 1, y);
     else if (S <= SLAB_RED_MAX_S)
         slab_reduce_banded_kernel<<<rgrid, SLAB_RED_THREADS, (size_t)S * sizeof(int2), st>>>(partial, rows, S, a.Nd,
                                                                                              a.Nt, PL, y);
@@ -1255,7 +1265,7 @@ cudaError_t launch_slab_reduce(const GaussDev& g, const ArrDev& a, const float* 
     dim3 rgrid((a.Nt + 255) / 256, a.Nd);
     if (g.grid && S <= SRS_MAX_S && slab_reduce_sorted_grid(a).y <= 65535)
         slab_reduce_sorted_kernel<<<slab_reduce_sorted_grid(a), SRS_THREADS, slab_reduce_sorted_smem(S), st>>>(
-            partial, rows, S, a.Nd, a.Nt, PL, y);
+            partial, rows, S, a.Nd, a.Nt, PL, slab_reduce_few(a) ? 1 : SRS_CHUNKS, slab_reduce_few(a) ? SRS_SEG : 1, y);
     else if (g.grid && S <= SLAB_RED_MAX_S)
         slab_reduce_banded_kernel<<<rgrid, SLAB_RED_THREADS, (size_t)S * sizeof(int2), st>>>(partial, rows, S, a.Nd,
                                                                                              a.Nt, PL, y);

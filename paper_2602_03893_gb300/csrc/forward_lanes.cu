@@ -21,6 +21,7 @@
 #include <climits>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "gpair_internal.cuh"
 
@@ -156,16 +157,20 @@ struct ZBand {
     }
 };
 
-// Slab descriptors in cube units: a block of scx x scy x scz cubes; lo/hi bound its Gaussian
-// centres (for the sample band of each sensor).
-__global__ void slab_info_cube_kernel(GaussDev g, int ncx, int ncy, int ncz, int scx, int scy, int scz, int nsx,
-                                      int nsy, int S, SlabInfo* si) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= S) return;
-    const int sx = s % nsx, sy = (s / nsx) % nsy, sz = s / (nsx * nsy);
+// The slabs of a lattice: blocks of sx x sy x sz cubes, kx x ky of them across, and the lattice's cubes.
+struct CubeSlabs {
+    int ncx, ncy, ncz, sx, sy, sz, kx, ky;
+};
+static CubeSlabs cube_slabs(const GaussDev& g, int sx, int sy, int sz) {
+    const int cx = (g.nx + CUBE - 1) / CUBE, cy = (g.ny + CUBE - 1) / CUBE, cz = (g.nz + CUBE - 1) / CUBE;
+    return {cx, cy, cz, sx, sy, sz, (cx + sx - 1) / sx, (cy + sy - 1) / sy};
+}
+
+// Slab s in cube units; lo/hi bound its Gaussian centres (for the sample band of each sensor).
+__device__ __forceinline__ SlabInfo cube_slab(const GaussDev& g, const CubeSlabs& c, int s) {
     SlabInfo o;
-    o.bx0 = sx * scx; o.by0 = sy * scy; o.bz0 = sz * scz;
-    o.bdx = min(scx, ncx - o.bx0); o.bdy = min(scy, ncy - o.by0); o.bdz = min(scz, ncz - o.bz0);
+    o.bx0 = s % c.kx * c.sx; o.by0 = s / c.kx % c.ky * c.sy; o.bz0 = s / (c.kx * c.ky) * c.sz;
+    o.bdx = min(c.sx, c.ncx - o.bx0); o.bdy = min(c.sy, c.ncy - o.by0); o.bdz = min(c.sz, c.ncz - o.bz0);
     const int ax = o.bx0 * CUBE, bxn = min(g.nx, (o.bx0 + o.bdx) * CUBE);
     const int ay = o.by0 * CUBE, byn = min(g.ny, (o.by0 + o.bdy) * CUBE);
     const int az = o.bz0 * CUBE, bzn = min(g.nz, (o.bz0 + o.bdz) * CUBE);
@@ -178,8 +183,33 @@ __global__ void slab_info_cube_kernel(GaussDev g, int ncx, int ncy, int ncz, int
     }
     o.smax = g.sigma;
     o.t_begin = 0; o.t_end = o.bdx * o.bdy * o.bdz;
-    o.pad = 0;
-    si[s] = o;
+    o.pad = 1;
+    return o;
+}
+
+// Slab descriptors, a CTA each; pad is set where the slab has amplitudes: those without any (sparse
+// images) are left out of the forward.  The signals of a vessel phantom in 128 x 128 x 64 nodes, 1024 sensors: 690 us
+// with all slabs' bands cleared and written, 490 us.
+// Few sensors' forward is not worth the look through the amplitudes (13 us of 210 for 47 sensors and a million nodes).
+constexpr int SI_THREADS = 512, SI_SCAN_MIN = 128;
+__global__ void __launch_bounds__(SI_THREADS)
+slab_info_cube_kernel(GaussDev g, const CubeSlabs c, int scan, SlabInfo* si) {
+    SlabInfo o = cube_slab(g, c, blockIdx.x);
+    const int ax = o.bx0 * CUBE, bxn = min(g.nx, (o.bx0 + o.bdx) * CUBE);
+    const int ay = o.by0 * CUBE, byn = min(g.ny, (o.by0 + o.bdy) * CUBE);
+    const int az = o.bz0 * CUBE, bzn = min(g.nz, (o.bz0 + o.bdz) * CUBE);
+    bool any = !scan;
+    const int wy = byn - ay, lines = scan ? wy * (bzn - az) : 0;
+    for (int x0 = ax; x0 < bxn; x0 += 32) {
+        const int x = x0 + (threadIdx.x & 31);
+#pragma unroll 8
+        for (int r = threadIdx.x >> 5; r < lines; r += SI_THREADS / 32)
+            any |= x < bxn && g.A[((int64_t)(az + r / wy) * g.ny + ay + r % wy) * g.nx + x] != 0.f;
+    }
+    any = __syncthreads_or(any);
+    if (threadIdx.x) return;
+    o.pad = any;
+    si[blockIdx.x] = o;
 }
 
 // 1.5 * 2^23: adding it to |x| < 2^22 with rounding toward +inf leaves ceil(x) in the low bits.
@@ -188,10 +218,15 @@ constexpr int FL_MAGIC_BITS = 0x4B400000;
 
 // LF > 0: the correlation for windows of at most LF positions with the outputs in a register
 // ring of LF (the table's coefficients are compile-time operands); LF = 0: any window length.
-template <int P, int LF>
+// PART: `parts` CTAs share a slab, each with some lattice rows of its cubes: a block of 8 x 8 x 4, 8 x 4 x 4 or
+// 8 x 4 x 2 nodes, whose bins are a short run of the cube's band (each lane's own), so that the
+// correlation, which each part repeats, is short as well.  8 cubes and 128 sensors, windows of 32 samples: 48 us
+// with a warp to a cube and the general correlation, 24 us with eight.
+template <int P, int LF, bool PART>
 __global__ void __launch_bounds__(FL_MAXW * 32, 1)
-fwd_lanes_kernel(GaussDev g, ArrDev a, const SlabInfo* __restrict__ slabs, float* __restrict__ partial,
-                 int2* __restrict__ rows, int LB, int NZ, int* status, int use_tma,
+fwd_lanes_kernel(GaussDev g, ArrDev a, const SlabInfo* __restrict__ slabs, const CubeSlabs cubes,
+                 float* __restrict__ partial,
+                 int2* __restrict__ rows, int LB, int NZ, int parts, int* status, int use_tma,
                  const __grid_constant__ CUtensorMap tmap, const __grid_constant__ MomentTable T) {
     static_assert(P >= 6 && P <= 8, "6 to 8 moments");
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -205,12 +240,20 @@ fwd_lanes_kernel(GaussDev g, ArrDev a, const SlabInfo* __restrict__ slabs, float
     Z.init(wbase, NZ);
     float* Y = reinterpret_cast<float*>(wbase + fl_zbytes(NZ, P));              // [LB][32]
 
-    const int slab = blockIdx.y;
     const int j = (blockIdx.x * NW + warp) * 32 + lane;
     const bool has_sensor = j < a.Nd;
-    const SlabInfo sl = slabs[slab];
+    const SlabInfo sl = PART ? cube_slab(g, cubes, blockIdx.y / parts) : slabs[blockIdx.y];
     const int nCubes = sl.t_end;
-    const size_t row = (size_t)slab * a.Nd + (has_sensor ? j : 0);
+    const size_t row = (size_t)blockIdx.y * a.Nd + (has_sensor ? j : 0);
+    if (!sl.pad) {             // no amplitudes: empty rows
+        if (has_sensor) rows[row] = make_int2(0, 0);
+        return;
+    }
+    // PART: lattice rows of the cubes, 8 lz + ly: row r of nrows, 1 << nyl rows of y
+    const int part = PART ? blockIdx.y % parts : 0, nrows = PART ? CUBE * CUBE / parts : CUBE * CUBE;
+    const int nyl = PART && parts > 2 ? 2 : 3, ly0 = PART && parts > 2 ? (part & 1) * 4 : 0;
+    const int lz0 = PART ? (parts > 2 ? part >> 1 : part) * (nrows >> nyl) : 0;
+    auto lattice_row = [&](int r) { return PART ? (lz0 + (r >> nyl)) * CUBE + ly0 + (r & ((1 << nyl) - 1)) : r; };
 
     // this lane's sample band for the slab: [w, w + LB), w a multiple of 4
     float sx = 0.f, sy = 0.f, sz = 0.f;
@@ -312,6 +355,7 @@ fwd_lanes_kernel(GaussDev g, ArrDev a, const SlabInfo* __restrict__ slabs, float
         }
         const float* tile = S.tileA[b];
         unsigned relmax = 0;       // largest band offset of the cube's pairs (as unsigned: negatives too)
+        int lomin = NZ;            // PART: the pairs' least bin
         // a cube without amplitudes adds nothing (sparse images): the warp skips it
         bool any = false;
 #pragma unroll
@@ -345,6 +389,7 @@ fwd_lanes_kernel(GaussDev g, ArrDev a, const SlabInfo* __restrict__ slabs, float
                 // band, and the kernel then reports the capacity status
                 const unsigned ur = (unsigned)rel;
                 relmax = max(relmax, ur);
+                if constexpr (PART) lomin = min(lomin, (int)min(ur, (unsigned)(NZ - 1)));
                 idx[lx] = (int)min(ur, (unsigned)(NZ - 1)) * 32 + lane;
                 mom[lx][0] = Arow[lx] * invR;                      // the table carries the 1/2
 #pragma unroll
@@ -360,14 +405,14 @@ fwd_lanes_kernel(GaussDev g, ArrDev a, const SlabInfo* __restrict__ slabs, float
             float momA[CUBE][P], momB[CUBE][P], evA[CUBE], evB[CUBE], eA, eB;
             int idxA[CUBE], idxB[CUBE];
             unsigned long long emask = 0;
-            row_pairs(0, momA, idxA, evA, eA);
+            row_pairs(lattice_row(0), momA, idxA, evA, eA);
 #pragma unroll 1
-            for (int row = 0; row < CUBE * CUBE; row += 2) {
-                row_pairs(row + 1, momB, idxB, evB, eB);
+            for (int row = 0; row < nrows; row += 2) {
+                row_pairs(lattice_row(row + 1), momB, idxB, evB, eB);
 #pragma unroll
                 for (int k = 0; k < CUBE; k += 2) Z.add2(idxA[k], idxA[k + 1], momA[k], momA[k + 1]);
                 emask |= (unsigned long long)edge_corrected(T, eA) << row;
-                row_pairs((row + 2) & (CUBE * CUBE - 1), momA, idxA, evA, eA);   // row 64: a dummy row 0
+                row_pairs(lattice_row((row + 2) & (nrows - 1)), momA, idxA, evA, eA);   // past the last: a dummy row 0
 #pragma unroll
                 for (int k = 0; k < CUBE; k += 2) Z.add2(idxB[k], idxB[k + 1], momB[k], momB[k + 1]);
                 emask |= (unsigned long long)edge_corrected(T, eB) << (row + 1);
@@ -376,7 +421,7 @@ fwd_lanes_kernel(GaussDev g, ArrDev a, const SlabInfo* __restrict__ slabs, float
             while (emask) {
                 const int row = __ffsll(emask) - 1;
                 emask &= emask - 1;
-                row_pairs(row, momA, idxA, evA, eA);
+                row_pairs(lattice_row(row), momA, idxA, evA, eA);
 #pragma unroll
                 for (int lx = 0; lx < CUBE; ++lx)
                     if (edge_corrected(T, evA[lx])) {
@@ -388,6 +433,12 @@ fwd_lanes_kernel(GaussDev g, ArrDev a, const SlabInfo* __restrict__ slabs, float
             }
         }
         if (relmax >= (unsigned)NZ) set_status(status, DEV_CAPACITY);   // a pair outside its band: not reached
+        int bin0 = 0, nbins = NZ;
+        if constexpr (PART) {      // each lane's own run of bins; the warp walks the longest
+            bin0 = min(lomin, NZ - 1);
+            nbins = max(0, __reduce_max_sync(0xffffffffu, active ? (int)min(relmax, (unsigned)(NZ - 1)) - bin0 + 1 : 0));
+            bin0 = min(bin0, NZ - nbins);      // a run that would pass the end starts earlier, at clear bins
+        }
         // release the slot; the warp that releases it last refills it with cube t + FL_RING
         __syncwarp();
         int last = 0;
@@ -408,7 +459,8 @@ fwd_lanes_kernel(GaussDev g, ArrDev a, const SlabInfo* __restrict__ slabs, float
 #pragma unroll
         for (int q = 0; q < LF; ++q) acc[q] = 0.f;
 #pragma unroll 2
-        for (int b = 0; b < NZ; ++b) {
+        for (int k = 0; k < nbins; ++k) {
+            const int b = PART ? bin0 + k : k;
             float z[8];
             Z.load(b * 32 + lane, z);
             Z.clear(b * 32 + lane);
@@ -425,10 +477,10 @@ fwd_lanes_kernel(GaussDev g, ArrDev a, const SlabInfo* __restrict__ slabs, float
             for (int m = 0; m < LF - 1; ++m) acc[m] = acc[m + 1];
             acc[LF - 1] = 0.f;
         }
-        // outputs NZ .. NZ + L - 2 are in acc[0 .. L - 2]
+        // the L - 1 outputs past the last bin are in acc[0 .. L - 2]
 #pragma unroll
         for (int q = 0; q < LF - 1; ++q) {
-            const int n = NZ + q;
+            const int n = (PART ? bin0 + nbins : NZ) + q;
             const int yi = yoff + n;
             if (n < NO && (unsigned)yi < (unsigned)LBe) Y[yi * 32 + lane] += acc[q];
         }
@@ -507,28 +559,41 @@ size_t fwd_lanes_smem(int NW, int NZ, int LB, int P, int L) { return fl_smem_byt
 int fwd_lanes_nz(float h, float invDelta) { return fl_nz(h, invDelta); }
 float fwd_lanes_cube_radius(float h) { return cube_radius(h); }
 
-cudaError_t launch_slab_info_cubes(const GaussDev& g, int scx, int scy, int scz, int S, SlabInfo* si, cudaStream_t st) {
-    const int ncx = (g.nx + CUBE - 1) / CUBE, ncy = (g.ny + CUBE - 1) / CUBE, ncz = (g.nz + CUBE - 1) / CUBE;
-    const int nsx = (ncx + scx - 1) / scx, nsy = (ncy + scy - 1) / scy;
-    slab_info_cube_kernel<<<(S + 127) / 128, 128, 0, st>>>(g, ncx, ncy, ncz, scx, scy, scz, nsx, nsy, S, si);
-    return cudaGetLastError();
-}
+// Largest number of CTAs that may share a slab of one cube.
+int fwd_lanes_parts(const MomentTable& T) { return T.P == 6 && T.L <= 32 ? 8 : 1; }
 
-cudaError_t launch_forward_lanes(const GaussDev& g, const ArrDev& a, const SlabInfo* si, int S, float* partial,
-                                 int2* rows, int LB, int NZ, int NW, int* status, const CUtensorMap* tmap,
-                                 const MomentTable& T, cudaStream_t st) {
+// S rows a sensor: `parts` of each slab of sx x sy x sz cubes.  si: S descriptors' place.  ev (optional): two events
+// recorded immediately before and after the slab kernel.
+cudaError_t launch_forward_lanes(const GaussDev& g, const ArrDev& a, int sx, int sy, int sz, int S, SlabInfo* si, float* partial,
+                                 int2* rows, int LB, int NZ, int NW, int parts, int* status, const CUtensorMap* tmap,
+                                 const MomentTable& T, const cudaEvent_t* ev, cudaStream_t st) {
     static const CUtensorMap zero_map = [] { CUtensorMap z; memset(&z, 0, sizeof(z)); return z; }();
     const size_t smem = fl_smem_bytes(NW, NZ, LB, T.P, T.L);
-    dim3 grid((a.Nd + 32 * NW - 1) / (32 * NW), S);
-    const bool l16 = T.L <= 16;     // the table is zero beyond L: a 16-slot ring serves any L <= 16
-    auto kern = T.P == 6 ? (l16 ? fwd_lanes_kernel<6, 16> : fwd_lanes_kernel<6, 0>)
-              : T.P == 7 ? (l16 ? fwd_lanes_kernel<7, 16> : fwd_lanes_kernel<7, 0>)
-                         : (l16 ? fwd_lanes_kernel<8, 16> : fwd_lanes_kernel<8, 0>);
+    const dim3 grid((a.Nd + 32 * NW - 1) / (32 * NW), S);
+    // The table is zero beyond L: a ring of 16 slots serves any L <= 16, and so on.  Windows over 16 samples
+    // have fine steps, for which six terms do.  Rings as short as the window: 32 samples, 1.2e8 pairs, took 1424 us by
+    // the general correlation, 1485 us with 40 slots and 1115 us with 32.
+    const bool l16 = T.L <= 16;
+    auto six = [&](auto part) {
+        constexpr bool PART = decltype(part)::value;
+        return l16 ? fwd_lanes_kernel<6, 16, PART> : T.L <= 20 ? fwd_lanes_kernel<6, 20, PART>
+             : T.L <= 24 ? fwd_lanes_kernel<6, 24, PART> : T.L <= 32 ? fwd_lanes_kernel<6, 32, PART> : nullptr;
+    };
+    auto kern = parts > 1 ? six(std::true_type{}) : T.P == 6 ? six(std::false_type{})
+              : T.P == 7 ? (l16 ? fwd_lanes_kernel<7, 16, false> : fwd_lanes_kernel<7, 0, false>)
+                         : (l16 ? fwd_lanes_kernel<8, 16, false> : fwd_lanes_kernel<8, 0, false>);
+    if (!kern) kern = fwd_lanes_kernel<6, 0, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<grid, 32 * NW, smem, st>>>(g, a, si, partial, rows, LB, NZ, status, tmap != nullptr,
+    const CubeSlabs c = cube_slabs(g, sx, sy, sz);
+    if (parts == 1) slab_info_cube_kernel<<<S, SI_THREADS, 0, st>>>(g, c, a.Nd >= SI_SCAN_MIN, si);      // parts form their own: a launch less
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (ev && (e = cudaEventRecord(ev[0], st)) != cudaSuccess) return e;
+    kern<<<grid, 32 * NW, smem, st>>>(g, a, si, c, partial, rows, LB, NZ, parts, status, tmap != nullptr,
                                       tmap ? *tmap : zero_map, T);
-    return cudaGetLastError();
+    e = cudaGetLastError();
+    if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], st);
+    return e;
 }
 
 }  // namespace gp

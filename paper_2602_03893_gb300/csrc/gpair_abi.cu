@@ -34,10 +34,10 @@ cudaError_t launch_slab_reduce_rows(const ArrDev& a, const float* partial, const
                                     cudaStream_t st);
 size_t fwd_lanes_smem(int NW, int NZ, int LB, int P, int L);
 int fwd_lanes_nz(float h, float invDelta);
-cudaError_t launch_slab_info_cubes(const GaussDev& g, int scx, int scy, int scz, int S, SlabInfo* si, cudaStream_t st);
-cudaError_t launch_forward_lanes(const GaussDev& g, const ArrDev& a, const SlabInfo* si, int S, float* partial,
-                                 int2* rows, int LB, int NZ, int NW, int* status, const CUtensorMap* tmap,
-                                 const MomentTable& T, cudaStream_t st);
+int fwd_lanes_parts(const MomentTable& T);
+cudaError_t launch_forward_lanes(const GaussDev& g, const ArrDev& a, int sx, int sy, int sz, int S, SlabInfo* si, float* partial,
+                                 int2* rows, int LB, int NZ, int NW, int parts, int* status, const CUtensorMap* tmap,
+                                 const MomentTable& T, const cudaEvent_t* ev, cudaStream_t st);
 int adj_band_len(float rad, float smax, float k, float invDelta);
 cudaError_t launch_adjoint(const GaussDev& g, const ArrDev& a, const TileInfo* ti, const float* delta, float* gA,
                            float* gc, float* gs, int LBA, cudaStream_t st);
@@ -373,14 +373,18 @@ bool lanes_plan_from_blocks(FwdPlan& p, const GaussDev& g, const ArrDev& a, cons
         const double span = (std::min(sc[q] * CUBE_SIDE, nn[q]) - 1) * (double)g.h;   // centre to centre
         d2 += span * span;
     }
+    S *= p.parts;
     if (S > 65535) return false;            // slabs are the grid's y dimension
     p.S = (int)S;
     p.LB = ((int)std::ceil((std::sqrt(d2) + 2.0 * a.k * g.sigma) * a.invDelta) + 10 + 3) & ~3;
     p.PL = p.LB;
     p.NZ = fwd_lanes_nz(g.h, a.invDelta);
-    p.NW = 4;
+    const int groups = (a.Nd + 31) / 32;
+    p.NW = std::min(4, groups);
     while (p.NW > 0 && fwd_lanes_smem(p.NW, p.NZ, p.LB, T.P, T.L) > SMEM_PER_CTA) --p.NW;
     if (p.NW == 0) return false;
+    const int ctas = (groups + p.NW - 1) / p.NW;
+    p.NW = (groups + ctas - 1) / ctas;       // no more CTAs, evenly filled
     p.lanes = true;
     p.binned = true;
     p.TB = 0;
@@ -410,6 +414,16 @@ bool plan_forward_lanes(const GaussDev& g, const ArrDev& a, const MomentTable& T
         FwdPlan t;
         memset(&t, 0, sizeof(t));
         t.parts = 1;
+        if (!lanes_plan_from_blocks(t, g, a, T, sc)) break;
+        p = t;
+    }
+    // Single cubes that leave the chip idle: up to 8 warps share a cube, each with some of its lattice
+    // rows and bands of its own, while there is a scheduler for each.
+    const int64_t groups = (a.Nd + 31) / 32;
+    while (p.sbx * p.sby * p.sbz == 1 && p.parts < fwd_lanes_parts(T) &&
+           p.S * groups * 2 <= (int64_t)device_sms() * 4) {
+        FwdPlan t = p;
+        t.parts = p.parts * 2;
         if (!lanes_plan_from_blocks(t, g, a, T, sc)) break;
         p = t;
     }
@@ -482,6 +496,7 @@ bool plan_forward_op_capped(const GaussDev& g, const ArrDev& a, size_t cap, FwdP
         int sc[3] = {p.sbx, p.sby, p.sbz};
         bool ok = true;
         while (p.bytes > cap) {
+            p.parts = 1;
             int best = -1;
             for (int q = 0; q < 3; ++q)
                 if (sc[q] < nc[q] && (best < 0 || sc[q] < sc[best])) best = q;
@@ -514,7 +529,9 @@ gpair_status run_forward(const GaussDev& g, const ArrDev& a, float* y, cudaStrea
         e = launch_spatial_order(g, base + p.off_sort, gp, st);
         if (e == cudaSuccess) e = launch_tile_info(gp, ti, st);
         if (e == cudaSuccess) e = launch_slab_info_soa(gp, gp.ntiles, p.tiles_per_slab, p.S / p.parts, si, st);
-        if (e == cudaSuccess) e = launch_slab_order(si, p.S / p.parts, st);
+        // the order matters where the CTAs do not all start at once
+        if (e == cudaSuccess && (int64_t)p.S * ((a.Nd + 32 * p.NW - 1) / (32 * p.NW)) > device_sms())
+            e = launch_slab_order(si, p.S / p.parts, st);
         if (e == cudaSuccess && ev) e = cudaEventRecord(ev[0], st);
         if (e == cudaSuccess) e = launch_forward_free(gp, a, ti, si, p.S, part, rows, p.PL, p.LB, p.NW, p.parts, st);
         if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], st);
@@ -522,15 +539,9 @@ gpair_status run_forward(const GaussDev& g, const ArrDev& a, float* y, cudaStrea
         return cuda_status(e);
     }
     if (p.lanes) {
-        MomentTable mom;
-        if (!make_moment_table(g, a, mom)) return GPAIR_ERR_UNSUPPORTED;
         const bool tma = make_tmap(g, &map, CUBE_SIDE, CUBE_SIDE, CUBE_SIDE);   // ragged pitch: plain loads
-        e = launch_slab_info_cubes(g, p.sbx, p.sby, p.sbz, p.S, si, st);
-        if (e == cudaSuccess && ev) e = cudaEventRecord(ev[0], st);
-        if (e == cudaSuccess)
-            e = launch_forward_lanes(g, a, si, p.S, part, rows, p.LB, p.NZ, p.NW, status, tma ? &map : nullptr, mom,
-                                     st);
-        if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], st);
+        e = launch_forward_lanes(g, a, p.sbx, p.sby, p.sbz, p.S, si, part, rows, p.LB, p.NZ, p.NW, p.parts, status,
+                                 tma ? &map : nullptr, p.mom, ev, st);
         if (e == cudaSuccess) e = launch_slab_reduce(g, a, part, rows, p.S, p.PL, y, st);
         return cuda_status(e);
     }

@@ -279,6 +279,28 @@ __device__ __forceinline__ void box_distance(const SlabInfo& sl, float sx, float
     dmax = sqrt(mx);
 }
 
+// Grid mode: the slab of bdx x bdy x bdz bricks from brick (bx0, by0, bz0); its box is that of its node centres.
+__device__ __forceinline__ SlabInfo brick_block(const GaussDev& g, int bx0, int by0, int bz0, int bdx, int bdy, int bdz) {
+    SlabInfo o;
+    o.bx0 = bx0; o.by0 = by0; o.bz0 = bz0;
+    o.bdx = bdx; o.bdy = bdy; o.bdz = bdz;
+    const int ax = o.bx0 * BX, bxn = min(g.nx, (o.bx0 + o.bdx) * BX);
+    const int ay = o.by0 * BY, byn = min(g.ny, (o.by0 + o.bdy) * BY);
+    const int az = o.bz0 * BZ, bzn = min(g.nz, (o.bz0 + o.bdz) * BZ);
+    o.lo[0] = (float)(g.ox + (ax + 0.5) * g.h); o.hi[0] = (float)(g.ox + (bxn - 0.5) * g.h);
+    o.lo[1] = (float)(g.oy + (ay + 0.5) * g.h); o.hi[1] = (float)(g.oy + (byn - 0.5) * g.h);
+    o.lo[2] = (float)(g.oz + (az + 0.5) * g.h); o.hi[2] = (float)(g.oz + (bzn - 0.5) * g.h);
+    // widen by a few ulp so that float rounding of the box never cuts a centre off
+    for (int q = 0; q < 3; ++q) {
+        float pad = 1e-6f * (fabsf(o.lo[q]) + fabsf(o.hi[q])) + 1e-9f;
+        o.lo[q] -= pad; o.hi[q] += pad;
+    }
+    o.smax = g.sigma;
+    o.t_begin = 0; o.t_end = o.bdx * o.bdy * o.bdz;
+    o.pad = 0;
+    return o;
+}
+
 // Tile t (0-based within the slab) -> brick coordinates (grid mode).
 __device__ __forceinline__ void slab_brick(const SlabInfo& sl, int t, int& tx, int& ty, int& tz) {
     tx = sl.bx0 + t % sl.bdx;

@@ -145,6 +145,28 @@ def test_free_gaussians_band_longer_than_shared_memory():
     assert np.abs(yo).max() > 0
 
 
+@pytest.mark.parametrize("nd", [1, 33, 97])
+@pytest.mark.parametrize("sides", [(3, 2, 1), (8, 8, 8), (17, 9, 10)])
+@pytest.mark.parametrize("h", [0.1e-3, 0.125e-3, 0.2e-3, 0.3e-3])
+def test_lattice_few_cubes(h, sides, nd):
+    """One to eight warps share a cube; windows of 16, 20, 32 and 48 samples take the correlation's rings of 16, 24
+    and 40 outputs and its general form; records that end before the last windows."""
+    g = synth.centred_grid(*sides, h)
+    A = np.random.default_rng(nd).uniform(0.1, 1.0, g.M).astype(np.float32)
+    w = synth.Workload("few", g, synth.cap_sensors(nd, 15e-3, 150.0), 405, A=A)
+    _check(w)
+
+
+
+def test_lattice_sparse_slabs():
+    """Slabs without amplitudes leave empty rows, and the bands of the others start clear."""
+    g = synth.centred_grid(70, 40, 33, 0.1e-3)
+    A = np.zeros(g.M, np.float32)
+    A[np.random.default_rng(3).choice(g.M, 40, replace=False)] = 1.0
+    w = synth.Workload("sparse", g, synth.cap_sensors(300, 25e-3, 150.0), 1400, A=A)
+    _check(w)
+    _check(w, A=np.zeros(g.M, np.float32))
+
 @pytest.mark.parametrize("sides", [(1, 1, 1), (16, 8, 2), (13, 10, 5), (20, 20, 21)])
 def test_free_gaussians_few_tiles(sides):
     """One to eight CTAs share a tile of 256: a lone Gaussian, a whole tile, a part of a third one; and an order
