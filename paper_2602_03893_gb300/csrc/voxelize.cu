@@ -6,6 +6,8 @@
 // separable gather passes, each one coalesced read and write of the volume (HBM-bound).
 // Any other Gaussian set: tiles of the volume gather the separable boxes of factors of the Gaussians that
 // reach them; very large sets, and calls under stream capture, scatter them instead.
+#include <algorithm>
+
 #include "gpair_internal.cuh"
 
 namespace gp {
@@ -101,92 +103,134 @@ vox_pass_run_kernel(const float* __restrict__ in, float* __restrict__ out, int n
     }
 }
 
-// All three passes in one kernel, for taps fixed at compile time.  A CTA owns a column block of
-// VF_TX x VF_TY outputs and VF_TZ planes, one thread per (x, y) column, and marches z through the
-// VF_TZ + 2 MM input planes it needs: each plane's input patch (with an MM halo in x and y, zero
-// outside the volume) is staged in shared memory, convolved along x into a second buffer, then
-// along y by each thread for its own column; the last 2 MM + 1 such values stay in registers,
-// and once a plane's z neighbours are in, the thread writes its output.  The volume is read once
-// from DRAM and written once (the halos come from L2), instead of three reads and writes through
-// a scratch volume.  Each output is the same three sums as the separate passes', in the same
-// order, so the result is the same.
-constexpr int VF_TX = 32, VF_TY = 8, VF_TZ = 16;
-constexpr int VF_THREADS = VF_TX * VF_TY;
+// All three passes in one kernel, for taps fixed at compile time.  A CTA owns VF_TX x VF_TY outputs of tz
+// planes, four outputs along x to a thread, and marches z through the tz + 2 MM input planes it needs.
+// A thread convolves up to two runs of four inputs of the next plane along x (16-byte loads where rows are
+// whole vectors) into one of two shared buffers, while it convolves its own outputs of the current
+// plane along y from the other; the last 2 MM + 1 such values stay in registers for the sum along z.
+// One barrier a plane.  The volume is read once from DRAM and written once (the halos come from L2).
+// Each output is the same three sums as the separate passes', in the same order, so the result is the
+// same.
+//
+// Bound by memory.  With one output to a thread, 32 x 8 columns and three barriers a plane it took 50 us
+// for 256 x 256 x 128 voxels.
+constexpr int VF_TX = 64, VF_TY = 16, VF_THREADS = VF_TX / 4 * VF_TY;
 
-template <int MM>
-__global__ void __launch_bounds__(VF_THREADS, 4)
-vox_fused_kernel(const float* __restrict__ in, float* __restrict__ out, int nx, int ny, int nz, Taps taps) {
-    constexpr int PX = VF_TX + 2 * MM, PY = VF_TY + 2 * MM, NPATCH = PX * PY;
-    constexpr int NLOAD = (NPATCH + VF_THREADS - 1) / VF_THREADS;            // patch values per thread
-    constexpr int NXP = (PY * VF_TX + VF_THREADS - 1) / VF_THREADS;          // x-pass outputs per thread
-    constexpr int NR = 2 * MM + 1;                                          // taps, and planes in the ring
-    __shared__ float P[PY][PX];
-    __shared__ float Sx[PY][VF_TX];
-    const int t = threadIdx.x, tx = t % VF_TX, ty = t / VF_TX;
-    const int x0 = blockIdx.x * VF_TX, y0 = blockIdx.y * VF_TY, z0 = blockIdx.z * VF_TZ;
+constexpr int vf_ctas(int mm) { return mm <= 3 ? 3 : 2; }       // resident per SM (registers)
+
+// VEC: nx a multiple of 4 and both volumes 16-byte aligned.
+template <int MM, bool VEC>
+__global__ void __launch_bounds__(VF_THREADS, vf_ctas(MM))
+vox_fused_kernel(const float* __restrict__ in, float* __restrict__ out, int nx, int ny, int nz, int tz, Taps taps) {
+    constexpr int ROWS = VF_TY + 2 * MM, GX = VF_TX / 4, ITEMS = ROWS * GX;
+    constexpr int NI = (ITEMS + VF_THREADS - 1) / VF_THREADS;               // runs of four a thread convolves along x
+    constexpr int HV = (MM + 3) / 4, NL = 4 + 8 * HV;                       // vectors of halo a side, values loaded
+    constexpr int NR = 2 * MM + 1;
+    __shared__ __align__(16) float Sx[2][ROWS][VF_TX];
+    const int t = threadIdx.x, gx = t % GX, ty = t / GX;
+    const int x0 = blockIdx.x * VF_TX, y0 = blockIdx.y * VF_TY, z0 = blockIdx.z * tz;
     const int64_t plane = (int64_t)nx * ny;
-    // this thread's patch values of input plane zi (zero outside the volume)
-    auto load = [&](int zi, float (&v)[NLOAD]) {
+    const int zn = min(tz, nz - z0);
+    float pre[NI][NL];
+    auto load = [&](int zi) {
 #pragma unroll
-        for (int u = 0; u < NLOAD; ++u) {
-            const int q = t + u * VF_THREADS;
-            const int px = q % PX, py = q / PX;
-            const int gx = x0 - MM + px, gy = y0 - MM + py;
-            const bool ok = q < NPATCH && (unsigned)gx < (unsigned)nx && (unsigned)gy < (unsigned)ny &&
-                            (unsigned)zi < (unsigned)nz;
-            v[u] = ok ? __ldg(in + zi * plane + (int64_t)gy * nx + gx) : 0.f;
-        }
-    };
-    float pre[NLOAD];
-    load(z0 - MM, pre);
-    float ring[NR];                          // ring[NR - 1] is the newest plane's value
+        for (int u = 0; u < NI; ++u) {
+            const int q = t + u * VF_THREADS, y = y0 - MM + q / GX, x = x0 + (q % GX) * 4 - 4 * HV;
+            const bool row = q < ITEMS && (unsigned)y < (unsigned)ny && (unsigned)zi < (unsigned)nz;
+            const float* src = in + (int64_t)zi * plane + (int64_t)y * nx;
+            if (VEC) {
 #pragma unroll
-    for (int m = 0; m < NR; ++m) ring[m] = 0.f;
-    const bool own = x0 + tx < nx && y0 + ty < ny;
-#pragma unroll 1
-    for (int i = 0; i < VF_TZ + 2 * MM; ++i) {
-        __syncthreads();      // the previous plane's x pass is done with P, its y pass with Sx
+                for (int v = 0; v < NL / 4; ++v) {
+                    const bool ok = row && (unsigned)(x + 4 * v) < (unsigned)nx;
+                    const float4 f = ok ? __ldg(reinterpret_cast<const float4*>(src + x + 4 * v)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    pre[u][4 * v] = f.x; pre[u][4 * v + 1] = f.y; pre[u][4 * v + 2] = f.z; pre[u][4 * v + 3] = f.w;
+                }
+            } else {
 #pragma unroll
-        for (int u = 0; u < NLOAD; ++u) {
-            const int q = t + u * VF_THREADS;
-            if (q < NPATCH) P[q / PX][q % PX] = pre[u];
-        }
-        __syncthreads();
-        if (i + 1 < VF_TZ + 2 * MM) load(z0 - MM + i + 1, pre);      // the next plane, in flight meanwhile
-#pragma unroll
-        for (int u = 0; u < NXP; ++u) {
-            const int q = t + u * VF_THREADS;
-            if (q < PY * VF_TX) {
-                const int r = q / VF_TX, x = q % VF_TX;
-                float acc = 0.f;
-#pragma unroll
-                for (int m = 0; m < NR; ++m) acc = fmaf(taps.t[m], P[r][x + m], acc);
-                Sx[r][x] = acc;
+                for (int v = 4 * HV - MM; v < 4 * HV + 4 + MM; ++v)
+                    pre[u][v] = row && (unsigned)(x + v) < (unsigned)nx ? __ldg(src + x + v) : 0.f;
             }
         }
-        __syncthreads();
-        float acc = 0.f;
+    };
+    auto along_x = [&](int buf) {
 #pragma unroll
-        for (int m = 0; m < NR; ++m) acc = fmaf(taps.t[m], Sx[ty + m][tx], acc);
+        for (int u = 0; u < NI; ++u) {
+            const int q = t + u * VF_THREADS;
+            if (q >= ITEMS) break;
+            float o[4];
 #pragma unroll
-        for (int m = 0; m < NR - 1; ++m) ring[m] = ring[m + 1];
-        ring[NR - 1] = acc;                  // the (x, y)-convolved value of plane z0 - MM + i
-        if (i >= 2 * MM) {                   // plane zo = z0 + i - 2 MM has all its z neighbours
-            const int zo = z0 + i - 2 * MM;
-            float o = 0.f;
+            for (int k = 0; k < 4; ++k) {
+                float acc = 0.f;
 #pragma unroll
-            for (int m = 0; m < NR; ++m) o = fmaf(taps.t[m], ring[m], o);
-            if (own && zo < nz) out[zo * plane + (int64_t)(y0 + ty) * nx + x0 + tx] = o;
+                for (int m = 0; m < NR; ++m) acc = fmaf(taps.t[m], pre[u][4 * HV - MM + k + m], acc);
+                o[k] = acc;
+            }
+            *reinterpret_cast<float4*>(&Sx[buf][q / GX][(q % GX) * 4]) = make_float4(o[0], o[1], o[2], o[3]);
         }
+    };
+    float ring[NR][4];                       // ring[NR - 1] is the newest plane's
+#pragma unroll
+    for (int m = 0; m < NR; ++m)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) ring[m][k] = 0.f;
+    const int xo = x0 + gx * 4, yo = y0 + ty;
+    load(z0 - MM);
+    along_x(0);
+    __syncthreads();
+    const int planes = zn + 2 * MM;
+#pragma unroll 1
+    for (int i = 0; i < planes; ++i) {
+        const bool more = i + 1 < planes;
+        if (more) load(z0 - MM + i + 1);     // in flight during this plane's sums
+#pragma unroll
+        for (int m = 0; m < NR - 1; ++m)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) ring[m][k] = ring[m + 1][k];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) ring[NR - 1][k] = 0.f;
+#pragma unroll
+        for (int m = 0; m < NR; ++m) {       // the (x, y)-convolved values of plane z0 - MM + i
+            const float4 v = *reinterpret_cast<const float4*>(&Sx[i & 1][ty + m][gx * 4]);
+            ring[NR - 1][0] = fmaf(taps.t[m], v.x, ring[NR - 1][0]);
+            ring[NR - 1][1] = fmaf(taps.t[m], v.y, ring[NR - 1][1]);
+            ring[NR - 1][2] = fmaf(taps.t[m], v.z, ring[NR - 1][2]);
+            ring[NR - 1][3] = fmaf(taps.t[m], v.w, ring[NR - 1][3]);
+        }
+        if (i >= 2 * MM && yo < ny) {        // plane z0 + i - 2 MM has all its z neighbours
+            float o[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                o[k] = 0.f;
+#pragma unroll
+                for (int m = 0; m < NR; ++m) o[k] = fmaf(taps.t[m], ring[m][k], o[k]);
+            }
+            float* dst = out + (int64_t)(z0 + i - 2 * MM) * plane + (int64_t)yo * nx + xo;
+            if (VEC) {
+                if (xo < nx) *reinterpret_cast<float4*>(dst) = make_float4(o[0], o[1], o[2], o[3]);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (xo + k < nx) dst[k] = o[k];
+            }
+        }
+        if (more) along_x((i + 1) & 1);
+        __syncthreads();
     }
 }
 
 template <int MM>
 static void vox_passes_fixed(const float* A, float* vol, float* tmp, const gpair_grid& og, const Taps& taps,
                              dim3 grid, cudaStream_t st) {
-    const dim3 fgrid((og.nx + VF_TX - 1) / VF_TX, (og.ny + VF_TY - 1) / VF_TY, (og.nz + VF_TZ - 1) / VF_TZ);
+    // planes a CTA: as few (but 4) as one wave of CTAs covers the volume with; 32 where the columns alone are more
+    // (each CTA reads the 2 MM planes of overlap again)
+    const int64_t cols = (int64_t)((og.nx + VF_TX - 1) / VF_TX) * ((og.ny + VF_TY - 1) / VF_TY);
+    const int64_t chunks = (int64_t)device_sms() * vf_ctas(MM) / cols;
+    const int tz = chunks < 1 ? 32 : (int)std::max<int64_t>(4, (og.nz + chunks - 1) / chunks);
+    const dim3 fgrid((og.nx + VF_TX - 1) / VF_TX, (og.ny + VF_TY - 1) / VF_TY, (og.nz + tz - 1) / tz);
     if (fgrid.y <= 65535 && fgrid.z <= 65535) {
-        vox_fused_kernel<MM><<<fgrid, VF_THREADS, 0, st>>>(A, vol, og.nx, og.ny, og.nz, taps);
+        const bool vec = og.nx % 4 == 0 && (((uintptr_t)A | (uintptr_t)vol) & 15) == 0;
+        if (vec) vox_fused_kernel<MM, true><<<fgrid, VF_THREADS, 0, st>>>(A, vol, og.nx, og.ny, og.nz, tz, taps);
+        else vox_fused_kernel<MM, false><<<fgrid, VF_THREADS, 0, st>>>(A, vol, og.nx, og.ny, og.nz, tz, taps);
         return;
     }
     vox_pass_fixed_kernel<0, MM><<<grid, VOX_THREADS, 0, st>>>(A, vol, og.nx, og.ny, og.nz, taps);

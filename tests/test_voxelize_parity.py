@@ -161,3 +161,13 @@ def test_free_gaussians_captured():
     graph.replay()
     # the same terms in another order: 300 of them, in single precision
     assert torch.allclose(one, two, rtol=300 * 2.0 ** -23, atol=300 * 2.0 ** -23 * float(one.max()))
+
+
+@pytest.mark.parametrize("dims", [(64, 16, 32), (65, 17, 5), (68, 15, 33), (4, 1, 1), (131, 40, 9)])
+@pytest.mark.parametrize("k", [1.5, 3.0, 6.0])
+def test_lattice_fused_tiles(dims, k):
+    """Whole and ragged 64 x 16 tiles, rows of whole vectors and not, planes fewer and more than a CTA's."""
+    g = synth.centred_grid(*dims, 0.1e-3)
+    A = np.random.default_rng(4).uniform(0, 1, g.M).astype(np.float32)
+    w = synth.Workload("tiles", g, synth.cap_sensors(1, 5e-3, 10.0), 16, A=A)
+    assert rel_l2(_gpu_vox(w, g, k), _ora_vox(w, g, k)) < 1e-4
