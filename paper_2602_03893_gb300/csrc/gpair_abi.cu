@@ -63,14 +63,13 @@ size_t assa_dconv_bytes(const ArrDev& a, const AssaTable& T);
 cudaError_t launch_assa_adjoint(const GaussDev& g, const ArrDev& a, const float* delta, float* gA, const AssaTable& T,
                                 float* dconv, const cudaEvent_t* ev, cudaStream_t st);
 cudaError_t launch_resid(const float* y, const float* b, float* delta, float scale, int64_t n, double* partial,
-                         double* out, cudaStream_t st);
+                         double* out, const SchedParams& p, StepSched* sd, cudaStream_t st);
 cudaError_t launch_reduce2(const float* a, const float* b, const float* c, int64_t n, double* partial, double* out,
                            cudaStream_t st);
 cudaError_t launch_ls(const float* r, const float* Fg, int64_t n, float* x, const float* g, int64_t M,
                       double* partial, double* nd, cudaStream_t st);
-cudaError_t launch_adam(float* z, float* m, float* v, const float* gx, int64_t M, int npc, float eps, float b1,
+cudaError_t launch_adam(float* z, float* m, float* v, float* x, const float* gx, int64_t M, int npc, float eps, float b1,
                         float b2, float adam_eps, const StepSched* sd, cudaStream_t st);
-cudaError_t launch_schedule(const SchedParams& p, StepSched* sd, cudaStream_t st);
 cudaError_t launch_set_step(StepSched* sd, int t, const SchedParams& p, cudaStream_t st);
 int red_blocks();
 bool vox_is_lattice(const GaussDev& g, const gpair_grid& og);
@@ -1105,6 +1104,7 @@ struct gpair_solver {
     ArrDev a;
     gpair_step_params p;
     int t = 0;
+    bool x_ready = false;    // x holds the amplitudes of z (Adam)
     float *z = nullptr, *m = nullptr, *v = nullptr, *x = nullptr, *gx = nullptr;
     float *y = nullptr, *delta = nullptr, *Fg = nullptr;
     double* red = nullptr;   // reduction partials (2 * red_blocks) + results (4)
@@ -1260,7 +1260,13 @@ gpair_status gpair_solver_timings(gpair_solver* S, double* ms, int* nsteps) {
 }  // extern "C"
 
 namespace {
-// The launches of one reconstruction step on st: no host synchronisation, S->t unchanged, and the
+// The amplitudes x of the iterate z, which every Adam step leaves for the next: formed here where z came from outside.
+gpair_status ensure_image(gpair_solver* S, cudaStream_t st) {
+    if (S->p.rule != GPAIR_RULE_ADAM || S->x_ready) return GPAIR_OK;
+    return cuda_status(launch_npc(S->z, S->x, S->g.M, S->p.npc != 0, S->p.npc_eps, st));
+}
+
+// The launches of one reconstruction step on st, given x: no host synchronisation, S->t unchanged, and the
 // same launches with the same arguments at every step (so that they can be replayed as a graph).
 gpair_status step_launches(gpair_solver* S, const float* b, const cudaEvent_t* ev, cudaStream_t st) {
     const int64_t M = S->g.M, N = (int64_t)S->a.Nd * S->a.Nt;
@@ -1270,25 +1276,24 @@ gpair_status step_launches(gpair_solver* S, const float* b, const cudaEvent_t* e
     gpair_status s;
     if (S->p.rule == GPAIR_RULE_ADAM) {
         const int npc = S->p.npc != 0;
-        if ((e = launch_npc(S->z, S->x, M, npc, S->p.npc_eps, st)) != cudaSuccess) return cuda_status(e);
         if ((s = solver_forward(S, S->y, ev ? ev + 1 : nullptr, st)) != GPAIR_OK) return s;
-        if ((e = launch_resid(S->y, b, S->delta, (float)(2.0 / (double)N), N, partial, res, st)) != cudaSuccess)
+        // and the CAWR step size and bias corrections of this step, from the device step count
+        if ((e = launch_resid(S->y, b, S->delta, (float)(2.0 / (double)N), N, partial, res, S->sched, S->sd, st)) != cudaSuccess)
             return cuda_status(e);
         if ((s = solver_adjoint(S, S->delta, S->gx, ev ? ev + 3 : nullptr, st)) != GPAIR_OK) return s;
         if (S->vcr &&    // grad_x += lambda grad R_VCR(x); R_VCR(x) into res[4]
             (e = launch_vcr(S->x, S->g.nx, S->g.ny, S->g.nz, S->p.vcr_beta, S->p.vcr_eps, S->p.vcr_lambda, partial,
                             res + 4, S->gx, st)) != cudaSuccess)
             return cuda_status(e);
-        // CAWR step size and bias corrections of this step, from the device step count
-        if ((e = launch_schedule(S->sched, S->sd, st)) != cudaSuccess) return cuda_status(e);
-        if ((e = launch_adam(S->z, S->m, S->v, S->gx, M, npc, S->p.npc_eps, S->p.beta1, S->p.beta2, S->p.adam_eps,
+        if ((e = launch_adam(S->z, S->m, S->v, S->x, S->gx, M, npc, S->p.npc_eps, S->p.beta1, S->p.beta2, S->p.adam_eps,
                              S->sd, st)) != cudaSuccess)
             return cuda_status(e);
     } else {
         // steepest descent on x = z with the exact line search alpha = <r, F g> / |F g|^2
         S->g.A = S->z;
         s = solver_forward(S, S->y, ev ? ev + 1 : nullptr, st);
-        if (s == GPAIR_OK && (e = launch_resid(S->y, b, S->delta, 1.0f, N, partial, res, st)) != cudaSuccess)
+        if (s == GPAIR_OK && (e = launch_resid(S->y, b, S->delta, 1.0f, N, partial, res, S->sched, nullptr, st)) !=
+                                    cudaSuccess)
             s = cuda_status(e);
         if (s == GPAIR_OK) s = solver_adjoint(S, S->delta, S->gx, ev ? ev + 3 : nullptr, st);
         S->g.A = S->gx;
@@ -1331,7 +1336,13 @@ gpair_status gpair_step(gpair_solver* S, const float* b, double* loss_out, doubl
         ev = &S->evs[6 * S->nrec];
         if (cudaEventRecord(ev[0], st) != cudaSuccess) return GPAIR_ERR_CUDA;
     }
-    gpair_status s = step_launches(S, b, ev, st);
+    // a step that a caller captures forms x itself: it may be replayed after a change of z
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const bool captured = cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
+    if (captured) S->x_ready = false;
+    gpair_status s = ensure_image(S, st);
+    S->x_ready = false;
+    if (s == GPAIR_OK) s = step_launches(S, b, ev, st);
     if (s != GPAIR_OK) {
         // the schedule kernel may have advanced the device step count before a later launch failed:
         // put it back to the host count, so that a checkpoint taken now resumes with the right step
@@ -1342,6 +1353,7 @@ gpair_status gpair_step(gpair_solver* S, const float* b, double* loss_out, doubl
         if (cudaEventRecord(ev[5], st) != cudaSuccess) return GPAIR_ERR_CUDA;
         S->nrec += 1;
     }
+    S->x_ready = !captured;
     S->t += 1;
     return read_loss(S, st, loss_out, resid_out);
 }
@@ -1384,11 +1396,15 @@ gpair_status gpair_solver_steps(gpair_solver* S, const float* b, int n, double* 
         }
         S->gb = b;
     }
+    const gpair_status si = ensure_image(S, st);
+    S->x_ready = false;
+    if (si != GPAIR_OK) return si;
     for (int k = 0; k < n; ++k)
         if (cudaGraphLaunch(S->gexec, st) != cudaSuccess) {
             S->t += k;      // the k replays already queued advance the device step count
             return GPAIR_ERR_CUDA;
         }
+    S->x_ready = true;
     S->t += n;
     return read_loss(S, st, loss_out, resid_out);
 }
@@ -1415,6 +1431,7 @@ gpair_status gpair_solver_set_state(gpair_solver* S, const float* z, const float
     if (!S || t < 0) return GPAIR_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const size_t bytes = (size_t)S->g.M * 4;
+    if (z) S->x_ready = false;
     if (z && cudaMemcpyAsync(S->z, z, bytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return GPAIR_ERR_CUDA;
     if (m && cudaMemcpyAsync(S->m, m, bytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return GPAIR_ERR_CUDA;
     if (v && cudaMemcpyAsync(S->v, v, bytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return GPAIR_ERR_CUDA;

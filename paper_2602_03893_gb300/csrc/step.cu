@@ -72,8 +72,8 @@ reduce2_kernel(const float* __restrict__ a, const float* __restrict__ b, const f
 }
 
 // out[q] = sum_blk partial[blk * stride + q] for q < nq, in block order (deterministic).
-__global__ void finish_kernel(const double* __restrict__ partial, int nblk, int stride, int nq,
-                              double* __restrict__ out) {
+__device__ __forceinline__ void finish_sums(const double* __restrict__ partial, int nblk, int stride, int nq,
+                                            double* __restrict__ out) {
     __shared__ double red[RED_THREADS / 32];
     for (int q = 0; q < nq; ++q) {
         double acc = 0.0;
@@ -83,15 +83,18 @@ __global__ void finish_kernel(const double* __restrict__ partial, int nblk, int 
         __syncthreads();
     }
 }
+__global__ void finish_kernel(const double* __restrict__ partial, int nblk, int stride, int nq,
+                              double* __restrict__ out) {
+    finish_sums(partial, nblk, stride, nq, out);
+}
 
 // Adam on z with gradient g_x (and the NPC chain rule g_z = g_x * 2 (z + eps)).
 // Per-step scalars of Algorithm 2 on the device, so that a step's launches do not change from one
 // step to the next (and can be replayed as a CUDA graph): the CAWR step size of step t and Adam's
 // bias corrections 1 / (1 - b1^(t+1)), 1 / sqrt(1 - b2^(t+1)), the powers kept as running
 // products.  One thread; FP64 only for the products (GB300's FP64 pipe is slow, and a chain of
-// FP64 pow / cos / divide took ~11 us).  schedule_kernel advances t.
-__global__ void schedule_kernel(SchedParams p, StepSched* __restrict__ sd) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// FP64 pow / cos / divide took ~11 us).  Advances t.
+__device__ __forceinline__ void schedule_step(const SchedParams& p, StepSched* __restrict__ sd) {
     const int t = sd->t;
     // SGDR: periods T0, T0 T_mult, ...; T_cur counts iterations since the last restart
     const int T0 = p.T0 > 0 ? p.T0 : 1;
@@ -115,6 +118,13 @@ __global__ void schedule_kernel(SchedParams p, StepSched* __restrict__ sd) {
     sd->t = t + 1;
 }
 
+// Block 0: out[0] = the sum of the residual's partials; block 1: the step's scalars, a launch less.
+__global__ void finish_schedule_kernel(const double* __restrict__ partial, int nblk, double* __restrict__ out,
+                                       SchedParams p, StepSched* __restrict__ sd) {
+    if (blockIdx.x == 0) finish_sums(partial, nblk, 1, 1, out);
+    else if (threadIdx.x == 0) schedule_step(p, sd);
+}
+
 __global__ void set_step_kernel(StepSched* __restrict__ sd, int t, double b1t, double b2t) {
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         sd->t = t;
@@ -123,7 +133,8 @@ __global__ void set_step_kernel(StepSched* __restrict__ sd, int t, double b1t, d
     }
 }
 
-__global__ void adam_kernel(float* __restrict__ z, float* __restrict__ m, float* __restrict__ v,
+// x: the amplitudes of the new iterate, as npc_kernel gives them.
+__global__ void adam_kernel(float* __restrict__ z, float* __restrict__ m, float* __restrict__ v, float* __restrict__ x,
                             const float* __restrict__ gx, int64_t M, int npc, float eps, float b1, float b2,
                             float adam_eps, const StepSched* __restrict__ sd) {
     const float eta = sd->eta, inv_c1 = sd->inv_c1, inv_sqrt_c2 = sd->inv_sqrt_c2;
@@ -135,7 +146,9 @@ __global__ void adam_kernel(float* __restrict__ z, float* __restrict__ m, float*
         float vi = b2 * v[i] + (1.f - b2) * g * g;
         m[i] = mi;
         v[i] = vi;
-        z[i] = zi - eta * (mi * inv_c1) / (sqrtf(vi) * inv_sqrt_c2 + adam_eps);
+        zi = zi - eta * (mi * inv_c1) / (sqrtf(vi) * inv_sqrt_c2 + adam_eps);
+        z[i] = zi;
+        x[i] = npc ? (zi + eps) * (zi + eps) : zi;
     }
 }
 
@@ -177,11 +190,12 @@ cudaError_t launch_npc(const float* z, float* x, int64_t M, int npc, float eps, 
     return cudaGetLastError();
 }
 
-// partial must hold RED_BLOCKS doubles; out[0] = sum r^2.
+// partial must hold RED_BLOCKS doubles; out[0] = sum r^2.  sd (optional): the schedule advances too.
 cudaError_t launch_resid(const float* y, const float* b, float* delta, float scale, int64_t n, double* partial,
-                         double* out, cudaStream_t st) {
+                         double* out, const SchedParams& p, StepSched* sd, cudaStream_t st) {
     resid_kernel<<<RED_BLOCKS, RED_THREADS, 0, st>>>(y, b, delta, scale, n, partial);
-    finish_kernel<<<1, RED_THREADS, 0, st>>>(partial, RED_BLOCKS, 1, 1, out);
+    if (sd) finish_schedule_kernel<<<2, RED_THREADS, 0, st>>>(partial, RED_BLOCKS, out, p, sd);
+    else finish_kernel<<<1, RED_THREADS, 0, st>>>(partial, RED_BLOCKS, 1, 1, out);
     return cudaGetLastError();
 }
 
@@ -201,20 +215,15 @@ cudaError_t launch_ls(const float* r, const float* Fg, int64_t n, float* x, cons
     return cudaGetLastError();
 }
 
-cudaError_t launch_schedule(const SchedParams& p, StepSched* sd, cudaStream_t st) {
-    schedule_kernel<<<1, 32, 0, st>>>(p, sd);
-    return cudaGetLastError();
-}
-
 // t steps taken: the running products are beta^t.
 cudaError_t launch_set_step(StepSched* sd, int t, const SchedParams& p, cudaStream_t st) {
     set_step_kernel<<<1, 32, 0, st>>>(sd, t, std::pow(p.beta1, (double)t), std::pow(p.beta2, (double)t));
     return cudaGetLastError();
 }
 
-cudaError_t launch_adam(float* z, float* m, float* v, const float* gx, int64_t M, int npc, float eps, float b1,
+cudaError_t launch_adam(float* z, float* m, float* v, float* x, const float* gx, int64_t M, int npc, float eps, float b1,
                         float b2, float adam_eps, const StepSched* sd, cudaStream_t st) {
-    adam_kernel<<<ew_blocks(M), 256, 0, st>>>(z, m, v, gx, M, npc, eps, b1, b2, adam_eps, sd);
+    adam_kernel<<<ew_blocks(M), 256, 0, st>>>(z, m, v, x, gx, M, npc, eps, b1, b2, adam_eps, sd);
     return cudaGetLastError();
 }
 
