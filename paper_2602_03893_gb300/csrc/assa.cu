@@ -23,6 +23,7 @@
 
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "adjoint_split.cuh"
 #include "gpair_internal.cuh"
@@ -267,6 +268,282 @@ assa_fwd_kernel(GaussDev g, ArrDev a, const SlabInfo* __restrict__ slabs, float*
     }
 }
 
+// The forward with the lanes of a warp owning 32 sensors, for slabs of at most ASSA_FLUSH bricks.  All lanes
+// take the same Gaussian; a lane adds its pair's mass, in fixed point as above, to an integer band of its
+// own, [sample][lane] in shared memory: 32 different banks whatever samples the lanes address, and a
+// shared-memory add that nothing waits for.  The band holds the fine samples between the
+// sensor's nearest and farthest distance to the slab, not the pulse's margins; an impulse outside the
+// record goes to the entry after the last.  After the slab a lane scales its band to floats and
+// convolves it, eight outputs at a time over a window of registers.  A lane whose masses have no bound
+// (sensor in the slab's box, amplitudes not finite) adds floats.
+//
+// Bound by the MUFU pipe (two operations a pair) and instruction issue; with a warp to a sensor the
+// lanes' samples met in the same banks and every pair had its own range tests (48 instructions a pair).
+constexpr int ASSA_LANES_MAXW = 4, ASSA_LANES_Q = 8;
+
+struct AssaLanesHdr {
+    float tileA[ASSA_RING][TILE];
+    uint64_t full[ASSA_RING];
+    int released[ASSA_RING];
+    int issued[ASSA_RING];
+    int abort;
+};
+constexpr size_t ASSA_LANES_HDR = (sizeof(AssaLanesHdr) + 127) & ~(size_t)127;
+
+// Entries of a lane's band for a slab whose centres span `diag` metres.
+int assa_lanes_nz(double diag, double invDelta, int alpha) { return (int)ceil(diag * 1.00001 * invDelta * alpha) + 6; }
+size_t assa_lanes_smem(int NW, int NZ) { return ASSA_LANES_HDR + (size_t)NW * (NZ + 1) * 32 * sizeof(int); }
+
+// Slabs of sb bricks that divide the blocks of qb bricks in which the kernel above walks the lattice: a slab's masses
+// take its block's scale, so that both kernels round each mass alike.  kx x ky slabs across.
+struct AssaSlabs {
+    int sb[3], qb[3], kx, ky;
+};
+
+__global__ void __launch_bounds__(ASSA_LANES_MAXW * 32, 2)
+assa_fwd_lanes_kernel(GaussDev g, ArrDev a, const AssaSlabs slabs, float* __restrict__ partial,
+                      int2* __restrict__ rows, int LB, int NZ, int* status, int use_tma,
+                      const __grid_constant__ CUtensorMap tmap, const __grid_constant__ AssaTable T,
+                      const unsigned* __restrict__ amax_bits) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    AssaLanesHdr& S = *reinterpret_cast<AssaLanesHdr*>(smem_raw);
+    const int NW = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int* Z = reinterpret_cast<int*>(smem_raw + ASSA_LANES_HDR) + (size_t)warp * (NZ + 1) * 32 + lane;    // [entry * 32]
+    const int alpha = T.alpha, K = T.K;
+    const int j = (blockIdx.x * NW + warp) * 32 + lane;
+    const bool has_sensor = j < a.Nd;
+    const size_t row = (size_t)blockIdx.y * a.Nd + (has_sensor ? j : 0);
+    const int Nup = alpha * a.Nt;
+    // this CTA's slab and its block
+    const int si[3] = {(int)(blockIdx.y % slabs.kx), (int)(blockIdx.y / slabs.kx % slabs.ky), (int)(blockIdx.y / (slabs.kx * slabs.ky))};
+    const int nt[3] = {g.ntx, g.nty, g.ntz};
+    int b0[3], bd[3], q0[3], qd[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const int per = (slabs.qb[q] + slabs.sb[q] - 1) / slabs.sb[q], sub = si[q] % per * slabs.sb[q];
+        q0[q] = si[q] / per * slabs.qb[q];
+        qd[q] = min(slabs.qb[q], nt[q] - q0[q]);
+        b0[q] = q0[q] + sub;
+        bd[q] = min(slabs.sb[q], qd[q] - sub);
+    }
+    if (bd[0] <= 0 || bd[1] <= 0 || bd[2] <= 0) {          // past the block's end at a ragged face
+        if (has_sensor) rows[row] = make_int2(0, 0);
+        return;
+    }
+    const SlabInfo sl = brick_block(g, b0[0], b0[1], b0[2], bd[0], bd[1], bd[2]);
+    const int nTiles = sl.t_end;
+
+    // the lane's samples of the slab, [w, w + LBe), and its impulses' fine samples, [lo, lo + cnt)
+    float sx = 0.f, sy = 0.f, sz = 0.f, qscale = 0.f;
+    int n_lo = 0, n_hi = -1, lo = 0, cnt = 0;
+    if (has_sensor) {
+        sx = a.xyz[3 * j]; sy = a.xyz[3 * j + 1]; sz = a.xyz[3 * j + 2];
+        double dmin, dmax;
+        box_distance(sl, sx, sy, sz, dmin, dmax);
+        const float amax = __int_as_float((int)*amax_bits);
+        double qmin, qmax;
+        box_distance(brick_block(g, q0[0], q0[1], q0[2], qd[0], qd[1], qd[2]), sx, sy, sz, qmin, qmax);
+        if (amax > 0.f && amax <= 3.0e38f && qmin > 0.0) qscale = (float)((double)ASSA_QMAX * qmin / (double)amax);
+        const double ks = (double)a.k * sl.smax;
+        double l = floor(((dmin - ks) / a.v - a.t0) * a.fs) - 2.0;
+        double u = ceil(((dmax + ks) / a.v - a.t0) * a.fs) + 2.0;
+        if (l < 0) l = 0;
+        if (u > a.Nt - 1) u = a.Nt - 1;
+        if (l <= u) { n_lo = (int)l; n_hi = (int)u; }
+        const double k0 = fmin(fmax(floor((dmin / a.v - a.t0) * a.fs * alpha) - 1.0, -1073741824.0), 1073741824.0);
+        lo = max((int)k0, 0);
+        cnt = max(0, min((int)k0 + NZ, Nup) - lo);
+    }
+    const int w = n_lo & ~3;
+    bool active = has_sensor && n_lo <= n_hi;
+    if (active && n_hi + 1 - w > LB) {     // cannot happen with the host's band bound
+        set_status(status, DEV_CAPACITY);
+        n_hi = w + LB - 1;
+    }
+    const int LBe = active ? min(min(LB, a.Nt - w), n_hi + 1 - w) : 0;
+    if (has_sensor) rows[row] = make_int2(w, LBe);
+    if (threadIdx.x == 0) {
+        S.abort = 0;
+        for (int b = 0; b < ASSA_RING; ++b) {
+            S.released[b] = 0;
+            S.issued[b] = -1;
+            mbar_init(&S.full[b], 1);
+        }
+        fence_mbar_init();
+    }
+    for (int q = 0; q <= NZ; ++q) Z[q * 32] = 0;       // 0 and 0.f
+    const bool fixedp = qscale > 0.f;
+    const bool all_fixed = __all_sync(0xffffffffu, fixedp || !active);
+    const float inv_q = fixedp ? 1.f / qscale : 0.f;
+    __syncthreads();
+
+    const bool tma = use_tma != 0;
+    auto fill = [&](int TT) {
+        const int b = TT % ASSA_RING;
+        int tx, ty, tz;
+        slab_brick(sl, TT, tx, ty, tz);
+        if (tma) {
+            if (lane == 0) {
+                S.issued[b] = TT;
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                mbar_arrive_expect_tx(&S.full[b], TILE * sizeof(float));
+                tma_load_3d(&S.tileA[b][0], &tmap, tx * BX, ty * BY, tz * BZ, &S.full[b]);
+            }
+        } else {
+            for (int q = lane; q < TILE; q += 32) {
+                const int gx = tx * BX + (q & (BX - 1)), gy = ty * BY + ((q / BX) & (BY - 1)), gz = tz * BZ + q / (BX * BY);
+                const bool ok = gx < g.nx && gy < g.ny && gz < g.nz;
+                S.tileA[b][q] = ok ? g.A[((int64_t)gz * g.ny + gy) * g.nx + gx] : 0.f;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&S.full[b]);
+        }
+    };
+    if (warp == 0)
+        for (int TT = 0; TT < ASSA_RING && TT < nTiles; ++TT) fill(TT);
+
+    auto both = [](float v) { return make_float2(v, v); };
+    const float h = g.h;
+    const float2 aD = both((float)alpha * a.invDelta), magic = both(SNAP_MAGIC), qs = both(qscale);
+    bool ok = true, touched = false;
+    for (int t = 0; t < nTiles; ++t) {
+        const int b = t % ASSA_RING;
+        if (!mbar_wait(&S.full[b], (uint32_t)((t / ASSA_RING) & 1))) {
+            ok = false;
+            break;
+        }
+        const float* tile = S.tileA[b];
+        bool any = false;                  // a brick without amplitudes adds nothing
+#pragma unroll
+        for (int q = 0; q < TILE / 32 / 4; ++q) {
+            const float4 v = reinterpret_cast<const float4*>(tile)[lane * (TILE / 32 / 4) + q];
+            any |= (v.x != 0.f) | (v.y != 0.f) | (v.z != 0.f) | (v.w != 0.f);
+        }
+        if (__any_sync(0xffffffffu, any) && active) {
+            touched = true;
+            int tx, ty, tz;
+            slab_brick(sl, t, tx, ty, tz);
+            const PairRef r = make_ref(g.ox + (tx * BX + BX / 2) * (double)h, g.oy + (ty * BY + BY / 2) * (double)h,
+                                       g.oz + (tz * BZ + BZ / 2) * (double)h, sx, sy, sz, a);
+            const unsigned base = (unsigned)assa_an0(alpha, r.n0) - SNAP_BITS - (unsigned)lo;
+            const float2 R0 = both(r.R0), phi0 = both(r.phi0);
+            float2 ax[BX / 2];
+#pragma unroll
+            for (int l = 0; l < BX; ++l) {
+                const float o = ((float)l - 0.5f * (BX - 1)) * h, v = o * fmaf(2.f, r.v0x, o);
+                if (l & 1) ax[l >> 1].y = v; else ax[l >> 1].x = v;
+            }
+            auto brick = [&](auto fx) {
+#pragma unroll 1
+                for (int ly = 0; ly < BY; ++ly) {
+                    const float oy = ((float)ly - 0.5f * (BY - 1)) * h;
+                    const float2 oy2 = both(oy), Yc = both(fmaf(2.f, r.v0y, oy));
+                    float2 axy[BX / 2];
+#pragma unroll
+                    for (int u = 0; u < BX / 2; ++u) axy[u] = __ffma2_rn(oy2, Yc, ax[u]);
+#pragma unroll
+                    for (int lz = 0; lz < BZ; ++lz) {
+                        const float oz = ((float)lz - 0.5f * (BZ - 1)) * h;
+                        const float2 az = both(__fmul_rn(oz, fmaf(2.f, r.v0z, oz)));
+                        const float4 a0 = *reinterpret_cast<const float4*>(tile + (lz * BY + ly) * BX);
+                        const float4 a1 = *reinterpret_cast<const float4*>(tile + (lz * BY + ly) * BX + 4);
+                        const float2 A[BX / 2] = {make_float2(a0.x, a0.y), make_float2(a0.z, a0.w), make_float2(a1.x, a1.y),
+                                                  make_float2(a1.z, a1.w)};
+#pragma unroll
+                        for (int u = 0; u < BX / 2; ++u) {
+                            const float2 num = __fadd2_rn(axy[u], az);
+                            const float2 R2 = __ffma2_rn(R0, R0, num);
+                            const float2 invR = make_float2(rsqrtf(R2.x), rsqrtf(R2.y));
+                            const float2 den = __ffma2_rn(R2, invR, R0);
+                            float2 rc;
+                            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc.x) : "f"(den.x));
+                            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc.y) : "f"(den.y));
+                            const float2 k = __ffma2_rn(__ffma2_rn(num, rc, phi0), aD, magic);
+                            int* z0 = Z + min((unsigned)__float_as_int(k.x) + base, (unsigned)cnt) * 32u;
+                            int* z1 = Z + min((unsigned)__float_as_int(k.y) + base, (unsigned)cnt) * 32u;
+                            const float2 mass = __fmul2_rn(A[u], invR);
+                            if (fx) {
+                                const float2 q = __ffma2_rn(mass, qs, magic);
+                                atomicAdd(z0, __float_as_int(q.x) - (int)SNAP_BITS);
+                                atomicAdd(z1, __float_as_int(q.y) - (int)SNAP_BITS);
+                            } else if (fixedp) {
+                                const float2 q = __ffma2_rn(mass, qs, magic);
+                                *z0 += __float_as_int(q.x) - (int)SNAP_BITS;
+                                *z1 += __float_as_int(q.y) - (int)SNAP_BITS;
+                            } else {
+                                if (A[u].x != 0.f) *z0 = __float_as_int(__int_as_float(*z0) + mass.x);
+                                if (A[u].y != 0.f) *z1 = __float_as_int(__int_as_float(*z1) + mass.y);
+                            }
+                        }
+                    }
+                }
+            };
+            if (all_fixed) brick(std::true_type{}); else brick(std::false_type{});
+        }
+        // release the slot; the warp that releases it last refills it with tile t + ASSA_RING
+        __syncwarp();
+        int last = 0;
+        if (lane == 0) {
+            __threadfence_block();
+            last = (atomicAdd(&S.released[b], 1) + 1) % NW == 0;
+            if (last) __threadfence_block();
+        }
+        last = __shfl_sync(0xffffffffu, last, 0);
+        if (last && t + ASSA_RING < nTiles) fill(t + ASSA_RING);
+    }
+    if (!ok && lane == 0) {
+        set_status(status, DEV_TIMEOUT);
+        S.abort = 1;
+    }
+    __syncthreads();
+    if (S.abort) {
+        if (tma && threadIdx.x == 0)
+            for (int b = 0; b < ASSA_RING; ++b)
+                if (S.issued[b] >= 0) mbar_wait(&S.full[b], (uint32_t)((S.issued[b] / ASSA_RING) & 1));
+        return;
+    }
+    if (!active) return;
+    if (!touched) {            // a slab without amplitudes: an empty row
+        rows[row] = make_int2(w, 0);
+        return;
+    }
+    float* F = reinterpret_cast<float*>(Z);
+    for (int q = 0; q <= NZ; ++q) F[q * 32] = q < cnt ? (fixedp ? (float)Z[q * 32] * inv_q : F[q * 32]) : 0.f;
+    // y[n] = sum_m z[m] h[alpha n - m]: output w + q sums entries alpha (w + q) - K - lo + tt, tt = 0 .. 2K, the
+    // taps tt = c, c + alpha, ... of one residue c at a time, so that the next tap's entries are this tap's
+    // shifted by one output
+    float4* prow = reinterpret_cast<float4*>(partial + row * LB);
+    for (int q0 = 0; q0 < LBe; q0 += ASSA_LANES_Q) {
+        float acc[ASSA_LANES_Q];
+#pragma unroll
+        for (int u = 0; u < ASSA_LANES_Q; ++u) acc[u] = 0.f;
+        for (int c = 0; c < alpha; ++c) {
+            int at = alpha * (w + q0) - K - lo + c;
+            auto entry = [&] {
+                const float v = F[min((unsigned)at, (unsigned)NZ) * 32u];        // entry NZ is zero
+                at += alpha;
+                return v;
+            };
+            float V[ASSA_LANES_Q];
+#pragma unroll
+            for (int u = 0; u < ASSA_LANES_Q - 1; ++u) V[u] = entry();
+            for (int tt = c; tt <= 2 * K;) {
+#pragma unroll
+                for (int i = 0; i < ASSA_LANES_Q; ++i, tt += alpha) {
+                    if (tt > 2 * K) break;
+                    V[(i + ASSA_LANES_Q - 1) % ASSA_LANES_Q] = entry();
+                    const float hv = T.hr[tt];                                 // h[alpha n - m] = h[K - tt]
+#pragma unroll
+                    for (int u = 0; u < ASSA_LANES_Q; ++u) acc[u] = fmaf(V[(i + u) % ASSA_LANES_Q], hv, acc[u]);
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < ASSA_LANES_Q; u += 4)          // LB is a multiple of 4; outputs past LBe are not read
+            if (q0 + u < LBe) prow[(q0 + u) >> 2] = make_float4(acc[u], acc[u + 1], acc[u + 2], acc[u + 3]);
+    }
+}
+
 // A sensor's row of dconv: its alpha N_t fine samples and a zero.
 __host__ __device__ __forceinline__ int assa_dconv_row(int alpha, int Nt) { return alpha * Nt + 1; }
 
@@ -427,6 +704,35 @@ cudaError_t launch_assa_forward(const GaussDev& g, const ArrDev& a, const SlabIn
     if (ev && (e = cudaEventRecord(ev[0], st)) != cudaSuccess) return e;
     assa_fwd_kernel<<<grid, ASSA_THREADS, smem, st>>>(g, a, si, partial, rows, LB, status, tmap != nullptr,
                                                       tmap ? *tmap : zero_map, T, amax);
+    e = cudaGetLastError();
+    if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], st);
+    return e;
+}
+
+// The same by the lanes kernel: S rows a sensor, slabs of sb bricks in blocks of qb, NW warps and NZ entries a lane.
+cudaError_t launch_assa_forward_lanes(const GaussDev& g, const ArrDev& a, const int sb[3], const int qb[3], int S,
+                                      float* partial, int2* rows, int LB, int NW, int NZ, int* status,
+                                      const CUtensorMap* tmap, const AssaTable& T, unsigned* amax, const cudaEvent_t* ev,
+                                      cudaStream_t st) {
+    static const CUtensorMap zero_map = [] { CUtensorMap z; memset(&z, 0, sizeof(z)); return z; }();
+    const size_t smem = assa_lanes_smem(NW, NZ);
+    cudaError_t e = cudaFuncSetAttribute(assa_fwd_lanes_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(amax, 0, sizeof(unsigned), st)) != cudaSuccess) return e;
+    assa_amax_kernel<<<4 * device_sms(), 256, 0, st>>>(g.A, g.M, amax);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    AssaSlabs s;
+    const int nt[3] = {g.ntx, g.nty, g.ntz};
+    int k[3];
+    for (int q = 0; q < 3; ++q) {
+        s.sb[q] = sb[q];
+        s.qb[q] = qb[q];
+        k[q] = (nt[q] + qb[q] - 1) / qb[q] * ((qb[q] + sb[q] - 1) / sb[q]);
+    }
+    s.kx = k[0]; s.ky = k[1];
+    if (ev && (e = cudaEventRecord(ev[0], st)) != cudaSuccess) return e;
+    assa_fwd_lanes_kernel<<<dim3((a.Nd + 32 * NW - 1) / (32 * NW), S), 32 * NW, smem, st>>>(
+        g, a, s, partial, rows, LB, NZ, status, tmap != nullptr, tmap ? *tmap : zero_map, T, amax);
     e = cudaGetLastError();
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], st);
     return e;

@@ -59,6 +59,12 @@ cudaError_t launch_vcr(const float* x, int nx, int ny, int nz, float beta, float
 cudaError_t launch_assa_forward(const GaussDev& g, const ArrDev& a, const SlabInfo* si, int S, float* partial,
                                 int2* rows, int LB, int* status, const CUtensorMap* tmap, const AssaTable& T,
                                 unsigned* amax, const cudaEvent_t* ev, cudaStream_t st);
+cudaError_t launch_assa_forward_lanes(const GaussDev& g, const ArrDev& a, const int sb[3], const int qb[3], int S,
+                                      float* partial, int2* rows, int LB, int NW, int NZ, int* status,
+                                      const CUtensorMap* tmap, const AssaTable& T, unsigned* amax, const cudaEvent_t* ev,
+                                      cudaStream_t st);
+int assa_lanes_nz(double diag, double invDelta, int alpha);
+size_t assa_lanes_smem(int NW, int NZ);
 size_t assa_dconv_bytes(const ArrDev& a, const AssaTable& T);
 cudaError_t launch_assa_adjoint(const GaussDev& g, const ArrDev& a, const float* delta, float* gA, const AssaTable& T,
                                 float* dconv, const cudaEvent_t* ev, cudaStream_t st);
@@ -237,6 +243,7 @@ struct FwdPlan {
     bool lanes;            // grid mode: the sensor-lane moment kernel (slabs of 8^3-node cubes)
     bool free_lanes;       // SoA mode: the sensor-lane direct kernel (slabs of tile ranges)
     int NW, NZ;            // warps per CTA of the lanes kernels; moment-band bins (grid)
+    int qbx, qby, qbz;     // ASSA lanes kernel: the blocks of bricks whose scale its slabs take
     size_t off_ti, off_si, off_rows, off_part, bytes;
     size_t off_sort;       // free-centre lanes plan: the spatial order's scratch (after the rest)
     bool has_mom;          // the expansion applies (grid mode); mom is its table
@@ -947,10 +954,60 @@ ArrDev assa_band_array(const GaussDev& g, const ArrDev& a, const AssaTable& T) {
     return aa;
 }
 
+// Plan of the ASSA forward: the lanes kernel with slabs of up to 2 x 2 x 4 bricks (16 x 16 x 16 nodes, what an integer
+// band holds), halved until the grid has about four CTAs per SM.  They divide the slabs of the kernel with a
+// warp to a sensor, whose scale their masses take (qb: those slabs' bricks).  A warp takes 32 sensors
+// whether they are there or not, so that fewer than ASSA_LANES_MIN go to the other kernel; so do slabs
+// too many for the sorted reduction and lattices so coarse that a brick's band does not fit.
+constexpr int ASSA_LANES_MIN = 12, ASSA_LANES_SLABS = 2048;
+FwdPlan plan_assa_forward(const GaussDev& g, const ArrDev& aa, const AssaTable& T) {
+    const FwdPlan wide = plan_forward(g, aa);
+    if (aa.Nd < ASSA_LANES_MIN) return wide;
+    const int nt[3] = {g.ntx, g.nty, g.ntz}, bn[3] = {BX, BY, BZ}, nn[3] = {g.nx, g.ny, g.nz};
+    const int qb[3] = {wide.sbx, wide.sby, wide.sbz};
+    int sb[3] = {std::min(2, qb[0]), std::min(2, qb[1]), std::min(4, qb[2])};
+    const int64_t groups = ((int64_t)aa.Nd + 31) / 32;
+    auto plan = [&](FwdPlan& p) {
+        memset(&p, 0, sizeof(p));
+        p.parts = 1;
+        int64_t S = 1;
+        double d2 = 0.0;
+        for (int q = 0; q < 3; ++q) {
+            S *= (int64_t)((nt[q] + qb[q] - 1) / qb[q]) * ((qb[q] + sb[q] - 1) / sb[q]);
+            const double span = (std::min(sb[q] * bn[q], nn[q]) - 1) * (double)g.h;
+            d2 += span * span;
+        }
+        if (S > ASSA_LANES_SLABS) return false;
+        grid_plan_from_blocks(p, g, aa, sb);
+        p.S = (int)S;
+        plan_offsets(p, g, aa);
+        p.qbx = qb[0]; p.qby = qb[1]; p.qbz = qb[2];
+        p.NZ = assa_lanes_nz(std::sqrt(d2), aa.invDelta, T.alpha);
+        p.NW = (int)std::min<int64_t>(4, groups);
+        while (p.NW > 0 && assa_lanes_smem(p.NW, p.NZ) > SMEM_PER_CTA) --p.NW;
+        p.lanes = p.NW > 0;
+        return p.lanes;
+    };
+    FwdPlan best;
+    bool any = plan(best);
+    for (;;) {
+        if (any && best.S * ((groups + best.NW - 1) / best.NW) >= (int64_t)device_sms() * 4) break;
+        int q = 0;
+        for (int k = 1; k < 3; ++k)
+            if (sb[k] * bn[k] > sb[q] * bn[q]) q = k;
+        if (sb[q] == 1) break;
+        sb[q] = (sb[q] + 1) / 2;
+        FwdPlan p;
+        if (plan(p)) { best = p; any = true; }
+        else if (any) break;
+    }
+    return any ? best : wide;
+}
+
 // Scratch of the ASSA forward beyond the plan: max |A| for the fixed-point bands.
 constexpr size_t ASSA_EXTRA_BYTES = 256;
 
-// ASSA forward into y with scratch of p.bytes + ASSA_EXTRA_BYTES (p = plan_forward(g, assa_band_array(...))).
+// ASSA forward into y with scratch of p.bytes + ASSA_EXTRA_BYTES (p = plan_assa_forward(...)).
 gpair_status run_assa_forward(const GaussDev& g, const ArrDev& aa, const AssaTable& T, const FwdPlan& p, float* y,
                               void* scratch, int* status, const cudaEvent_t* ev, cudaStream_t st) {
     char* base = static_cast<char*>(scratch);
@@ -960,10 +1017,13 @@ gpair_status run_assa_forward(const GaussDev& g, const ArrDev& aa, const AssaTab
     CUtensorMap map;
     memset(&map, 0, sizeof(map));
     const bool tma = make_tmap(g, &map);
-    cudaError_t e = launch_slab_info_grid(g, p.sbx, p.sby, p.sbz, p.S, si, st);
+    const int sb[3] = {p.sbx, p.sby, p.sbz}, qb[3] = {p.qbx, p.qby, p.qbz};
+    cudaError_t e = p.lanes ? cudaSuccess : launch_slab_info_grid(g, p.sbx, p.sby, p.sbz, p.S, si, st);
+    unsigned* amax = reinterpret_cast<unsigned*>(base + p.bytes);
     if (e == cudaSuccess)
-        e = launch_assa_forward(g, aa, si, p.S, part, rows, p.LB, status, tma ? &map : nullptr, T,
-                                reinterpret_cast<unsigned*>(base + p.bytes), ev, st);
+        e = p.lanes ? launch_assa_forward_lanes(g, aa, sb, qb, p.S, part, rows, p.LB, p.NW, p.NZ, status, tma ? &map : nullptr,
+                                                T, amax, ev, st)
+                    : launch_assa_forward(g, aa, si, p.S, part, rows, p.LB, status, tma ? &map : nullptr, T, amax, ev, st);
     if (e == cudaSuccess) e = launch_slab_reduce(g, aa, part, rows, p.S, p.PL, y, st);
     return cuda_status(e);
 }
@@ -981,7 +1041,7 @@ gpair_status gpair_assa_forward(const gpair_gaussians* gi, const gpair_array* ai
     if (!y) return GPAIR_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const ArrDev aa = assa_band_array(g, a, T);
-    FwdPlan p = plan_forward(g, aa);
+    FwdPlan p = plan_assa_forward(g, aa, T);
     void* scratch = nullptr;
     int* status = nullptr;
     if ((s = get_scratch(st, p.bytes + ASSA_EXTRA_BYTES, &scratch, &status)) != GPAIR_OK) return s;
@@ -1188,7 +1248,7 @@ gpair_status gpair_solver_create(const gpair_gaussians* gi, const gpair_array* a
     }
     const size_t M = (size_t)g.M, N = (size_t)a.Nd * a.Nt;
     if (assa) S->aa = assa_band_array(g, a, S->T);
-    S->plan = assa ? plan_forward(g, S->aa) : plan_forward_op(g, a);
+    S->plan = assa ? plan_assa_forward(g, S->aa, S->T) : plan_forward_op(g, a);
     const size_t qbytes = !assa && S->plan.has_mom ? adjoint_q_bytes(a, S->plan.mom) : 0;
     bool ok = cudaMalloc(&S->z, M * 4) == cudaSuccess && cudaMalloc(&S->m, M * 4) == cudaSuccess &&
               cudaMalloc(&S->v, M * 4) == cudaSuccess && cudaMalloc(&S->x, M * 4) == cudaSuccess &&

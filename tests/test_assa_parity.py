@@ -157,3 +157,31 @@ def test_paper_scale_adjoint_sampled_gaussians():
     g_ora, amb = oracle.assa_adjoint(Gs, G.sigma[0], w.sensors, w.v, w.fs, w.t0, w.Nt, delta, tau=TAU_SNAP,
                                      want_amb=True)
     assert np.linalg.norm(g[idx] - g_ora) <= 1e-4 * np.linalg.norm(g_ora) + np.linalg.norm(amb)
+
+
+@pytest.mark.parametrize("nd", [11, 12, 33, 130])
+@pytest.mark.parametrize("n_min", [1, 25, 61])
+@pytest.mark.parametrize("sides", [(8, 8, 4), (17, 9, 10), (35, 20, 17)])
+def test_few_sensors_and_slabs(sides, n_min, nd):
+    """The last count with a warp to a sensor and the first with a lane to one, a group of 32 with a remainder; fine
+    grids of alpha = 1, 2 and 4; one brick, ragged bricks, several slabs of 16; records that end early."""
+    g = synth.centred_grid(*sides, 0.1e-3)
+    w = synth.Workload("assa-few", g, synth.cap_sensors(nd, 15e-3, 150.0), 410, A=None)
+    _check_forward(w, A=_dense(w), n_min=n_min)
+
+
+def test_sensors_in_the_volume_and_large_amplitudes():
+    """Sensors inside a slab's box have no bound on A / r: their lanes add floats beside the others' integers."""
+    g = synth.centred_grid(20, 18, 9, 0.1e-3)
+    xyz = synth.cap_sensors(40, 12e-3, 120.0)
+    xyz[::7] = (np.array([0.21, -0.33, 0.08]) * 1e-3 + np.arange(6)[:, None] * 1.7e-5).astype(np.float32)
+    w = synth.Workload("assa-in", g, xyz, 400, A=None)
+    _check_forward(w, A=_dense(w) * 1e6)
+
+
+def test_sparse_slabs():
+    """Slabs and bricks without amplitudes."""
+    g = synth.centred_grid(40, 33, 40, 0.1e-3)
+    A = np.zeros(g.M, np.float32)
+    A[np.random.default_rng(3).choice(g.M, 25, replace=False)] = 1.0
+    _check_forward(synth.Workload("assa-sparse", g, synth.cap_sensors(40, 20e-3, 120.0), 900, A=None), A=A)
