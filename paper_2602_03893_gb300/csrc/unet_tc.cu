@@ -609,26 +609,260 @@ conv3d_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_co
     }
 }
 
-// dw[co][t][ci] += sum over splits (in order) of partial[split][t Cin + ci][co]
-__global__ void wgrad_reduce_kernel(const float* __restrict__ partial, int n_splits, int rows, int Cout,
-                                    float* __restrict__ dw) {
-    const int64_t n = (int64_t)rows * Cout;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int co = (int)(i / rows), m = (int)(i - (int64_t)co * rows);   // dw index co * rows + m
-        const float* src = partial + (size_t)m * Cout + co;
-        const size_t step = (size_t)rows * Cout;
-        float acc = 0.f;
-        int s = 0;
-        for (; s + 8 <= n_splits; s += 8) {      // eight loads in flight, added in split order
-            float v[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) v[q] = src[(size_t)(s + q) * step];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) acc += v[q];
-        }
-        for (; s < n_splits; ++s) acc += src[(size_t)s * step];
-        dw[i] += acc;
+// The same for narrow layers (3 Cout <= 96), whose boxes' traffic, not the MMAs, bounds the kernel above: a unit's box
+// is fetched for each of its nine (dz, dy) shifts, in 32-byte rows.  Here a tile fetches one box per 16
+// channels with its halo in y and z, and a shift is a place in it: a row of x (8 voxels) is one
+// swizzle atom of 256 bytes, so that dy moves an operand by 256 bytes and dz by the 18 rows of a plane.
+// The 8 atoms of M = 128 are 256 bytes apart, the shifts dy = 0 .. 7 of one (16 channels, dz), of which the first
+// three are wanted: the others' sums stay in tensor memory (and read rows past the box, inside the
+// stage).  ZCOL, 16 output channels: the dz shifts too are columns.  A tile is one plane; each dout box has the
+// planes z0 - 1 .. z0 + 1, its 16-channel atoms a plane apart, so that the nine (dx, dz) shifts are one operand
+// of N = 144 and the MMAs a third as many.
+//
+// Bound by the MMAs' operand reads from shared memory.  48 -> 16 channels of 64 x 128 x 128 voxels: 153 us with a box
+// per shift, 136 us with dz in the rows.
+constexpr int WH_MAX_N = 96;                          // columns: wider layers are bound by the MMAs
+constexpr int WH_ROWS = TC_TY + 2;                    // rows of x per plane of a box
+constexpr uint32_t WH_ROW_BYTES = TC_TX * 16 * 2;     // one swizzle atom
+static_assert(WH_ROW_BYTES == 256 && (WH_ROWS * WH_ROW_BYTES) % 256 == 0, "shifts keep the swizzle's phase");
+
+struct WgradHaloArgs {
+    int Cin, Cout, ZS;
+    int tiles_x, tiles_y, n_tiles;        // voxel tiles of 8 x 16 x ZS
+    int N;                                // columns = 3 Cout, 9 Cout with ZCOL
+    int ncp, n_groups, n_splits;          // 16-channel groups per CTA, their groups, voxel-tile splits
+    int nstages;
+    uint32_t a_bytes, b_atom, b_bytes, stage_bytes, tmem_cols;     // a_bytes: a box; b_bytes: one dout box, b_atom 16 of its channels
+    float* partial;                       // [split][27 Cin][Cout]
+};
+
+template <bool ZCOL>
+__global__ void __launch_bounds__(WG_THREADS, 1)
+conv3d_wgrad_halo_kernel(const __grid_constant__ CUtensorMap tmIn, const __grid_constant__ CUtensorMap tmOut,
+                         const WgradHaloArgs p) {
+    extern __shared__ __align__(1024) unsigned char sm[];
+    constexpr int DZ = ZCOL ? 1 : 3;      // dz shifts in the rows
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int NS = p.nstages;
+    uint64_t* full = reinterpret_cast<uint64_t*>(sm + (size_t)NS * p.stage_bytes);
+    uint64_t* empty = full + TC_MAX_STAGES;
+    uint64_t* done = empty + TC_MAX_STAGES;
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
+    const int grp = (int)(blockIdx.x % p.n_groups), split = (int)(blockIdx.x / p.n_groups);
+    const int cp0 = grp * p.ncp, ncp = min(p.ncp, p.Cin / 16 - cp0);
+    const int t0 = (int)((int64_t)split * p.n_tiles / p.n_splits), t1 = (int)((int64_t)(split + 1) * p.n_tiles / p.n_splits);
+
+    if (threadIdx.x == 0) {
+        for (int q = 0; q < NS; ++q) { mbar_init(&full[q], 1); mbar_init(&empty[q], 1); }
+        mbar_init(done, 1);
+        fence_mbar_init();
     }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
+                     "r"(p.tmem_cols));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tslot;
+    bool ok = true;
+
+    if (warp == 0) {
+        // lane 0 claims the slot and posts the byte count; one lane a box issues them
+        int s = 0;
+        uint32_t ph = 0;
+        for (int tile = t0; tile < t1; ++tile) {
+            const int tx = tile % p.tiles_x, ty = (tile / p.tiles_x) % p.tiles_y, tz = tile / (p.tiles_x * p.tiles_y);
+            const int x0 = tx * TC_TX, y0 = ty * TC_TY, z0 = tz * p.ZS;
+            const uint32_t dst = smem_u32(sm + (size_t)s * p.stage_bytes);
+            if (lane == 0) {
+                if (ok && !mbar_wait(&empty[s], ph ^ 1u)) ok = false;
+                mbar_arrive_expect_tx(&full[s], (uint32_t)ncp * p.a_bytes + 3 * p.b_bytes);
+            }
+            __syncwarp();
+            if (lane < ncp) {
+                tma_load_5d(dst + (uint32_t)lane * p.a_bytes, &tmIn, 0, x0, y0 - 1, ZCOL ? z0 : z0 - 1, cp0 + lane,
+                            &full[s]);
+            } else if (lane >= 8 && lane < 11) {
+                const int j = lane - 8;             // dout box of x-tap j: dout[u - j + 1]
+                tma_load_5d(dst + (uint32_t)p.ncp * p.a_bytes + (uint32_t)j * p.b_bytes, &tmOut, 0, x0 + 1 - j, y0,
+                            ZCOL ? z0 - 1 : z0, 0, &full[s]);
+            }
+            if (++s == NS) { s = 0; ph ^= 1u; }
+        }
+        if (lane == 0)
+            for (int q = 0; q < NS; ++q) {      // every load issued has landed before the CTA ends
+                int s2 = s - 1 - q;
+                uint32_t ph2 = ph;
+                if (s2 < 0) { s2 += NS; ph2 ^= 1u; }
+                mbar_wait_n(&full[s2], ph2, WAIT_LIMIT / 16);
+            }
+    } else if (warp == 1 && lane == 0) {
+        const uint32_t idesc = tc_idesc_mn(p.N, 128);
+        int s = 0;
+        uint32_t ph = 0;
+        for (int tile = t0; tile < t1; ++tile) {
+            if (ok && !mbar_wait(&full[s], ph)) ok = false;
+            tc_fence_after();
+            const uint32_t aaddr = smem_u32(sm + (size_t)s * p.stage_bytes);
+            const uint64_t b0 = smem_desc_sw32(aaddr + (uint32_t)p.ncp * p.a_bytes, p.b_atom, WH_ROW_BYTES);
+            for (int blk = 0; blk < DZ * ncp; ++blk) {
+                const int cp = blk / DZ, dz = blk - DZ * cp;
+                const uint64_t a0 = smem_desc_sw32(aaddr + (uint32_t)cp * p.a_bytes + (uint32_t)(dz * WH_ROWS) * WH_ROW_BYTES,
+                                                   WH_ROW_BYTES, WH_ROW_BYTES);
+                for (int z = 0; z < p.ZS; ++z)
+                    for (int y = 0; y < TC_TY; y += 2)      // K = 16 voxels: two rows of x
+                        tc_mma(tmem + (uint32_t)(blk * p.N), a0 + (uint64_t)((z * WH_ROWS + y) * (WH_ROW_BYTES / 16)),
+                               b0 + (uint64_t)((z * TC_TY + y) * (WH_ROW_BYTES / 16)), idesc,
+                               (tile > t0 || z > 0 || y > 0) ? 1u : 0u);
+            }
+            tc_commit(&empty[s]);
+            if (++s == NS) { s = 0; ph ^= 1u; }
+        }
+        tc_commit(done);
+    }
+    __syncwarp();
+    // drain: TMEM lane 16 dy + ci of block (cp, dz), column j Cout + co: tap (dz, dy, j); warps 0 and 1 hold dy < 3
+    if (t1 > t0 && warp < 2) {
+        if (ok && !mbar_wait(done, 0)) ok = false;
+        tc_fence_after();
+        const int rows = 27 * p.Cin;
+        const int mi = 32 * warp + lane, dy = mi / 16, ci = mi & 15;
+        const bool valid = dy < 3;
+        for (int blk = 0; blk < DZ * ncp; ++blk) {
+            const int cp = cp0 + blk / DZ;
+            // ZCOL: columns (dx, plane of the dout box), plane 2 - dz
+            for (int c = 0; c < (ZCOL ? 9 : 3); ++c) {
+                const int j = ZCOL ? c / 3 : c, dz = ZCOL ? 2 - c % 3 : blk % DZ;
+                const int t = dz * 9 + (valid ? dy : 0) * 3 + j;
+                float* dst = p.partial + ((size_t)split * rows + (size_t)t * p.Cin + cp * 16 + ci) * p.Cout;
+                for (int c0 = 0; c0 < p.Cout; c0 += 16) {
+                    uint32_t r[16];
+                    tc_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(blk * p.N + c * p.Cout + c0), r);
+                    if (valid) {
+                        float4* d4 = reinterpret_cast<float4*>(dst + c0);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            d4[i] = make_float4(__uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1]),
+                                                __uint_as_float(r[4 * i + 2]), __uint_as_float(r[4 * i + 3]));
+                    }
+                }
+            }
+        }
+    }
+    if (!ok) atomicMax(&g_conv_tc_status, 1);
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        __syncwarp();
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(p.tmem_cols));
+    }
+}
+
+// dw[co][t][ci] += sum over splits of partial[split][t Cin + ci][co].  Threads run along the partials' memory,
+// WR_SEG of them to an element, each with a run of the splits (in order); their sums are added in order.
+constexpr int WR_SEG = 8, WR_ELEMS = 32;
+__global__ void __launch_bounds__(WR_SEG * WR_ELEMS)
+wgrad_reduce_kernel(const float* __restrict__ partial, int n_splits, int rows, int Cout, float* __restrict__ dw) {
+    __shared__ float part[WR_SEG][WR_ELEMS];
+    const int64_t n = (int64_t)rows * Cout;
+    const int e = threadIdx.x % WR_ELEMS, seg = threadIdx.x / WR_ELEMS;
+    const int s0 = (int)((int64_t)seg * n_splits / WR_SEG), s1 = (int)((int64_t)(seg + 1) * n_splits / WR_SEG);
+    for (int64_t i0 = blockIdx.x * (int64_t)WR_ELEMS; i0 < n; i0 += (int64_t)gridDim.x * WR_ELEMS) {
+        const int64_t i = i0 + e;
+        float acc = 0.f;
+        if (i < n) {
+            const float* src = partial + i;
+            int s = s0;
+            for (; s + 8 <= s1; s += 8) {        // eight loads in flight, added in split order
+                float v[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) v[q] = src[(size_t)(s + q) * n];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) acc += v[q];
+            }
+            for (; s < s1; ++s) acc += src[(size_t)s * n];
+        }
+        part[seg][e] = acc;
+        __syncthreads();
+        if (seg == 0 && i < n) {
+#pragma unroll
+            for (int q = 1; q < WR_SEG; ++q) acc += part[q][e];
+            const int m = (int)(i / Cout), co = (int)(i - (int64_t)m * Cout);
+            dw[(size_t)co * rows + m] += acc;
+        }
+        __syncthreads();
+    }
+}
+
+static cudaError_t launch_wgrad_reduce(const float* partial, int n_splits, int rows, int Cout, float* dw, cudaStream_t st) {
+    int64_t blocks = ((int64_t)rows * Cout + WR_ELEMS - 1) / WR_ELEMS;
+    if (blocks > (int64_t)device_sms() * 32) blocks = (int64_t)device_sms() * 32;
+    wgrad_reduce_kernel<<<(unsigned)blocks, WR_SEG * WR_ELEMS, 0, st>>>(partial, n_splits, rows, Cout, dw);
+    return cudaGetLastError();
+}
+
+// Tensor map of a voxel-major tensor in boxes of 16 channels x 8 x ny x nz voxels x `groups` 16-channel groups,
+// 32-byte swizzle: dims (16 channels, x, y, z, 16-channel group).
+static bool wgrad_map(PFN_cuTensorMapEncodeTiled_v12000 enc, CUtensorMap* m, const uint16_t* t, int D, int H, int W, int C,
+                      int ny, int nz, int groups) {
+    cuuint64_t dims[5] = {16, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)D, (cuuint64_t)(C / 16)};
+    cuuint64_t strides[4] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2, 32};
+    cuuint32_t box[5] = {16, TC_TX, (cuuint32_t)ny, (cuuint32_t)nz, (cuuint32_t)groups};
+    cuuint32_t es[5] = {1, 1, 1, 1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<uint16_t*>(t), dims, strides, box, es,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+static cudaError_t launch_wgrad_halo(PFN_cuTensorMapEncodeTiled_v12000 enc, const uint16_t* in, const uint16_t* dout, int D,
+                                     int H, int W, int Cin, int Cout, float* dw, cudaStream_t st) {
+    WgradHaloArgs a{};
+    const size_t bar_bytes = 8 * (2 * TC_MAX_STAGES + 1) + 16;
+    const int sms = device_sms(), cps = Cin / 16;
+    const bool zcol = Cout == 16;
+    const int dz = zcol ? 1 : 3;
+    a.Cin = Cin; a.Cout = Cout; a.ZS = zcol ? 1 : 2; a.N = (zcol ? 9 : 3) * Cout;
+    a.tiles_x = (W + TC_TX - 1) / TC_TX; a.tiles_y = (H + TC_TY - 1) / TC_TY;
+    a.n_tiles = a.tiles_x * a.tiles_y * ((D + a.ZS - 1) / a.ZS);
+    const int a_planes = zcol ? 1 : a.ZS + 2, b_planes = zcol ? 3 : a.ZS;
+    a.a_bytes = (uint32_t)(a_planes * WH_ROWS) * WH_ROW_BYTES;
+    a.b_atom = (uint32_t)((zcol ? 1 : b_planes) * TC_TY) * WH_ROW_BYTES;
+    a.b_bytes = (uint32_t)(b_planes * TC_TY) * WH_ROW_BYTES * (uint32_t)(Cout / 16);
+    // 16-channel groups per CTA: what tensor memory and two stages hold, evenly
+    int ncp = 512 / (dz * a.N);
+    auto stage = [&](int n) { return ((uint32_t)n * a.a_bytes + 3 * a.b_bytes + 1023u) & ~1023u; };
+    while (ncp > 1 && 2 * (size_t)stage(ncp) + bar_bytes > TC_SMEM_MAX) --ncp;
+    if (ncp > cps) ncp = cps;
+    a.n_groups = (cps + ncp - 1) / ncp;
+    a.ncp = (cps + a.n_groups - 1) / a.n_groups;
+    a.stage_bytes = stage(a.ncp);
+    const int nst = (int)((TC_SMEM_MAX - bar_bytes) / a.stage_bytes);
+    a.nstages = nst < TC_MAX_STAGES ? nst : TC_MAX_STAGES;
+    if (a.nstages < 2) return cudaErrorNotSupported;
+    a.tmem_cols = tmem_columns(dz * a.ncp * a.N);
+    int ns = sms / a.n_groups;
+    if (ns < 1) ns = 1;
+    if (ns > a.n_tiles) ns = a.n_tiles;
+    a.n_splits = ns;
+    const int rows = 27 * Cin;
+    void* scratch = nullptr;
+    if (stream_scratch(st, (size_t)a.n_splits * rows * Cout * sizeof(float), &scratch) != GPAIR_OK)
+        return cudaErrorMemoryAllocation;
+    a.partial = static_cast<float*>(scratch);
+    CUtensorMap mI, mO;
+    if (!wgrad_map(enc, &mI, in, D, H, W, Cin, WH_ROWS, a_planes, 1) ||
+        !wgrad_map(enc, &mO, dout, D, H, W, Cout, TC_TY, b_planes, Cout / 16))
+        return cudaErrorNotSupported;
+    const size_t smem = (size_t)a.nstages * a.stage_bytes + bar_bytes;
+    auto kern = zcol ? conv3d_wgrad_halo_kernel<true> : conv3d_wgrad_halo_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)(a.n_groups * a.n_splits), WG_THREADS, smem, st>>>(mI, mO, a);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return launch_wgrad_reduce(a.partial, a.n_splits, rows, Cout, dw, st);
 }
 
 // Eligible: Cin and Cout multiples of 16, Cout <= 256, 1 or 27 taps, 16-byte aligned tensors.
@@ -639,6 +873,7 @@ cudaError_t launch_conv3d_wgrad_tc(const uint16_t* in, const uint16_t* dout, int
     if (((uintptr_t)in | (uintptr_t)dout) & 15) return cudaErrorNotSupported;
     auto enc = conv_encoder();
     if (!enc) return cudaErrorNotSupported;
+    if (taps == 27 && 3 * Cout <= WH_MAX_N) return launch_wgrad_halo(enc, in, dout, D, H, W, Cin, Cout, dw, st);
     const int sms = device_sms();
     WgradTcArgs a{};
     const size_t bar_bytes = 8 * (2 * TC_MAX_STAGES + 1) + 16;
@@ -675,41 +910,16 @@ cudaError_t launch_conv3d_wgrad_tc(const uint16_t* in, const uint16_t* dout, int
         return cudaErrorMemoryAllocation;
     a.partial = static_cast<float*>(scratch);
 
+    // the input: one 16-channel group per load; dout: all groups
     CUtensorMap mI, mO;
-    const int R = taps == 27 ? 1 : 0;
-    (void)R;
-    // input and dout: dims (16 channels, x, y, z, 16-channel group), boxes of 16 channels x 8 x 16 x
-    // ZS voxels (the input: one group per load; dout: all groups), 32-byte swizzle
-    {
-        cuuint64_t dims[5] = {16, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)D, (cuuint64_t)(Cin / 16)};
-        cuuint64_t strides[4] = {(cuuint64_t)Cin * 2, (cuuint64_t)W * Cin * 2, (cuuint64_t)H * W * Cin * 2, 32};
-        cuuint32_t box[5] = {16, TC_TX, TC_TY, (cuuint32_t)a.ZS, 1};
-        cuuint32_t es[5] = {1, 1, 1, 1, 1};
-        if (enc(&mI, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<uint16_t*>(in), dims, strides, box, es,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return cudaErrorNotSupported;
-    }
-    {
-        cuuint64_t dims[5] = {16, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)D, (cuuint64_t)(Cout / 16)};
-        cuuint64_t strides[4] = {(cuuint64_t)Cout * 2, (cuuint64_t)W * Cout * 2, (cuuint64_t)H * W * Cout * 2, 32};
-        cuuint32_t box[5] = {16, TC_TX, TC_TY, (cuuint32_t)a.ZS, (cuuint32_t)(Cout / 16)};
-        cuuint32_t es[5] = {1, 1, 1, 1, 1};
-        if (enc(&mO, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<uint16_t*>(dout), dims, strides, box, es,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return cudaErrorNotSupported;
-    }
+    if (!wgrad_map(enc, &mI, in, D, H, W, Cin, TC_TY, a.ZS, 1) || !wgrad_map(enc, &mO, dout, D, H, W, Cout, TC_TY, a.ZS, Cout / 16))
+        return cudaErrorNotSupported;
     auto kern = taps == 27 ? conv3d_wgrad_tc_kernel<27> : conv3d_wgrad_tc_kernel<1>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)(a.n_groups * a.n_splits), WG_THREADS, smem, st>>>(mI, mO, a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const int64_t n = (int64_t)rows * Cout;
-    int64_t blocks = (n + 255) / 256;
-    if (blocks > (int64_t)sms * 8) blocks = (int64_t)sms * 8;
-    wgrad_reduce_kernel<<<(unsigned)blocks, 256, 0, st>>>(a.partial, a.n_splits, rows, Cout, dw);
-    return cudaGetLastError();
+    return launch_wgrad_reduce(a.partial, a.n_splits, rows, Cout, dw, st);
 }
 
 int conv_tc_status_and_clear() {

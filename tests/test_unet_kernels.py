@@ -77,6 +77,30 @@ def _conv_case(dims, cin, cout, taps, relu):
     _close(db.cpu(), dout.double().sum(0), rel=1e-4)
 
 
+@pytest.mark.parametrize("cin,cout", [(16, 16), (48, 16), (64, 16), (80, 32), (96, 32), (32, 48)])
+@pytest.mark.parametrize("dims", [(1, 1, 1), (2, 16, 8), (3, 17, 9), (5, 33, 20)])
+def test_wgrad_tiles(dims, cin, cout):
+    """One voxel, whole 8 x 16 x 2 tiles and remainders; one to several groups of 16 channels a CTA, one and two
+    groups of them; the last width with haloed boxes (32) and the first without (48)."""
+    gen = torch.Generator().manual_seed(sum(dims) + cin)
+    nv = int(np.prod(dims))
+    x, dout = _bf((nv, cin), gen), _bf((nv, cout), gen)
+    w = torch.zeros((cout, cin, 3, 3, 3), dtype=torch.float64, requires_grad=True)
+    F.conv3d(_cl_to_cf(x, dims), w, padding=1).backward(_cl_to_cf(dout, dims))
+    ref = w.grad.reshape(cout, cin, 27).permute(0, 2, 1)
+    dw, db = torch.ones((cout, 27, cin), device="cuda"), torch.zeros(cout, device="cuda")
+    before = unet.gpair_unet_tensor_path()
+    unet.gpair_unet_tensor_path(2)
+    try:
+        unet.gpair_conv3d_wgrad(x.cuda(), dout.cuda(), dims, cin, cout, 27, dw, db)
+    finally:
+        unet.gpair_unet_tensor_path(before)
+    # FP32 sums of exact products, at most nv of them: 2^-24 each, on sums of the products' sizes
+    bound = nv * 2.0 ** -22 * float((x.double().abs().amax() * dout.double().abs().amax()))
+    assert float((dw.cpu().double() - 1 - ref).abs().max()) <= bound + 1e-6
+    assert unet.gpair_unet_tc_status() == 0
+
+
 def test_tensor_core_paths_agree_on_the_unet_layers():
     """The tcgen05 and mma.sync convolutions on the U-Net's own layer shapes (128 x 128 x 64 level
     halved to keep the test short): both accumulate in FP32, so their BF16 outputs differ by at most
