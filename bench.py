@@ -38,7 +38,7 @@ UNIT = "s/iter"
 FP32_LANES_PER_SM = 128
 SM_MAX_MHZ = 2070.0
 MUFU_LANES_PER_SM = 32          # MUFU lanes per SM (ex2 measured at ~30 lane-ops / clk / SM)
-LAUNCHES_PER_STEP = 10          # npc, slab info, forward, slab reduce, resid, finish, Q table, adjoint, schedule, adam
+LAUNCHES_PER_STEP = 8           # slab info, forward, slab reduce, resid, finish, Q table, adjoint, adam
 ASSA_NMIN = 25                  # the paper's minimum number of fine samples across the pulse
 
 

@@ -27,17 +27,20 @@ __device__ __forceinline__ bool split_sum(float (&sum)[N], float* part, int at) 
     return blockIdx.y == 0;
 }
 
-// CTAs that share a tile's sensors, a power of two up to 8, for grids of less than one wave of `ctas` per SM: doubled
-// while the CTAs stay within a wave and keep `least` sensors each (idle SMs), and while they stay within four
-// waves and keep 64 (few warps on each SM).  The amplitude adjoint's time with 1, 2, 4, 8 CTAs a tile: 16 bricks, 128
-// sensors: 74 us for 1, 17 us for 8; 184 bricks, 33 sensors: 24, ..., 12, 19 us; 675 bricks, 952 sensors: 609, 600,
-// 441, 370 us; 1024 bricks, 512 sensors: 337, 316, 305, 279 us.  From a wave on it costs: CTAs that walk the
-// sensors in the same order share their rows in L1 (3900 bricks, 47 sensors: 76, ..., 154, 241 us).
-inline int adj_split(int64_t ntiles, int Nd, int ctas, int least) {
+// CTAs that share a tile's sensors, a power of two up to 8: doubled while the CTAs stay within a wave of `ctas` per SM and
+// keep `least` sensors each (idle SMs), and while they stay within some waves and keep 64.
+// rows: the tiles gather the sensors' rows of a table through L1, and CTAs that walk the sensors in the same order share
+// them there.  Such grids are split only where unsplit they are less than a wave, up to four waves.  The amplitude
+// adjoint with 1, 2, 4 and 8 CTAs a tile: 16 bricks, 128 sensors: 74 us with 1, 17 us with 8; 675 bricks, 952
+// sensors: 609, 600, 441, 370 us; 1024 bricks, 512 sensors: 337, 316, 305, 279 us; but 3900 bricks, 47 sensors: 76 us
+// with 1, 154 with 4, 241 with 8.  Without such rows up to 16 waves, for the last wave's sake: the gradient step
+// of 1024 tiles of free centres and 512 sensors 3498, 3435, 3424, 3413 us.
+inline int adj_split(int64_t ntiles, int Nd, int ctas, int least, bool rows) {
     const int64_t wave = (int64_t)device_sms() * ctas;
+    const int64_t most = rows ? (ntiles < wave ? 4 * wave : 0) : 16 * wave;
     int split = 1;
-    while (split < 8 && ntiles < wave &&
-           ((ntiles * split * 2 <= wave && Nd >= 2 * least * split) || (ntiles * split * 2 <= 4 * wave && Nd >= 128 * split)))
+    while (split < 8 && ((ntiles * split * 2 <= wave && Nd >= 2 * least * split) ||
+                         (ntiles * split * 2 <= most && Nd >= 128 * split)))
         split *= 2;
     return split;
 }

