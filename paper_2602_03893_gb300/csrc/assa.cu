@@ -549,37 +549,47 @@ assa_fwd_lanes_kernel(GaussDev g, ArrDev a, const AssaSlabs slabs, float* __rest
 __host__ __device__ __forceinline__ int assa_dconv_row(int alpha, int Nt) { return alpha * Nt + 1; }
 
 // dconv_j[k] = sum_n h[alpha n - k] delta_j[n], k = 0 .. alpha Nt - 1 (zero filling and the
-// correlation with the flipped pulse in one pass).  Block: 256 fine samples of one sensor.
+// correlation with the flipped pulse in one pass).  The outputs of one residue, k = alpha q + r, are a filter of delta
+// with taps of their own: a block takes DC_PER samples q from each of its threads, residue by residue, so that
+// the taps are uniform and serve DC_PER outputs each.  4.2e6 samples, alpha = 2: 87 us with a thread to an
+// output, 28 us.
+constexpr int DC_THREADS = 256, DC_PER = 4;
 __device__ __forceinline__ int floor_div(int a, int b) { return (a >= 0) ? a / b : -((-a + b - 1) / b); }
 
-__global__ void assa_dconv_kernel(const float* __restrict__ delta, int Nt, const __grid_constant__ AssaTable T,
-                                  float* __restrict__ dconv) {
-    extern __shared__ float sd[];
-    const int j = blockIdx.y;
-    const int alpha = T.alpha, K = T.K;
-    const int Nup = alpha * Nt;
-    const int k0 = blockIdx.x * 256;
-    const int na = -floor_div(-(k0 - K), alpha);            // ceil((k0 - K) / alpha)
-    const int nb = floor_div(k0 + 255 + K, alpha);
+__global__ void __launch_bounds__(DC_THREADS)
+assa_dconv_kernel(const float* __restrict__ delta, int Nt, const __grid_constant__ AssaTable T,
+                  float* __restrict__ dconv) {
+    extern __shared__ float sd[];                  // samples q0 - M .. q0 + DC_THREADS DC_PER + M
+    const int j = blockIdx.y, t = threadIdx.x;
+    const int alpha = T.alpha, K = T.K, M = K / alpha + 1;
+    const int q0 = blockIdx.x * DC_THREADS * DC_PER;
     const float* dj = delta + (size_t)j * Nt;
-    for (int q = threadIdx.x; q <= nb - na; q += blockDim.x) {
-        const int n = na + q;
-        sd[q] = (n >= 0 && n < Nt) ? dj[n] : 0.f;
+    for (int c = t; c < DC_THREADS * DC_PER + 2 * M + 1; c += DC_THREADS) {
+        const int n = q0 - M + c;
+        sd[c] = (n >= 0 && n < Nt) ? dj[n] : 0.f;
     }
     __syncthreads();
-    const int k = k0 + (int)threadIdx.x;
-    if (k > Nup) return;
-    if (k == Nup) {              // the entry of every sample outside the record
-        dconv[(size_t)j * assa_dconv_row(alpha, Nt) + k] = 0.f;
-        return;
+    float* row = dconv + (size_t)j * assa_dconv_row(alpha, Nt);
+    for (int r = 0; r < alpha; ++r) {
+        const int i1 = -floor_div(-(r - K), alpha), i2 = (r + K) / alpha;      // n - q with |alpha n - k| <= K
+        float acc[DC_PER];
+#pragma unroll
+        for (int u = 0; u < DC_PER; ++u) acc[u] = 0.f;
+        for (int i = i1; i <= i2; ++i) {
+            const float h = T.hr[K - alpha * i + r];
+#pragma unroll
+            for (int u = 0; u < DC_PER; ++u) acc[u] = fmaf(h, sd[t + u * DC_THREADS + M + i], acc[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < DC_PER; ++u) {
+            const int q = q0 + t + u * DC_THREADS;
+            if (q < Nt) row[(size_t)alpha * q + r] = acc[u];
+        }
     }
-    const int n1 = -floor_div(-(k - K), alpha), n2 = floor_div(k + K, alpha);
-    float acc = 0.f;
-    for (int n = n1; n <= n2; ++n) acc = fmaf(T.hr[K - (alpha * n - k)], sd[n - na], acc);
-    dconv[(size_t)j * assa_dconv_row(alpha, Nt) + k] = acc;
+    if (blockIdx.x == 0 && t == 0) row[(size_t)alpha * Nt] = 0.f;      // the entry of every sample outside the record
 }
 
-size_t assa_dconv_smem(const AssaTable& T) { return (size_t)((255 + 2 * T.K) / T.alpha + 3) * sizeof(float); }
+size_t assa_dconv_smem(const AssaTable& T) { return (size_t)(DC_THREADS * DC_PER + 2 * (T.K / T.alpha + 1) + 1) * sizeof(float); }
 
 // g_i = sum_j dconv_j[k_ij] / r_ij.  One CTA of 64 threads per brick, four Gaussians to a thread (x and
 // x + 4, two planes each; the planes through packed FP32 arithmetic, which rounds each half as the scalar
@@ -743,8 +753,8 @@ size_t assa_dconv_bytes(const ArrDev& a, const AssaTable& T) { return (size_t)a.
 
 cudaError_t launch_assa_adjoint(const GaussDev& g, const ArrDev& a, const float* delta, float* gA, const AssaTable& T,
                                 float* dconv, const cudaEvent_t* ev, cudaStream_t st) {
-    dim3 dgrid((T.alpha * a.Nt + 256) / 256, a.Nd);
-    assa_dconv_kernel<<<dgrid, 256, assa_dconv_smem(T), st>>>(delta, a.Nt, T, dconv);
+    dim3 dgrid((a.Nt + DC_THREADS * DC_PER - 1) / (DC_THREADS * DC_PER), a.Nd);
+    assa_dconv_kernel<<<dgrid, DC_THREADS, assa_dconv_smem(T), st>>>(delta, a.Nt, T, dconv);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (ev && (e = cudaEventRecord(ev[0], st)) != cudaSuccess) return e;
