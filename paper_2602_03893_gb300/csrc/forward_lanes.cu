@@ -83,22 +83,6 @@ struct ZBand {
         c1 = reinterpret_cast<float*>(rest + (size_t)(NZ + 1) * 32 * 8);
         b4 = reinterpret_cast<float4*>(rest);
     }
-    // Z[bin][lane] += (m0 .. m_{P-1})
-    __device__ __forceinline__ void add(int idx, const float* m) {
-        float4 z = a[idx];
-        z.x += m[0]; z.y += m[1]; z.z += m[2]; z.w += m[3];
-        a[idx] = z;
-        if constexpr (P == 8) {
-            float4 y = b4[idx];
-            y.x += m[4]; y.y += m[5]; y.z += m[6]; y.w += m[7];
-            b4[idx] = y;
-        } else {
-            float2 y = b2[idx];
-            y.x += m[4]; y.y += m[5];
-            b2[idx] = y;
-            if constexpr (P == 7) c1[idx] += m[6];
-        }
-    }
     // Two pairs at once: Z[i1] += m1 and Z[i2] += m2.  All loads come before all stores, so the two
     // read-modify-writes (and the parts of each) form one dependency step instead of a chain of
     // four; when i1 == i2 the second store, which lands last, carries both pairs.
@@ -572,7 +556,6 @@ fwd_lanes_kernel(GaussDev g, ArrDev a, const SlabInfo* __restrict__ slabs, const
 
 size_t fwd_lanes_smem(int NW, int NZ, int LB, int P, int L) { return fl_smem_bytes(NW, NZ, LB, P, L); }
 int fwd_lanes_nz(float h, float invDelta) { return fl_nz(h, invDelta); }
-float fwd_lanes_cube_radius(float h) { return cube_radius(h); }
 
 // Largest number of CTAs that may share a slab of one cube.
 int fwd_lanes_parts(const MomentTable& T) { return T.P == 6 && T.L <= 32 ? 8 : 1; }
