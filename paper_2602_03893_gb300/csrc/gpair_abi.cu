@@ -1164,7 +1164,6 @@ struct gpair_solver {
     ArrDev a;
     gpair_step_params p;
     int t = 0;
-    bool x_ready = false;    // x holds the amplitudes of z (Adam)
     float *z = nullptr, *m = nullptr, *v = nullptr, *x = nullptr, *gx = nullptr;
     float *y = nullptr, *delta = nullptr, *Fg = nullptr;
     double* red = nullptr;   // reduction partials (2 * red_blocks) + results (4)
@@ -1205,6 +1204,14 @@ gpair_status solver_adjoint(gpair_solver* S, const float* delta, float* gA, cons
     if (S->assa) return cuda_status(launch_assa_adjoint(S->g, S->a, delta, gA, S->T, S->dconv, ev, st));
     // the amplitude adjoint needs only the tile summaries of the forward scratch (same layout)
     return run_adjoint(S->g, S->a, delta, gA, nullptr, nullptr, st, S->fwd_scratch, ev, S->qbuf, &S->plan.mom);
+}
+
+// Adam: x, the amplitudes of the iterate z.  Whatever changes z leaves x with it, in the order of the stream and under
+// capture too, so that a step needs no look at where z came from: the creation and gpair_solver_set_state here,
+// a step in its Adam pass.
+cudaError_t image_of_z(gpair_solver* S, cudaStream_t st) {
+    if (S->p.rule != GPAIR_RULE_ADAM) return cudaSuccess;
+    return launch_npc(S->z, S->x, S->g.M, S->p.npc != 0, S->p.npc_eps, st);
 }
 }  // namespace
 
@@ -1273,6 +1280,7 @@ gpair_status gpair_solver_create(const gpair_gaussians* gi, const gpair_array* a
     S->sched = SchedParams{prm->eta_max, prm->eta_min, prm->T_mult, prm->beta1, prm->beta2, prm->T0};
     cudaMemset(S->sd, 0, sizeof(StepSched));
     launch_set_step(S->sd, 0, S->sched, 0);
+    image_of_z(S, 0);
     if (cudaDeviceSynchronize() != cudaSuccess) {
         gpair_solver_destroy(S);
         return GPAIR_ERR_CUDA;
@@ -1320,14 +1328,8 @@ gpair_status gpair_solver_timings(gpair_solver* S, double* ms, int* nsteps) {
 }  // extern "C"
 
 namespace {
-// The amplitudes x of the iterate z, which every Adam step leaves for the next: formed here where z came from outside.
-gpair_status ensure_image(gpair_solver* S, cudaStream_t st) {
-    if (S->p.rule != GPAIR_RULE_ADAM || S->x_ready) return GPAIR_OK;
-    return cuda_status(launch_npc(S->z, S->x, S->g.M, S->p.npc != 0, S->p.npc_eps, st));
-}
-
-// The launches of one reconstruction step on st, given x: no host synchronisation, S->t unchanged, and the
-// same launches with the same arguments at every step (so that they can be replayed as a graph).
+// The launches of one reconstruction step on st: no host synchronisation, S->t unchanged, and the same launches
+// with the same arguments at every step (so that they can be replayed as a graph).  Adam: x is image_of_z.
 gpair_status step_launches(gpair_solver* S, const float* b, const cudaEvent_t* ev, cudaStream_t st) {
     const int64_t M = S->g.M, N = (int64_t)S->a.Nd * S->a.Nt;
     double* partial = S->red;
@@ -1396,13 +1398,7 @@ gpair_status gpair_step(gpair_solver* S, const float* b, double* loss_out, doubl
         ev = &S->evs[6 * S->nrec];
         if (cudaEventRecord(ev[0], st) != cudaSuccess) return GPAIR_ERR_CUDA;
     }
-    // a step that a caller captures forms x itself: it may be replayed after a change of z
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    const bool captured = cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
-    if (captured) S->x_ready = false;
-    gpair_status s = ensure_image(S, st);
-    S->x_ready = false;
-    if (s == GPAIR_OK) s = step_launches(S, b, ev, st);
+    gpair_status s = step_launches(S, b, ev, st);
     if (s != GPAIR_OK) {
         // the schedule kernel may have advanced the device step count before a later launch failed:
         // put it back to the host count, so that a checkpoint taken now resumes with the right step
@@ -1413,7 +1409,6 @@ gpair_status gpair_step(gpair_solver* S, const float* b, double* loss_out, doubl
         if (cudaEventRecord(ev[5], st) != cudaSuccess) return GPAIR_ERR_CUDA;
         S->nrec += 1;
     }
-    S->x_ready = !captured;
     S->t += 1;
     return read_loss(S, st, loss_out, resid_out);
 }
@@ -1456,15 +1451,11 @@ gpair_status gpair_solver_steps(gpair_solver* S, const float* b, int n, double* 
         }
         S->gb = b;
     }
-    const gpair_status si = ensure_image(S, st);
-    S->x_ready = false;
-    if (si != GPAIR_OK) return si;
     for (int k = 0; k < n; ++k)
         if (cudaGraphLaunch(S->gexec, st) != cudaSuccess) {
             S->t += k;      // the k replays already queued advance the device step count
             return GPAIR_ERR_CUDA;
         }
-    S->x_ready = true;
     S->t += n;
     return read_loss(S, st, loss_out, resid_out);
 }
@@ -1491,8 +1482,8 @@ gpair_status gpair_solver_set_state(gpair_solver* S, const float* z, const float
     if (!S || t < 0) return GPAIR_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const size_t bytes = (size_t)S->g.M * 4;
-    if (z) S->x_ready = false;
     if (z && cudaMemcpyAsync(S->z, z, bytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return GPAIR_ERR_CUDA;
+    if (z && image_of_z(S, st) != cudaSuccess) return GPAIR_ERR_CUDA;
     if (m && cudaMemcpyAsync(S->m, m, bytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return GPAIR_ERR_CUDA;
     if (v && cudaMemcpyAsync(S->v, v, bytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return GPAIR_ERR_CUDA;
     if (launch_set_step(S->sd, t, S->sched, st) != cudaSuccess) return GPAIR_ERR_CUDA;

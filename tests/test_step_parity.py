@@ -273,3 +273,42 @@ def test_graph_replayed_steps_equal_single_steps(problem, kind):
     assert tb == 8 and rel_l2(zb.cpu().numpy(), za.cpu().numpy()) < 1e-5
     for s in (s1, s2, s3):
         s.close()
+
+
+@pytest.mark.parametrize("kind", ["step", "steps"])
+def test_captured_state_and_captured_steps_mix_with_eager_ones(problem, kind):
+    """A set_state recorded in a graph changes the iterate when the graph runs, not when it is recorded, and so do
+    recorded steps: whatever comes after works on the iterate that the device then has.  Losses of the
+    iterates tell which amplitudes a step used."""
+    w, G, b = problem
+    p = _lib.StepParams(rule=_lib.RULE_ADAM, npc=1, eta_max=0.03, T0=50, adam_eps=1e-20)
+    gs, arr = device_inputs(w)
+    bt = torch.as_tensor(b, device="cuda")
+    z0 = torch.as_tensor(np.random.default_rng(5).uniform(0.2, 1.0, w.M).astype(np.float32), device="cuda")
+    zero = torch.zeros_like(z0)
+
+    def eager(s):
+        return s.gpair_step(bt)[0] if kind == "step" else s.gpair_solver_steps(bt, 1)[0]
+
+    ref = _lib.Solver(gs, arr, p)
+    ref.gpair_solver_set_state(z0, zero, zero, 0)
+    want = [eager(ref) for _ in range(3)]
+    z_ref = ref.gpair_solver_get_state()[0]
+    s = _lib.Solver(gs, arr, p)
+    eager(s)
+    graph, steps = torch.cuda.CUDAGraph(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        s.gpair_solver_set_state(z0, zero, zero, 0)
+    eager(s)
+    graph.replay()
+    got = [eager(s)]
+    with torch.cuda.graph(steps):
+        s.gpair_step(bt, want_loss=False)
+    graph.replay()                       # the recorded step has not run: back to z0
+    steps.replay()
+    got += [eager(s), eager(s)]
+    z = s.gpair_solver_get_state()[0]
+    assert np.allclose(got, want, rtol=1e-5), (got, want)
+    assert rel_l2(z.cpu().numpy(), z_ref.cpu().numpy()) < 1e-5
+    ref.close()
+    s.close()
