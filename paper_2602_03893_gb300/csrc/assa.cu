@@ -291,8 +291,13 @@ struct AssaLanesHdr {
 };
 constexpr size_t ASSA_LANES_HDR = (sizeof(AssaLanesHdr) + 127) & ~(size_t)127;
 
-// Entries of a lane's band for a slab whose centres span `diag` metres.
-int assa_lanes_nz(double diag, double invDelta, int alpha) { return (int)ceil(diag * 1.00001 * invDelta * alpha) + 6; }
+// Entries of a lane's band for a slab whose centres span `diag` metres.  The band starts up to two samples before
+// the nearest distance to the slab's box, which lies up to `widened` metres before the nearest centre
+// (brick_block): the six entries more than the span cover the first and a sample of the second.
+int assa_lanes_nz(double diag, double widened, double invDelta, int alpha) {
+    const double fine = invDelta * alpha, extra = fmax(0.0, ceil(widened * fine) - 1.0);
+    return (int)fmin(ceil(diag * 1.00001 * fine) + 6.0 + extra, (double)(1 << 24));
+}
 size_t assa_lanes_smem(int NW, int NZ) { return ASSA_LANES_HDR + (size_t)NW * (NZ + 1) * 32 * sizeof(int); }
 
 // Slabs of sb bricks that divide the blocks of qb bricks in which the kernel above walks the lattice: a slab's masses

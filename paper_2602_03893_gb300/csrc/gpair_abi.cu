@@ -63,7 +63,7 @@ cudaError_t launch_assa_forward_lanes(const GaussDev& g, const ArrDev& a, const 
                                       float* partial, int2* rows, int LB, int NW, int NZ, int* status,
                                       const CUtensorMap* tmap, const AssaTable& T, unsigned* amax, const cudaEvent_t* ev,
                                       cudaStream_t st);
-int assa_lanes_nz(double diag, double invDelta, int alpha);
+int assa_lanes_nz(double diag, double widened, double invDelta, int alpha);
 size_t assa_lanes_smem(int NW, int NZ);
 size_t assa_dconv_bytes(const ArrDev& a, const AssaTable& T);
 cudaError_t launch_assa_adjoint(const GaussDev& g, const ArrDev& a, const float* delta, float* gA, const AssaTable& T,
@@ -982,7 +982,7 @@ FwdPlan plan_assa_forward(const GaussDev& g, const ArrDev& aa, const AssaTable& 
         p.S = (int)S;
         plan_offsets(p, g, aa);
         p.qbx = qb[0]; p.qby = qb[1]; p.qbz = qb[2];
-        p.NZ = assa_lanes_nz(std::sqrt(d2), aa.invDelta, T.alpha);
+        p.NZ = assa_lanes_nz(std::sqrt(d2), brick_block_widening(g), aa.invDelta, T.alpha);
         p.NW = (int)std::min<int64_t>(4, groups);
         while (p.NW > 0 && assa_lanes_smem(p.NW, p.NZ) > SMEM_PER_CTA) --p.NW;
         p.lanes = p.NW > 0;

@@ -267,6 +267,18 @@ __device__ __forceinline__ SlabInfo brick_block(const GaussDev& g, int bx0, int 
     return o;
 }
 
+// By how much the distance to a brick_block may fall short of the distance to its nearest centre, for any block of the
+// lattice: the widening along the three axes, with the rounding of its ends.
+inline double brick_block_widening(const GaussDev& g) {
+    const double o[3] = {g.ox, g.oy, g.oz}, n[3] = {(double)g.nx, (double)g.ny, (double)g.nz};
+    double s = 0.0;
+    for (int q = 0; q < 3; ++q) {
+        const double far = fmax(fabs(o[q]), fabs(o[q] + n[q] * (double)g.h)), w = 1.2 * (2e-6 * far + 1e-9);
+        s += w * w;
+    }
+    return sqrt(s);
+}
+
 // Tile t (0-based within the slab) -> brick coordinates (grid mode).
 __device__ __forceinline__ void slab_brick(const SlabInfo& sl, int t, int& tx, int& ty, int& tz) {
     tx = sl.bx0 + t % sl.bdx;

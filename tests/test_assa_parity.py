@@ -185,3 +185,21 @@ def test_sparse_slabs():
     A = np.zeros(g.M, np.float32)
     A[np.random.default_rng(3).choice(g.M, 25, replace=False)] = 1.0
     _check_forward(synth.Workload("assa-sparse", g, synth.cap_sensors(40, 20e-3, 120.0), 900, A=None), A=A)
+
+
+@pytest.mark.parametrize("sides,h,sigma,n_min,off", [((16, 16, 16), 1e-4, 1e-4, 513, 2.0), ((35, 20, 17), 1e-4, 1e-4, 513, 4.0),
+                                                     ((16, 16, 16), 1.2e-5, 1.2e-5, 513, 0.25)])
+def test_lattice_far_from_the_origin(sides, h, sigma, n_min, off):
+    """Fine grids of alpha = 32 and 256, lattices so far out that the slabs' boxes, widened by a part of their
+    coordinates, start several fine samples before the nearest node: the farthest nodes' masses, seen along
+    the diagonals of two bricks, stay in the band.  Only nodes at the bricks' corners have amplitudes."""
+    g = synth.centred_grid(*sides, h, sigma=sigma, centre=(off, -off, off))
+    ix, iy, iz = (np.arange(n) for n in sides)
+    at = [(np.isin(q % b, (0, b - 1)) | (q == n - 1)) for q, b, n in ((iz, 4, sides[2]), (iy, 8, sides[1]), (ix, 8, sides[0]))]
+    A = (at[0][:, None, None] & at[1][None, :, None] & at[2][None, None, :]).astype(np.float32).ravel()
+    d = np.array([[7.0 * x, 7.0 * y, 3.0 * z] for x in (-1, 1) for y in (-1, 1) for z in (-1, 1)])
+    d /= np.linalg.norm(d, axis=1, keepdims=True)
+    o = np.array([g.ox, g.oy, g.oz])
+    xyz = np.concatenate([o + np.array([4.0, 4.0, 2.0]) * h * (2 * q + 1) + 10e-3 * d for q in (0, 1)])
+    w = synth.Workload("assa-far", g, xyz.astype(np.float32), 400, A=A)
+    _check_forward(w, A=A, n_min=n_min)
