@@ -10,6 +10,8 @@
 // global atomics.  Free-centre Gaussians are taken in the order of their window length (a
 // counting sort of the tile in shared memory), so the 32 threads of a warp walk windows of about
 // the same length.
+#include <type_traits>
+
 #include "adjoint_split.cuh"
 #include "gpair_internal.cuh"
 
@@ -307,6 +309,10 @@ adj_q_kernel(const float* __restrict__ delta, int Nt, const __grid_constant__ Mo
 //
 // A brick's sensors are divided over the CTAs of a cluster where there are too few bricks to fill the
 // chip; their sums meet in the first CTA's shared memory, in the order of the ranks.
+//
+// A node on which a sensor lies has neither phase nor 1 / R.  Where the window start of the brick's centre is outside
+// the record it adds nothing, as every start there; it reads the zero entry, but 0 / 0 is not a number: a CTA that
+// finds such a sum gathers again and leaves these pairs out (CHECK).
 constexpr int ADJM_THREADS = 64, ADJM_PER = TILE / ADJM_THREADS;
 constexpr int ADJM_SC = 64;              // sensors per chunk; sums are compensated every 32
 constexpr int ADJM_CTAS = 16;            // resident per SM (12: 1 to 3 % slower)
@@ -372,78 +378,95 @@ adj_moment_kernel(GaussDev g, ArrDev a, const float* __restrict__ delta, const f
     const float2 magic = both(ADJ_MAGIC), mmagic = both(-ADJ_MAGIC), iD = both(invDelta), mksi = both(-ksi),
                  mD = both(-Delta), mdstar = both(-T.dstar), ihalf = both(T.inv_half);
     KahanF kA[ADJM_PER];
-    // References are double-buffered: after each barrier the threads form the next chunk's.
-    if (jb + l < je) refs2[0][l] = ref(jb + l);
-    int cur = 0;
-    for (int j0 = jb; j0 < je; j0 += ADJM_SC, cur ^= 1) {
-        const int nsc = min(ADJM_SC, je - j0);
-        __syncthreads();
-        if (j0 + ADJM_SC + l < je) refs2[cur ^ 1][l] = ref(j0 + ADJM_SC + l);
-        for (int q0 = 0; q0 < nsc; q0 += 32) {
-            float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};   // FP32 over 32 sensors
-            const AdjmRef* rp = refs2[cur] + q0;
-            const int nq = min(32, nsc - q0);
+    auto gather = [&](auto CHECK) {
+#pragma unroll
+        for (int u = 0; u < ADJM_PER; ++u) kA[u] = KahanF();
+        // References are double-buffered: after each barrier the threads form the next chunk's.
+        if (jb + l < je) refs2[0][l] = ref(jb + l);
+        int cur = 0;
+        for (int j0 = jb; j0 < je; j0 += ADJM_SC, cur ^= 1) {
+            const int nsc = min(ADJM_SC, je - j0);
+            __syncthreads();
+            if (j0 + ADJM_SC + l < je) refs2[cur ^ 1][l] = ref(j0 + ADJM_SC + l);
+            for (int q0 = 0; q0 < nsc; q0 += 32) {
+                float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};   // FP32 over 32 sensors
+                const AdjmRef* rp = refs2[cur] + q0;
+                const int nq = min(32, nsc - q0);
 #pragma unroll 1
-            for (int q = 0; q < nq; ++q) {
-                const AdjmRef r = rp[q];
-                const float2 R0 = both(r.R0);
-                float2 e[2], iR[2];
-                unsigned rel[ADJM_PER];
+                for (int q = 0; q < nq; ++q) {
+                    const AdjmRef r = rp[q];
+                    const float2 R0 = both(r.R0);
+                    float2 e[2], iR[2];
+                    unsigned rel[ADJM_PER];
 #pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const float2 num = __ffma2_rn(dx[u], both(r.v2x), __ffma2_rn(dy2, both(r.v2y), __ffma2_rn(dz, both(r.v2z), d2[u])));
-                    const float2 R2 = __ffma2_rn(R0, R0, num);
-                    iR[u] = make_float2(rsqrtf(R2.x), rsqrtf(R2.y));
-                    const float2 den = __ffma2_rn(R2, iR[u], R0);
-                    float2 rc;
-                    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc.x) : "f"(den.x));
-                    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc.y) : "f"(den.y));
-                    const float2 phi = __ffma2_rn(num, rc, both(r.phi0));
-                    const float2 up = __fadd2_ru(__ffma2_rn(phi, iD, mksi), magic);      // as the forward
-                    const float2 mf = __fadd2_rn(up, mmagic);
-                    rel[2 * u] = (unsigned)__float_as_int(up.x) + r.n0;
-                    rel[2 * u + 1] = (unsigned)__float_as_int(up.y) + r.n0;
-                    const float2 d0 = __ffma2_rn(mf, mD, phi);
-                    e[u] = __fmul2_rn(__fadd2_rn(d0, mdstar), ihalf);
-                }
-                float s[ADJM_PER];
-#pragma unroll
-                for (int u = 0; u < ADJM_PER; ++u) {
-                    const float x = (u & 1) ? e[u >> 1].y : e[u >> 1].x;
-                    const unsigned at = min(rel[u], zero_row);
-                    const float4 q0v = __ldg(r.qa + at);
-                    float v;
-                    if constexpr (P == 6) {
-                        const float2 q1 = __ldg(reinterpret_cast<const float2*>(r.qb) + at);
-                        v = fmaf(q1.y, x, q1.x);
-                    } else {
-                        const float4 q1 = __ldg(reinterpret_cast<const float4*>(r.qb) + at);
-                        if constexpr (P == 8) v = fmaf(fmaf(fmaf(q1.w, x, q1.z), x, q1.y), x, q1.x);
-                        else v = fmaf(fmaf(q1.z, x, q1.y), x, q1.x);
+                    for (int u = 0; u < 2; ++u) {
+                        const float2 num = __ffma2_rn(dx[u], both(r.v2x), __ffma2_rn(dy2, both(r.v2y), __ffma2_rn(dz, both(r.v2z), d2[u])));
+                        const float2 R2 = __ffma2_rn(R0, R0, num);
+                        iR[u] = make_float2(rsqrtf(R2.x), rsqrtf(R2.y));
+                        const float2 den = __ffma2_rn(R2, iR[u], R0);
+                        float2 rc;
+                        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc.x) : "f"(den.x));
+                        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc.y) : "f"(den.y));
+                        const float2 phi = __ffma2_rn(num, rc, both(r.phi0));
+                        const float2 up = __fadd2_ru(__ffma2_rn(phi, iD, mksi), magic);      // as the forward
+                        const float2 mf = __fadd2_rn(up, mmagic);
+                        rel[2 * u] = (unsigned)__float_as_int(up.x) + r.n0;
+                        rel[2 * u + 1] = (unsigned)__float_as_int(up.y) + r.n0;
+                        const float2 d0 = __ffma2_rn(mf, mD, phi);
+                        e[u] = __fmul2_rn(__fadd2_rn(d0, mdstar), ihalf);
                     }
-                    s[u] = fmaf(fmaf(fmaf(fmaf(v, x, q0v.w), x, q0v.z), x, q0v.y), x, q0v.x);
-                }
-                bool edge = false;
-#pragma unroll
-                for (int u = 0; u < ADJM_PER; ++u) edge |= edge_corrected(T, (u & 1) ? e[u >> 1].y : e[u >> 1].x);
-                if (edge) {            // edge position E: rare direct correction
+                    float s[ADJM_PER];
 #pragma unroll
                     for (int u = 0; u < ADJM_PER; ++u) {
                         const float x = (u & 1) ? e[u >> 1].y : e[u >> 1].x;
-                        const int n = (int)(rel[u] - (unsigned)L) + T.E;
-                        if (edge_corrected(T, x) && n >= 0 && n < Nt) {
-                            const float dE = fmaf(x, 0.5f * Delta, T.dstar) - ED;
-                            s[u] = fmaf(edge_factor(T) * delta[(size_t)r.j * Nt + n] * dE, ex2_approx(dE * dE * c2), s[u]);
+                        const unsigned at = min(rel[u], zero_row);
+                        const float4 q0v = __ldg(r.qa + at);
+                        float v;
+                        if constexpr (P == 6) {
+                            const float2 q1 = __ldg(reinterpret_cast<const float2*>(r.qb) + at);
+                            v = fmaf(q1.y, x, q1.x);
+                        } else {
+                            const float4 q1 = __ldg(reinterpret_cast<const float4*>(r.qb) + at);
+                            if constexpr (P == 8) v = fmaf(fmaf(fmaf(q1.w, x, q1.z), x, q1.y), x, q1.x);
+                            else v = fmaf(fmaf(q1.z, x, q1.y), x, q1.x);
+                        }
+                        s[u] = fmaf(fmaf(fmaf(fmaf(v, x, q0v.w), x, q0v.z), x, q0v.y), x, q0v.x);
+                    }
+                    bool edge = false;
+#pragma unroll
+                    for (int u = 0; u < ADJM_PER; ++u) edge |= edge_corrected(T, (u & 1) ? e[u >> 1].y : e[u >> 1].x);
+                    if (CHECK && r.n0 + (unsigned)ADJ_MAGIC_BITS >= zero_row) {
+#pragma unroll
+                        for (int u = 0; u < ADJM_PER; ++u) {
+                            float& x = (u & 1) ? e[u >> 1].y : e[u >> 1].x;
+                            float& w = (u & 1) ? iR[u >> 1].y : iR[u >> 1].x;
+                            if (x != x) x = s[u] = w = 0.f;
                         }
                     }
+                    if (edge) {            // edge position E: rare direct correction
+#pragma unroll
+                        for (int u = 0; u < ADJM_PER; ++u) {
+                            const float x = (u & 1) ? e[u >> 1].y : e[u >> 1].x;
+                            const int n = (int)(rel[u] - (unsigned)L) + T.E;
+                            if (edge_corrected(T, x) && n >= 0 && n < Nt) {
+                                const float dE = fmaf(x, 0.5f * Delta, T.dstar) - ED;
+                                s[u] = fmaf(edge_factor(T) * delta[(size_t)r.j * Nt + n] * dE, ex2_approx(dE * dE * c2), s[u]);
+                            }
+                        }
+                    }
+                    acc[0] = __ffma2_rn(make_float2(s[0], s[1]), iR[0], acc[0]);
+                    acc[1] = __ffma2_rn(make_float2(s[2], s[3]), iR[1], acc[1]);
                 }
-                acc[0] = __ffma2_rn(make_float2(s[0], s[1]), iR[0], acc[0]);
-                acc[1] = __ffma2_rn(make_float2(s[2], s[3]), iR[1], acc[1]);
+                kA[0].add(acc[0].x); kA[1].add(acc[0].y);
+                kA[2].add(acc[1].x); kA[3].add(acc[1].y);
             }
-            kA[0].add(acc[0].x); kA[1].add(acc[0].y);
-            kA[2].add(acc[1].x); kA[3].add(acc[1].y);
         }
-    }
+    };
+    gather(std::false_type{});
+    bool nan = false;
+#pragma unroll
+    for (int u = 0; u < ADJM_PER; ++u) nan |= kA[u].s != kA[u].s;
+    if (__syncthreads_or(nan)) gather(std::true_type{});
     float sum[ADJM_PER];
 #pragma unroll
     for (int u = 0; u < ADJM_PER; ++u) sum[u] = kA[u].s;

@@ -602,6 +602,9 @@ size_t assa_dconv_smem(const AssaTable& T) { return (size_t)(DC_THREADS * DC_PER
 // double-buffered.  A snapped sample outside the record reads the sensor's zero entry, one past its end.
 // A brick's sensors may be divided over the CTAs of a cluster.
 //
+// A node on which a sensor lies has no time of flight and adds nothing.  It reads the zero entry, but 0 / 0 is not
+// a number: a CTA that finds such a sum gathers again, dropping 1 / R at the zero entry (CHECK).
+//
 // Bound by instruction issue.  With a Gaussian to a thread 25 instructions a pair; 1.07e9 pairs: 955 us, 771 us now.
 constexpr int ASSA_ADJ_THREADS = 64, ASSA_ADJ_PER = TILE / ASSA_ADJ_THREADS, ASSA_ADJ_CTAS = 14;
 constexpr int ASSA_ADJ_SC = 64;
@@ -653,39 +656,52 @@ assa_adj_kernel(GaussDev g, ArrDev a, const float* __restrict__ dconv, const __g
     const float2 magic = both(SNAP_MAGIC), aD = both(aInvD);
     KahanF kA[ASSA_ADJ_PER];         // FP32 over 32 sensors, compensated from there on
     const int jb = SPLIT ? blockIdx.y * per : 0, je = SPLIT ? min(a.Nd, jb + per) : a.Nd;
-    if (jb + l < je) refs2[0][l] = ref(jb + l);
-    int cur = 0;
-    for (int j0 = jb; j0 < je; j0 += ASSA_ADJ_SC, cur ^= 1) {
-        const int nsc = min(ASSA_ADJ_SC, je - j0);
-        __syncthreads();
-        if (j0 + ASSA_ADJ_SC + l < je) refs2[cur ^ 1][l] = ref(j0 + ASSA_ADJ_SC + l);
-        for (int q0 = 0; q0 < nsc; q0 += 32) {
-            float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-            const AssaRef* rp = refs2[cur] + q0;
-            const int nq = min(32, nsc - q0);
-#pragma unroll 4
-            for (int q = 0; q < nq; ++q) {
-                const AssaRef r = rp[q];
-                const float2 R0 = both(r.R0);
+    auto gather = [&](auto CHECK) {
 #pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const float2 num = __ffma2_rn(dx[u], both(r.v2x), __ffma2_rn(dy2, both(r.v2y), __ffma2_rn(dz, both(r.v2z), d2[u])));
-                    const float2 R2 = __ffma2_rn(R0, R0, num);
-                    const float2 iR = make_float2(rsqrtf(R2.x), rsqrtf(R2.y));
-                    const float2 den = __ffma2_rn(R2, iR, R0);
-                    float2 rc;
-                    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc.x) : "f"(den.x));
-                    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc.y) : "f"(den.y));
-                    const float2 s = __ffma2_rn(__ffma2_rn(num, rc, both(r.phi0)), aD, magic);
-                    const unsigned ka = min((unsigned)__float_as_int(s.x) + r.base, zero_entry);
-                    const unsigned kb = min((unsigned)__float_as_int(s.y) + r.base, zero_entry);
-                    acc[u] = __ffma2_rn(make_float2(__ldg(r.row + ka), __ldg(r.row + kb)), iR, acc[u]);
+        for (int u = 0; u < ASSA_ADJ_PER; ++u) kA[u] = KahanF();
+        if (jb + l < je) refs2[0][l] = ref(jb + l);
+        int cur = 0;
+        for (int j0 = jb; j0 < je; j0 += ASSA_ADJ_SC, cur ^= 1) {
+            const int nsc = min(ASSA_ADJ_SC, je - j0);
+            __syncthreads();
+            if (j0 + ASSA_ADJ_SC + l < je) refs2[cur ^ 1][l] = ref(j0 + ASSA_ADJ_SC + l);
+            for (int q0 = 0; q0 < nsc; q0 += 32) {
+                float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+                const AssaRef* rp = refs2[cur] + q0;
+                const int nq = min(32, nsc - q0);
+#pragma unroll 4
+                for (int q = 0; q < nq; ++q) {
+                    const AssaRef r = rp[q];
+                    const float2 R0 = both(r.R0);
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const float2 num = __ffma2_rn(dx[u], both(r.v2x), __ffma2_rn(dy2, both(r.v2y), __ffma2_rn(dz, both(r.v2z), d2[u])));
+                        const float2 R2 = __ffma2_rn(R0, R0, num);
+                        float2 iR = make_float2(rsqrtf(R2.x), rsqrtf(R2.y));
+                        const float2 den = __ffma2_rn(R2, iR, R0);
+                        float2 rc;
+                        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc.x) : "f"(den.x));
+                        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc.y) : "f"(den.y));
+                        const float2 s = __ffma2_rn(__ffma2_rn(num, rc, both(r.phi0)), aD, magic);
+                        const unsigned ka = min((unsigned)__float_as_int(s.x) + r.base, zero_entry);
+                        const unsigned kb = min((unsigned)__float_as_int(s.y) + r.base, zero_entry);
+                        if (CHECK) {
+                            if (ka == zero_entry) iR.x = 0.f;
+                            if (kb == zero_entry) iR.y = 0.f;
+                        }
+                        acc[u] = __ffma2_rn(make_float2(__ldg(r.row + ka), __ldg(r.row + kb)), iR, acc[u]);
+                    }
                 }
+                kA[0].add(acc[0].x); kA[1].add(acc[0].y);
+                kA[2].add(acc[1].x); kA[3].add(acc[1].y);
             }
-            kA[0].add(acc[0].x); kA[1].add(acc[0].y);
-            kA[2].add(acc[1].x); kA[3].add(acc[1].y);
         }
-    }
+    };
+    gather(std::false_type{});
+    bool nan = false;
+#pragma unroll
+    for (int u = 0; u < ASSA_ADJ_PER; ++u) nan |= kA[u].s != kA[u].s;
+    if (__syncthreads_or(nan)) gather(std::true_type{});
     float sum[ASSA_ADJ_PER];
 #pragma unroll
     for (int u = 0; u < ASSA_ADJ_PER; ++u) sum[u] = kA[u].s;

@@ -114,3 +114,37 @@ def test_moment_adjoint_few_tiles(nd, sides):
     delta = np.random.default_rng(nd).normal(size=(w.Nd, w.Nt)).astype(np.float32)
     _check(w, delta, full=False, A=w.A)
 
+
+@pytest.mark.parametrize("assa", [False, True])
+@pytest.mark.parametrize("nd", [3, 130])
+def test_sensor_on_a_node_with_a_record_that_begins_later(assa, nd):
+    """Sensors on lattice nodes add nothing to the nodes' gradients where their records do not reach back to the
+    time of flight 0; the parts of the others stay.  Coordinates that are exact in FP32, so that the distance of
+    node and sensor comes out as 0, or its square just below it."""
+    import torch
+    from gpair_testutil import device_inputs
+    from paper_2602_03893_gb300 import _lib
+
+    h = 2.0 ** -13
+    g = synth.Grid(17, 9, 10, h, h, 0.0, 0.0, 0.0)
+    on = np.random.default_rng(1).choice(g.M, 40, replace=False)
+    nodes = (np.stack([on % g.nx, on // g.nx % g.ny, on // (g.nx * g.ny)], axis=1) + 0.5) * h
+    far = synth.cap_sensors(nd, 12e-3, 140.0) + np.float32(1e-3)
+    xyz = np.concatenate([nodes, far]).astype(np.float32)
+    w = synth.Workload("on-a-node", g, xyz, 400, A=np.ones(g.M, np.float32), t0=4e-6)
+    delta = np.random.default_rng(nd).normal(size=(w.Nd, w.Nt)).astype(np.float32)
+    # 4 us is 6 mm, beyond the lattice: these sensors see nothing of it
+    wf = synth.Workload("far", g, xyz[40:], 400, A=w.A, t0=4e-6)
+
+    def grad(work, d):
+        if not assa:
+            return gpu_adjoint(work, d, False, A=work.A)["A"]
+        gs, arr = device_inputs(work)
+        gA = torch.full((work.M,), float("nan"), device="cuda")
+        _lib.gpair_assa_adjoint(gs, arr, torch.as_tensor(d, device="cuda"), gA)
+        return gA.cpu().numpy()
+
+    got, want = grad(w, delta), grad(wf, np.ascontiguousarray(delta[40:]))
+    assert np.all(np.isfinite(got)), np.flatnonzero(~np.isfinite(got))
+    # the same terms, summed in chunks of 32 that begin elsewhere
+    assert rel_l2(got, want) < 1e-6
