@@ -65,6 +65,7 @@ cudaError_t launch_assa_forward_lanes(const GaussDev& g, const ArrDev& a, const 
                                       cudaStream_t st);
 int assa_lanes_nz(double diag, double widened, double invDelta, int alpha);
 size_t assa_lanes_smem(int NW, int NZ);
+size_t assa_fwd_smem(int LB, const AssaTable& T);
 size_t assa_dconv_bytes(const ArrDev& a, const AssaTable& T);
 cudaError_t launch_assa_adjoint(const GaussDev& g, const ArrDev& a, const float* delta, float* gA, const AssaTable& T,
                                 float* dconv, const cudaEvent_t* ev, cudaStream_t st);
@@ -959,7 +960,24 @@ ArrDev assa_band_array(const GaussDev& g, const ArrDev& a, const AssaTable& T) {
 // warp to a sensor, whose scale their masses take (qb: those slabs' bricks).  A warp takes 32 sensors
 // whether they are there or not, so that fewer than ASSA_LANES_MIN go to the other kernel; so do slabs
 // too many for the sorted reduction and lattices so coarse that a brick's band does not fit.
+//
+// The other kernel also takes what it is faster at.  Over 8 x 8 x 4 to 128^3 nodes, 12 to 1024 sensors, fine grids
+// of alpha = 1 to 32 and three spacings (1160 plans, of which the three rules leave 491 to the lanes):
+//  - fewer than ASSA_LANES_WARPS warps in all: eight sensors a CTA fill more of the chip.  16^3 nodes, 48 sensors, 32
+//    warps: 38 us, lanes 43 at alpha = 2 and 65 at alpha = 7; from 192 warps on lanes took 0.2 to 1.0 of the time;
+//  - fewer than ASSA_LANES_RESIDENT warps on an SM, for bands of many fine samples: 128 x 128 x 64 nodes, 48 sensors,
+//    alpha = 10, two warps: 372 us, lanes 710;
+//  - its smaller slabs convolve more: by ASSA_LANES_TAPS products a pair and over it loses.  128 x 128 x 64 nodes, 96
+//    sensors, alpha = 7 (8.4 against 2.6 products): 344 us, lanes 589.
+// What is left took 0.19 to 1.01 of the other kernel's time.  Where the other kernel's bands do not fit, lanes stay.
 constexpr int ASSA_LANES_MIN = 12, ASSA_LANES_SLABS = 2048;
+constexpr int ASSA_LANES_WARPS = 192, ASSA_LANES_RESIDENT = 6;
+constexpr double ASSA_LANES_TAPS = 4.0;
+// Products of the bands' convolutions a pair, for slabs of sb bricks.
+double assa_conv_per_pair(const FwdPlan& p, const GaussDev& g, const AssaTable& T) {
+    const double nodes = (double)std::min(p.sbx * BX, g.nx) * std::min(p.sby * BY, g.ny) * std::min(p.sbz * BZ, g.nz);
+    return p.LB * (2.0 * T.K + 1.0) / nodes;
+}
 FwdPlan plan_assa_forward(const GaussDev& g, const ArrDev& aa, const AssaTable& T) {
     const FwdPlan wide = plan_forward(g, aa);
     if (aa.Nd < ASSA_LANES_MIN) return wide;
@@ -1001,7 +1019,12 @@ FwdPlan plan_assa_forward(const GaussDev& g, const ArrDev& aa, const AssaTable& 
         if (plan(p)) { best = p; any = true; }
         else if (any) break;
     }
-    return any ? best : wide;
+    if (!any) return wide;
+    if (assa_fwd_smem(wide.LB, T) > SMEM_PER_CTA) return best;
+    const int64_t resident = best.NW * (int64_t)(SMEM_PER_CTA / (assa_lanes_smem(best.NW, best.NZ) + 1024));
+    const double extra = assa_conv_per_pair(best, g, T) - assa_conv_per_pair(wide, g, T);
+    const bool faster = best.S * groups >= ASSA_LANES_WARPS && resident >= ASSA_LANES_RESIDENT && extra <= ASSA_LANES_TAPS;
+    return faster ? best : wide;
 }
 
 // Scratch of the ASSA forward beyond the plan: max |A| for the fixed-point bands.

@@ -187,9 +187,10 @@ def test_sparse_slabs():
     _check_forward(synth.Workload("assa-sparse", g, synth.cap_sensors(40, 20e-3, 120.0), 900, A=None), A=A)
 
 
-@pytest.mark.parametrize("sides,h,sigma,n_min,off", [((16, 16, 16), 1e-4, 1e-4, 513, 2.0), ((35, 20, 17), 1e-4, 1e-4, 513, 4.0),
-                                                     ((16, 16, 16), 1.2e-5, 1.2e-5, 513, 0.25)])
-def test_lattice_far_from_the_origin(sides, h, sigma, n_min, off):
+@pytest.mark.parametrize("sides,h,sigma,n_min,off,shells",
+                         [((16, 16, 16), 1e-4, 1e-4, 513, 2.0, 1), ((35, 20, 17), 1e-4, 1e-4, 513, 4.0, 1),
+                          ((16, 16, 16), 1.2e-5, 1.2e-5, 513, 0.25, 1), ((16, 16, 16), 2.4e-5, 2.4e-5, 129, 2.0, 24)])
+def test_lattice_far_from_the_origin(sides, h, sigma, n_min, off, shells):
     """Fine grids of alpha = 32 and 256, lattices so far out that the slabs' boxes, widened by a part of their
     coordinates, start several fine samples before the nearest node: the farthest nodes' masses, seen along
     the diagonals of two bricks, stay in the band.  Only nodes at the bricks' corners have amplitudes."""
@@ -200,6 +201,29 @@ def test_lattice_far_from_the_origin(sides, h, sigma, n_min, off):
     d = np.array([[7.0 * x, 7.0 * y, 3.0 * z] for x in (-1, 1) for y in (-1, 1) for z in (-1, 1)])
     d /= np.linalg.norm(d, axis=1, keepdims=True)
     o = np.array([g.ox, g.oy, g.oz])
-    xyz = np.concatenate([o + np.array([4.0, 4.0, 2.0]) * h * (2 * q + 1) + 10e-3 * d for q in (0, 1)])
+    xyz = np.concatenate([o + np.array([4.0, 4.0, 2.0]) * h * (2 * q + 1) + (10e-3 + 1e-5 * r) * d
+                          for q in (0, 1) for r in range(shells)])
     w = synth.Workload("assa-far", g, xyz.astype(np.float32), 400, A=A)
     _check_forward(w, A=A, n_min=n_min)
+
+
+@pytest.mark.parametrize("nd", [33, 65, 230])
+@pytest.mark.parametrize("n_min", [1, 25, 61, 101, 257])
+@pytest.mark.parametrize("sides", [(35, 20, 17), (40, 24, 40)])
+def test_lanes_and_the_other_kernel(sides, n_min, nd):
+    """On both sides of the rules that choose the kernel: 150 to 192 and more warps, fine grids of alpha = 1 to 16
+    whose bands leave room for many and for few warps, slabs of one and of several bricks."""
+    g = synth.centred_grid(*sides, 0.1e-3)
+    w = synth.Workload("assa-rules", g, synth.cap_sensors(nd, 15e-3, 150.0), 410, A=None)
+    _check_forward(w, A=_dense(w), n_min=n_min)
+
+
+def test_lanes_with_sensors_in_the_volume():
+    """Lanes without a bound on A / r beside lanes with one, and a brick without amplitudes."""
+    g = synth.centred_grid(24, 24, 12, 0.1e-3)
+    xyz = synth.cap_sensors(300, 12e-3, 120.0)
+    xyz[::29] = (np.array([0.21, -0.33, 0.08]) * 1e-3 + np.arange(len(xyz[::29]))[:, None] * 1.7e-5).astype(np.float32)
+    w = synth.Workload("assa-in-lanes", g, xyz, 400, A=None)
+    A = _dense(w) * 1e6
+    A.reshape(12, 24, 24)[:4, :8, :8] = 0.0
+    _check_forward(w, A=A)
