@@ -1232,11 +1232,15 @@ cudaError_t launch_forward(const GaussDev& g, const ArrDev& a, const TileInfo* t
 }
 
 constexpr int SRS_SEG = 4;
-static bool slab_reduce_few(const ArrDev& a) {      // the grid of four chunks a block is under two blocks an SM
-    return (int64_t)a.Nd * ((a.Nt + SRS_CHUNKS * SRS_THREADS - 1) / (SRS_CHUNKS * SRS_THREADS)) <= (int64_t)device_sms() * 2;
+// Blocks of 64 samples and four warps to 32: where the grid of four chunks a block is under two blocks an SM; but not for
+// a few slabs and many blocks, whose start costs more than it saves (one slab, 128 sensors, 1500 samples: 6 us more).
+static bool slab_reduce_few(const ArrDev& a, int S) {
+    const int64_t sms = device_sms(), per = SRS_THREADS / SRS_SEG;
+    return (int64_t)a.Nd * ((a.Nt + SRS_CHUNKS * SRS_THREADS - 1) / (SRS_CHUNKS * SRS_THREADS)) <= sms * 2 &&
+           (S >= 16 || (int64_t)a.Nd * ((a.Nt + per - 1) / per) <= sms * 8);
 }
-static dim3 slab_reduce_sorted_grid(const ArrDev& a) {
-    const int per = slab_reduce_few(a) ? SRS_THREADS / SRS_SEG : SRS_CHUNKS * SRS_THREADS;
+static dim3 slab_reduce_sorted_grid(const ArrDev& a, int S) {
+    const int per = slab_reduce_few(a, S) ? SRS_THREADS / SRS_SEG : SRS_CHUNKS * SRS_THREADS;
     return dim3(a.Nd, (a.Nt + per - 1) / per);
 }
 
@@ -1250,9 +1254,9 @@ static size_t slab_reduce_sorted_smem(int S) {
 cudaError_t launch_slab_reduce_rows(const ArrDev& a, const float* partial, const int2* rows, int S, int PL, float* y,
                                     cudaStream_t st) {
     dim3 rgrid((a.Nt + 255) / 256, a.Nd);
-    if (S <= SRS_MAX_S && slab_reduce_sorted_grid(a).y <= 65535)
-        slab_reduce_sorted_kernel<<<slab_reduce_sorted_grid(a), SRS_THREADS, slab_reduce_sorted_smem(S), st>>>(
-            partial, rows, S, a.Nd, a.Nt, PL, slab_reduce_few(a) ? 1 : SRS_CHUNKS, slab_reduce_few(a) ? SRS_SEG : 1, y);
+    if (S <= SRS_MAX_S && slab_reduce_sorted_grid(a, S).y <= 65535)
+        slab_reduce_sorted_kernel<<<slab_reduce_sorted_grid(a, S), SRS_THREADS, slab_reduce_sorted_smem(S), st>>>(
+            partial, rows, S, a.Nd, a.Nt, PL, slab_reduce_few(a, S) ? 1 : SRS_CHUNKS, slab_reduce_few(a, S) ? SRS_SEG : 1, y);
     else if (S <= SLAB_RED_MAX_S)
         slab_reduce_banded_kernel<<<rgrid, SLAB_RED_THREADS, (size_t)S * sizeof(int2), st>>>(partial, rows, S, a.Nd,
                                                                                              a.Nt, PL, y);
@@ -1264,9 +1268,9 @@ cudaError_t launch_slab_reduce_rows(const ArrDev& a, const float* partial, const
 cudaError_t launch_slab_reduce(const GaussDev& g, const ArrDev& a, const float* partial, const int2* rows, int S,
                                int PL, float* y, cudaStream_t st) {
     dim3 rgrid((a.Nt + 255) / 256, a.Nd);
-    if (g.grid && S <= SRS_MAX_S && slab_reduce_sorted_grid(a).y <= 65535)
-        slab_reduce_sorted_kernel<<<slab_reduce_sorted_grid(a), SRS_THREADS, slab_reduce_sorted_smem(S), st>>>(
-            partial, rows, S, a.Nd, a.Nt, PL, slab_reduce_few(a) ? 1 : SRS_CHUNKS, slab_reduce_few(a) ? SRS_SEG : 1, y);
+    if (g.grid && S <= SRS_MAX_S && slab_reduce_sorted_grid(a, S).y <= 65535)
+        slab_reduce_sorted_kernel<<<slab_reduce_sorted_grid(a, S), SRS_THREADS, slab_reduce_sorted_smem(S), st>>>(
+            partial, rows, S, a.Nd, a.Nt, PL, slab_reduce_few(a, S) ? 1 : SRS_CHUNKS, slab_reduce_few(a, S) ? SRS_SEG : 1, y);
     else if (g.grid && S <= SLAB_RED_MAX_S)
         slab_reduce_banded_kernel<<<rgrid, SLAB_RED_THREADS, (size_t)S * sizeof(int2), st>>>(partial, rows, S, a.Nd,
                                                                                              a.Nt, PL, y);

@@ -175,3 +175,14 @@ def test_free_gaussians_few_tiles(sides):
     free = synth.free_gaussians(g, 7, A=np.random.default_rng(8).uniform(0.2, 1.0, g.M))
     w = synth.Workload("free-few", g, synth.cap_sensors(35, 20e-3, 160.0), 900, free=free)
     _check(w)
+
+
+@pytest.mark.parametrize("nd,nt", [(19, 4099), (20, 4099), (128, 607), (128, 609)])
+@pytest.mark.parametrize("sides", [(8, 8, 8), (16, 8, 8)])
+def test_reduction_of_few_slabs(sides, nd, nt):
+    """Under 16 rows a sensor: the last grid of 8 blocks of 64 samples an SM (152 of them) and the first beyond; the
+    second lattice has two cubes."""
+    g = synth.centred_grid(*sides, 0.1e-3)
+    A = np.random.default_rng(nd).uniform(0.1, 1.0, g.M).astype(np.float32)
+    w = synth.Workload("few-slabs", g, synth.cap_sensors(nd, 15e-3, 150.0), nt, A=A)
+    _check(w)
