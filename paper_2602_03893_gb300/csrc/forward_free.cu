@@ -262,15 +262,14 @@ fwd_free_lanes_kernel(GaussDev g, ArrDev a, const TileInfo* __restrict__ ti, con
 // Longest slabs first: the slab descriptors permuted in place by decreasing box diagonal (ties
 // by index), so that the CTAs of the slabs with the longest sample bands -- those that may need
 // several passes, such as a tile range that jumps across the Morton order -- start in the first
-// wave instead of extending the last; by_count: by decreasing pad, for lattices' slabs of cubes with and without
-// amplitudes.  The slab reduction sums the rows of all slabs, so only the
+// wave instead of extending the last.  The slab reduction sums the rows of all slabs, so only the
 // order of its (fixed-order) sum changes.  One CTA; S <= FF_ORDER_MAX.
 constexpr int FF_ORDER_THREADS = 1024;
 constexpr int FF_ORDER_MAX = 2048;
 constexpr int FF_ORDER_PER = FF_ORDER_MAX / FF_ORDER_THREADS;
 
 __global__ void __launch_bounds__(FF_ORDER_THREADS)
-slab_order_kernel(SlabInfo* __restrict__ si, int S, int by_count) {
+slab_order_kernel(SlabInfo* __restrict__ si, int S) {
     __shared__ float key[FF_ORDER_MAX];
     SlabInfo mine[FF_ORDER_PER];
     int rank[FF_ORDER_PER];
@@ -281,7 +280,7 @@ slab_order_kernel(SlabInfo* __restrict__ si, int S, int by_count) {
             mine[u] = si[s];
             const float dx = mine[u].hi[0] - mine[u].lo[0], dy = mine[u].hi[1] - mine[u].lo[1],
                         dz = mine[u].hi[2] - mine[u].lo[2];
-            key[s] = by_count ? (float)mine[u].pad : (mine[u].t_end > mine[u].t_begin) ? dx * dx + dy * dy + dz * dz : -1.f;
+            key[s] = (mine[u].t_end > mine[u].t_begin) ? dx * dx + dy * dy + dz * dz : -1.f;
         }
     }
     __syncthreads();
@@ -312,9 +311,9 @@ slab_order_kernel(SlabInfo* __restrict__ si, int S, int by_count) {
 
 size_t fwd_free_smem(int NW, int LB) { return ff_smem_bytes(NW, LB); }
 
-cudaError_t launch_slab_order(SlabInfo* si, int S, bool by_count, cudaStream_t st) {
+cudaError_t launch_slab_order(SlabInfo* si, int S, cudaStream_t st) {
     if (S <= 1 || S > FF_ORDER_MAX) return cudaSuccess;     // more slabs: kept in tile order
-    slab_order_kernel<<<1, FF_ORDER_THREADS, 0, st>>>(si, S, by_count);
+    slab_order_kernel<<<1, FF_ORDER_THREADS, 0, st>>>(si, S);
     return cudaGetLastError();
 }
 

@@ -27,8 +27,6 @@
 
 namespace gp {
 
-cudaError_t launch_slab_order(SlabInfo* si, int S, bool by_count, cudaStream_t st);
-
 constexpr int CUBE = 8;                        // cube side, lattice nodes
 constexpr int CUBE_N = CUBE * CUBE * CUBE;     // Gaussians per cube
 constexpr int FL_RING = 4;                     // cube buffers in flight
@@ -174,11 +172,13 @@ __device__ __forceinline__ SlabInfo cube_slab(const GaussDev& g, const CubeSlabs
 }
 
 // Slab descriptors, a CTA each; pad is the number of cubes with amplitudes: slabs without any (sparse
-// images) are left out of the forward, and those with most of them come first (launch_slab_order).  The signals of a
+// images) are left out of the forward, and those with most of them come first (cube_slab_order_kernel).  The signals of a
 // vessel phantom in 128 x 128 x 64 nodes, 1024 sensors: 714 us with all slabs' bands cleared and written, 450 us
 // without, 430 us in that order.
 // Few sensors' forward is not worth the look through the amplitudes (13 us of 210 for 47 sensors and a million nodes).
-constexpr int SI_THREADS = 512, SI_SCAN_MIN = 128;
+// Blocks of 32 nodes a thread, narrow lines sharing a warp: 2048 slabs of 512 nodes take 9 us, 20 with blocks of 512 and
+// a warp to a line.
+constexpr int SI_THREADS = 512, SI_THREADS_MIN = 128, SI_SCAN_MIN = 128;
 constexpr int SI_CUBES = 512;            // cubes told apart; a slab of more counts as one
 __global__ void __launch_bounds__(SI_THREADS)
 slab_info_cube_kernel(GaussDev g, const CubeSlabs c, int scan, SlabInfo* si) {
@@ -188,27 +188,53 @@ slab_info_cube_kernel(GaussDev g, const CubeSlabs c, int scan, SlabInfo* si) {
     const int ay = o.by0 * CUBE, byn = min(g.ny, (o.by0 + o.bdy) * CUBE);
     const int az = o.bz0 * CUBE, bzn = min(g.nz, (o.bz0 + o.bdz) * CUBE);
     const bool each = o.t_end <= SI_CUBES;
-    for (int q = threadIdx.x; q < SI_CUBES; q += SI_THREADS) on[q] = 0;
+    for (int q = threadIdx.x; q < SI_CUBES; q += blockDim.x) on[q] = 0;
     __syncthreads();
     bool any = !scan;
+    // 8, 16 or 32 lanes to a line of x, so that narrow slabs' lines share a warp; a thread's lines are `step` apart
     const int wy = byn - ay, lines = scan ? wy * (bzn - az) : 0;
+    const int sh = bxn - ax <= 8 ? 3 : bxn - ax <= 16 ? 4 : 5, step = blockDim.x >> sh, dy = step % wy, dz = step / wy;
     for (int x0 = ax; x0 < bxn; x0 += 32) {
-        const int x = x0 + (threadIdx.x & 31);
+        const int x = x0 + (threadIdx.x & ((1 << sh) - 1));
+        int y = (threadIdx.x >> sh) % wy, z = (threadIdx.x >> sh) / wy;
 #pragma unroll 8
-        for (int r = threadIdx.x >> 5; r < lines; r += SI_THREADS / 32) {
-            const int y = r % wy, z = r / wy;
+        for (int r = threadIdx.x >> sh; r < lines; r += step) {
             if (x < bxn && g.A[((int64_t)(az + z) * g.ny + ay + y) * g.nx + x] != 0.f) {
                 any = true;
                 if (each) on[((z / CUBE) * o.bdy + y / CUBE) * o.bdx + (x - ax) / CUBE] = 1;
             }
+            y += dy;
+            z += dz;
+            if (y >= wy) { y -= wy; ++z; }
         }
     }
     const int slab_on = __syncthreads_or(any);
-    static_assert(SI_CUBES <= SI_THREADS, "a thread to a cube");
-    const int count = __syncthreads_count(threadIdx.x < SI_CUBES && on[threadIdx.x]);
+    static_assert(SI_CUBES % SI_THREADS == 0 && SI_THREADS % SI_THREADS_MIN == 0, "every thread takes as many cubes");
+    int count = 0;
+    for (int q = threadIdx.x; q < SI_CUBES; q += blockDim.x) count += __syncthreads_count(on[q]);
     if (threadIdx.x) return;
     o.pad = slab_on ? max(1, count) : 0;
     si[blockIdx.x] = o;
+}
+
+// out: the descriptors by decreasing pad, ties by index.  Each CTA counts the ranks of 32 slabs, eight threads to one.
+// The slab reduction sums the rows of all slabs, so only the order of its (fixed-order) sum changes.  2048 slabs:
+// 135 us with one CTA for all of them, 7 us.
+constexpr int SO_SLABS = 2048, SO_SLAB_THREADS = 256, SO_SLAB_PER = SO_SLAB_THREADS / 8;
+__global__ void __launch_bounds__(SO_SLAB_THREADS)
+cube_slab_order_kernel(const SlabInfo* __restrict__ in, int S, SlabInfo* __restrict__ out) {
+    __shared__ int key[SO_SLABS];
+    for (int q = threadIdx.x; q < S; q += SO_SLAB_THREADS) key[q] = in[q].pad;
+    __syncthreads();
+    const int s = blockIdx.x * SO_SLAB_PER + threadIdx.x / 8, part = threadIdx.x % 8;
+    int r = 0;
+    if (s < S) {
+        const int k = key[s];
+#pragma unroll 4
+        for (int t = part; t < S; t += 8) r += key[t] > k || (key[t] == k && t < s);
+    }
+    for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+    if (s < S && part == 0) out[r] = in[s];
 }
 
 // 1.5 * 2^23: adding it to |x| < 2^22 with rounding toward +inf leaves ceil(x) in the low bits.
@@ -560,7 +586,8 @@ int fwd_lanes_nz(float h, float invDelta) { return fl_nz(h, invDelta); }
 // Largest number of CTAs that may share a slab of one cube.
 int fwd_lanes_parts(const MomentTable& T) { return T.P == 6 && T.L <= 32 ? 8 : 1; }
 
-// S rows a sensor: `parts` of each slab of sx x sy x sz cubes.  si: S descriptors' place.  ev (optional): two events
+// S rows a sensor: `parts` of each slab of sx x sy x sz cubes.  si: S descriptors' place; before they are in order they
+// stand in that of the rows (8 bytes a sensor and row), which the slab kernel writes.  ev (optional): two events
 // recorded immediately before and after the slab kernel.
 cudaError_t launch_forward_lanes(const GaussDev& g, const ArrDev& a, int sx, int sy, int sz, int S, SlabInfo* si, float* partial,
                                  int2* rows, int LB, int NZ, int NW, int parts, int* status, const CUtensorMap* tmap,
@@ -584,9 +611,18 @@ cudaError_t launch_forward_lanes(const GaussDev& g, const ArrDev& a, int sx, int
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const CubeSlabs c = cube_slabs(g, sx, sy, sz);
-    if (parts == 1) slab_info_cube_kernel<<<S, SI_THREADS, 0, st>>>(g, c, a.Nd >= SI_SCAN_MIN, si);      // parts form their own: a launch less
+    if (parts == 1) {          // parts form their own: a launch less
+        const bool scan = a.Nd >= SI_SCAN_MIN, order = scan && S > 1 && S <= SO_SLABS;
+        static_assert(SI_SCAN_MIN * sizeof(int2) >= sizeof(SlabInfo), "a row's place holds a descriptor");
+        SlabInfo* first = order ? reinterpret_cast<SlabInfo*>(rows) : si;
+        const int64_t nodes = (int64_t)sx * sy * sz * CUBE_N;
+        int threads = SI_THREADS_MIN;
+        while (threads < SI_THREADS && scan && nodes > 32 * threads) threads *= 2;
+        slab_info_cube_kernel<<<S, threads, 0, st>>>(g, c, scan, first);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if (order) cube_slab_order_kernel<<<(S + SO_SLAB_PER - 1) / SO_SLAB_PER, SO_SLAB_THREADS, 0, st>>>(first, S, si);
+    }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (parts == 1 && a.Nd >= SI_SCAN_MIN && (e = launch_slab_order(si, S, true, st)) != cudaSuccess) return e;
     if (ev && (e = cudaEventRecord(ev[0], st)) != cudaSuccess) return e;
     kern<<<grid, 32 * NW, smem, st>>>(g, a, si, c, partial, rows, LB, NZ, parts, status, tmap != nullptr,
                                       tmap ? *tmap : zero_map, T);

@@ -186,3 +186,24 @@ def test_reduction_of_few_slabs(sides, nd, nt):
     A = np.random.default_rng(nd).uniform(0.1, 1.0, g.M).astype(np.float32)
     w = synth.Workload("few-slabs", g, synth.cap_sensors(nd, 15e-3, 150.0), nt, A=A)
     _check(w)
+
+
+@pytest.mark.parametrize("free", [False, True])
+@pytest.mark.parametrize("n", [9, 10, 13])
+def test_order_of_many_slabs(free, n):
+    """The slabs' order with S just under, at and over a power of two, up to its 2048 words (n^3 cubes, or tiles of
+    free centres, and 128 sensors): every slab is in the sum once, with all amplitudes and with few."""
+    if free:
+        g = synth.centred_grid(16, 16, n, 0.1e-3)
+        w = synth.Workload("order", g, synth.cap_sensors(128, 15e-3, 150.0), 500,
+                           free=synth.free_gaussians(g, n, A=np.random.default_rng(8).uniform(0.2, 1.0, g.M)))
+        _check(w)
+        return
+    side = 8 * n - 3
+    g = synth.centred_grid(side, side, side, 0.1e-3)
+    rng = np.random.default_rng(n)
+    w = synth.Workload("order", g, synth.cap_sensors(128, 15e-3, 150.0), 700, A=rng.uniform(0.1, 1.0, g.M).astype(np.float32))
+    idx = np.array([0, 31, 77, 127])
+    _check(w, sensors_idx=idx)
+    few = np.where(rng.uniform(size=g.M) < 3e-5, w.A, 0).astype(np.float32)
+    _check(w, A=few, sensors_idx=idx)
