@@ -11,6 +11,7 @@
 // the tcgen05 kernels (unet_tc.cu) do not take, and tensor path 0.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "../../include/gpair_unet.h"
@@ -271,8 +272,8 @@ __global__ void bias_grad_sum_kernel(const float* __restrict__ part, int nblocks
 // The elementwise passes below are HBM-bound: what they cost is their bytes, provided that each
 // thread moves 16 bytes at a time and spends few instructions on indices.  V channels per access:
 // 8 (one 16-byte load or store) where the channel counts are multiples of 8 and the tensors 16-byte
-// aligned, else 1.  Blocks are 128 units along a row of voxels x 2 rows, so a unit costs one 32-bit
-// division.  The copies of one prediction at 64 x 128 x 128 voxels (packing, three poolings, three
+// aligned, else 1.  Blocks are up to 128 units along a row of voxels x the rows that fill 256 threads, and few long
+// rows are shared by blocks (row_launch), so a unit costs one 32-bit division.  The copies of one prediction at 64 x 128 x 128 voxels (packing, three poolings, three
 // upsamplings with their concatenations): 444 us with one channel per access and 64-bit index
 // divisions, 58 us like this.
 template <int V>
@@ -301,14 +302,30 @@ __device__ __forceinline__ Chunk<8> narrow(const float (&f)[8]) {
     return c;
 }
 
-constexpr int EW_X = 128, EW_Y = 2;      // block of the row kernels
+constexpr int EW_X = 128, EW_THREADS = 256;      // units along a row, at most, and threads of a block of the row kernels
 // u / d of a unit in a row of n units (64 bits only for rows that need them)
 __device__ __forceinline__ int64_t unit_div(int64_t u, int d, int64_t n) {
     return n <= 0xFFFFFFFFll ? (int64_t)((uint32_t)u / (uint32_t)d) : u / d;
 }
-inline unsigned row_blocks(int64_t rows) {
-    const int64_t b = (rows + EW_Y - 1) / EW_Y, most = (int64_t)gp::device_sms() * 64;
-    return (unsigned)(b < most ? b : most);
+// Block and grid of a row kernel: narrow rows take as many lanes as they have units (2 units a row, 65,536 rows: 23 us
+// with 128 lanes to each, 7 us), and the units of a long row are shared by blocks where the rows are few (one
+// row of 4096 units: 18 us with one block, 7 us).
+// WIDE, blocks of 128 lanes and a block to a row: strides that the compiler knows (64 x 128 x 128 voxels, 32 + 16 channels:
+// 20.5 us, 23.2 without).
+struct RowLaunch {
+    dim3 grid, block;
+    bool wide() const { return block.x == EW_X && grid.y == 1; }
+};
+template <bool WIDE> __device__ __forceinline__ unsigned row_lanes() { return WIDE ? EW_X : blockDim.x; }
+template <bool WIDE> __device__ __forceinline__ unsigned rows_per_block() { return WIDE ? EW_THREADS / EW_X : blockDim.y; }
+template <bool WIDE> __device__ __forceinline__ unsigned row_sharers() { return WIDE ? 1u : gridDim.y; }
+inline RowLaunch row_launch(int64_t rows, int64_t units) {
+    unsigned bx = 1;
+    while (bx < EW_X && (int64_t)bx < units) bx *= 2;
+    const unsigned by = EW_THREADS / bx;
+    const int64_t most = (int64_t)gp::device_sms() * 64, b = std::min((rows + by - 1) / by, most);
+    const int64_t along = std::min((units + bx - 1) / bx, std::max<int64_t>(1, gp::device_sms() * 4 / b));
+    return {dim3((unsigned)b, (unsigned)along), dim3(bx, by)};
 }
 inline bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
 
@@ -331,15 +348,15 @@ __global__ void relu_bwd8_kernel(const bf16_t* __restrict__ act, bf16_t* __restr
     }
 }
 
-template <int V>
-__global__ void __launch_bounds__(EW_X * EW_Y)
+template <int V, bool WIDE>
+__global__ void __launch_bounds__(EW_THREADS)
 pool2_fwd_kernel(const bf16_t* __restrict__ in, int D, int H, int W, int C, bf16_t* __restrict__ out) {
     const int h = H / 2, w = W / 2, CV = C / V;
     const int64_t rows = (int64_t)(D / 2) * h, units = (int64_t)w * CV;
-    for (int64_t r = blockIdx.x * (int64_t)EW_Y + threadIdx.y; r < rows; r += (int64_t)gridDim.x * EW_Y) {
+    for (int64_t r = blockIdx.x * (int64_t)rows_per_block<WIDE>() + threadIdx.y; r < rows; r += (int64_t)gridDim.x * rows_per_block<WIDE>()) {
         const int64_t z = r / h, y = r - z * h;
         const Chunk<V>* src = chunks<V>(in) + ((2 * z * H + 2 * y) * W) * CV;
-        for (int64_t u = threadIdx.x; u < units; u += EW_X) {
+        for (int64_t u = (WIDE ? 0u : blockIdx.y * blockDim.x) + threadIdx.x; u < units; u += row_sharers<WIDE>() * row_lanes<WIDE>()) {
             const int64_t x = unit_div(u, CV, units), c = u - x * CV;
             float s[V];
 #pragma unroll
@@ -372,17 +389,17 @@ __global__ void pool2_bwd_kernel(const bf16_t* __restrict__ dout, int D, int H, 
 // out[v] = (a upsampled x2 (Ca channels), b[v] (Cb channels)), Cb = 0: the upsampling alone.  Level 0
 // of the network (32 + 16 channels): 155.9 us for the upsampling and 113.1 us for the concatenation
 // as two passes through a tensor of their own.
-template <int V>
-__global__ void __launch_bounds__(EW_X * EW_Y)
+template <int V, bool WIDE>
+__global__ void __launch_bounds__(EW_THREADS)
 up2_concat_kernel(const bf16_t* __restrict__ a, int D, int H, int W, int Ca, const bf16_t* __restrict__ b, int Cb,
                   bf16_t* __restrict__ out) {
     const int H2 = 2 * H, W2 = 2 * W, CaV = Ca / V, CbV = Cb / V, CV = CaV + CbV;
     const int64_t rows = (int64_t)2 * D * H2, units = (int64_t)W2 * CV;
-    for (int64_t r = blockIdx.x * (int64_t)EW_Y + threadIdx.y; r < rows; r += (int64_t)gridDim.x * EW_Y) {
+    for (int64_t r = blockIdx.x * (int64_t)rows_per_block<WIDE>() + threadIdx.y; r < rows; r += (int64_t)gridDim.x * rows_per_block<WIDE>()) {
         const int64_t z = r / H2, y = r - z * H2;
         const Chunk<V>* sa = chunks<V>(a) + ((z / 2) * H + y / 2) * W * CaV;
         const Chunk<V>* sb = chunks<V>(b) + r * W2 * CbV;
-        for (int64_t u = threadIdx.x; u < units; u += EW_X) {
+        for (int64_t u = (WIDE ? 0u : blockIdx.y * blockDim.x) + threadIdx.x; u < units; u += row_sharers<WIDE>() * row_lanes<WIDE>()) {
             const int64_t x = unit_div(u, CV, units);
             const int c = (int)(u - x * CV);
             chunks<V>(out)[r * units + u] = c < CaV ? sa[(x >> 1) * CaV + c] : sb[x * CbV + (c - CaV)];
@@ -508,13 +525,12 @@ bool dims_ok(int D, int H, int W, int C) { return D > 0 && H > 0 && W > 0 && C >
 constexpr int64_t MOST32 = ((int64_t)1 << 32) - ((int64_t)1 << 24);
 
 gpair_status up2_concat(const bf16_t* a, int D, int H, int W, int Ca, const bf16_t* b, int Cb, bf16_t* out, void* stream) {
-    const dim3 blk(EW_X, EW_Y);
-    const unsigned nb = row_blocks((int64_t)4 * D * H);
+    const bool vec = Ca % 8 == 0 && Cb % 8 == 0 && aligned16(a) && aligned16(b) && aligned16(out);
+    const RowLaunch l = row_launch((int64_t)4 * D * H, (int64_t)2 * W * (((int64_t)Ca + Cb) / (vec ? 8 : 1)));
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (Ca % 8 == 0 && Cb % 8 == 0 && aligned16(a) && aligned16(b) && aligned16(out))
-        up2_concat_kernel<8><<<nb, blk, 0, s>>>(a, D, H, W, Ca, b, Cb, out);
-    else
-        up2_concat_kernel<1><<<nb, blk, 0, s>>>(a, D, H, W, Ca, b, Cb, out);
+    auto kern = vec ? (l.wide() ? up2_concat_kernel<8, true> : up2_concat_kernel<8, false>)
+                    : (l.wide() ? up2_concat_kernel<1, true> : up2_concat_kernel<1, false>);
+    kern<<<l.grid, l.block, 0, s>>>(a, D, H, W, Ca, b, Cb, out);
     return st(cudaGetLastError());
 }
 
@@ -633,11 +649,12 @@ gpair_status gpair_relu_bwd(const gpair_bf16* act, gpair_bf16* g, int64_t n, voi
 
 gpair_status gpair_pool2_fwd(const gpair_bf16* in, int D, int H, int W, int C, gpair_bf16* out, void* stream) {
     if (!in || !out || !dims_ok(D, H, W, C) || (D | H | W) & 1) return GPAIR_ERR_INVALID_ARG;
-    const dim3 blk(EW_X, EW_Y);
-    const unsigned nb = row_blocks((int64_t)(D / 2) * (H / 2));
+    const bool vec = C % 8 == 0 && aligned16(in) && aligned16(out);
+    const RowLaunch l = row_launch((int64_t)(D / 2) * (H / 2), (int64_t)(W / 2) * (C / (vec ? 8 : 1)));
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (C % 8 == 0 && aligned16(in) && aligned16(out)) pool2_fwd_kernel<8><<<nb, blk, 0, s>>>(in, D, H, W, C, out);
-    else pool2_fwd_kernel<1><<<nb, blk, 0, s>>>(in, D, H, W, C, out);
+    auto kern = vec ? (l.wide() ? pool2_fwd_kernel<8, true> : pool2_fwd_kernel<8, false>)
+                    : (l.wide() ? pool2_fwd_kernel<1, true> : pool2_fwd_kernel<1, false>);
+    kern<<<l.grid, l.block, 0, s>>>(in, D, H, W, C, out);
     return st(cudaGetLastError());
 }
 

@@ -265,3 +265,20 @@ def test_training_reduces_loss():
         first = l if first is None else first
         last = l
     assert last < 0.3 * first, (first, last)
+
+
+@pytest.mark.parametrize("dims,C", [((2, 2, 1), 1), ((70, 90, 1), 8), ((65, 3, 1), 3), ((1, 1, 256), 128), ((1, 2, 64), 8),
+                                    ((1, 3, 129), 8), ((1, 1, 1021), 5), ((3, 40, 65), 16)])
+def test_row_kernels_on_narrow_and_long_rows(dims, C):
+    """Upsampling and pooling with one unit to a row, rows of powers of two and beside them, many rows of few units
+    and few rows of thousands that several blocks share."""
+    D, H, W = dims
+    gen = torch.Generator().manual_seed(C)
+    a = _bf((D * H * W, C), gen)
+    up = torch.full((8 * D * H * W, C), float("nan"), dtype=torch.bfloat16, device="cuda")
+    unet.gpair_up2_fwd(a.cuda(), dims, C, up)
+    ref = a.reshape(D, H, W, C).repeat_interleave(2, 0).repeat_interleave(2, 1).repeat_interleave(2, 2).reshape(-1, C)
+    assert torch.equal(up.cpu(), ref)
+    p = torch.full((D * H * W, C), float("nan"), dtype=torch.bfloat16, device="cuda")
+    unet.gpair_pool2_fwd(up, (2 * D, 2 * H, 2 * W), C, p)
+    assert torch.equal(p.cpu(), a)              # the mean of eight equal values: exact in single precision
