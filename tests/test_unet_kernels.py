@@ -282,3 +282,34 @@ def test_row_kernels_on_narrow_and_long_rows(dims, C):
     p = torch.full((D * H * W, C), float("nan"), dtype=torch.bfloat16, device="cuda")
     unet.gpair_pool2_fwd(up, (2 * D, 2 * H, 2 * W), C, p)
     assert torch.equal(p.cpu(), a)              # the mean of eight equal values: exact in single precision
+
+
+@pytest.mark.parametrize("cin,cout,taps", [(16, 16, 27), (64, 16, 1), (96, 32, 27), (32, 48, 27), (64, 64, 1), (80, 64, 27),
+                                            (128, 128, 27)])
+@pytest.mark.parametrize("dims", [(1, 1, 1), (3, 17, 9), (12, 24, 24), (40, 64, 61)])
+def test_wgrad_many_tiles_and_bias(dims, cin, cout, taps):
+    """One to dozens of voxel tiles a CTA, so that the ring's stages are used again and sums go on from tile to tile;
+    few and many splits of the sum over CTAs, in tiles of 32 and of 16 output channels; bias gradients of blocks with
+    one to dozens of voxels a thread."""
+    gen = torch.Generator().manual_seed(sum(dims) + cin)
+    nv = int(np.prod(dims))
+    x, dout = _bf((nv, cin), gen), _bf((nv, cout), gen)
+    # integers of up to 3 in size: every product and sum is exact, so the kernels must give the reference's bits
+    x, dout = (q.float().mul(2).round().clamp(-3, 3).to(torch.bfloat16) for q in (x, dout))
+    xg, gg = x.cuda(), dout.cuda()
+    dw, db = torch.ones((cout, taps, cin), device="cuda"), torch.ones(cout, device="cuda")
+    before = unet.gpair_unet_tensor_path()
+    unet.gpair_unet_tensor_path(2)
+    try:
+        unet.gpair_conv3d_wgrad(xg, gg, dims, cin, cout, taps, dw, db)
+    finally:
+        unet.gpair_unet_tensor_path(before)
+    assert unet.gpair_unet_tc_status() == 0
+    assert torch.equal(db.cpu().double() - 1, dout.double().sum(0))
+    X = F.pad(xg.double().reshape(*dims, cin), (0, 0, 1, 1, 1, 1, 1, 1))
+    G = gg.double()
+    D, H, W = dims
+    for t in range(taps):
+        dz, dy, dx = (t // 9, t // 3 % 3, t % 3) if taps == 27 else (1, 1, 1)
+        ref = G.T @ X[dz:dz + D, dy:dy + H, dx:dx + W].reshape(nv, cin)
+        assert torch.equal(dw[:, t].double() - 1, ref), t
