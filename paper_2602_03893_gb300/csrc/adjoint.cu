@@ -491,7 +491,7 @@ cudaError_t launch_adjoint_moment(const GaussDev& g, const ArrDev& a, const floa
     if (e != cudaSuccess) return e;
     if (ev && (e = cudaEventRecord(ev[0], st)) != cudaSuccess) return e;
     auto kern = T.P == 6 ? adj_moment_kernel<6> : T.P == 7 ? adj_moment_kernel<7> : adj_moment_kernel<8>;
-    const int split = adj_split(g.ntiles, a.Nd, ADJM_CTAS, 8, true);
+    const int split = adj_split_rows(g.ntiles, a.Nd);
     e = launch_split(kern, (unsigned)g.ntiles, split, ADJM_THREADS, 0, st, g, a, delta, (const float*)Q, T, gA,
                      (a.Nd + split - 1) / split);
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], st);
@@ -510,7 +510,7 @@ cudaError_t launch_adjoint(const GaussDev& g, const ArrDev& a, const TileInfo* t
     size_t smem = (size_t)ADJ_SC * LBA * sizeof(float);
     smem = smem < 5 * TILE * sizeof(float) ? 5 * TILE * sizeof(float) : smem;     // the split's sums
     unsigned blocks = (unsigned)g.ntiles;
-    const int split = adj_split(g.ntiles, a.Nd, ADJ_CTAS, 4, false);
+    const int split = adj_split(g.ntiles, a.Nd, ADJ_CTAS, 4);
     cudaError_t e = cudaSuccess;
 #define GP_LAUNCH_ADJ(G, F)                                                                                   \
     do {                                                                                                      \

@@ -28,21 +28,34 @@ __device__ __forceinline__ bool split_sum(float (&sum)[N], float* part, int at) 
 }
 
 // CTAs that share a tile's sensors, a power of two up to 8: doubled while the CTAs stay within a wave of `ctas` per SM and
-// keep `least` sensors each (idle SMs), and while they stay within some waves and keep 64.
-// rows: the tiles gather the sensors' rows of a table through L1, and CTAs that walk the sensors in the same order share
-// them there.  Such grids are split only where unsplit they are less than a wave, up to four waves.  The amplitude
-// adjoint with 1, 2, 4 and 8 CTAs a tile: 16 bricks, 128 sensors: 74 us with 1, 17 us with 8; 675 bricks, 952
-// sensors: 609, 600, 441, 370 us; 1024 bricks, 512 sensors: 337, 316, 305, 279 us; but 3900 bricks, 47 sensors: 76 us
-// with 1, 154 with 4, 241 with 8.  Without such rows up to 16 waves, for the last wave's sake: the gradient step
-// of 1024 tiles of free centres and 512 sensors 3498, 3435, 3424, 3413 us.
-inline int adj_split(int64_t ntiles, int Nd, int ctas, int least, bool rows) {
+// keep `least` sensors each (idle SMs), and while they stay within 16 waves and keep 64, for the last wave's sake: the
+// gradient step of 1024 tiles of free centres and 512 sensors 3498, 3435, 3424, 3413 us.
+inline int adj_split(int64_t ntiles, int Nd, int ctas, int least) {
     const int64_t wave = (int64_t)device_sms() * ctas;
-    const int64_t most = rows ? (ntiles < wave ? 4 * wave : 0) : 16 * wave;
     int split = 1;
     while (split < 8 && ((ntiles * split * 2 <= wave && Nd >= 2 * least * split) ||
-                         (ntiles * split * 2 <= most && Nd >= 128 * split)))
+                         (ntiles * split * 2 <= 16 * wave && Nd >= 128 * split)))
         split *= 2;
     return split;
+}
+
+// The same for the amplitude adjoints of lattices, whose tiles gather the sensors' rows of a table through L1: CTAs that
+// walk the sensors in the same order share them there, so that a split costs more than its barrier, and grids that
+// fill half of the chip's warps already lose by it.  Microseconds with 1, 2, 4 and 8 CTAs a tile, exact adjoint (the
+// discretised one is alike), at the lines of the rule (152 SMs):
+//    54 tiles,  128 sensors:   70   43   29   21        768 tiles,  128 sensors:   72   79   70   87
+//   150         128            70   41   27   33        768         300           160  172  140  155 (84 100 83 96)
+//   288         128            70   43   31   46        768         512           266  290  231  226
+//   512         128            69   45   51   62       1024         300           169  176  180  194
+//   512        1024           496  295  310  308       1352         512           305  428  365  360
+//  1024          33            28   33   45   70       2048        1024           761 1089  965  984
+inline int adj_split_rows(int64_t ntiles, int Nd) {
+    const int64_t sms = device_sms();
+    if (ntiles * 8 <= 4 * sms && Nd >= 64) return 8;
+    if (ntiles * 4 <= 8 * sms && Nd >= 32) return 4;
+    if (ntiles * 2 <= 8 * sms) return Nd >= 16 ? 2 : 1;
+    if (ntiles <= 6 * sms) return Nd >= 512 ? 8 : Nd >= 300 ? 4 : 1;
+    return 1;
 }
 
 template <typename... Args>

@@ -779,7 +779,7 @@ cudaError_t launch_assa_adjoint(const GaussDev& g, const ArrDev& a, const float*
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (ev && (e = cudaEventRecord(ev[0], st)) != cudaSuccess) return e;
-    const int split = adj_split(g.ntiles, a.Nd, ASSA_ADJ_CTAS, 8, true);
+    const int split = adj_split_rows(g.ntiles, a.Nd);
     e = launch_split(split > 1 ? assa_adj_kernel<true> : assa_adj_kernel<false>, (unsigned)g.ntiles, split, ASSA_ADJ_THREADS, 0, st, g, a, (const float*)dconv, T,
                      gA, (a.Nd + split - 1) / split);
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], st);

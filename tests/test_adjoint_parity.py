@@ -148,3 +148,14 @@ def test_sensor_on_a_node_with_a_record_that_begins_later(assa, nd):
     assert np.all(np.isfinite(got)), np.flatnonzero(~np.isfinite(got))
     # the same terms, summed in chunks of 32 that begin elsewhere
     assert rel_l2(got, want) < 1e-6
+
+
+@pytest.mark.parametrize("sides,nds", [((35, 33, 18), (31, 64, 70)), ((50, 44, 30), (40, 130)), ((62, 55, 31), (15, 16, 130)),
+                                       ((60, 60, 47), (299, 300, 512))])
+def test_moment_adjoint_more_tiles(sides, nds):
+    """The rule that divides a brick's sensors over CTAs, at its lines: 125, 336, 448 and 768 bricks."""
+    for nd in nds:
+        g = synth.centred_grid(*sides, 0.1e-3)
+        w = synth.Workload("more", g, synth.cap_sensors(nd, 15e-3, 150.0), 605, A=np.ones(g.M, np.float32))
+        delta = np.random.default_rng(nd).normal(size=(w.Nd, w.Nt)).astype(np.float32)
+        _check(w, delta, full=False, gauss_idx=np.sort(np.random.default_rng(7).choice(w.M, 400, replace=False)))

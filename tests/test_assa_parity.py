@@ -227,3 +227,22 @@ def test_lanes_with_sensors_in_the_volume():
     A = _dense(w) * 1e6
     A.reshape(12, 24, 24)[:4, :8, :8] = 0.0
     _check_forward(w, A=A)
+
+
+@pytest.mark.parametrize("nd", [1, 15, 16, 33, 63, 130])
+@pytest.mark.parametrize("n_min", [1, 25, 61])
+@pytest.mark.parametrize("sides", [(3, 2, 1), (17, 9, 10), (62, 55, 31)])
+def test_adjoint_few_tiles(sides, n_min, nd):
+    """One, two, four and eight CTAs to a brick's sensors, counts that leave the last CTA short; fine grids of alpha =
+    1, 2 and 4 whose residual is correlated residue by residue; records that end before the last windows."""
+    g = synth.centred_grid(*sides, 0.1e-3)
+    w = synth.Workload("assa-adj-few", g, synth.cap_sensors(nd, 15e-3, 150.0), 405, A=np.ones(g.M, np.float32))
+    delta = np.random.default_rng(nd).normal(size=(w.Nd, w.Nt)).astype(np.float32)
+    idx = np.sort(np.random.default_rng(7).choice(w.M, min(w.M, 1500), replace=False))
+    G = oracle_gaussians(w)
+    Gs = oracle.Gaussians(G.c[idx], G.sigma[idx], G.A[idx])
+    g_ora, amb = oracle.assa_adjoint(Gs, G.sigma[0], w.sensors, w.v, w.fs, w.t0, w.Nt, delta, n_min=n_min, tau=TAU_SNAP,
+                                     want_amb=True)
+    gg = gpu_assa_adjoint(w, delta, n_min=n_min)
+    assert np.all(np.isfinite(gg))
+    assert np.linalg.norm(gg[idx] - g_ora) <= 1e-4 * np.linalg.norm(g_ora) + np.linalg.norm(amb)
