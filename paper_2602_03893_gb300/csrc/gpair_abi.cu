@@ -438,6 +438,12 @@ bool plan_forward_lanes(const GaussDev& g, const ArrDev& a, const MomentTable& T
     return true;
 }
 
+void free_plan_offsets(FwdPlan& p, const GaussDev& g, const ArrDev& a) {
+    plan_offsets(p, g, a);
+    p.off_sort = p.bytes;
+    p.bytes += align256(spatial_order_bytes(g.M));
+}
+
 constexpr int FREE_LANES_WARPS = 8;    // warps (sensor groups of 32) per CTA of the free-centre kernel
 
 // Free-centre Gaussians with the sensor-lane direct kernel: slabs of contiguous tile ranges,
@@ -467,9 +473,16 @@ bool plan_forward_free(const GaussDev& g, const ArrDev& a, FwdPlan& p) {
         p.S *= 2;
     }
     p.free_lanes = true;
-    plan_offsets(p, g, a);
-    p.off_sort = p.bytes;
-    p.bytes += align256(spatial_order_bytes(g.M));
+    free_plan_offsets(p, g, a);
+    return true;
+}
+
+// For where the memory for p is not there: p with one CTA to a slab.  False when it has that already.
+bool plan_without_parts(FwdPlan& p, const GaussDev& g, const ArrDev& a) {
+    if (!p.free_lanes || p.parts == 1) return false;
+    p.S /= p.parts;
+    p.parts = 1;
+    free_plan_offsets(p, g, a);
     return true;
 }
 
@@ -754,7 +767,9 @@ gpair_status gpair_forward(const gpair_gaussians* gi, const gpair_array* ai, flo
     FwdPlan p = plan_forward_op(g, a);
     void* scratch = nullptr;
     int* status = nullptr;
-    if ((s = get_scratch(st, p.bytes, &scratch, &status)) != GPAIR_OK) return s;
+    s = get_scratch(st, p.bytes, &scratch, &status);
+    if (s == GPAIR_ERR_NOMEM && plan_without_parts(p, g, a)) s = get_scratch(st, p.bytes, &scratch, &status);
+    if (s != GPAIR_OK) return s;
     return run_forward(g, a, y, st, scratch, status, p);
 }
 
@@ -1027,6 +1042,16 @@ FwdPlan plan_assa_forward(const GaussDev& g, const ArrDev& aa, const AssaTable& 
     return faster ? best : wide;
 }
 
+// For where the memory for p is not there: the plan of the kernel with a warp to a sensor, whose larger slabs leave fewer
+// rows (1024 sensors of 256 x 256 x 128 nodes: 175 MB, lanes 784 MB).  False when p is it already.
+bool plan_assa_fewer_rows(FwdPlan& p, const GaussDev& g, const ArrDev& aa, const AssaTable& T) {
+    if (!p.lanes) return false;
+    const FwdPlan wide = plan_forward(g, aa);
+    if (wide.bytes >= p.bytes || assa_fwd_smem(wide.LB, T) > SMEM_PER_CTA) return false;
+    p = wide;
+    return true;
+}
+
 // Scratch of the ASSA forward beyond the plan: max |A| for the fixed-point bands.
 constexpr size_t ASSA_EXTRA_BYTES = 256;
 
@@ -1067,7 +1092,10 @@ gpair_status gpair_assa_forward(const gpair_gaussians* gi, const gpair_array* ai
     FwdPlan p = plan_assa_forward(g, aa, T);
     void* scratch = nullptr;
     int* status = nullptr;
-    if ((s = get_scratch(st, p.bytes + ASSA_EXTRA_BYTES, &scratch, &status)) != GPAIR_OK) return s;
+    s = get_scratch(st, p.bytes + ASSA_EXTRA_BYTES, &scratch, &status);
+    if (s == GPAIR_ERR_NOMEM && plan_assa_fewer_rows(p, g, aa, T))
+        s = get_scratch(st, p.bytes + ASSA_EXTRA_BYTES, &scratch, &status);
+    if (s != GPAIR_OK) return s;
     return run_assa_forward(g, aa, T, p, y, scratch, status, nullptr, st);
 }
 
@@ -1286,11 +1314,19 @@ gpair_status gpair_solver_create(const gpair_gaussians* gi, const gpair_array* a
               cudaMalloc(&S->delta, N * 4) == cudaSuccess &&
               (prm->rule != GPAIR_RULE_GD_LINESEARCH || cudaMalloc(&S->Fg, N * 4) == cudaSuccess) &&
               cudaMalloc(&S->red, sizeof(double) * (2 * red_blocks() + 8)) == cudaSuccess &&
-              cudaMalloc(&S->fwd_scratch, S->plan.bytes + (assa ? ASSA_EXTRA_BYTES : 0)) == cudaSuccess &&
               (qbytes == 0 || cudaMalloc(&S->qbuf, qbytes) == cudaSuccess) &&
               (!assa || cudaMalloc(&S->dconv, assa_dconv_bytes(a, S->T)) == cudaSuccess) &&
               cudaMalloc(&S->status, sizeof(int)) == cudaSuccess &&
               cudaMalloc(&S->sd, sizeof(StepSched)) == cudaSuccess;
+    // the forward's scratch last: where it does not fit, a plan that takes less may
+    auto forward_scratch = [&] {
+        return cudaMalloc(&S->fwd_scratch, S->plan.bytes + (assa ? ASSA_EXTRA_BYTES : 0)) == cudaSuccess;
+    };
+    if (ok && !(ok = forward_scratch())) {
+        cudaGetLastError();
+        S->fwd_scratch = nullptr;
+        ok = (assa ? plan_assa_fewer_rows(S->plan, g, S->aa, S->T) : plan_without_parts(S->plan, g, a)) && forward_scratch();
+    }
     if (!ok) {
         cudaGetLastError();
         gpair_solver_destroy(S);
