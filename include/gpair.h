@@ -163,8 +163,11 @@ gpair_status gpair_adjoint_shard(const gpair_gaussians* g, const gpair_array* ar
  *     V[v] = sum_i A_i prod_a [|r_a - c_a| <= k sigma_i] exp(-(r_a - c_a)^2 / 2 sigma_i^2)
  * at voxel centres of out_grid (host pointer; its sigma field is ignored), box-truncated at
  * k sigma_i per axis with k = window_k.  vol: device [nz][ny][nx] float32, overwritten.
- * Grid-implicit Gaussians on the same lattice use three separable 1-D passes; any other set
- * uses a cell-binned gather. */
+ * Grid-implicit Gaussians on the same lattice use three separable 1-D passes (one kernel up to six taps a side).  Any
+ * other set scatters small boxes and gathers large ones by tiles of the volume, with scratch of its own kept per stream:
+ * 46 bytes a Gaussian, 0.8 GB for the largest set that has any, until gpair_release_scratch or until another call of the
+ * library finds no memory.  Calls under stream capture and calls that find no memory take none and scatter all boxes.
+ * The order of the sums differs from call to call. */
 gpair_status gpair_voxelize(const gpair_gaussians* g, const gpair_grid* out_grid, float window_k,
                             float* vol, void* stream);
 

@@ -80,7 +80,7 @@ cudaError_t launch_adam(float* z, float* m, float* v, float* x, const float* gx,
 cudaError_t launch_set_step(StepSched* sd, int t, const SchedParams& p, cudaStream_t st);
 int red_blocks();
 bool vox_is_lattice(const GaussDev& g, const gpair_grid& og);
-size_t vox_tile_bytes(const GaussDev& g, const gpair_grid& og);
+size_t vox_tile_bytes(const GaussDev& g, const gpair_grid& og, float k);
 cudaError_t launch_voxelize(const GaussDev& g, const gpair_grid& og, float k, float* vol, float* tmp, void* prep,
                             cudaStream_t st);
 }  // namespace gp
@@ -886,7 +886,7 @@ gpair_status gpair_voxelize(const gpair_gaussians* gi, const gpair_grid* og, flo
     // launches: calls of several threads on one stream follow one another in it.  The scatter needs no
     // scratch; it takes captured calls (a graph must not hold a buffer that a later call may replace),
     // and those that find no memory.
-    const size_t bytes = vox_tile_bytes(g, *og);
+    const size_t bytes = vox_tile_bytes(g, *og, window_k);
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (bytes && cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone) {
         int dev = 0;

@@ -6,7 +6,7 @@
 // The order is a stable sort of 18-bit Morton keys (64 cells per axis, finer than a tile of 256
 // Gaussians needs): equal keys keep their index order, so the result is deterministic.
 // Up to SO_ONE_MAX Gaussians one CTA does all of it, a bitonic sort of (key, index) words in shared
-// memory: ten launches less.  Larger sets go through an LSD radix sort in two passes of 9 bits:
+// memory: seven launches less.  Larger sets go through an LSD radix sort in two passes of 9 bits:
 // per-block digit counts, a scan of each digit's counts over the blocks, and a scatter whose
 // ranks inside a block follow the index order through warp-level match masks.  Then one gather
 // writes the permuted centres, widths and amplitudes.
@@ -122,9 +122,9 @@ __device__ __forceinline__ void so_gather_one(const GaussDev& g, int64_t i, int6
 }
 
 // The whole order of up to SO_ONE_MAX Gaussians: Mp words (a power of two of at least 64) of dynamic
-// shared memory.  out (may be null): the permuted arrays.
+// shared memory.  out: the permuted arrays.
 __global__ void __launch_bounds__(SO_ONE_THREADS)
-so_one_kernel(GaussDev g, int Mp, int* __restrict__ perm, float* __restrict__ out) {
+so_one_kernel(GaussDev g, int Mp, float* __restrict__ out) {
     extern __shared__ uint32_t so_word[];
     __shared__ SoBox sh[SO_ONE_THREADS / 32];
     const int M = (int)g.M, t = threadIdx.x;
@@ -143,9 +143,7 @@ so_one_kernel(GaussDev g, int Mp, int* __restrict__ perm, float* __restrict__ ou
             if (h > 32 || h == 1) __syncthreads(); else __syncwarp();
         }
     for (int i = t; i < M; i += SO_ONE_THREADS) {
-        const int j = (int)(so_word[i] & (SO_ONE_MAX - 1));
-        perm[i] = j;
-        if (out) so_gather_one(g, i, j, out);
+        so_gather_one(g, i, (int)(so_word[i] & (SO_ONE_MAX - 1)), out);
     }
 }
 
@@ -264,21 +262,27 @@ __global__ void so_gather_kernel(GaussDev g, const int* __restrict__ perm, float
     if (i < g.M) so_gather_one(g, i, perm[i], out);
 }
 
-// The order as indices of g, in scratch; out (may be null): the permuted arrays.
-static cudaError_t spatial_sort(const GaussDev& g, void* scratch, const int** perm, float* out, cudaStream_t st) {
+// gp: g with its arrays replaced by the permuted copies in scratch (spatial_order_bytes(g.M)).
+cudaError_t launch_spatial_order(const GaussDev& g, void* scratch, GaussDev& gp, cudaStream_t st) {
     const int64_t M = g.M;
     if (M > 0x7FFFFFFF) return cudaErrorNotSupported;
     const size_t a = align256_sz((size_t)M * 4);
     char* p = static_cast<char*>(scratch);
-    uint32_t* keys[2] = {reinterpret_cast<uint32_t*>(p), reinterpret_cast<uint32_t*>(p + a)};
-    int* vals[2] = {reinterpret_cast<int*>(p + 2 * a), reinterpret_cast<int*>(p + 3 * a)};
-    *perm = vals[0];
+    float* out = reinterpret_cast<float*>(p + spatial_order_bytes(M) - 5 * a);
+    gp = g;
+    gp.cx = out;
+    gp.cy = out + M;
+    gp.cz = out + 2 * M;
+    gp.sg = out + 3 * M;
+    gp.A = out + 4 * M;
     if (M <= SO_ONE_MAX) {
         int Mp = 64;
         while (Mp < M) Mp <<= 1;
-        so_one_kernel<<<1, SO_ONE_THREADS, (size_t)Mp * 4, st>>>(g, Mp, vals[0], out);
+        so_one_kernel<<<1, SO_ONE_THREADS, (size_t)Mp * 4, st>>>(g, Mp, out);
         return cudaGetLastError();
     }
+    uint32_t* keys[2] = {reinterpret_cast<uint32_t*>(p), reinterpret_cast<uint32_t*>(p + a)};
+    int* vals[2] = {reinterpret_cast<int*>(p + 2 * a), reinterpret_cast<int*>(p + 3 * a)};
     const int nb = so_blocks(M);
     const int64_t chunk = so_chunk(M);
     int* hist = reinterpret_cast<int*>(p + 4 * a);
@@ -294,29 +298,7 @@ static cudaError_t spatial_sort(const GaussDev& g, void* scratch, const int** pe
                                                      vals[in ^ 1]);
     }
     static_assert(SO_PASSES % 2 == 0, "the order ends in buffer 0");
-    if (out) so_gather_kernel<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(g, vals[0], out);
-    return cudaGetLastError();
-}
-
-// perm: the order as indices of g, in scratch (spatial_order_bytes(g.M)).
-cudaError_t launch_spatial_perm(const GaussDev& g, void* scratch, const int** perm, cudaStream_t st) {
-    return spatial_sort(g, scratch, perm, nullptr, st);
-}
-
-// gp: g with its arrays replaced by the permuted copies in scratch (spatial_order_bytes(g.M)).
-cudaError_t launch_spatial_order(const GaussDev& g, void* scratch, GaussDev& gp, cudaStream_t st) {
-    const int64_t M = g.M;
-    const int* perm = nullptr;
-    float* out = reinterpret_cast<float*>(static_cast<char*>(scratch) + spatial_order_bytes(M) -
-                                          5 * align256_sz((size_t)M * 4));
-    const cudaError_t e = spatial_sort(g, scratch, &perm, out, st);
-    if (e != cudaSuccess) return e;
-    gp = g;
-    gp.cx = out;
-    gp.cy = out + M;
-    gp.cz = out + 2 * M;
-    gp.sg = out + 3 * M;
-    gp.A = out + 4 * M;
+    so_gather_kernel<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(g, vals[0], out);
     return cudaGetLastError();
 }
 

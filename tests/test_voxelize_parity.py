@@ -171,3 +171,59 @@ def test_lattice_fused_tiles(dims, k):
     A = np.random.default_rng(4).uniform(0, 1, g.M).astype(np.float32)
     w = synth.Workload("tiles", g, synth.cap_sensors(1, 5e-3, 10.0), 16, A=A)
     assert rel_l2(_gpu_vox(w, g, k), _ora_vox(w, g, k)) < 1e-4
+
+
+def _set(M, ext, lo, hi, seed, spread=0.55):
+    rng = np.random.default_rng(seed)
+    c = (rng.uniform(-spread, spread, (M, 3)) * np.asarray(ext)).astype(np.float32)      # some lie outside
+    sig = np.exp(rng.uniform(np.log(lo), np.log(hi), M)).astype(np.float32)
+    A = rng.uniform(0.2, 1, M).astype(np.float32)
+    A[::11] = 0.0
+    return c, sig, A
+
+
+# Sides of the boxes in voxels (6 sigma / dx): all scattered by threads, on both sides of VOX_SMALL's 4, all listed; few
+# enough for a warp to each box and enough for the tiles, in one super of 1024 and in several, with whole and ragged
+# tiles; sets that go to the tiles as they are (4096 of them at most, M times the tiles up to 2^21).
+@pytest.mark.parametrize("M,dims", [(5, (257, 40, 37)), (2048, (88, 80, 77)), (4096, (64, 64, 64)), (4097, (33, 24, 41)),
+                                    (2100, (81, 81, 81)), (9000, (64, 17, 40)), (20000, (40, 64, 33))])
+@pytest.mark.parametrize("lo,hi", [(1.0, 2.5), (3.0, 5.5), (6.0, 9.0), (2.0, 26.0)])
+def test_free_gaussians_small_and_large_boxes(M, dims, lo, hi):
+    dx = 0.07e-3
+    ext = np.array(dims) * dx
+    c, sig, A = _set(M, ext, lo * dx / 6, hi * dx / 6, M)
+    gs = _lib.Gaussians(A=_cuda(A), cx=_cuda(c[:, 0]), cy=_cuda(c[:, 1]), cz=_cuda(c[:, 2]), sigma=_cuda(sig))
+    o = [float(np.float32(-e / 2)) for e in ext]
+    og = _lib.Grid(*dims, *o, dx, dx)
+    ref = oracle.voxelize(oracle.gaussians_from_soa(c[:, 0], c[:, 1], c[:, 2], sig, A), 3.0, *dims, *o, float(np.float32(dx)))
+    for _ in range(2):                       # the second call finds the first one's scratch
+        vol = torch.full(dims[::-1], float("nan"), device="cuda")
+        _lib.gpair_voxelize(gs, og, 3.0, vol)
+        got = vol.cpu().numpy()
+        # a voxel at a box's edge may count on one side only: a term below e^-4.5 of its amplitude
+        bad = np.abs(got - ref) > 1e-4 * max(1e-30, np.abs(ref).max())
+        assert bad.mean() < 1e-3 and np.linalg.norm((got - ref)[~bad]) <= 1e-4 * np.linalg.norm(ref) + 1e-30
+
+
+@pytest.mark.parametrize("M", [40, 5000])
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), 1e38])
+def test_free_gaussians_odd_values_by_either_path(M, value):
+    """A few Gaussians with a centre, width or amplitude that is not finite (or not in voxel units) among others: by
+    tiles of the set as it is and after the split, the volume of the captured call (all scattered)."""
+    dx, n = 1e-4, 40
+    c, sig, A = _set(M, [n * dx] * 3, 0.3e-4, 3e-4, 3)
+    c[3, 0], A[8], c[9, 2] = value, value, -value
+    gs = _lib.Gaussians(A=_cuda(A), cx=_cuda(c[:, 0]), cy=_cuda(c[:, 1]), cz=_cuda(c[:, 2]), sigma=_cuda(sig))
+    og = _lib.Grid(n, n, n, -n * dx / 2, -n * dx / 2, -n * dx / 2, dx, dx)
+    one, two = torch.empty((n, n, n), device="cuda"), torch.empty((n, n, n), device="cuda")
+    _lib.gpair_voxelize(gs, og, 3.0, one)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        _lib.gpair_voxelize(gs, og, 3.0, two)
+    graph.replay()
+    same = torch.isfinite(one) & torch.isfinite(two)
+    assert torch.equal(torch.isfinite(one), torch.isfinite(two))
+    assert torch.equal(torch.isnan(one), torch.isnan(two))
+    lim = M * 2.0 ** -23 * float(two[same].abs().max())
+    assert float((one - two)[same].abs().max()) <= lim
