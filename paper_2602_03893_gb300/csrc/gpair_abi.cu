@@ -893,7 +893,12 @@ gpair_status gpair_voxelize(const gpair_gaussians* gi, const gpair_grid* og, flo
         if (cudaGetDevice(&dev) != cudaSuccess) return GPAIR_ERR_CUDA;
         std::lock_guard<std::mutex> lk(g_vox_mu);
         Scratch& b = g_vox_pool[pool_key(dev, st)];
-        if (grow_scratch(b, st, bytes) == GPAIR_OK)
+        // an allocation here must not end a capture that another thread has under way
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        const gpair_status grown = grow_scratch(b, st, bytes);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (grown == GPAIR_OK)
             return cuda_status(launch_voxelize(g, *og, window_k, vol, nullptr, b.buf, st));
     }
     cudaGetLastError();

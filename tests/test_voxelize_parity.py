@@ -227,3 +227,37 @@ def test_free_gaussians_odd_values_by_either_path(M, value):
     assert torch.equal(torch.isnan(one), torch.isnan(two))
     lim = M * 2.0 ** -23 * float(two[same].abs().max())
     assert float((one - two)[same].abs().max()) <= lim
+
+
+def test_allocation_does_not_end_another_threads_capture():
+    """A first call on a stream allocates its scratch while another thread records a graph."""
+    import threading
+
+    dx, n, M = 1e-4, 64, 20000
+    c, sig, A = _set(M, [n * dx] * 3, 0.5e-4, 3e-4, 5)
+    gs = _lib.Gaussians(A=_cuda(A), cx=_cuda(c[:, 0]), cy=_cuda(c[:, 1]), cz=_cuda(c[:, 2]), sigma=_cuda(sig))
+    og = _lib.Grid(n, n, n, -n * dx / 2, -n * dx / 2, -n * dx / 2, dx, dx)
+    vol, x = torch.empty((n, n, n), device="cuda"), torch.zeros(8, device="cuda")
+    other = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    err = []
+
+    def call():
+        try:
+            _lib.gpair_voxelize(gs, og, 3.0, vol, stream=other)
+        except Exception as e:               # noqa: BLE001 -- reported below, in the test's own thread
+            err.append(e)
+
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        x += 1
+        t = threading.Thread(target=call)
+        t.start()
+        t.join()
+        x += 1
+    graph.replay()
+    torch.cuda.synchronize()
+    assert not err and float(x[0]) == 2.0
+    ref = torch.empty_like(vol)
+    _lib.gpair_voxelize(gs, og, 3.0, ref)
+    assert torch.allclose(vol, ref, rtol=M * 2.0 ** -23, atol=M * 2.0 ** -23 * float(ref.max()))
