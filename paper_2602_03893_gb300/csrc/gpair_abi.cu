@@ -121,6 +121,24 @@ gpair_status grow_scratch(Scratch& s, cudaStream_t st, size_t bytes) {
     return GPAIR_OK;
 }
 
+// The voxelisation's scratch of the current device freed, for who finds no memory; false when there is none.
+bool release_vox_scratch() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    bool any = false;
+    std::lock_guard<std::mutex> lk(g_vox_mu);       // the calls that use it have been launched
+    for (auto it = g_vox_pool.begin(); it != g_vox_pool.end();) {
+        if ((it->first >> 48) != (uint64_t)(uint32_t)dev) { ++it; continue; }
+        if (it->second.buf) {
+            cudaDeviceSynchronize();
+            cudaFree(it->second.buf);
+            any = true;
+        }
+        it = g_vox_pool.erase(it);
+    }
+    return any;
+}
+
 gpair_status get_scratch(cudaStream_t st, size_t bytes, void** out_buf, int** out_status) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return GPAIR_ERR_CUDA;
@@ -130,7 +148,8 @@ gpair_status get_scratch(cudaStream_t st, size_t bytes, void** out_buf, int** ou
         if (cudaMalloc(&s.status, sizeof(int)) != cudaSuccess) { s.status = nullptr; return GPAIR_ERR_NOMEM; }
         if (cudaMemsetAsync(s.status, 0, sizeof(int), st) != cudaSuccess) return GPAIR_ERR_CUDA;
     }
-    const gpair_status g = grow_scratch(s, st, bytes);
+    gpair_status g = grow_scratch(s, st, bytes);
+    if (g == GPAIR_ERR_NOMEM && release_vox_scratch()) g = grow_scratch(s, st, bytes);
     if (g != GPAIR_OK) return g;
     if (out_buf) *out_buf = s.buf;
     if (out_status) *out_status = s.status;
@@ -1193,21 +1212,18 @@ gpair_status gpair_wait_selftest(int polls, void* stream) {
 void gpair_release_scratch(void) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return;
-    auto release = [dev](std::mutex& mu, std::unordered_map<uint64_t, Scratch>& pool) {
-        std::lock_guard<std::mutex> lk(mu);
-        for (auto it = pool.begin(); it != pool.end();) {
-            if ((it->first >> 48) == (uint64_t)(uint32_t)dev) {
-                cudaDeviceSynchronize();
-                if (it->second.buf) cudaFree(it->second.buf);
-                if (it->second.status) cudaFree(it->second.status);
-                it = pool.erase(it);
-            } else {
-                ++it;
-            }
+    release_vox_scratch();
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    for (auto it = g_pool.begin(); it != g_pool.end();) {
+        if ((it->first >> 48) == (uint64_t)(uint32_t)dev) {
+            cudaDeviceSynchronize();
+            if (it->second.buf) cudaFree(it->second.buf);
+            if (it->second.status) cudaFree(it->second.status);
+            it = g_pool.erase(it);
+        } else {
+            ++it;
         }
-    };
-    release(g_pool_mu, g_pool);
-    release(g_vox_mu, g_vox_pool);
+    }
 }
 
 }  // extern "C"
@@ -1335,7 +1351,7 @@ gpair_status gpair_solver_create(const gpair_gaussians* gi, const gpair_array* a
     if (!ok) {
         cudaGetLastError();
         gpair_solver_destroy(S);
-        return GPAIR_ERR_NOMEM;
+        return release_vox_scratch() ? gpair_solver_create(gi, ai, prm, out) : GPAIR_ERR_NOMEM;
     }
     cudaMemset(S->z, 0, M * 4);
     cudaMemset(S->m, 0, M * 4);

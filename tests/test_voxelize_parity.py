@@ -261,3 +261,37 @@ def test_allocation_does_not_end_another_threads_capture():
     ref = torch.empty_like(vol)
     _lib.gpair_voxelize(gs, og, 3.0, ref)
     assert torch.allclose(vol, ref, rtol=M * 2.0 ** -23, atol=M * 2.0 ** -23 * float(ref.max()))
+
+
+def test_scratch_of_the_tiles_gives_way_to_other_calls():
+    """A set of eight million leaves 370 MB of scratch on its stream; with 150 MB left on the device, a call that needs
+    300 MB has it."""
+    rng = np.random.default_rng(2)
+    M, n, dx = 8_000_000, 256, 1e-4
+    u = lambda lo, hi: _cuda(rng.uniform(lo, hi, M).astype(np.float32))
+    gs = _lib.Gaussians(A=u(0.2, 1), cx=u(0, n * dx), cy=u(0, n * dx), cz=u(0, n * dx), sigma=u(2e-5, 3e-5))
+    og = _lib.Grid(n, n, n, 0.0, 0.0, 0.0, dx, dx)
+    vol = torch.empty((n, n, n), device="cuda")
+    w = synth.Workload("long", synth.centred_grid(8, 8, 4, 1e-4), synth.cap_sensors(64, 12e-3, 140.0), 1 << 20)
+    gl, arr = device_inputs(w, A=np.ones(w.M, np.float32))
+    delta = torch.randn((w.Nd, w.Nt), device="cuda")
+    want, got = torch.empty(w.M, device="cuda"), torch.empty(w.M, device="cuda")
+    _lib.gpair_assa_adjoint(gl, arr, delta, want, n_min=1)
+    _lib.gpair_release_scratch()
+    _lib.gpair_voxelize(gs, og, 3.0, vol)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    left, hog = 150 << 20, []
+    try:
+        while True:
+            free = torch.cuda.mem_get_info()[0]
+            if free <= left + (64 << 20):
+                break
+            hog.append(torch.empty(max(free - left - (32 << 20), 32 << 20) // 4 * 4, dtype=torch.uint8, device="cuda"))
+        _lib.gpair_assa_adjoint(gl, arr, delta, got, n_min=1)
+        torch.cuda.synchronize()
+    finally:
+        hog.clear()
+        _lib.gpair_release_scratch()
+        torch.cuda.empty_cache()
+    assert torch.equal(got, want)            # the same launches on the same data
