@@ -207,3 +207,18 @@ def test_order_of_many_slabs(free, n):
     _check(w, sensors_idx=idx)
     few = np.where(rng.uniform(size=g.M) < 3e-5, w.A, 0).astype(np.float32)
     _check(w, A=few, sensors_idx=idx)
+
+
+@pytest.mark.parametrize("nd", [97, 130])
+@pytest.mark.parametrize("h,window", [(0.1e-3, 16), (0.125e-3, 20), (0.15e-3, 24), (0.2e-3, 32), (0.3e-3, 48)])
+def test_lattice_rings_without_parts(h, window, nd):
+    """120 cubes and four or five groups of sensors, so that a warp has whole cubes: the correlation's rings of 16, 20, 24
+    and 32 outputs and its general form, with fewer sensors than the amplitude scan and the slab order take and with
+    more; an image with empty cubes, records cut at both ends."""
+    g = synth.centred_grid(45, 37, 29, h)
+    assert int(2 * 3.0 * g.sigma * 40e6 / 1500.0 + 1e-6) == window
+    rng = np.random.default_rng(nd)
+    A = rng.uniform(0.1, 1.0, g.M).astype(np.float32)
+    A.reshape(29, 37, 45)[8:, 16:24, :] = 0.0
+    w = synth.Workload("rings", g, synth.cap_sensors(nd, 20e-3, 150.0), 330, A=A, t0=10.2e-6)
+    _check(w, sensors_idx=np.array([0, 31, 32, 64, 90, nd - 1]))
