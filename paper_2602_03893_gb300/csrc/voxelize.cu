@@ -323,14 +323,15 @@ __global__ void vox_scatter_kernel(GaussDev g, gpair_grid og, float k, float* __
 // Bound by FMA issue and shared-memory reads, no longer by the L2's atomics: 262,144 Gaussians of 6 to 24 voxels a side
 // into 128^3 took 3992 us as a scatter (857 M atomics) and take 305.  Microseconds with a thread's scatter for every box,
 // with tiles for every box of sorted sets, and now (side of the volume, Gaussians, mean side of their boxes):
-//   128  262144  8   643  195  169        256    1000  6    57   231   24        512  100000  2     95   1924   103
-//   128  262144 18  7300  456  453        256  100000  2    21   325   30        512  100000  6    532   2063   449
-//    64    4096 12   267   29   21        256  100000  8   296   385  208        512  100000 30  53157   3047  3222
-//   128  100000  2    16  100   25        256 1000000  2    51  1057   69        512 4000000  2    579  23025   586
-//   128 1000000  6  1022  438  347        256 1000000 12  8025  1616 1230        512 4000000  8  29146  24401 27331
+//   128  262144  8   643  195  169        256    1000  6    57   231   26        512  100000  2     95   1924   101
+//   128  262144 18  7300  456  453        256  100000  2    21   325   27        512  100000  6    532   2063   478
+//    64    4096 12   267   29   21        256  100000  8   296   385  195        512  100000 30  53157   3047  3222
+//   128  100000  2    16  100   21        256 1000000  2    51  1057   59        512 4000000  2    579  23025   585
+//   128 1000000  6  1022  438  349        256 1000000 12  8025  1616 1229        512 4000000  8  29146  24401 27670
+// The sets of two-voxel boxes pay for the three launches that leave, 6 to 9 us.
 //
 // In thin sets of many (VOX_THIN: under 64 Gaussians a tile) in volumes of over VOX_THIN_TILES tiles, boxes of up to
-// VOX_SMALL_THIN voxels are scattered: 100,000 Gaussians of 6 voxels a side into 256^3 take 131 us, listed 395.
+// VOX_SMALL_THIN voxels are scattered: 100,000 Gaussians of 6 voxels a side into 256^3 take 141 us, listed 395.
 //
 // The scatter takes all of sets whose prepared entries would need more than about 0.8 GB (VOX_TILE_MAX) and where
 // Gaussians crowd the voxels (more than VOX_TILE_PER_VOXEL each): there are too few tiles then to fill the chip, and
@@ -433,32 +434,34 @@ vox_split_kernel(GaussDev g, gpair_grid og, float k, float small, float* __restr
             const float w = min((float)(X.y - X.x + 1), side), h = min((float)(Y.y - Y.x + 1), side),
                         d = min((float)(Z.y - Z.x + 1), side);
             if (w > 0.f && h > 0.f && d > 0.f) voxels = (unsigned)fminf(fmaxf(w * h * d, 1.f), 16777216.f);
-        } else {
-            vox_scatter_one(q, og, k, vol);
+            q.A = 0.f;                        // not for the scatter
         }
     }
-    __syncwarp();
     const unsigned listed = __ballot_sync(0xffffffffu, voxels > 0);
     const unsigned sum = __reduce_add_sync(0xffffffffu, voxels);
     if (lane == 0) { wn[warp] = __popc(listed); wv[warp] = sum; }
-    if (!__syncthreads_or(listed != 0)) return;
-    if (threadIdx.x == 0) {                   // one place for the block, the warps' parts of it after another
-        unsigned n = 0;
-        unsigned long long v = 0;
-        for (int w = 0; w < VC_THREADS / 32; ++w) {
-            const unsigned m = wn[w];
-            wn[w] = n;
-            n += m;
-            v += wv[w];
+    if (__syncthreads_or(listed != 0)) {
+        if (threadIdx.x == 0) {               // one place for the block, the warps' parts of it after another
+            unsigned n = 0;
+            unsigned long long v = 0;
+            for (int w = 0; w < VC_THREADS / 32; ++w) {
+                const unsigned m = wn[w];
+                wn[w] = n;
+                n += m;
+                v += wv[w];
+            }
+            base = atomicAdd(&V.n->count, n);
+            atomicAdd(&V.n->voxels, v);
         }
-        base = atomicAdd(&V.n->count, n);
-        atomicAdd(&V.n->voxels, v);
+        __syncthreads();
+        if (voxels) {
+            V.list[base + wn[warp] + __popc(listed & ((1u << lane) - 1u))] = (int)i;
+            atomicAdd(&V.n->cell[vox_cell(q, og)], 1);
+        }
     }
-    __syncthreads();
-    if (voxels) {
-        V.list[base + wn[warp] + __popc(listed & ((1u << lane) - 1u))] = (int)i;
-        atomicAdd(&V.n->cell[vox_cell(q, og)], 1);
-    }
+    // last: with anything after it, the warps' lanes would wait for one another at the ends of the loops (4,000,000 boxes of
+    // two voxels a side: 187 us, 150 like this)
+    if (q.A != 0.f) vox_scatter_one(q, og, k, vol);
 }
 
 __global__ void __launch_bounds__(VC_PLACE)
