@@ -177,7 +177,7 @@ __device__ __forceinline__ SlabInfo cube_slab(const GaussDev& g, const CubeSlabs
 // without, 430 us in that order.
 // Few sensors' forward is not worth the look through the amplitudes (13 us of 210 for 47 sensors and a million nodes).
 // Blocks of 32 nodes a thread, narrow lines sharing a warp: 2048 slabs of 512 nodes take 9 us, 20 with blocks of 512 and
-// a warp to a line.
+// a warp to a line; of 8 nodes, one batch of loads, while a wave holds them all: 256 slabs of 4096 nodes take 9 us, 20 with 32.
 constexpr int SI_THREADS = 512, SI_THREADS_MIN = 128, SI_SCAN_MIN = 128;
 constexpr int SI_CUBES = 512;            // cubes told apart; a slab of more counts as one
 __global__ void __launch_bounds__(SI_THREADS)
@@ -617,7 +617,9 @@ cudaError_t launch_forward_lanes(const GaussDev& g, const ArrDev& a, int sx, int
         SlabInfo* first = order ? reinterpret_cast<SlabInfo*>(rows) : si;
         const int64_t nodes = (int64_t)sx * sy * sz * CUBE_N;
         int threads = SI_THREADS_MIN;
-        while (threads < SI_THREADS && scan && nodes > 32 * threads) threads *= 2;
+        while (threads < SI_THREADS && scan &&
+               (nodes > 32 * threads || (nodes > 8 * threads && (int64_t)S * threads * 2 <= (int64_t)device_sms() * 2048)))
+            threads *= 2;
         slab_info_cube_kernel<<<S, threads, 0, st>>>(g, c, scan, first);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if (order) cube_slab_order_kernel<<<(S + SO_SLAB_PER - 1) / SO_SLAB_PER, SO_SLAB_THREADS, 0, st>>>(first, S, si);
