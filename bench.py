@@ -38,7 +38,8 @@ UNIT = "s/iter"
 FP32_LANES_PER_SM = 128
 SM_MAX_MHZ = 2070.0
 MUFU_LANES_PER_SM = 32          # MUFU lanes per SM (ex2 measured at ~30 lane-ops / clk / SM)
-LAUNCHES_PER_STEP = 8           # slab info, forward, slab reduce, resid, finish, Q table, adjoint, adam
+# slab info, slab order, forward, slab reduce, resid, finish, Q table, adjoint, adam (the first two not in the tiny one)
+LAUNCHES_PER_STEP = 9
 ASSA_NMIN = 25                  # the paper's minimum number of fine samples across the pulse
 
 
@@ -545,7 +546,7 @@ def main():
         vbytes = 4.0 * (1 + 2) * w.M
         vcr = {"ms": vms, "alg_bytes": vbytes, "achieved_GBs": vbytes / (vms / 1e3) / 1e9,
                "peak_GBs": HBM_GBS, "frac": vbytes / (vms / 1e3) / 1e9 / HBM_GBS,
-               "includes": "vcr_march_kernel (fields in shared memory + transposed-stencil gradient + FP64 "
+               "includes": "vcr_march_kernel (fields in registers + transposed-stencil gradient + FP64 "
                            "block partials); no host sync"}
 
     # ---- voxelization of the image (Eq. 2 sampled on the lattice: three separable gather passes) and

@@ -259,7 +259,7 @@ void gpair_release_scratch(void);
  * (p != q) the four-point central mixed difference / 4 (counted for (p,q) and (q,p)), with Neumann
  * boundaries (neighbour indices clamped) and unit voxel spacing.  value_out (host, may be NULL):
  * R_VCR in FP64 (the call then synchronises `stream`); grad (device [M], may be NULL):
- * grad += lam * dR_VCR/dx.  One fused pass: the difference fields stay in shared memory, so only x
+ * grad += lam * dR_VCR/dx.  One fused pass: the difference fields stay on the chip, so only x
  * and grad cross device memory; scratch is a few KB of FP64 block partials from the library's
  * per-stream pool.  Errors:
  * GPAIR_ERR_INVALID_ARG for a NULL x, non-positive sizes or eps < 0; GPAIR_ERR_UNSUPPORTED when

@@ -305,7 +305,7 @@ adj_q_kernel(const float* __restrict__ delta, int Nt, const __grid_constant__ Mo
 //
 // Bound by instruction issue and by the gathers' L1 wavefronts.  With one Gaussian to a thread and scalar
 // arithmetic it took 57 instructions a pair: 14.96 ms for 256 x 256 x 128 Gaussians and 1024 sensors,
-// 9.7 ms now.
+// 9.5 ms now.
 //
 // A brick's sensors are divided over the CTAs of a cluster where there are too few bricks to fill the
 // chip; their sums meet in the first CTA's shared memory, in the order of the ranks.

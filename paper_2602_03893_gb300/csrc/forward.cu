@@ -1046,7 +1046,7 @@ slab_reduce_banded_kernel(const float* __restrict__ partial, const int2* __restr
 // each 32 of them, a run of the slabs each, added in their order.
 //
 // Bound by the latency of the rows' loads.  512 slabs, 1024 sensors: 256 us with all rows sorted and runs for 256
-// samples, 195 us; 1300 slabs, 47 sensors: 257 us before, 182 us with a warp to 32
+// samples, 165 us; 1300 slabs, 47 sensors: 257 us before, 182 us with a warp to 32
 // samples, 104 us with four.
 constexpr int SRS_THREADS = 256;
 constexpr int SRS_MAX_S = 2048;             // sorted keys and descriptors: 32 KB

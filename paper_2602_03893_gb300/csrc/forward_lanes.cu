@@ -177,7 +177,8 @@ __device__ __forceinline__ SlabInfo cube_slab(const GaussDev& g, const CubeSlabs
 // without, 430 us in that order.
 // Few sensors' forward is not worth the look through the amplitudes (13 us of 210 for 47 sensors and a million nodes).
 // Blocks of 32 nodes a thread, narrow lines sharing a warp: 2048 slabs of 512 nodes take 9 us, 20 with blocks of 512 and
-// a warp to a line; of 8 nodes, one batch of loads, while a wave holds them all: 256 slabs of 4096 nodes take 9 us, 20 with 32.
+// a warp to a line; of 8 nodes, one batch of loads, while a wave holds them all: 256 slabs of 4096 nodes take 9 us, 20
+// with 32.
 constexpr int SI_THREADS = 512, SI_THREADS_MIN = 128, SI_SCAN_MIN = 128;
 constexpr int SI_CUBES = 512;            // cubes told apart; a slab of more counts as one
 __global__ void __launch_bounds__(SI_THREADS)

@@ -4,8 +4,8 @@
 // uniform window of `win` samples per axis, sample (N / (N - 1)) variances and covariance,
 // C1 = (0.01 R)^2, C2 = (0.03 R)^2 for the data range R, averaged over the positions whose window
 // lies inside the image.  The local sums are separable box filters (x, then y, then z) of five
-// fields (x, y, x^2, y^2, x y): fused in shared memory for windows up to 15 (ssim_march_kernel,
-// which also sums the squared differences), else one coalesced pass per axis through device memory.
+// fields (x, y, x^2, y^2, x y): fused for windows up to 9 (ssim_zfirst_kernel) and up to 15
+// (ssim_march_kernel), which also sum the squared differences, else one coalesced pass per axis through device memory.
 #include "gpair_internal.cuh"
 
 namespace gp {
